@@ -119,8 +119,8 @@ SENTRY_API int sentry_gate_select(sentry_ctx* ctx, const float* scores, int S, i
  * the channels of a layer, or the units of several layers): every member of
  * `sets` (host array, 1 <= n_sets <= SENTRY_GATE_MAX_SETS) has the meaning of
  * the like-named sentry_gate_select arguments, and the result of each set is
- * what sentry_gate_select would write for it.  A set with n_masks * k > 16384
- * needs one more launch for its fan-out.  Workspace: the sum over the sets of
+ * what sentry_gate_select would write for it.  With a row of more than 8192
+ * units the sets run one after the other, two launches each.  Workspace: the sum over the sets of
  * S*k*4 + S*4 bytes, each rounded up to 256. */
 #define SENTRY_GATE_MAX_SETS 4
 typedef struct sentry_gate_set {

@@ -1,33 +1,207 @@
 // SentryGate selection (Section 4.6): per modality-mask row of the score
 // table, keep the k best-scoring units; then fan the per-row result out to the
 // per-sample masks.  Selection is exact and deterministic: scores are mapped to
-// order-preserving integer keys, the k-th key is found by a bitwise threshold
-// search with warp-ballot counting, and the kept indices are compacted in
-// ascending order (equal scores: lower index first).
+// order-preserving integer keys, the k-th key is found by counting against
+// candidate thresholds, and the kept indices are compacted in ascending order
+// (equal scores: lower index first).
 #include "common.cuh"
 
 namespace {
 
-constexpr int kGateMaxThreads = 1024;
+// ------------------------------------------------------------------------------------------
+// Rows of up to kGateMaxRegUnits units: a thread holds KPT consecutive keys in registers, and one launch does the
+// selection and the fan-out to the samples.
+//
+// Bound by latency: a row is a few KB, and what takes the time is the chain of block-wide steps.  A counting step costs
+// about 270 cycles at 256 threads (warp votes, a barrier, a 56-cycle warp reduction), so a step settles TWO bits of the
+// k-th key (three candidate thresholds at once), the search starts at the first bit in which the keys differ and ends as
+// soon as exactly k keys lie above a candidate: 6 to 8 steps.  Few threads with several keys each, because the barrier
+// of 1024 threads costs 87 cycles and that of 256 costs 39.
+// grid (S * sets, y): the y blocks of a row each make the row's selection and serve their share of the samples -- one
+// launch whatever the fan-out, where a second launch for large fan-outs cost more than the repeated selection.
+struct GateSetDev {
+    const float* scores;
+    int n_units, k;
+    int heads_per_group;
+    const uint32_t* masks;
+    int n_masks;
+    int32_t* kept;
+    uint32_t* kv_groups;
+};
+struct GateSetsDev { GateSetDev set[SENTRY_GATE_MAX_SETS]; };
 
-// Block size of the per-row selection: one key per thread up to 1024 threads.
-inline int gate_threads(int n_units) {
-    int t = (n_units + 31) / 32 * 32;
-    return t < 64 ? 64 : (t > kGateMaxThreads ? kGateMaxThreads : t);
+constexpr int kGateMaxRegUnits = 8192;
+
+template <int KPT>
+__global__ void __launch_bounds__(1024)
+gate_select_kernel(const __grid_constant__ GateSetsDev sets, int S, unsigned int* status) {
+    extern __shared__ int32_t s_list[];            // [k] kept units, ascending
+    __shared__ uint32_t s_red[2][3][32];           // per-warp partial results of a counting step, two steps in turn
+    __shared__ uint32_t s_bits;
+    const GateSetDev& g = sets.set[blockIdx.x / S];
+    const int s = (int)(blockIdx.x % S), n = g.n_units, k = g.k;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const float* row = g.scores + (size_t)s * n;
+    const int i0 = threadIdx.x * KPT;
+    uint32_t key[KPT];
+    uint32_t hi = 0u, lo = 0xffffffffu;
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+        // padding ranks with NaN, below every number; it is kept out of the list by its index
+        key[j] = i0 + j < n ? sentry_order_key(__ldg(row + i0 + j)) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < KPT; ++j)
+        if (i0 + j < n) { hi = max(hi, key[j]); lo = min(lo, key[j]); }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    if (lane == 0) { s_red[0][0][warp] = hi; s_red[0][1][warp] = lo; }
+    if (threadIdx.x == 0) s_bits = 0u;
+    __syncthreads();
+    hi = __reduce_max_sync(0xffffffffu, lane < nw ? s_red[0][0][lane] : 0u);
+    lo = __reduce_min_sync(0xffffffffu, lane < nw ? s_red[0][1][lane] : 0xffffffffu);
+
+    uint32_t t = lo;
+    bool cut = k == n;                             // exactly k units have keys >= t
+    int above = 0;                                 // units with keys >= the next candidate above t's range
+    if (!cut && hi != lo) {
+        int b = (31 - __clz((int)(hi ^ lo))) | 1;  // digits of two bits, aligned
+        t = b == 31 ? 0u : hi & ~((2u << b) - 1u);
+        int buf = 1;
+#pragma unroll 1
+        for (b -= 1; b >= 0 && !cut; b -= 2, buf ^= 1) {
+            const uint32_t c1 = t + (1u << b), c2 = t + (2u << b), c3 = t + (3u << b);
+            uint32_t n1 = 0u, n2 = 0u, n3 = 0u;
+#pragma unroll
+            for (int j = 0; j < KPT; ++j) {
+                n1 += __popc(__ballot_sync(0xffffffffu, key[j] >= c1));
+                n2 += __popc(__ballot_sync(0xffffffffu, key[j] >= c2));
+                n3 += __popc(__ballot_sync(0xffffffffu, key[j] >= c3));
+            }
+            if (lane == 0) { s_red[buf][0][warp] = n1; s_red[buf][1][warp] = n2; s_red[buf][2][warp] = n3; }
+            __syncthreads();                       // (the other buffer's readers are past the barrier before)
+            const int k1 = (int)__reduce_add_sync(0xffffffffu, lane < nw ? s_red[buf][0][lane] : 0u);
+            const int k2 = (int)__reduce_add_sync(0xffffffffu, lane < nw ? s_red[buf][1][lane] : 0u);
+            const int k3 = (int)__reduce_add_sync(0xffffffffu, lane < nw ? s_red[buf][2][lane] : 0u);
+            if (k3 >= k) { t = c3; cut = k3 == k; }
+            else if (k2 >= k) { t = c2; cut = k2 == k; above = k3; }
+            else if (k1 >= k) { t = c1; cut = k1 == k; above = k2; }
+            else above = k1;
+        }
+        __syncthreads();
+    } else {
+        __syncthreads();
+    }
+    // ordered compaction.  cut: everything >= t (t may be 0 only with k == n).  Otherwise t is the k-th key itself: all
+    // keys above it (`above` of them) and, in index order, as many of the equal ones as are wanted
+    const int need_eq = cut ? 0x7fffffff : k - above;
+    uint32_t mine = 0u;                            // keys above t: low half, equal to t: high half
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+        const bool in = i0 + j < n;
+        mine += (in && key[j] > t ? 1u : 0u) + (in && key[j] == t ? 65536u : 0u);
+    }
+    uint32_t incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) s_red[0][2][warp] = incl;
+    __syncthreads();
+    const uint32_t warps_before = __reduce_add_sync(0xffffffffu, lane < warp ? s_red[0][2][lane] : 0u);
+    const uint32_t before = warps_before + incl - mine;
+    int gt_n = (int)(before & 0xffffu), eq_n = (int)(before >> 16);
+    uint32_t bits = 0u;
+#pragma unroll
+    for (int j = 0; j < KPT; ++j) {
+        const bool in = i0 + j < n, gt = in && key[j] > t, eq = in && key[j] == t;
+        if (gt || (eq && eq_n < need_eq)) {
+            s_list[gt_n + min(eq_n, need_eq)] = i0 + j;
+            if (g.kv_groups != nullptr) bits |= 1u << ((i0 + j) / g.heads_per_group);
+        }
+        gt_n += gt;
+        eq_n += eq;
+    }
+    if (g.kv_groups != nullptr && bits) atomicOr(&s_bits, bits);
+    __syncthreads();
+
+    // fan-out over this block's share of the samples
+    const int per = (g.n_masks + (int)gridDim.y - 1) / (int)gridDim.y;
+    const int m_end = min(g.n_masks, ((int)blockIdx.y + 1) * per);
+    if (k <= 16) {                                 // short lists (heads): a thread per sample
+        for (int m = (int)blockIdx.y * per + threadIdx.x; m < m_end; m += blockDim.x) {
+            const uint32_t ms = g.masks[m];
+            if (ms == (uint32_t)s) {
+                for (int j = 0; j < k; ++j) g.kept[(size_t)m * k + j] = s_list[j];
+                if (g.kv_groups != nullptr) g.kv_groups[m] = s_bits;
+            } else if (s == 0 && ms >= (uint32_t)S) {
+                atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+            }
+        }
+        return;
+    }
+    for (int m0 = (int)blockIdx.y * per; m0 < m_end; m0 += 32) {   // longer ones: the block copies the list to each match
+        const uint32_t ms = m0 + lane < m_end ? g.masks[m0 + lane] : 0xfffffffeu;
+        if (s == 0 && warp == 0 && m0 + lane < m_end && ms >= (uint32_t)S) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+        unsigned hits = __ballot_sync(0xffffffffu, m0 + lane < m_end && ms == (uint32_t)s);
+        while (hits) {
+            const int m = m0 + __ffs(hits) - 1;
+            hits &= hits - 1;
+            for (int j = threadIdx.x; j < k; j += blockDim.x) g.kept[(size_t)m * k + j] = s_list[j];
+            if (g.kv_groups != nullptr && threadIdx.x == 0) g.kv_groups[m] = s_bits;
+        }
+    }
 }
 
-// One block per score-table row s: rows[s, 0..k) and groups[s].  With fan_masks given (a small
-// fan-out), the block also copies its row to every sample whose mask selects it, which saves
-// the second launch: kept[m, :] = rows[s, :] for masks[m] == s.
-__device__ __forceinline__ void
-gate_row_block(int s, const float* __restrict__ scores, int n_units, int k,
-               int32_t* __restrict__ rows, uint32_t* __restrict__ groups,
-               int heads_per_group, const uint32_t* __restrict__ fan_masks,
-               int n_masks, int S, int32_t* __restrict__ kept,
-               uint32_t* __restrict__ kv_groups, unsigned int* status) {
+// Launch of the register form: keys per thread and threads from the longest row, blocks per row from the fan-out.
+int launch_gate_reg(int S, const sentry_gate_set* sets, int n_sets, unsigned int* status, int sm_count,
+                    cudaStream_t st) {
+    GateSetsDev dev = {};
+    int n_max = 1, k_max = 1, m_max = 1;
+    long long out_max = 1;
+    for (int i = 0; i < n_sets; ++i) {
+        const sentry_gate_set& g = sets[i];
+        dev.set[i] = {g.scores, g.n_units, g.k, g.heads_per_group > 0 ? g.heads_per_group : 1, g.masks, g.n_masks, g.kept, g.kv_groups};
+        if (g.n_units > n_max) n_max = g.n_units;
+        if (g.k > k_max) k_max = g.k;
+        if (g.n_masks > m_max) m_max = g.n_masks;
+        if ((long long)g.n_masks * g.k > out_max) out_max = (long long)g.n_masks * g.k;
+    }
+    // a share of 4096 list entries and 512 samples per block, as long as the blocks of all rows together about fill the GPU once
+    long long y = (out_max / S + 4095) / 4096;
+    if (y < (m_max + 511) / 512) y = (m_max + 511) / 512;
+    const long long most = (sm_count + S * n_sets - 1) / (S * n_sets);
+    if (y > most) y = most;
+    if (y < 1) y = 1;
+    const dim3 grid((unsigned)(S * n_sets), (unsigned)y);
+    const size_t smem = (size_t)k_max * sizeof(int32_t);
+    auto threads_for = [&](int kpt) { return ((n_max + kpt - 1) / kpt + 31) / 32 * 32; };
+    if (n_max <= 256) {
+        const int th = n_max <= 64 ? (out_max >= 1024 ? 256 : 64) : threads_for(1);
+        gate_select_kernel<1><<<grid, th, smem, st>>>(dev, S, status);
+    } else if (n_max <= 1024) {
+        gate_select_kernel<4><<<grid, threads_for(4), smem, st>>>(dev, S, status);
+    } else {
+        gate_select_kernel<8><<<grid, threads_for(8), smem, st>>>(dev, S, status);
+    }
+    SENTRY_CUDA_TRY(cudaGetLastError());
+    return SENTRY_OK;
+}
+
+
+constexpr int kGateMaxThreads = 1024;
+
+// ------------------------------------------------------------------------------------------
+// Longer rows: keys in shared memory, the rows to scratch, a second launch fans them out.
+// One block per score-table row s: rows[s, 0..k) and groups[s].
+__global__ void __launch_bounds__(kGateMaxThreads)
+gate_rows_kernel(const float* __restrict__ scores, int n_units, int k, int32_t* __restrict__ rows,
+                 uint32_t* __restrict__ groups, int heads_per_group) {
     extern __shared__ uint32_t s_keys[];
     __shared__ int red[66];
     __shared__ uint32_t s_bits;
+    const int s = blockIdx.x;
     const float* row = scores + (size_t)s * n_units;
     for (int i = threadIdx.x; i < n_units; i += blockDim.x) s_keys[i] = sentry_order_key(row[i]);
     if (threadIdx.x == 0) s_bits = 0u;
@@ -43,66 +217,6 @@ gate_row_block(int s, const float* __restrict__ scores, int n_units, int k,
         __syncthreads();
         if (threadIdx.x == 0) groups[s] = s_bits;
     }
-    if (fan_masks == nullptr) return;
-    __syncthreads();   // out[] (global, written by this block) is complete
-    if (k <= 32) {
-        // short lists (heads): one thread per mask -- one independent load of the mask per
-        // thread instead of a chain of dependent loads down an element loop
-        for (int m = threadIdx.x; m < n_masks; m += blockDim.x) {
-            const uint32_t ms = fan_masks[m];
-            if (ms == (uint32_t)s) {
-                int32_t* dst = kept + (size_t)m * k;
-                for (int j = 0; j < k; ++j) dst[j] = out[j];
-                if (kv_groups != nullptr) kv_groups[m] = s_bits;
-            } else if (s == 0 && ms >= (uint32_t)S) {
-                atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
-            }
-        }
-        return;
-    }
-    const long long total = (long long)n_masks * k;
-    for (long long i = threadIdx.x; i < total; i += blockDim.x) {
-        const int m = (int)(i / k), j = (int)(i % k);
-        const uint32_t ms = fan_masks[m];
-        if (ms == (uint32_t)s) {
-            kept[i] = out[j];
-            if (j == 0 && kv_groups != nullptr) kv_groups[m] = s_bits;
-        } else if (s == 0 && j == 0 && ms >= (uint32_t)S) {
-            atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kGateMaxThreads)
-gate_rows_kernel(const float* __restrict__ scores, int n_units, int k,
-                 int32_t* __restrict__ rows, uint32_t* __restrict__ groups,
-                 int heads_per_group, const uint32_t* __restrict__ fan_masks = nullptr,
-                 int n_masks = 0, int S = 0, int32_t* __restrict__ kept = nullptr,
-                 uint32_t* __restrict__ kv_groups = nullptr, unsigned int* status = nullptr) {
-    gate_row_block(blockIdx.x, scores, n_units, k, rows, groups, heads_per_group, fan_masks, n_masks, S, kept,
-                   kv_groups, status);
-}
-
-// Several selections over the same S mask values (heads and channels of a layer, or several
-// layers) in one launch: block b works on row b % S of set b / S.
-struct GateSetDev {
-    const float* scores;
-    int n_units, k;
-    int32_t* rows;
-    uint32_t* groups;
-    int heads_per_group;
-    const uint32_t* fan_masks;   // null: no fan-out in this launch (the set is expanded afterwards)
-    int n_masks;
-    int32_t* kept;
-    uint32_t* kv_groups;
-};
-struct GateSetsDev { GateSetDev set[SENTRY_GATE_MAX_SETS]; };
-
-__global__ void __launch_bounds__(kGateMaxThreads)
-gate_rows_multi_kernel(const __grid_constant__ GateSetsDev sets, int S, unsigned int* status) {
-    const GateSetDev& g = sets.set[blockIdx.x / S];
-    gate_row_block((int)(blockIdx.x % S), g.scores, g.n_units, g.k, g.rows, g.groups, g.heads_per_group,
-                   g.fan_masks, g.n_masks, S, g.kept, g.kv_groups, status);
 }
 
 // kept[m, :] = rows[masks[m], :]  (and kv_groups[m] = groups[masks[m]]).
@@ -131,28 +245,20 @@ int launch_gate_select(sentry_ctx* ctx, const float* scores, int S, int n_units,
                        const uint32_t* masks, int n_masks, int k, int32_t* kept,
                        uint32_t* kv_groups, int heads_per_group, int32_t* ws_rows,
                        uint32_t* ws_groups, cudaStream_t st) {
+    if (n_units <= kGateMaxRegUnits) {
+        const sentry_gate_set g = {scores, n_units, k, masks, n_masks, kept, kv_groups, heads_per_group};
+        LaunchScope ls(ctx, KS_GATE_ROWS, st);
+        return launch_gate_reg(S, &g, 1, ctx->d_status, ctx->sm_count, st);
+    }
     const size_t smem = (size_t)n_units * sizeof(uint32_t);
     if (smem > 48 * 1024)
         SENTRY_CUDA_TRY(cudaFuncSetAttribute(gate_rows_kernel,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const size_t total = (size_t)n_masks * k;
-    if (total <= 16384) {   // small fan-out: one launch does both steps
-        // enough threads for the fan-out as well as for the selection
-        int threads = gate_threads(n_units);
-        const int fan = k <= 32 ? n_masks : (int)(total < 1024 ? total : 1024);
-        while (threads < 256 && threads < fan) threads *= 2;
-        LaunchScope ls(ctx, KS_GATE_ROWS, st);
-        gate_rows_kernel<<<S, threads, smem, st>>>(
-            scores, n_units, k, ws_rows, kv_groups ? ws_groups : nullptr,
-            heads_per_group > 0 ? heads_per_group : 1, masks, n_masks, S, kept, kv_groups, ctx->d_status);
-        SENTRY_CUDA_TRY(cudaGetLastError());
-        return SENTRY_OK;
-    }
     {
         LaunchScope ls(ctx, KS_GATE_ROWS, st);
-        gate_rows_kernel<<<S, gate_threads(n_units), smem, st>>>(scores, n_units, k, ws_rows,
-                                                         kv_groups ? ws_groups : nullptr,
-                                                         heads_per_group > 0 ? heads_per_group : 1);
+        gate_rows_kernel<<<S, kGateMaxThreads, smem, st>>>(scores, n_units, k, ws_rows, kv_groups ? ws_groups : nullptr,
+                                                           heads_per_group > 0 ? heads_per_group : 1);
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
     int blocks = (int)((total + 255) / 256);
@@ -168,51 +274,21 @@ int launch_gate_select(sentry_ctx* ctx, const float* scores, int S, int n_units,
     return SENTRY_OK;
 }
 
-// All sets in one launch; a set whose fan-out is large gets its rows there and one expand launch.
+// All sets in one launch; with a row too long for the register form, set after set.
 int launch_gate_select_multi(sentry_ctx* ctx, int S, const sentry_gate_set* sets, int n_sets, int32_t* const* ws_rows,
                              uint32_t* const* ws_groups, cudaStream_t st) {
-    GateSetsDev dev = {};
-    size_t smem = 0;
-    int threads = 64;
-    bool expand[SENTRY_GATE_MAX_SETS] = {};
-    for (int i = 0; i < n_sets; ++i) {
-        const sentry_gate_set& g = sets[i];
-        const size_t total = (size_t)g.n_masks * g.k;
-        expand[i] = total > 16384;
-        GateSetDev& d = dev.set[i];
-        d.scores = g.scores; d.n_units = g.n_units; d.k = g.k;
-        d.rows = ws_rows[i];
-        d.groups = g.kv_groups ? ws_groups[i] : nullptr;
-        d.heads_per_group = g.heads_per_group > 0 ? g.heads_per_group : 1;
-        d.fan_masks = expand[i] ? nullptr : g.masks;
-        d.n_masks = g.n_masks; d.kept = g.kept; d.kv_groups = g.kv_groups;
-        if ((size_t)g.n_units * sizeof(uint32_t) > smem) smem = (size_t)g.n_units * sizeof(uint32_t);
-        int t = gate_threads(g.n_units);
-        if (!expand[i]) {
-            const int fan = g.k <= 32 ? g.n_masks : (int)(total < 1024 ? total : 1024);
-            while (t < 256 && t < fan) t *= 2;
-        }
-        if (t > threads) threads = t;
-    }
-    if (smem > 48 * 1024)
-        SENTRY_CUDA_TRY(cudaFuncSetAttribute(gate_rows_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem));
-    {
+    bool all_short = true;
+    for (int i = 0; i < n_sets; ++i) all_short = all_short && sets[i].n_units <= kGateMaxRegUnits;
+    if (all_short) {
         LaunchScope ls(ctx, KS_GATE_ROWS, st);
-        gate_rows_multi_kernel<<<S * n_sets, threads, smem, st>>>(dev, S, ctx->d_status);
+        return launch_gate_reg(S, sets, n_sets, ctx->d_status, ctx->sm_count, st);
     }
-    SENTRY_CUDA_TRY(cudaGetLastError());
     for (int i = 0; i < n_sets; ++i) {
-        if (!expand[i]) continue;
         const sentry_gate_set& g = sets[i];
-        const size_t total = (size_t)g.n_masks * g.k;
-        int blocks = (int)((total + 255) / 256);
-        const int cap = ctx->sm_count * 8;
-        if (blocks > cap) blocks = cap;
-        LaunchScope ls(ctx, KS_GATE_EXPAND, st);
-        gate_expand_kernel<<<blocks, 256, 0, st>>>(ws_rows[i], ws_groups[i], g.masks, S, g.n_masks, g.k, g.kept,
-                                                   g.kv_groups, ctx->d_status);
-        SENTRY_CUDA_TRY(cudaGetLastError());
+        if (g.n_masks == 0) continue;
+        const int rc = launch_gate_select(ctx, g.scores, S, g.n_units, g.masks, g.n_masks, g.k, g.kept, g.kv_groups,
+                                          g.heads_per_group, ws_rows[i], ws_groups[i], st);
+        if (rc != SENTRY_OK) return rc;
     }
     return SENTRY_OK;
 }
@@ -300,10 +376,14 @@ extern "C" int sentry_gate_select_static(int device, const float* scores, int S,
     unsigned int* own_status = reinterpret_cast<unsigned int*>(sd.scratch);
     int32_t* rows = reinterpret_cast<int32_t*>(sd.scratch + kStaticHeader);
     uint32_t* groups = reinterpret_cast<uint32_t*>(sd.scratch + kStaticHeader + rows_bytes);
+    if (n_units <= kGateMaxRegUnits) {   // no scratch wanted
+        const sentry_gate_set g = {scores, n_units, k, masks, n_masks, kept, kv_groups, heads_per_group};
+        return launch_gate_reg(S, &g, 1, status != nullptr ? status : own_status, sd.sm_count, st);
+    }
     // The array keeps whatever the previous call left.  rows/groups are rewritten in full for
     // all S score rows before the fan-out reads them; only the status word must start at zero.
     SENTRY_CUDA_TRY(cudaMemsetAsync(own_status, 0, sizeof(unsigned int), st));
-    gate_rows_kernel<<<S, gate_threads(n_units), (size_t)n_units * sizeof(uint32_t), st>>>(
+    gate_rows_kernel<<<S, kGateMaxThreads, (size_t)n_units * sizeof(uint32_t), st>>>(
         scores, n_units, k, rows, kv_groups ? groups : nullptr, heads_per_group > 0 ? heads_per_group : 1);
     SENTRY_CUDA_TRY(cudaGetLastError());
     const size_t total = (size_t)n_masks * k;
