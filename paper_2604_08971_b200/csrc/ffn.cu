@@ -21,16 +21,161 @@ constexpr int kGenericThreads = 256;
 constexpr int kTcTileRows = 128;
 
 // One launch prepares everything the main kernel needs.  Block ranges:
-//   [0, B)              row table of sample b: every block finds by itself where its sample's
-//                       rows start (a scan over all samples' lists and present-row counts, so no
-//                       separate planning launch is needed); block 0 also writes the per-list
-//                       offsets and tile counts
-//   [B, B + B*zsplit)   zero rows of Y for the absent tokens of a sample (slices of its rows)
+//   [0, P)              row tables of G samples each (P = ceil(B / G)): every block finds by itself where its samples'
+//                       rows start (a scan over all samples' lists and present-row counts, so no separate planning
+//                       launch is needed); block 0 also writes the per-list offsets and tile counts.  G = 1 for small
+//                       batches, whose blocks are then all in flight at once; from kGroupPlanB samples on the scan is
+//                       what a block does, and eight samples share it
+//   [P, P + B*zsplit)   plain-ALU kernel only: zero rows of Y for the absent tokens of a sample (slices of its rows;
+//                       the tensor-core kernel writes them itself, beside its arithmetic)
 //   [.., + prepack)     the weight gather, which "materialises" the pruned W1', W2' per list:
 //     layout 0 (plain-ALU kernel): W1g [l][D][kc_pad], W2g [l][kc_pad][D]
 //     layout 1 (tensor-core kernel, both K-major): W1c [l][kc_pad][D], W2c [l][D][kc_pad]
 //     columns / rows n >= k_c are zero.
-template <typename T>
+constexpr int kGroupPlanB = 1024;
+constexpr int kPlanListsSmem = 1024;   // lists whose row counts block 0 keeps in shared memory
+
+template <int G>
+__device__ __forceinline__ void plan_block(const int32_t* __restrict__ ids, const uint32_t* __restrict__ masks,
+                                           const int32_t* __restrict__ list_of_sample, int B, int Tlen, int tile_rows,
+                                           const FfnPlan& p, int n_lists, unsigned int* status) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __shared__ int s_cnt[32];
+    __shared__ int red[66];
+    __shared__ int s_before[G][8];
+    __shared__ int s_rows[kPlanListsSmem];
+    const int b0 = blockIdx.x * G;
+    const bool first_block = blockIdx.x == 0;
+    if (threadIdx.x < 32) s_cnt[threadIdx.x] = 0;
+    if (first_block)
+        for (int l = threadIdx.x; l < min(n_lists, kPlanListsSmem); l += blockDim.x) s_rows[l] = 0;
+    __syncthreads();
+    if (ids != nullptr) {
+        for (int t0 = 0; t0 < Tlen; t0 += blockDim.x) {
+            const int t = t0 + threadIdx.x;
+            const int m = t < Tlen ? ids[t] : -1;
+            if (t < Tlen && (m < 0 || m >= 32) && first_block) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+            // tokens of a modality lie together: one shared-memory atomic per warp and modality
+            const unsigned peers = __match_any_sync(0xffffffffu, m);
+            if (m >= 0 && m < 32 && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[m], __popc(peers));
+        }
+        __syncthreads();
+    }
+    auto present_rows = [&](int bb) {
+        if (ids == nullptr) return Tlen;
+        uint32_t mask = masks[bb];
+        int n = 0;
+        while (mask) { const int m = __ffs(mask) - 1; n += s_cnt[m]; mask &= mask - 1; }
+        return n;
+    };
+    auto list_of = [&](int bb) {
+        int l = list_of_sample ? list_of_sample[bb] : 0;
+        if (l < 0 || l >= n_lists) {
+            if (first_block) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+            l = 0;
+        }
+        return l;
+    };
+    // rows of all samples in earlier lists, and of earlier samples in the sample's list
+    int my_list[G], before[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) { my_list[g] = b0 + g < B ? list_of(b0 + g) : -1; before[g] = 0; }
+    for (int bb = threadIdx.x; bb < B; bb += blockDim.x) {
+        const int l = list_of(bb), r = present_rows(bb);
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            if (l < my_list[g] || (l == my_list[g] && bb < b0 + g)) before[g] += r;
+        if (first_block) {
+            if (r == 0) atomicOr(status, SENTRY_STATUS_BIT_EMPTY_MASK);
+            if (n_lists <= kPlanListsSmem) atomicAdd(&s_rows[l], r);
+        }
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        before[g] = __reduce_add_sync(0xffffffffu, before[g]);
+        if (lane == 0) s_before[g][wid] = before[g];
+    }
+    __syncthreads();
+    if (first_block) {
+        // per-list totals -> list offsets and tile counts
+        if (n_lists <= kPlanListsSmem) {
+            if (wid == 0) {
+                int row0 = 0, tile0 = 0;
+                for (int l0 = 0; l0 < n_lists; l0 += 32) {
+                    const int l = l0 + lane;
+                    const int r = l < n_lists ? s_rows[l] : 0, c = (r + tile_rows - 1) / tile_rows;
+                    int ir = r, ic = c;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int vr = __shfl_up_sync(0xffffffffu, ir, o), vc = __shfl_up_sync(0xffffffffu, ic, o);
+                        if (lane >= o) { ir += vr; ic += vc; }
+                    }
+                    if (l < n_lists) { p.list_row0[l] = row0 + ir - r; p.tile_start[l] = tile0 + ic - c; }
+                    row0 += __shfl_sync(0xffffffffu, ir, 31);
+                    tile0 += __shfl_sync(0xffffffffu, ic, 31);
+                }
+                if (lane == 0) { p.list_row0[n_lists] = row0; p.tile_start[n_lists] = tile0; }
+            }
+        } else {   // very many lists: a pass over the samples for each
+            int row0 = 0, tile0 = 0;
+            for (int l = 0; l < n_lists; ++l) {
+                int rows = 0;
+                for (int bb = threadIdx.x; bb < B; bb += blockDim.x)
+                    if (list_of(bb) == l) rows += present_rows(bb);
+                rows = block_sum_int(rows, red);
+                if (threadIdx.x == 0) { p.list_row0[l] = row0; p.tile_start[l] = tile0; }
+                row0 += rows;
+                tile0 += (rows + tile_rows - 1) / tile_rows;
+            }
+            if (threadIdx.x == 0) { p.list_row0[n_lists] = row0; p.tile_start[n_lists] = tile0; }
+        }
+    }
+    // present tokens of the samples, ascending -> row table
+    auto present = [&](int t, uint32_t mask) {
+        if (t >= Tlen) return false;
+        if (ids == nullptr) return true;
+        const int m = ids[t];
+        return m >= 0 && m < 32 && ((mask >> m) & 1u);
+    };
+    if constexpr (G > 1) {   // a warp per sample
+        static_assert(G <= 8, "one warp per sample of the group");
+        const int b = b0 + wid;
+        if (wid < G && b < B) {
+            int base = 0;
+            for (int w = 0; w < nw; ++w) base += s_before[wid][w];
+            if (lane == 0) p.sample_row0[b] = base;
+            const uint32_t mask = ids != nullptr ? masks[b] : 0xffffffffu;
+            for (int t0 = 0; t0 < Tlen; t0 += 32) {
+                const bool ok = present(t0 + lane, mask);
+                const unsigned bm = __ballot_sync(0xffffffffu, ok);
+                if (ok) p.rowidx[base + __popc(bm & ((1u << lane) - 1u))] = b * Tlen + t0 + lane;
+                base += __popc(bm);
+            }
+        }
+    } else {                 // the whole block: every warp a run of 32-token pieces, after one count of what comes before
+        const int b = b0;
+        int base = 0;
+        for (int w = 0; w < nw; ++w) base += s_before[0][w];
+        if (threadIdx.x == 0) p.sample_row0[b] = base;
+        const uint32_t mask = ids != nullptr ? masks[b] : 0xffffffffu;
+        const int per = ((Tlen + 31) / 32 + nw - 1) / nw;
+        const int p0 = wid * per, p1 = min(p0 + per, (Tlen + 31) / 32);
+        int mine = 0;
+        for (int pc = p0; pc < p1; ++pc) mine += __popc(__ballot_sync(0xffffffffu, present(pc * 32 + lane, mask)));
+        if (lane == 0) red[wid] = mine;
+        __syncthreads();
+        for (int w = 0; w < wid; ++w) base += red[w];
+        for (int pc = p0; pc < p1; ++pc) {
+            const int t = pc * 32 + lane;
+            const bool ok = present(t, mask);
+            const unsigned bm = __ballot_sync(0xffffffffu, ok);
+            if (ok) p.rowidx[base + __popc(bm & ((1u << lane) - 1u))] = b * Tlen + t;
+            base += __popc(bm);
+        }
+    }
+}
+
+template <typename T, int G>
 __global__ void __launch_bounds__(256)
 ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__ masks,
                    const int32_t* __restrict__ list_of_sample, int B, int Tlen, int zsplit,
@@ -41,86 +186,12 @@ ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__
                    unsigned int* status) {
     // w_stride: elements between the weight matrices of consecutive lists (0: every list gathers
     // from the same W1, W2; D*F: list l has its own, as the experts of a Sparse-MoE block do)
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if ((int)blockIdx.x < B) {
-        __shared__ int s_cnt[32];
-        __shared__ int red[66];
-        const int b = blockIdx.x;
-        if (threadIdx.x < 32) s_cnt[threadIdx.x] = 0;
-        __syncthreads();
-        if (ids != nullptr) {
-            for (int t = threadIdx.x; t < Tlen; t += blockDim.x) {
-                const int m = ids[t];
-                if (m >= 0 && m < 32) atomicAdd(&s_cnt[m], 1);
-                else if (b == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
-            }
-            __syncthreads();
-        }
-        auto present_rows = [&](int bb) {
-            if (ids == nullptr) return Tlen;
-            uint32_t mask = masks[bb];
-            int n = 0;
-            while (mask) { const int m = __ffs(mask) - 1; n += s_cnt[m]; mask &= mask - 1; }
-            return n;
-        };
-        auto list_of = [&](int bb) {
-            int l = list_of_sample ? list_of_sample[bb] : 0;
-            if (l < 0 || l >= n_lists) {
-                if (b == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
-                l = 0;
-            }
-            return l;
-        };
-        // rows of all samples in earlier lists, and of earlier samples in this sample's list
-        const int my_list = list_of(b);
-        int before = 0;
-        for (int bb = threadIdx.x; bb < B; bb += blockDim.x) {
-            const int l = list_of(bb);
-            if (l < my_list || (l == my_list && bb < b)) before += present_rows(bb);
-        }
-        before = block_sum_int(before, red);
-        if (threadIdx.x == 0) p.sample_row0[b] = before;
-        if (b == 0) {
-            // per-list totals -> list offsets and tile counts (lists are few: one pass each)
-            int row0 = 0, tile0 = 0;
-            for (int l = 0; l < n_lists; ++l) {
-                int rows = 0;
-                for (int bb = threadIdx.x; bb < B; bb += blockDim.x)
-                    if (list_of(bb) == l) {
-                        const int r = present_rows(bb);
-                        rows += r;
-                        if (r == 0) atomicOr(status, SENTRY_STATUS_BIT_EMPTY_MASK);
-                    }
-                rows = block_sum_int(rows, red);
-                if (threadIdx.x == 0) { p.list_row0[l] = row0; p.tile_start[l] = tile0; }
-                row0 += rows;
-                tile0 += (rows + tile_rows - 1) / tile_rows;
-            }
-            if (threadIdx.x == 0) { p.list_row0[n_lists] = row0; p.tile_start[n_lists] = tile0; }
-        }
-        // present tokens of this sample, ascending -> row table
-        const uint32_t mask = (ids != nullptr) ? masks[b] : 0xffffffffu;
-        int32_t* rows = p.rowidx + before;
-        int base = 0;
-        for (int t0 = 0; t0 < Tlen; t0 += blockDim.x) {
-            const int t = t0 + threadIdx.x;
-            bool ok = false;
-            if (t < Tlen) {
-                if (ids == nullptr) ok = true;
-                else { const int m = ids[t]; ok = (m >= 0 && m < 32) && ((mask >> m) & 1u); }
-            }
-            const unsigned bm = __ballot_sync(0xffffffffu, ok);
-            __syncthreads();
-            if (lane == 0) red[wid] = __popc(bm);
-            __syncthreads();
-            int pos = base, tot = 0;
-            for (int w = 0; w < nw; ++w) { if (w < wid) pos += red[w]; tot += red[w]; }
-            if (ok) rows[pos + __popc(bm & ((1u << lane) - 1u))] = b * Tlen + t;
-            base += tot;
-        }
+    const int plan_blocks = (B + G - 1) / G;
+    if ((int)blockIdx.x < plan_blocks) {
+        plan_block<G>(ids, masks, list_of_sample, B, Tlen, tile_rows, p, n_lists, status);
         return;
     }
-    size_t pb = (size_t)blockIdx.x - B;
+    size_t pb = (size_t)blockIdx.x - plan_blocks;
     const size_t zero_blocks = (ids != nullptr) ? (size_t)B * zsplit : 0;
     if (pb < zero_blocks) {
         // zero the rows of absent tokens, 16 bytes per store
@@ -364,6 +435,10 @@ FfnWs carve(const sentry_ffn_desc& d, int kc_pad, void* ws, size_t bytes, bool w
     w.plan.tile_start = a.take<int32_t>(d.n_lists + 1);
     w.plan.rowidx = a.take<int32_t>((size_t)d.B * d.T);
     w.plan.rowout = nullptr;
+    w.plan.zero_ids = nullptr;
+    w.plan.zero_masks = nullptr;
+    w.plan.n_rows = 0;
+    w.plan.Tlen = d.T;
     w.w1p = w.w2p = nullptr;
     if (with_weights) {
         w.w1p = a.take<uint8_t>(packed_half_bytes(d, kc_pad));
@@ -405,15 +480,15 @@ int launch_ffn_prepack(sentry_ctx* ctx, const FfnArgs& a, void* packed, cudaStre
     // no row-table and no zero-fill blocks (B = 0, no ids): every block gathers weights
     if (d.dtype == SENTRY_FP8_E4M3) {
         if (!tc) return SENTRY_ERR_UNSUPPORTED;
-        ffn_prepare_kernel<uint8_t><<<(unsigned)pack_blocks, 256, 0, st>>>(
+        ffn_prepare_kernel<uint8_t, 1><<<(unsigned)pack_blocks, 256, 0, st>>>(
             nullptr, nullptr, nullptr, 0, d.T, 1, kTcTileRows, none, nullptr, (const uint8_t*)a.W1, (const uint8_t*)a.W2,
             a.kept, d.n_lists, d.D, d.F, d.k_c, kc_pad, 1, a.w_stride, w1p, w2p, a.status);
     } else if (d.dtype == SENTRY_F32)
-        ffn_prepare_kernel<float><<<(unsigned)pack_blocks, 256, 0, st>>>(
+        ffn_prepare_kernel<float, 1><<<(unsigned)pack_blocks, 256, 0, st>>>(
             nullptr, nullptr, nullptr, 0, d.T, 1, kGenericTileRows, none, nullptr, (const float*)a.W1,
             (const float*)a.W2, a.kept, d.n_lists, d.D, d.F, d.k_c, kc_pad, 0, a.w_stride, (float*)w1p, (float*)w2p, a.status);
     else
-        ffn_prepare_kernel<__nv_bfloat16><<<(unsigned)pack_blocks, 256, 0, st>>>(
+        ffn_prepare_kernel<__nv_bfloat16, 1><<<(unsigned)pack_blocks, 256, 0, st>>>(
             nullptr, nullptr, nullptr, 0, d.T, 1, tc ? kTcTileRows : kGenericTileRows, none, nullptr,
             (const __nv_bfloat16*)a.W1, (const __nv_bfloat16*)a.W2, a.kept, d.n_lists, d.D, d.F, d.k_c, kc_pad,
             tc ? 1 : 0, a.w_stride, (__nv_bfloat16*)w1p, (__nv_bfloat16*)w2p, a.status);
@@ -502,28 +577,31 @@ int launch_ffn(sentry_ctx* ctx, const FfnArgs& a, void* ws, size_t ws_bytes, con
         w.w2p = (uint8_t*)w.w1p + packed_half_bytes(d, kc_pad);
     }
     const int tile_rows = tc ? kTcTileRows : kGenericTileRows;
+    if (tc && a.ids != nullptr) {
+        w.plan.zero_ids = a.ids;
+        w.plan.zero_masks = a.masks;
+        w.plan.n_rows = d.B * d.T;
+    }
 
     {
         const size_t per = (size_t)kc_pad * d.D;
-        // enough zero-fill blocks to cover the GPU a few times over when the batch is small
-        int zsplit = (4 * ctx->sm_count + d.B - 1) / d.B;
-        if (zsplit < 1) zsplit = 1;
+        // plain-ALU kernel: enough zero-fill blocks to cover the GPU a few times over when the batch is small
+        int zsplit = tc ? 0 : (4 * ctx->sm_count + d.B - 1) / d.B;
+        if (!tc && zsplit < 1) zsplit = 1;
         if (zsplit > 32) zsplit = 32;
         const size_t pack_blocks = packed != nullptr ? 0
                                    : (tc ? 2 * (size_t)d.n_lists * (kc_pad / 32) * (d.D / 64)
                                          : 2 * (size_t)d.n_lists * ((per + 255) / 256));
-        const size_t grid = (size_t)d.B + (a.ids != nullptr ? (size_t)d.B * zsplit : 0) + pack_blocks;
+        const bool grouped = d.B >= kGroupPlanB;
+        const size_t plan_blocks = grouped ? ((size_t)d.B + 7) / 8 : (size_t)d.B;
+        const size_t grid = plan_blocks + (a.ids != nullptr ? (size_t)d.B * zsplit : 0) + pack_blocks;
         LaunchScope ls(ctx, KS_FFN_PREPARE, st);
-        if (d.dtype == SENTRY_F32)
-            ffn_prepare_kernel<float><<<(unsigned)grid, 256, 0, st>>>(
-                a.ids, a.masks, a.list_of_sample, d.B, d.T, zsplit, tile_rows, w.plan, (uint8_t*)a.Y,
-                (const float*)a.W1, (const float*)a.W2, a.kept, d.n_lists, d.D, d.F, d.k_c, kc_pad, 0, a.w_stride,
-                (float*)w.w1p, (float*)w.w2p, a.status);
-        else
-            ffn_prepare_kernel<__nv_bfloat16><<<(unsigned)grid, 256, 0, st>>>(
-                a.ids, a.masks, a.list_of_sample, d.B, d.T, zsplit, tile_rows, w.plan, (uint8_t*)a.Y,
-                (const __nv_bfloat16*)a.W1, (const __nv_bfloat16*)a.W2, a.kept, d.n_lists, d.D, d.F,
-                d.k_c, kc_pad, tc ? 1 : 0, a.w_stride, (__nv_bfloat16*)w.w1p, (__nv_bfloat16*)w.w2p, a.status);
+#define PREPARE(TT, G) ffn_prepare_kernel<TT, G><<<(unsigned)grid, 256, 0, st>>>(                                      \
+            a.ids, a.masks, a.list_of_sample, d.B, d.T, zsplit, tile_rows, w.plan, (uint8_t*)a.Y, (const TT*)a.W1,    \
+            (const TT*)a.W2, a.kept, d.n_lists, d.D, d.F, d.k_c, kc_pad, tc ? 1 : 0, a.w_stride, (TT*)w.w1p, (TT*)w.w2p, a.status)
+        if (d.dtype == SENTRY_F32) { if (grouped) PREPARE(float, 8); else PREPARE(float, 1); }
+        else { if (grouped) PREPARE(__nv_bfloat16, 8); else PREPARE(__nv_bfloat16, 1); }
+#undef PREPARE
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
     const long long rows = (long long)d.B * d.T;

@@ -16,6 +16,10 @@ struct FfnPlan {
     int32_t* rowidx;        // [B*T]        global row (b*T + t) of every present row, list-major
     int32_t* rowout;        // same shape or null: row of Y a result goes to, if not the row of X it came from
                             //              (Sparse-MoE: X row = token, Y row = (token, routing slot))
+    // zero rows of Y (tensor-core kernel): those of absent tokens among rows 0 .. n_rows-1 = b*Tlen + t; null: none
+    const int32_t* zero_ids;
+    const uint32_t* zero_masks;
+    int n_rows, Tlen;
 };
 
 // The fused pair alone, on a row plan and materialised weights that are already in place.

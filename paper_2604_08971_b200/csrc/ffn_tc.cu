@@ -24,8 +24,8 @@
 // and stores one 128-column third of Y (see the kernel).
 //
 // Warp roles (512 threads): warps 0 and 2 = weight TMA producers (warp 0 owns TMEM),
-// warp 1 = UMMA issuer (warp 15 is idle), warps 3-6 = X row
-// gather, warps 7-14 = epilogue (two warps per TMEM lane quarter).  Producer and issuer warps stay
+// warp 1 = UMMA issuer, warps 3-6 = X row
+// gather, warps 7-14 = epilogue (two warps per TMEM lane quarter), warp 15 = zero rows of absent tokens.  Producer and issuer warps stay
 // converged and elect one lane per instruction.  Every wait is bounded; on expiry the CTA raises SENTRY_STATUS_BIT_TIMEOUT
 // and unwinds.
 #include <cuda.h>
@@ -45,6 +45,7 @@ constexpr int kStages = 3;
 constexpr int kThreads = 512;
 constexpr int kLoaderWarp0 = 3, kLoaderWarps = 4, kLoaderThreads = kLoaderWarps * 32;
 constexpr int kEpiWarp0 = 7, kEpiWarps = 8;
+constexpr int kZeroWarp = 15, kZeroBytes = 1024;   // zeros at the end of the misc block
 constexpr int kTmemCols = 512;
 
 // FP8: X, the weights and the hidden activations are e4m3 bytes (a 128-byte operand row then
@@ -81,7 +82,7 @@ struct Misc {
     uint32_t tmem_base;
     int abort_flag;
 };
-static_assert(sizeof(Misc) <= 2048, "misc block too large");
+static_assert(sizeof(Misc) <= 2048 - kZeroBytes, "misc block too large");
 
 // ---- lean forms for the single-thread roles -------------------------------------------------
 // A warp that walks a chain of dependent scalar instructions with shared-memory round trips in
@@ -655,6 +656,46 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__
             }
         }
         if (ok && ti > 0) drain_y(ti - 1, my_row, my_third);
+    } else if (warp == kZeroWarp && plan.zero_ids != nullptr) {
+        // ------------------------------------------------- zero rows of Y for absent tokens
+        // The CTAs share the rows out evenly; runs of absent rows are written by bulk copies from a block of zeros, an
+        // instruction per kilobyte.  As blocks of the prepare launch these stores were a pass of their own over the absent
+        // part of Y (65 of 85 us at 4096 x 256 tokens, 3/7 absent); here they run beside the arithmetic.
+        const uint32_t zsm = ptx::smem_u32(misc) + 2048u - kZeroBytes;
+        for (int i = lane; i < kZeroBytes / 16; i += 32)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(zsm + i * 16), "r"(0) : "memory");
+        ptx::fence_proxy_async_smem();
+        __syncwarp();
+        const int per = (plan.n_rows + (int)gridDim.x - 1) / (int)gridDim.x;
+        const int r1 = min(plan.n_rows, ((int)blockIdx.x + 1) * per);
+        for (int r0 = (int)blockIdx.x * per; r0 < r1; r0 += 128) {
+            // 128 rows at a time: their ids and masks are requested together (a round trip per 32 rows made this warp
+            // the last to finish)
+            int m[4];
+            uint32_t mask[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int r = min(r0 + u * 32 + lane, plan.n_rows - 1), bb = r / plan.Tlen;
+                m[u] = __ldg(plan.zero_ids + (r - bb * plan.Tlen));
+                mask[u] = __ldg(plan.zero_masks + bb);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool absent = r0 + u * 32 + lane < r1 && !(m[u] >= 0 && m[u] < 32 && ((mask[u] >> m[u]) & 1u));
+                unsigned todo = __ballot_sync(0xffffffffu, absent);
+                while (todo) {   // runs of absent rows: contiguous in Y, kZeroBytes per lane (32 rows are at most 24 KB)
+                    const int first = __ffs(todo) - 1;
+                    const unsigned rest = ~(todo >> first);
+                    const int len = rest ? min(__ffs(rest) - 1, 32 - first) : 32 - first;
+                    todo &= ~((len == 32 ? 0xffffffffu : (1u << len) - 1u) << first);
+                    const int off = lane * kZeroBytes, bytes = min(len * D * 2 - off, kZeroBytes);
+                    if (bytes > 0)
+                        ptx::bulk_store(reinterpret_cast<uint8_t*>(Y) + (size_t)(r0 + u * 32 + first) * D * 2 + off, zsm,
+                                        (uint32_t)bytes);
+                }
+            }
+        }
+        ptx::bulk_store_wait();   // the zeros have been read (and the rows are written before the grid ends)
     }
 
     cta_teardown(abort_flag, status, tmem, kTmemCols);

@@ -305,6 +305,10 @@ MoeWs carve(const sentry_moe_desc& m, void* ws, size_t bytes, bool with_weights)
     w.plan.tile_start = a.take<int32_t>((size_t)m.E + 1);
     w.plan.rowidx = a.take<int32_t>(slots);
     w.plan.rowout = a.take<int32_t>(slots);
+    w.plan.zero_ids = nullptr;
+    w.plan.zero_masks = nullptr;
+    w.plan.n_rows = 0;
+    w.plan.Tlen = 1;
     w.counts = a.take<int32_t>((size_t)2 * m.E);
     w.cursor = w.counts ? w.counts + m.E : nullptr;
     w.staged = a.take<uint8_t>(slots * m.D * esz);
