@@ -122,6 +122,7 @@ attend_score_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
                          const int64_t* __restrict__ offsets, int n_subsets, int Tlen, int Hq, int Hk,
                          int k_h, int c, int score_mode, int seg_shift, float* __restrict__ mscore,
                          unsigned int* status) {
+    grid_dependency_wait();
     extern __shared__ __align__(128) uint8_t s_raw[];
     __shared__ int red[66];
     uint16_t* s_valid = reinterpret_cast<uint16_t*>(s_raw);
@@ -211,6 +212,7 @@ attend_core_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16
                         const float* __restrict__ mscore, const int32_t* __restrict__ active_in,
                         int32_t* __restrict__ active_out, int Tlen, int Hq, int Hk, int k_h, int c,
                         int U_max, __nv_bfloat16* __restrict__ O, unsigned int* status) {
+    grid_dependency_wait();
     using S = Sw<D>;
     using CS = CoreSmem<D>;
     constexpr int NT = D / 8;        // n-tiles of the output (8 dims each)
@@ -605,6 +607,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
                          int32_t* __restrict__ active_out, int Tlen, int Hq, int Hk, int k_h, int c,
                          int score_mode, int U_max, __nv_bfloat16* __restrict__ O, unsigned int* status,
                          const float* __restrict__ gate_scores, int gate_S, int32_t* __restrict__ kept_out) {
+    grid_dependency_wait();
     using S = Sw<D>;
     constexpr int NT = D / 8;        // n-tiles of the output (8 dims each)
     constexpr int KS = D / 16;       // k-steps of q.k
@@ -1050,12 +1053,12 @@ int launch_d(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
         // phases are a few barrier-separated microseconds each, so concurrency is what helps)
         const int threads = fused_bytes > 100 * 1024 ? 512 : (d.T <= kSmallT ? 128 : 256);
         LaunchScope ls(ctx, KS_ATT_CORE, st);
-        kern<<<d.B * d.Hk, threads, fused_bytes, st>>>(
+        SENTRY_CUDA_TRY(launch_chained(kern, dim3(d.B * d.Hk), dim3(threads), fused_bytes, st,
             (const __nv_bfloat16*)a.Q, (const __nv_bfloat16*)a.K, (const __nv_bfloat16*)a.V, a.kept_heads,
             a.ids, a.masks, a.sample_table, a.sample_offsets, a.n_subsets,
             a.selection_given ? a.active : nullptr, a.selection_given ? nullptr : a.active_out_user, d.T,
             d.Hq, d.Hk, d.k_h, d.c, d.score_mode, a.U_max, (__nv_bfloat16*)a.O, a.status, a.gate_scores, a.gate_S,
-            a.kept_out);
+            a.kept_out));
         SENTRY_CUDA_TRY(cudaGetLastError());
         return SENTRY_OK;
     }
@@ -1082,10 +1085,10 @@ int launch_d(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
         SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         dim3 grid(d.B * d.Hk, (d.T + kScoreThreads - 1) / kScoreThreads);   // (sample, group) on x: no 65535 limit
         LaunchScope ls(ctx, KS_ATT_SCORE, st);
-        kern<<<grid, kScoreThreads, smem, st>>>((const __nv_bfloat16*)a.Q, (const __nv_bfloat16*)a.K,
+        SENTRY_CUDA_TRY(launch_chained(kern, dim3(grid), dim3(kScoreThreads), smem, st, (const __nv_bfloat16*)a.Q, (const __nv_bfloat16*)a.K,
                                                  a.kept_heads, a.ids, a.masks, a.sample_table,
                                                  a.sample_offsets, a.n_subsets, d.T, d.Hq, d.Hk, d.k_h,
-                                                 d.c, d.score_mode, seg_shift, a.mscore, a.status);
+                                                 d.c, d.score_mode, seg_shift, a.mscore, a.status));
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
     {
@@ -1099,11 +1102,11 @@ int launch_d(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
         auto kern = attend_core_bf16_kernel<D>;
         SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         LaunchScope ls(ctx, KS_ATT_CORE, st);
-        kern<<<d.B * d.Hk, kCoreThreads, smem, st>>>(
+        SENTRY_CUDA_TRY(launch_chained(kern, dim3(d.B * d.Hk), dim3(kCoreThreads), smem, st,
             (const __nv_bfloat16*)a.Q, (const __nv_bfloat16*)a.K, (const __nv_bfloat16*)a.V, a.kept_heads,
             a.ids, a.masks, a.mscore, given ? a.active : nullptr,
             given ? nullptr : a.active_out_user, d.T, d.Hq, d.Hk, d.k_h, d.c, a.U_max,
-            (__nv_bfloat16*)a.O, a.status);
+            (__nv_bfloat16*)a.O, a.status));
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;

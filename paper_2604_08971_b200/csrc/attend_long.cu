@@ -86,6 +86,7 @@ attend_long_select_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat
                           const int64_t* __restrict__ offsets, int n_subsets, int Tlen, int Hq, int Hk,
                           int k_h, int c, int score_mode, int U_max, int smem_bytes,
                           int32_t* __restrict__ active, unsigned int* status) {
+    grid_dependency_wait();
     using S = Sw<D>;
     extern __shared__ __align__(128) uint8_t s_raw[];
     __shared__ int red[66];
@@ -214,9 +215,9 @@ int launch_long_d(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
     auto kern = attend_long_select_kernel<D>;
     SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     LaunchScope ls(ctx, KS_ATT_SCORE, st);
-    kern<<<d.B * d.Hk, kLongThreads, smem, st>>>(
+    SENTRY_CUDA_TRY(launch_chained(kern, dim3(d.B * d.Hk), dim3(kLongThreads), smem, st,
         (const __nv_bfloat16*)a.Q, (const __nv_bfloat16*)a.K, a.kept_heads, a.ids, a.masks, a.sample_table,
-        a.sample_offsets, a.n_subsets, d.T, d.Hq, d.Hk, d.k_h, d.c, d.score_mode, a.U_max, (int)smem, a.active, a.status);
+        a.sample_offsets, a.n_subsets, d.T, d.Hq, d.Hk, d.k_h, d.c, d.score_mode, a.U_max, (int)smem, a.active, a.status));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
 }

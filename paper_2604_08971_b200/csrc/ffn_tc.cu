@@ -165,21 +165,6 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int NC = kc_pad / C::CH;
-    const int total_tiles = plan.tile_start[n_lists];
-    // Column-split tail (d_model = 384, 16-bit and FP8 operands).  The tiles of the last, partial round leave most CTAs idle
-    // (340 tiles on 148 CTAs: 44 in the third round).  When three times their number still fits
-    // one round, each of them is taken by three CTAs: all three form the tile's hidden
-    // activations, and each accumulates and stores one 128-column third of Y (GEMM2 of a third =
-    // the N = 128 stage alone).  Nothing is exchanged; a third costs 4/6 of the tensor work of a
-    // whole tile.  Virtual tile v < full_v is tile v; the others are (tile, third) pairs.  A CTA's
-    // split tile, if it has one, is its last.
-    int full_v = total_tiles, n_vt = total_tiles;
-    if constexpr (C::COLSPLIT) {
-        const int rem = total_tiles % (int)gridDim.x;
-        if (rem > 0 && 3 * rem <= (int)gridDim.x) { full_v = total_tiles - rem; n_vt = full_v + 3 * rem; }
-    }
-    auto tile_of = [&](int v) { return v < full_v ? v : full_v + (v - full_v) / 3; };
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             ptx::mbar_init(ptx::smem_u32(&misc->w_full[s]), 1);
@@ -208,6 +193,22 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = misc->tmem_base;
+    grid_dependency_wait();   // barriers and tensor memory are set up before the plan is there
+
+    const int total_tiles = plan.tile_start[n_lists];
+    // Column-split tail (d_model = 384, 16-bit and FP8 operands).  The tiles of the last, partial round leave most CTAs idle
+    // (340 tiles on 148 CTAs: 44 in the third round).  When three times their number still fits
+    // one round, each of them is taken by three CTAs: all three form the tile's hidden
+    // activations, and each accumulates and stores one 128-column third of Y (GEMM2 of a third =
+    // the N = 128 stage alone).  Nothing is exchanged; a third costs 4/6 of the tensor work of a
+    // whole tile.  Virtual tile v < full_v is tile v; the others are (tile, third) pairs.  A CTA's
+    // split tile, if it has one, is its last.
+    int full_v = total_tiles, n_vt = total_tiles;
+    if constexpr (C::COLSPLIT) {
+        const int rem = total_tiles % (int)gridDim.x;
+        if (rem > 0 && 3 * rem <= (int)gridDim.x) { full_v = total_tiles - rem; n_vt = full_v + 3 * rem; }
+    }
+    auto tile_of = [&](int v) { return v < full_v ? v : full_v + (v - full_v) / 3; };
 
     constexpr int SPG = C::SPG;
     const uint32_t mb = ptx::smem_u32(misc);
@@ -743,8 +744,8 @@ int launch_d(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, 
     int grid = max_tiles < ctx->sm_count ? max_tiles : ctx->sm_count;
     if (grid < 1) grid = 1;
     LaunchScope ls(ctx, KS_FFN_MAIN, st);
-    kern<<<grid, kThreads, Cfg<D>::SMEM_BYTES, st>>>(m1, m2a, m2b, (const __nv_bfloat16*)a.X,
-                                                      (__nv_bfloat16*)a.Y, plan, d.n_lists, kc_pad, a.status, 1.f, 1.f, 1.f);
+    SENTRY_CUDA_TRY(launch_chained(kern, dim3(grid), dim3(kThreads), Cfg<D>::SMEM_BYTES, st, m1, m2a, m2b, (const __nv_bfloat16*)a.X,
+                                                      (__nv_bfloat16*)a.Y, plan, d.n_lists, kc_pad, a.status, 1.f, 1.f, 1.f));
     return SENTRY_OK;
 }
 
@@ -763,9 +764,9 @@ int launch_fp8(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c
     int grid = max_tiles < ctx->sm_count ? max_tiles : ctx->sm_count;
     if (grid < 1) grid = 1;
     LaunchScope ls(ctx, KS_FFN_MAIN, st);
-    kern<<<grid, kThreads, Cfg<D, true>::SMEM_BYTES, st>>>(m1, m2a, m2b, (const __nv_bfloat16*)a.X, (__nv_bfloat16*)a.Y,
+    SENTRY_CUDA_TRY(launch_chained(kern, dim3(grid), dim3(kThreads), (size_t)Cfg<D, true>::SMEM_BYTES, st, m1, m2a, m2b, (const __nv_bfloat16*)a.X, (__nv_bfloat16*)a.Y,
                                                            plan, d.n_lists, kc_pad, a.status, a.fp8_a_scale,
-                                                           a.fp8_h_inv, a.fp8_y_scale);
+                                                           a.fp8_h_inv, a.fp8_y_scale));
     return SENTRY_OK;
 }
 

@@ -35,6 +35,8 @@ constexpr int kGateMaxRegUnits = 8192;
 template <int KPT>
 __global__ void __launch_bounds__(1024)
 gate_select_kernel(const __grid_constant__ GateSetsDev sets, int S, unsigned int* status) {
+    grid_dependents_start();
+    grid_dependency_wait();
     extern __shared__ int32_t s_list[];            // [k] kept units, ascending
     __shared__ uint32_t s_red[2][3][32];           // per-warp partial results of a counting step, two steps in turn
     __shared__ uint32_t s_bits;
@@ -179,11 +181,11 @@ int launch_gate_reg(int S, const sentry_gate_set* sets, int n_sets, unsigned int
     auto threads_for = [&](int kpt) { return ((n_max + kpt - 1) / kpt + 31) / 32 * 32; };
     if (n_max <= 256) {
         const int th = n_max <= 64 ? (out_max >= 1024 ? 256 : 64) : threads_for(1);
-        gate_select_kernel<1><<<grid, th, smem, st>>>(dev, S, status);
+        SENTRY_CUDA_TRY(launch_chained(gate_select_kernel<1>, dim3(grid), dim3(th), smem, st, dev, S, status));
     } else if (n_max <= 1024) {
-        gate_select_kernel<4><<<grid, threads_for(4), smem, st>>>(dev, S, status);
+        SENTRY_CUDA_TRY(launch_chained(gate_select_kernel<4>, dim3(grid), dim3(threads_for(4)), smem, st, dev, S, status));
     } else {
-        gate_select_kernel<8><<<grid, threads_for(8), smem, st>>>(dev, S, status);
+        SENTRY_CUDA_TRY(launch_chained(gate_select_kernel<8>, dim3(grid), dim3(threads_for(8)), smem, st, dev, S, status));
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;

@@ -21,6 +21,8 @@ gate_eval_kernel(const float* __restrict__ zeta, const float* __restrict__ gamma
                  const int32_t* __restrict__ layer_offsets, int n_layers, const float* __restrict__ W1,
                  const float* __restrict__ b1, const float* __restrict__ w2, const float* __restrict__ b2,
                  int M, int hidden, int jc, int N, int S, float* __restrict__ logits, float* __restrict__ gates) {
+    grid_dependents_start();
+    grid_dependency_wait();
     extern __shared__ float s_par[];               // [32][stride]: W1 piece [jc][M] | b1 piece [jc] | w2 piece [jc]
     const int stride = (jc * (M + 2)) | 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -79,6 +81,8 @@ gate_eval_kernel(const float* __restrict__ zeta, const float* __restrict__ gamma
 __global__ void __launch_bounds__(256)
 layer_count_kernel(const int32_t* __restrict__ kept, int n_masks, int k, const int32_t* __restrict__ layer_offsets,
                    int n_layers, int32_t* __restrict__ counts) {
+    grid_dependents_start();
+    grid_dependency_wait();
     extern __shared__ int s_pos[];                 // [n_layers + 1]
     const int m = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t* row = kept + (size_t)m * k;
@@ -111,8 +115,8 @@ int launch_gate_eval(sentry_ctx* ctx, const float* zeta, const float* gamma, con
     const size_t smem = (size_t)kEvalUnits * ((jc * (M + 2)) | 1) * sizeof(float);   // at most 33 KB
     const dim3 grid((unsigned)((N + kEvalUnits - 1) / kEvalUnits), (unsigned)((S + kEvalMasks - 1) / kEvalMasks));
     LaunchScope ls(ctx, KS_GATE_EVAL, st);
-    gate_eval_kernel<<<grid, 256, smem, st>>>(zeta, gamma, layer_offsets, n_layers, W1, b1, w2, b2, M, hidden, jc, N, S,
-                                              logits, gates);
+    SENTRY_CUDA_TRY(launch_chained(gate_eval_kernel, dim3(grid), dim3(256), smem, st, zeta, gamma, layer_offsets, n_layers, W1, b1, w2, b2, M, hidden, jc, N, S,
+                                              logits, gates));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
 }
@@ -125,7 +129,7 @@ int launch_layer_counts(sentry_ctx* ctx, const int32_t* kept, int n_masks, int k
         if (smem > 220 * 1024) return SENTRY_ERR_UNSUPPORTED;
         SENTRY_CUDA_TRY(cudaFuncSetAttribute(layer_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
-    layer_count_kernel<<<n_masks, 256, smem, st>>>(kept, n_masks, k, layer_offsets, n_layers, counts);
+    SENTRY_CUDA_TRY(launch_chained(layer_count_kernel, dim3(n_masks), dim3(256), smem, st, kept, n_masks, k, layer_offsets, n_layers, counts));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
 }

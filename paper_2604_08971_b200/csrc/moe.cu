@@ -21,6 +21,8 @@ constexpr int kPlanThreads = 256;
 __global__ void __launch_bounds__(kPlanThreads)
 moe_route_kernel(const int32_t* __restrict__ expert_ids, long long n_slots, int E, int top_k, int phase,
                  int32_t* __restrict__ counts, int32_t* __restrict__ cursor, FfnPlan plan, unsigned int* status) {
+    grid_dependents_start();
+    grid_dependency_wait();
     extern __shared__ int s_int[];
     int* s_cnt = s_int;        // [E] slots of this block per expert
     int* s_base = s_int + E;   // [E] first position of this block's range in the expert's rows
@@ -74,6 +76,8 @@ moe_route_kernel(const int32_t* __restrict__ expert_ids, long long n_slots, int 
 __global__ void __launch_bounds__(kPlanThreads)
 moe_offsets_kernel(const int32_t* __restrict__ counts, int E, int tile_rows, FfnPlan plan,
                    int32_t* __restrict__ cursor) {
+    grid_dependents_start();
+    grid_dependency_wait();
     __shared__ int s_rows[kPlanThreads], s_tiles[kPlanThreads];
     const int per = (E + kPlanThreads - 1) / kPlanThreads;
     const int e0 = threadIdx.x * per, e1 = min(E, e0 + per);
@@ -108,6 +112,8 @@ constexpr long long kPlanOneMaxSlots = 8192;   // one round of the block; beyond
 __global__ void __launch_bounds__(kPlanOneThreads)
 moe_plan_one_kernel(const int32_t* __restrict__ expert_ids, int n_slots, int E, int top_k, int tile_rows,
                     FfnPlan plan, unsigned int* status) {
+    grid_dependents_start();
+    grid_dependency_wait();
     extern __shared__ int s_int[];
     int* s_cnt = s_int;          // [E] slots per expert
     int* s_cur = s_int + E;      // [E] next free row of the expert
@@ -236,6 +242,8 @@ __global__ void __launch_bounds__(256)
 moe_combine_kernel(const uint4* __restrict__ staged, const int32_t* __restrict__ expert_ids,
                    const float* __restrict__ weights, long long N, int vpr, int E, int top_k,
                    uint4* __restrict__ Y) {
+    grid_dependents_start();
+    grid_dependency_wait();
     constexpr int NV = Vec16<T>::N;
     constexpr bool IS_BF16 = sizeof(T) == 2 && Vec16<T>::N == 8 && __is_same(T, __nv_bfloat16);
     const long long total = N * vpr;
@@ -351,16 +359,16 @@ int launch_moe_ffn(sentry_ctx* ctx, const MoeArgs& m, void* ws, size_t ws_bytes,
     }
     if (slots <= kPlanOneMaxSlots && route_smem <= 48 * 1024) {
         LaunchScope ls(ctx, KS_MOE_PLAN, st);
-        moe_plan_one_kernel<<<1, kPlanOneThreads, route_smem, st>>>(m.expert_ids, (int)slots, d.E, d.top_k, tile_rows,
-                                                                    w.plan, m.status);
+        SENTRY_CUDA_TRY(launch_chained(moe_plan_one_kernel, dim3(1), dim3(kPlanOneThreads), route_smem, st, m.expert_ids, (int)slots, d.E, d.top_k, tile_rows,
+                                                                    w.plan, m.status));
     } else {
         SENTRY_CUDA_TRY(cudaMemsetAsync(w.counts, 0, (size_t)d.E * sizeof(int32_t), st));
         LaunchScope ls(ctx, KS_MOE_PLAN, st, 3);
-        moe_route_kernel<<<route_blocks, kPlanThreads, route_smem, st>>>(m.expert_ids, slots, d.E, d.top_k, 0,
-                                                                         w.counts, w.cursor, w.plan, m.status);
-        moe_offsets_kernel<<<1, kPlanThreads, 0, st>>>(w.counts, d.E, tile_rows, w.plan, w.cursor);
-        moe_route_kernel<<<route_blocks, kPlanThreads, route_smem, st>>>(m.expert_ids, slots, d.E, d.top_k, 1,
-                                                                         w.counts, w.cursor, w.plan, m.status);
+        SENTRY_CUDA_TRY(launch_chained(moe_route_kernel, dim3(route_blocks), dim3(kPlanThreads), route_smem, st, m.expert_ids, slots, d.E, d.top_k, 0,
+                                                                         w.counts, w.cursor, w.plan, m.status));
+        SENTRY_CUDA_TRY(launch_chained(moe_offsets_kernel, dim3(1), dim3(kPlanThreads), 0, st, w.counts, d.E, tile_rows, w.plan, w.cursor));
+        SENTRY_CUDA_TRY(launch_chained(moe_route_kernel, dim3(route_blocks), dim3(kPlanThreads), route_smem, st, m.expert_ids, slots, d.E, d.top_k, 1,
+                                                                         w.counts, w.cursor, w.plan, m.status));
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
 
@@ -385,14 +393,14 @@ int launch_moe_ffn(sentry_ctx* ctx, const MoeArgs& m, void* ws, size_t ws_bytes,
         if (blocks > cap) blocks = cap;
         LaunchScope ls(ctx, KS_MOE_COMBINE, st);
         if (d.dtype == SENTRY_F32)
-            moe_combine_kernel<float><<<(unsigned)blocks, 256, 0, st>>>(
-                (const uint4*)w.staged, m.expert_ids, m.expert_weights, d.N, vpr, d.E, d.top_k, (uint4*)m.Y);
+            SENTRY_CUDA_TRY(launch_chained(moe_combine_kernel<float>, dim3((unsigned)blocks), dim3(256), 0, st,
+                (const uint4*)w.staged, m.expert_ids, m.expert_weights, d.N, vpr, d.E, d.top_k, (uint4*)m.Y));
         else if (d.dtype == SENTRY_F16)
-            moe_combine_kernel<__half><<<(unsigned)blocks, 256, 0, st>>>(
-                (const uint4*)w.staged, m.expert_ids, m.expert_weights, d.N, vpr, d.E, d.top_k, (uint4*)m.Y);
+            SENTRY_CUDA_TRY(launch_chained(moe_combine_kernel<__half>, dim3((unsigned)blocks), dim3(256), 0, st,
+                (const uint4*)w.staged, m.expert_ids, m.expert_weights, d.N, vpr, d.E, d.top_k, (uint4*)m.Y));
         else
-            moe_combine_kernel<__nv_bfloat16><<<(unsigned)blocks, 256, 0, st>>>(
-                (const uint4*)w.staged, m.expert_ids, m.expert_weights, d.N, vpr, d.E, d.top_k, (uint4*)m.Y);
+            SENTRY_CUDA_TRY(launch_chained(moe_combine_kernel<__nv_bfloat16>, dim3((unsigned)blocks), dim3(256), 0, st,
+                (const uint4*)w.staged, m.expert_ids, m.expert_weights, d.N, vpr, d.E, d.top_k, (uint4*)m.Y));
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;

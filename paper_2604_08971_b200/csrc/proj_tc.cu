@@ -48,6 +48,7 @@ proj_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                    const uint32_t* __restrict__ masks, int Tlen, int D, int Hq, int Hk, int k_h,
                    __nv_bfloat16* __restrict__ Q, __nv_bfloat16* __restrict__ K, __nv_bfloat16* __restrict__ V,
                    unsigned int* status) {
+    grid_dependency_wait();
     constexpr int RB = DH * 2;
     constexpr int NS = 512 / DH;                    // slices whose accumulators fit in tensor memory at once
     extern __shared__ uint8_t smem_raw[];
@@ -227,6 +228,7 @@ proj_out_tc_kernel(const __grid_constant__ CUtensorMap tm_o, const __nv_bfloat16
                    const int32_t* __restrict__ kept_heads, const int32_t* __restrict__ ids,
                    const uint32_t* __restrict__ masks, int Tlen, int D, int Hq, int k_h,
                    __nv_bfloat16* __restrict__ out, unsigned int* status) {
+    grid_dependency_wait();
     using S = Sw<DH>;
     constexpr int RB = DH * 2;
     extern __shared__ uint8_t smem_raw[];
@@ -397,8 +399,8 @@ int launch_out_d(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t st) {
     SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const unsigned grid = (unsigned)((size_t)d.B * ((d.T + 127) / 128));
     LaunchScope ls(ctx, KS_PROJ_OUT, st);
-    kern<<<grid, kPThreads, smem, st>>>(mo, (const __nv_bfloat16*)a.A, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq,
-                                        d.k_h, (__nv_bfloat16*)a.out, a.status);
+    SENTRY_CUDA_TRY(launch_chained(kern, dim3(grid), dim3(kPThreads), smem, st, mo, (const __nv_bfloat16*)a.A, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq,
+                                        d.k_h, (__nv_bfloat16*)a.out, a.status));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
 }
@@ -420,9 +422,9 @@ int launch_qkv_d(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t st) {
     SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const unsigned grid = (unsigned)((size_t)d.B * ((d.T + 127) / 128));
     LaunchScope ls(ctx, KS_PROJ_QKV, st);
-    kern<<<grid, kPThreads, smem, st>>>(mq, mk, mv, (const __nv_bfloat16*)a.X, a.kept_heads, a.ids, a.masks, d.T, d.D,
+    SENTRY_CUDA_TRY(launch_chained(kern, dim3(grid), dim3(kPThreads), smem, st, mq, mk, mv, (const __nv_bfloat16*)a.X, a.kept_heads, a.ids, a.masks, d.T, d.D,
                                         d.Hq, d.Hk, d.k_h, (__nv_bfloat16*)a.Q, (__nv_bfloat16*)a.K,
-                                        (__nv_bfloat16*)a.V, a.status);
+                                        (__nv_bfloat16*)a.V, a.status));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
 }
