@@ -346,7 +346,7 @@ SENTRY_API int sentry_ffn_fwd_packed(sentry_ctx* ctx, const sentry_ffn_desc* des
  *   expert_weights [N,top_k] fp32 (whatever the router produced; not renormalised)
  *   Y out [N,D] dtype; a token with no routed slot gets zeros
  * All device pointers, 16-byte aligned; D % 8 == 0, D <= 1024, E <= 4096,
- * N*top_k < 2^31.  bf16 with D in {128,256,384} runs on the tcgen05 kernel of
+ * N*top_k < 2^31.  16-bit types with D % 64 == 0 run on the tcgen05 kernels of
  * sentry_ffn_fwd with one weight set per expert; other shapes on the plain
  * ALUs.  Scratch (row plan, per-slot results, and W1', W2' unless `packed` is
  * given) comes from the workspace: sentry_moe_workspace_bytes.
@@ -446,8 +446,8 @@ typedef struct sentry_ffn_desc {
     int B, T, D, F; /* batch, tokens per sample, d_model, d_ff */
     int k_c;        /* kept channels per list */
     int n_lists;    /* number of kept-channel lists (one per modality subset in use) */
-    int dtype;      /* sentry_dtype of X, W1, W2, Y (F32, BF16 or F16; the 16-bit types with D in
-                       {128,256,384} run on tcgen05, everything else on the plain ALUs) */
+    int dtype;      /* sentry_dtype of X, W1, W2, Y (F32, BF16 or F16; the 16-bit types run on tcgen05 where
+                       D is a multiple of 64, everything else on the plain ALUs) */
 } sentry_ffn_desc;
 
 /*   X [B,T,D]; W1 [D,F]; W2 [F,D]; Y out [B,T,D]
@@ -459,8 +459,9 @@ typedef struct sentry_ffn_desc {
  * every call (the "materialised" pruned weights), then a fused GEMM pair runs
  * over the present rows.  Supported: D % 8 == 0, D <= 1024.
  * bf16 with D in {128, 256, 384} runs on the tcgen05 tensor cores, one
- * persistent CTA per SM; every other shape and fp32 run on the plain ALUs with
- * fp32 accumulation.  The GELU of the bf16 path evaluates
+ * persistent CTA per SM; with any other multiple of 64 as two tcgen05 GEMMs
+ * whose hidden activations keep 16 bits of precision beyond bf16's 8; other
+ * shapes and fp32 run on the plain ALUs with fp32 accumulation.  The GELU of the bf16 path evaluates
  * erf through the hardware tanh: within 4e-4 of gelu(|z|), below the rounding
  * of the bf16 hidden value it is stored as; fp32 uses erff.  Results are
  * bit-identical from call to call for identical inputs.

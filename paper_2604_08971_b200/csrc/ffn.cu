@@ -9,11 +9,6 @@
 
 #include "ffn_plan.cuh"
 
-int launch_ffn_tc(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c,
-                  int kc_pad, int max_tiles, cudaStream_t st);  // ffn_tc.cu
-bool ffn_tc_supported(const sentry_ffn_desc& d);
-int ffn_tc_kc_pad(int D, int k_c);
-
 namespace {
 
 constexpr int kGenericTileRows = 16;
@@ -26,8 +21,7 @@ constexpr int kTcTileRows = 128;
 //                       launch is needed); block 0 also writes the per-list offsets and tile counts.  G = 1 for small
 //                       batches, whose blocks are then all in flight at once; from kGroupPlanB samples on the scan is
 //                       what a block does, and eight samples share it
-//   [P, P + B*zsplit)   plain-ALU kernel only: zero rows of Y for the absent tokens of a sample (slices of its rows;
-//                       the tensor-core kernel writes them itself, beside its arithmetic)
+//   [P, P + B*zsplit)   (not with the fused kernel, which does it itself) zero rows of Y for the absent tokens of a sample (slices of its rows)
 //   [.., + prepack)     the weight gather, which "materialises" the pruned W1', W2' per list:
 //     layout 0 (plain-ALU kernel): W1g [l][D][kc_pad], W2g [l][kc_pad][D]
 //     layout 1 (tensor-core kernel, both K-major): W1c [l][kc_pad][D], W2c [l][D][kc_pad]
@@ -453,13 +447,26 @@ FfnWs carve(const sentry_ffn_desc& d, int kc_pad, void* ws, size_t bytes, bool w
 
 int kc_pad_for(const sentry_ffn_desc& d) {
     if (ffn_tc_supported(d)) return ffn_tc_kc_pad(d.D, d.k_c);
+    if (ffn_wide_supported(d)) return ffn_wide_kc_pad(d.k_c);
     return (d.k_c + 7) / 8 * 8;
+}
+
+// Weights as K-major chunk-padded copies (either tensor-core form), tiles of 128 rows.
+bool k_major(const sentry_ffn_desc& d) { return ffn_tc_supported(d) || ffn_wide_supported(d); }
+long long tiles_bound(const sentry_ffn_desc& d) {
+    const int tile_rows = k_major(d) ? kTcTileRows : kGenericTileRows;
+    return ((long long)d.B * d.T + tile_rows - 1) / tile_rows + d.n_lists;
 }
 
 }  // namespace
 
 size_t ffn_workspace_bytes(const sentry_ffn_desc& d) {
-    return carve(d, kc_pad_for(d), nullptr, 0, true).used + 256;
+    return carve(d, kc_pad_for(d), nullptr, 0, true).used + ffn_hidden_bytes(d, tiles_bound(d)) + 512;
+}
+
+// Scratch for the hidden activations where they leave the SM.
+size_t ffn_hidden_bytes(const sentry_ffn_desc& d, long long max_tiles) {
+    return ffn_wide_supported(d) ? ffn_wide_hidden_bytes(kc_pad_for(d), max_tiles) : 0;
 }
 
 size_t ffn_packed_bytes(const sentry_ffn_desc& d) { return 2 * packed_half_bytes(d, kc_pad_for(d)); }
@@ -469,7 +476,7 @@ size_t ffn_packed_bytes(const sentry_ffn_desc& d) { return 2 * packed_half_bytes
 // instantiation unchanged.)
 int launch_ffn_prepack(sentry_ctx* ctx, const FfnArgs& a, void* packed, cudaStream_t st) {
     const sentry_ffn_desc& d = a.d;
-    const bool tc = ffn_tc_supported(d);
+    const bool tc = k_major(d);
     const int kc_pad = kc_pad_for(d);
     const size_t per = (size_t)kc_pad * d.D;
     const size_t pack_blocks = tc ? 2 * (size_t)d.n_lists * (kc_pad / 32) * (d.D / 64)
@@ -500,7 +507,7 @@ int launch_ffn_prepack(sentry_ctx* ctx, const FfnArgs& a, void* packed, cudaStre
 
 int launch_ffn_prepack_fp8(sentry_ctx* ctx, const sentry_ffn_desc& d, const uint8_t* W1q, const uint8_t* W2q, float s1,
                            float s2, const int32_t* kept, void* packed, cudaStream_t st) {
-    const bool tc = ffn_tc_supported(d);
+    const bool tc = k_major(d);
     const int kc_pad = kc_pad_for(d);
     const size_t per = (size_t)kc_pad * d.D;
     const unsigned grid = (unsigned)(2 * (size_t)d.n_lists * ((per + 255) / 256));
@@ -524,15 +531,17 @@ int launch_ffn_prepack_fp8(sentry_ctx* ctx, const sentry_ffn_desc& d, const uint
 
 int ffn_kc_pad(const sentry_ffn_desc& d) { return kc_pad_for(d); }
 int ffn_tile_rows(const sentry_ffn_desc& d) {
-    return ffn_tc_supported(d) ? kTcTileRows : kGenericTileRows;
+    return k_major(d) ? kTcTileRows : kGenericTileRows;
 }
 
 // The fused pair alone, on a row plan and materialised weights that are already in place.
 int launch_ffn_main(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1p, void* w2p, int kc_pad,
-                    int max_tiles, cudaStream_t st) {
+                    int max_tiles, void* hidden, cudaStream_t st) {
     const sentry_ffn_desc& d = a.d;
-    const bool tc = ffn_tc_supported(d);
-    if (tc) {
+    if (ffn_wide_supported(d)) {
+        int rc = launch_ffn_wide(ctx, a, plan, w1p, w2p, kc_pad, max_tiles, hidden, st);
+        if (rc != SENTRY_OK) return rc;
+    } else if (ffn_tc_supported(d)) {
         int rc = launch_ffn_tc(ctx, a, plan, w1p, w2p, kc_pad, max_tiles, st);
         if (rc != SENTRY_OK) return rc;
     } else {
@@ -540,21 +549,21 @@ int launch_ffn_main(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void
         LaunchScope ls(ctx, KS_FFN_MAIN, st);
         if (d.dtype == SENTRY_F32) {
             auto kern = ffn_generic_kernel<float>;
-            if (smem > 48 * 1024)
+            if (smem > 40 * 1024)   // (beside the static arrays)
                 SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             kern<<<max_tiles, kGenericThreads, smem, st>>>((const float*)a.X, (const float*)w1p,
                                                             (const float*)w2p, plan, d.n_lists,
                                                             d.T, d.D, d.k_c, kc_pad, (float*)a.Y);
         } else if (d.dtype == SENTRY_F16) {
             auto kern = ffn_generic_kernel<__half>;
-            if (smem > 48 * 1024)
+            if (smem > 40 * 1024)   // (beside the static arrays)
                 SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             kern<<<max_tiles, kGenericThreads, smem, st>>>(
                 (const __half*)a.X, (const __half*)w1p, (const __half*)w2p,
                 plan, d.n_lists, d.T, d.D, d.k_c, kc_pad, (__half*)a.Y);
         } else {
             auto kern = ffn_generic_kernel<__nv_bfloat16>;
-            if (smem > 48 * 1024)
+            if (smem > 40 * 1024)   // (beside the static arrays)
                 SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             kern<<<max_tiles, kGenericThreads, smem, st>>>(
                 (const __nv_bfloat16*)a.X, (const __nv_bfloat16*)w1p, (const __nv_bfloat16*)w2p,
@@ -569,17 +578,19 @@ int launch_ffn_main(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void
 // caller's materialised W1', W2' (launch_ffn_prepack) and only build the row plan.
 int launch_ffn(sentry_ctx* ctx, const FfnArgs& a, void* ws, size_t ws_bytes, const void* packed, cudaStream_t st) {
     const sentry_ffn_desc& d = a.d;
-    const bool tc = ffn_tc_supported(d);
+    const bool fused = ffn_tc_supported(d), tc = k_major(d);   // tc: K-major weights, 128-row tiles
     const int kc_pad = kc_pad_for(d);
-    if (d.dtype == SENTRY_FP8_E4M3 && (packed == nullptr || !tc)) return SENTRY_ERR_UNSUPPORTED;   // FP8: prepacked weights only
+    if (d.dtype == SENTRY_FP8_E4M3 && (packed == nullptr || !fused)) return SENTRY_ERR_UNSUPPORTED;   // FP8: prepacked weights only
     FfnWs w = carve(d, kc_pad, ws, ws_bytes, packed == nullptr);
-    if (!w.ok) return SENTRY_ERR_WORKSPACE;
+    const size_t h_at = align_up(w.used, 256), h_bytes = ffn_hidden_bytes(d, tiles_bound(d));
+    if (!w.ok || h_at + h_bytes > ws_bytes) return SENTRY_ERR_WORKSPACE;
+    void* hidden = (uint8_t*)ws + h_at;
     if (packed != nullptr) {
         w.w1p = const_cast<void*>(packed);
         w.w2p = (uint8_t*)w.w1p + packed_half_bytes(d, kc_pad);
     }
     const int tile_rows = tc ? kTcTileRows : kGenericTileRows;
-    if (tc && a.ids != nullptr) {
+    if (fused && a.ids != nullptr) {   // the fused kernel writes the zero rows
         w.plan.zero_ids = a.ids;
         w.plan.zero_masks = a.masks;
         w.plan.n_rows = d.B * d.T;
@@ -587,9 +598,9 @@ int launch_ffn(sentry_ctx* ctx, const FfnArgs& a, void* ws, size_t ws_bytes, con
 
     {
         const size_t per = (size_t)kc_pad * d.D;
-        // plain-ALU kernel: enough zero-fill blocks to cover the GPU a few times over when the batch is small
-        int zsplit = tc ? 0 : (4 * ctx->sm_count + d.B - 1) / d.B;
-        if (!tc && zsplit < 1) zsplit = 1;
+        // other kernels: enough zero-fill blocks to cover the GPU a few times over when the batch is small
+        int zsplit = fused ? 0 : (4 * ctx->sm_count + d.B - 1) / d.B;
+        if (!fused && zsplit < 1) zsplit = 1;
         if (zsplit > 32) zsplit = 32;
         const size_t pack_blocks = packed != nullptr ? 0
                                    : (tc ? 2 * (size_t)d.n_lists * (kc_pad / 32) * (d.D / 64)
@@ -606,7 +617,6 @@ int launch_ffn(sentry_ctx* ctx, const FfnArgs& a, void* ws, size_t ws_bytes, con
 #undef PREPARE
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
-    const long long rows = (long long)d.B * d.T;
-    const int max_tiles = (int)((rows + tile_rows - 1) / tile_rows) + d.n_lists;
-    return launch_ffn_main(ctx, a, w.plan, w.w1p, w.w2p, kc_pad, max_tiles, st);
+    const int max_tiles = (int)tiles_bound(d);
+    return launch_ffn_main(ctx, a, w.plan, w.w1p, w.w2p, kc_pad, max_tiles, hidden, st);
 }

@@ -22,9 +22,20 @@ struct FfnPlan {
     int n_rows, Tlen;
 };
 
-// The fused pair alone, on a row plan and materialised weights that are already in place.
+// The pair alone, on a row plan and materialised weights that are already in place.  hidden: ffn_hidden_bytes of scratch.
 int launch_ffn_main(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1p, void* w2p, int kc_pad,
-                    int max_tiles, cudaStream_t st);
+                    int max_tiles, void* hidden, cudaStream_t st);
+size_t ffn_hidden_bytes(const sentry_ffn_desc& d, long long max_tiles);
+// ffn_tc.cu / ffn_wide.cu: the tensor-core forms, fused for d_model 128, 256, 384 and as two GEMMs for other multiples of 64
+bool ffn_tc_supported(const sentry_ffn_desc& d);
+int ffn_tc_kc_pad(int D, int k_c);
+int launch_ffn_tc(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c, int kc_pad, int max_tiles,
+                  cudaStream_t st);
+bool ffn_wide_supported(const sentry_ffn_desc& d);
+int ffn_wide_kc_pad(int k_c);
+size_t ffn_wide_hidden_bytes(int kc_pad, long long max_tiles);
+int launch_ffn_wide(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c, int kc_pad, int max_tiles,
+                    void* hidden, cudaStream_t st);
 
 #ifdef __CUDACC__
 // Locate tile `tile` -> list l, offset of its first row in rowidx, and its row count;

@@ -127,24 +127,6 @@ static __device__ __noinline__ bool wait_each_slow(uint32_t b0, uint32_t p0, uin
     return ok;
 }
 
-// End of a CTA: if any wait ran out, raise the status bit and give copies and UMMAs that may
-// still be in flight time to land before shared memory and TMEM go away; then free the TMEM.
-__device__ __forceinline__ void cta_teardown(volatile int* abort_flag, unsigned int* status, uint32_t tmem,
-                                             uint32_t tmem_cols) {
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    if (*abort_flag) {
-        if (threadIdx.x == 0) atomicOr(status, SENTRY_STATUS_BIT_TIMEOUT);
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000LL) __nanosleep(1000);
-        __syncthreads();
-    }
-    if ((threadIdx.x >> 5) == 0) {
-        ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem, tmem_cols);
-    }
-}
-
 // F16: X, W and Y are IEEE half instead of bf16.  FP8: X and the weights are e4m3 bytes with
 // per-tensor scales, the hidden activations are requantised to e4m3 (gelu(acc * a_scale) * h_inv),
 // Y = acc * y_scale is stored as bf16.
@@ -699,7 +681,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__
         ptx::bulk_store_wait();   // the zeros have been read (and the rows are written before the grid ends)
     }
 
-    cta_teardown(abort_flag, status, tmem, kTmemCols);
+    tc_cta_teardown(abort_flag, status, tmem, kTmemCols);
 }
 
 // One CTA that waits, through the same bounded wait as the kernels above, on a barrier nobody
@@ -727,7 +709,7 @@ __global__ void __launch_bounds__(128, 1) wait_expiry_selftest_kernel(long long 
     // must be released by the abort flag that warp 1 raises
     const long long limit = (threadIdx.x >> 5) == 1 ? limit_cycles : ptx::kWaitLimitCycles;
     (void)ptx::mbar_wait(ptx::smem_u32(&never), 0u, abort_flag, limit);
-    cta_teardown(abort_flag, status, tmem, 32);
+    tc_cta_teardown(abort_flag, status, tmem, 32);
 }
 
 template <int D, bool F16>

@@ -291,6 +291,7 @@ struct MoeWs {
     int32_t *counts, *cursor;
     void* staged;
     void* packed;
+    void* hidden;
     bool ok;
     size_t used;
 };
@@ -301,6 +302,11 @@ sentry_ffn_desc as_ffn_desc(const sentry_moe_desc& m) {
     d.T = 1;   // the row count of the plan is N * top_k; the fused-pair kernels read it from the plan
     d.D = m.D; d.F = m.F; d.k_c = m.k_c; d.n_lists = m.E; d.dtype = m.dtype;
     return d;
+}
+
+long long tiles_bound(const sentry_moe_desc& m) {
+    const int tile_rows = ffn_tile_rows(as_ffn_desc(m));
+    return ((long long)m.N * m.top_k + tile_rows - 1) / tile_rows + m.E;
 }
 
 MoeWs carve(const sentry_moe_desc& m, void* ws, size_t bytes, bool with_weights) {
@@ -321,6 +327,7 @@ MoeWs carve(const sentry_moe_desc& m, void* ws, size_t bytes, bool with_weights)
     w.cursor = w.counts ? w.counts + m.E : nullptr;
     w.staged = a.take<uint8_t>(slots * m.D * esz);
     w.packed = with_weights ? a.take<uint8_t>(ffn_packed_bytes(as_ffn_desc(m))) : nullptr;
+    w.hidden = a.take<uint8_t>(ffn_hidden_bytes(as_ffn_desc(m), tiles_bound(m)));
     w.ok = a.ok;
     w.used = a.off;
     return w;
@@ -378,10 +385,10 @@ int launch_moe_ffn(sentry_ctx* ctx, const MoeArgs& m, void* ws, size_t ws_bytes,
     a.Y = w.staged;
     a.status = m.status;
     const int kc_pad = ffn_kc_pad(fd);
-    const int max_tiles = (int)((slots + tile_rows - 1) / tile_rows) + d.E;
+    const int max_tiles = (int)tiles_bound(d);
     void* w1p = const_cast<void*>(packed);
     void* w2p = (uint8_t*)w1p + ffn_packed_bytes(fd) / 2;
-    int rc = launch_ffn_main(ctx, a, w.plan, w1p, w2p, kc_pad, max_tiles, st);
+    int rc = launch_ffn_main(ctx, a, w.plan, w1p, w2p, kc_pad, max_tiles, w.hidden, st);
     if (rc != SENTRY_OK) return rc;
 
     {

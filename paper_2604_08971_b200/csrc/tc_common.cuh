@@ -123,6 +123,24 @@ __device__ __forceinline__ bool elect_one() {
 }
 
 
+// End of a CTA: if any wait ran out, raise the status bit and give copies and UMMAs that may
+// still be in flight time to land before shared memory and TMEM go away; then free the TMEM.
+__device__ __forceinline__ void tc_cta_teardown(volatile int* abort_flag, unsigned int* status, uint32_t tmem,
+                                             uint32_t tmem_cols) {
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    if (*abort_flag) {
+        if (threadIdx.x == 0) atomicOr(status, SENTRY_STATUS_BIT_TIMEOUT);
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000LL) __nanosleep(1000);
+        __syncthreads();
+    }
+    if ((threadIdx.x >> 5) == 0) {
+        ptx::tc_fence_after_sync();
+        ptx::tmem_dealloc(tmem, tmem_cols);
+    }
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,

@@ -1,0 +1,59 @@
+"""The channel-compacted FFN as two tensor-core GEMMs (d_model a multiple of 64 other than 128, 256, 384) against the
+float64 oracle, where its tiles can go wrong: one K block, column tiles that end half way, ragged channel counts, row
+tiles of several lists, more row tiles than the hidden buffer holds, and as the experts' FFN of a Sparse-MoE block."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2604_08971_b200 as sentry
+import synth
+from tests import parity
+from tests.parity import TOL
+
+pytestmark = pytest.mark.gpu
+
+
+def n_s_of(tv):
+    return sentry.num_active_queries(tv, 5)
+
+
+def _w(name, dtype, B, lengths, D, F, k_c, rule="cycle7"):
+    return synth.Workload(name, dtype, B, lengths, D, 4, 2, 16, F, 2, k_c, rule, 7, w_std=0.05)
+
+
+@pytest.mark.parametrize("w", [
+    _w("wide_d64_one_row", "bf16", 1, (1, 1, 1), 64, 128, 8),
+    _w("wide_d192_ragged", "bf16", 9, (37, 5, 91), 192, 400, 201),
+    _w("wide_d768_lists", "bf16", 8, (61, 47, 20), 768, 1024, 300),
+    _w("wide_d1024_f16", "f16", 3, (40, 50, 39), 1024, 512, 129),
+    _w("wide_d320_turns", "bf16", 70, (100, 100, 100), 320, 256, 128, "all"),   # 165 row tiles: two turns of the buffer
+], ids=lambda w: w.name)
+def test_wide_ffn_matches_oracle(w):
+    sn = sentry.Sentry(0)
+    try:
+        inp = synth.generate(w, n_s_of)
+        _, kept_c = parity.gate_lists(sn, inp)
+        assert parity.ffn_parity(sn, inp, kept_c) <= TOL[w.dtype]
+        # materialised once: the same bits, and the same again
+        los, ids, masks = (parity.dev(inp.list_of_sample), parity.dev(inp.ids), parity.masks_dev(inp.masks))
+        X, W1, W2 = inp.X.cuda(), inp.W1.cuda(), inp.W2.cuda()
+        Y = sn.ffn_fwd(X, W1, W2, kept_c, los, ids, masks)
+        packed = sn.ffn_prepack(W1, W2, kept_c)
+        Y2 = sn.ffn_fwd_packed(X, packed, w.F, w.k_c, kept_c.shape[0], los, ids, masks)
+        assert torch.equal(Y, Y2) and sn.last_status() == 0
+    finally:
+        sn.close()
+
+
+def test_wide_moe_matches_oracle():
+    m = synth.generate_moe(300, 512, 256, 5, 2, 100, "bf16", seed=3, skew=1.0)
+    sn = sentry.Sentry(0)
+    try:
+        ids, wts = torch.from_numpy(m.expert_ids).cuda(), torch.from_numpy(m.expert_weights).cuda()
+        Y = sn.moe_ffn_fwd(m.X.cuda(), ids, wts, W1=m.W1.cuda(), W2=m.W2.cuda(), kept_channels=torch.from_numpy(m.kept).cuda())
+        want = oracle.moe_ffn(m.X, m.W1, m.W2, m.kept, m.expert_ids, m.expert_weights)
+        assert parity.rel_err(Y.float().cpu().numpy(), want, "bf16", np.ones(300, dtype=bool)) <= TOL["bf16"]
+        assert sn.last_status() == 0
+    finally:
+        sn.close()
