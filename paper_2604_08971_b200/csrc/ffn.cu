@@ -207,22 +207,24 @@ ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__
     }
     pb -= zero_blocks;
     if (layout == 1) {
-        // K-major copies for the tensor-core kernel, one 32-channel x 64-column tile per block,
-        // transposed through shared memory so that both the gather and the store touch whole
-        // sectors:  W1c[l][n][e] = W1[e][N[n]],  W2c[l][e][n] = W2[N[n]][e].
-        __shared__ T s_tile[64][33];
-        __shared__ int s_ch[32];
-        const int tiles_n = kc_pad / 32, tiles_e = D / 64;
+        // K-major copies for the tensor-core kernels, one tile of 64 channels x 64 columns per block, transposed through
+        // shared memory:  W1c[l][n][e] = W1[e][N[n]],  W2c[l][e][n] = W2[N[n]][e].  Bound by latency (a few MB in all), so
+        // a thread has all its loads in flight at once: 16 single elements of W1 (kept columns are scattered), 16-byte
+        // pieces of W2's rows; both copies are written 16 bytes at a time.
+        constexpr int VEC = 16 / (int)sizeof(T);           // elements of a 16-byte piece
+        constexpr int PITCH = 64 + (sizeof(T) == 1 ? 4 : 2);   // elements; odd number of words
+        __shared__ __align__(16) T s_tile[64 * PITCH];
+        __shared__ int s_ch[64];
+        const int tiles_n = kc_pad / 64, tiles_e = D / 64;
         const size_t per_list = (size_t)tiles_n * tiles_e;
         const int which = (int)(pb / (per_list * n_lists));
         pb -= (size_t)which * per_list * n_lists;
         const int l = (int)(pb / per_list);
         const int tn = (int)((pb % per_list) / tiles_e), te = (int)(pb % tiles_e);
-        const int n0 = tn * 32, e0 = te * 64;
+        const int n0 = tn * 64, e0 = te * 64;
         const T* W1l = W1 + (size_t)l * w_stride;
         const T* W2l = W2 + (size_t)l * w_stride;
-        const int tx = threadIdx.x & 31, wy = threadIdx.x >> 5;   // 8 warps
-        if (threadIdx.x < 32) {
+        if (threadIdx.x < 64) {
             const int n = n0 + threadIdx.x;
             int ch = -1;
             if (n < k_c) {
@@ -236,25 +238,52 @@ ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__
         }
         __syncthreads();
         const T zero = from_f32<T>(0.f);
+        T* dst;
+        size_t ld;
         if (which == 0) {
-            const int ch = s_ch[tx];
-            for (int ee = wy; ee < 64; ee += 8)
-                s_tile[ee][tx] = ch >= 0 ? W1l[(size_t)(e0 + ee) * F + ch] : zero;
-            __syncthreads();
-            T* dst = out1 + ((size_t)l * kc_pad + n0) * D + e0;
-            for (int nn = wy; nn < 32; nn += 8) {
-                dst[(size_t)nn * D + tx] = s_tile[tx][nn];
-                dst[(size_t)nn * D + 32 + tx] = s_tile[32 + tx][nn];
+            // s_tile[e][n]
+            const int tx = threadIdx.x & 31, wy = threadIdx.x >> 5;   // 8 warps
+            const int c0 = s_ch[tx], c1 = s_ch[tx + 32];
+            T v0[8], v1[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const T* row = W1l + (size_t)(e0 + wy + 8 * i) * F;
+                v0[i] = c0 >= 0 ? row[c0] : zero;
+                v1[i] = c1 >= 0 ? row[c1] : zero;
             }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                s_tile[(wy + 8 * i) * PITCH + tx] = v0[i];
+                s_tile[(wy + 8 * i) * PITCH + tx + 32] = v1[i];
+            }
+            dst = out1 + ((size_t)l * kc_pad + n0) * D + e0;
+            ld = D;
         } else {
-            for (int nn = wy; nn < 32; nn += 8) {
+            // s_tile[n][e]
+            for (int i = threadIdx.x; i < 64 * 64 / VEC; i += 256) {
+                const int nn = i / (64 / VEC), c = i % (64 / VEC);
                 const int ch = s_ch[nn];
-                s_tile[tx][nn] = ch >= 0 ? W2l[(size_t)ch * D + e0 + tx] : zero;
-                s_tile[32 + tx][nn] = ch >= 0 ? W2l[(size_t)ch * D + e0 + 32 + tx] : zero;
+                uint4 v = make_uint4(0, 0, 0, 0);
+                if (ch >= 0) {
+                    const T* src = W2l + (size_t)ch * D + e0 + c * VEC;
+                    v = *reinterpret_cast<const uint4*>(src);
+                }
+                const T* p8 = reinterpret_cast<const T*>(&v);
+#pragma unroll
+                for (int e = 0; e < VEC; ++e) s_tile[nn * PITCH + c * VEC + e] = p8[e];
             }
-            __syncthreads();
-            T* dst = out2 + ((size_t)l * D + e0) * kc_pad + n0;
-            for (int ee = wy; ee < 64; ee += 8) dst[(size_t)ee * kc_pad + tx] = s_tile[ee][tx];
+            dst = out2 + ((size_t)l * D + e0) * kc_pad + n0;
+            ld = kc_pad;
+        }
+        __syncthreads();
+        // column r of s_tile -> row r of the copy
+        for (int i = threadIdx.x; i < 64 * 64 / VEC; i += 256) {
+            const int r = i % 64, c = i / 64;
+            uint4 v;
+            T* p8 = reinterpret_cast<T*>(&v);
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) p8[e] = s_tile[(c * VEC + e) * PITCH + r];
+            *reinterpret_cast<uint4*>(dst + (size_t)r * ld + c * VEC) = v;
         }
         return;
     }
@@ -479,7 +508,7 @@ int launch_ffn_prepack(sentry_ctx* ctx, const FfnArgs& a, void* packed, cudaStre
     const bool tc = k_major(d);
     const int kc_pad = kc_pad_for(d);
     const size_t per = (size_t)kc_pad * d.D;
-    const size_t pack_blocks = tc ? 2 * (size_t)d.n_lists * (kc_pad / 32) * (d.D / 64)
+    const size_t pack_blocks = tc ? 2 * (size_t)d.n_lists * (kc_pad / 64) * (d.D / 64)
                                   : 2 * (size_t)d.n_lists * ((per + 255) / 256);
     uint8_t* w1p = (uint8_t*)packed;
     uint8_t* w2p = w1p + packed_half_bytes(d, kc_pad);
@@ -603,7 +632,7 @@ int launch_ffn(sentry_ctx* ctx, const FfnArgs& a, void* ws, size_t ws_bytes, con
         if (!fused && zsplit < 1) zsplit = 1;
         if (zsplit > 32) zsplit = 32;
         const size_t pack_blocks = packed != nullptr ? 0
-                                   : (tc ? 2 * (size_t)d.n_lists * (kc_pad / 32) * (d.D / 64)
+                                   : (tc ? 2 * (size_t)d.n_lists * (kc_pad / 64) * (d.D / 64)
                                          : 2 * (size_t)d.n_lists * ((per + 255) / 256));
         const bool grouped = d.B >= kGroupPlanB;
         const size_t plan_blocks = grouped ? ((size_t)d.B + 7) / 8 : (size_t)d.B;

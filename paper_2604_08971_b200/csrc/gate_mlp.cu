@@ -41,13 +41,26 @@ gate_eval_kernel(const float* __restrict__ zeta, const float* __restrict__ gamma
     for (int j0 = 0; j0 < hidden; j0 += jc) {
         const int nj = min(jc, hidden - j0);
         __syncthreads();
-        for (int u = warp; u < nu; u += 8) {       // a warp per unit: its pieces are contiguous
-            const float* src = W1 + ((size_t)(u0 + u) * hidden + j0) * M;
-            float* dst = s_par + u * stride;
-            for (int e = lane; e < nj * M; e += 32) dst[e] = src[e];
-            for (int e = lane; e < nj; e += 32) {
-                dst[jc * M + e] = b1[(size_t)(u0 + u) * hidden + j0 + e];
-                dst[jc * (M + 1) + e] = w2[(size_t)(u0 + u) * hidden + j0 + e];
+        if (jc == hidden) {                        // whole units: one contiguous piece, every thread's loads in flight at once
+            const float* src = W1 + (size_t)u0 * hidden * M;
+            const int hm = hidden * M;
+#pragma unroll 8
+            for (int e = threadIdx.x; e < nu * hm; e += 256) s_par[(e / hm) * stride + e % hm] = src[e];
+#pragma unroll 4
+            for (int e = threadIdx.x; e < nu * hidden; e += 256) {
+                const int u = e / hidden, j = e % hidden;
+                s_par[u * stride + hm + j] = b1[(size_t)u0 * hidden + e];
+                s_par[u * stride + hm + hidden + j] = w2[(size_t)u0 * hidden + e];
+            }
+        } else {
+            for (int u = warp; u < nu; u += 8) {   // a warp per unit
+                const float* src = W1 + ((size_t)(u0 + u) * hidden + j0) * M;
+                float* dst = s_par + u * stride;
+                for (int e = lane; e < nj * M; e += 32) dst[e] = src[e];
+                for (int e = lane; e < nj; e += 32) {
+                    dst[jc * M + e] = b1[(size_t)(u0 + u) * hidden + j0 + e];
+                    dst[jc * (M + 1) + e] = w2[(size_t)(u0 + u) * hidden + j0 + e];
+                }
             }
         }
         __syncthreads();
