@@ -418,9 +418,12 @@ SENTRY_API int sentry_project_out(sentry_ctx* ctx, const sentry_proj_desc* desc,
  *                           weights in tensor memory, two-pass softmax
  * Both split every softmax weight into a bf16 head and a bf16 remainder, so the
  * results agree to well below the bf16 rounding of the stored output.
- * SENTRY_ATTEND_AUTO (default) takes the one that measured faster for the
- * shape.  Other shapes: bf16 with longer T runs a score kernel and a streamed
- * warp-MMA kernel; fp32, Hq/Hk > 4, U > 48 or T > 8192 run on the plain ALUs. */
+ * Both take one CTA per (sample, KV head).  SENTRY_ATTEND_AUTO (default) takes
+ * the form that measured faster for the shape: WARP_MMA, or, where a CTA per
+ * group would leave SMs idle and for most longer T, four launches (scores,
+ * top-U, Eq. 6 rows, context rows) that spread over the whole GPU.  Otherwise
+ * bf16 with longer T runs a score kernel and a streamed warp-MMA kernel; fp32,
+ * Hq/Hk > 4, U > 48 or T > 8192 run on the plain ALUs. */
 #define SENTRY_OPT_ATTEND_KERNEL 1
 #define SENTRY_ATTEND_AUTO 0
 #define SENTRY_ATTEND_WARP_MMA 1
@@ -430,7 +433,8 @@ SENTRY_API int sentry_project_out(sentry_ctx* ctx, const sentry_proj_desc* desc,
  * 256-query blocks per (sample, KV group) (QUERY_BLOCKS) or from one CTA per
  * group with the group's K rows resident (PER_GROUP: K staged once instead of
  * once per query block; needs about a group per SM to pay).  AUTO: PER_GROUP
- * when B*Hk >= the number of SMs.  Same results either way. */
+ * when B*Hk >= the number of SMs, unless the four-launch form above is faster.
+ * Same results either way. */
 #define SENTRY_OPT_LONG_SELECT 2
 #define SENTRY_LONG_SELECT_AUTO 0
 #define SENTRY_LONG_SELECT_QUERY_BLOCKS 1

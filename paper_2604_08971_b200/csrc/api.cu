@@ -17,7 +17,23 @@ size_t attend_workspace_bytes(const sentry_attend_desc& d) {
     WsAlloc a(nullptr, 0);
     a.take<float>((size_t)d.B * d.k_h * d.T);
     a.take<int32_t>((size_t)d.B * d.k_h * U_max);
-    return a.off + 256;
+    const size_t split = attend_bf16_supported(d) || attend_f16_supported(d) ? attend_split_ws_bytes(d) : 0;
+    return a.off + split + 512;
+}
+
+// Which form 16-bit attention takes: a CTA per (sample, KV head) group, or four launches spread over all SMs.  Measured, the
+// CTA per group against the four launches, us per call:
+//   K and V of a group fit in shared memory: 64 groups of T = 1024, d = 32: 70 / 52, T = 512: 46 / 43; 128 groups 72 / 78
+//     and 46 / 50; d = 64: 128 groups of T = 256 58 / 45, 256 groups 67 / 70.  Below 16 groups a call is latency, and one
+//     launch does it all (2 groups of T = 768: 21 / 26).
+//   longer sequences (the sampled keys of several CTA waves stay in shared memory there): T = 2048, d = 32: 128 groups
+//     234 / 133, 384 groups 334 / 315, 512 groups 402 / 422; T = 4096, d = 16: 128 groups 343 / 219, 256 groups 366 / 388;
+//     d = 64: 800 groups of T = 2048 1935 / 1751.
+bool attend_split_faster(const sentry_attend_desc& d, int sm_count) {
+    const long long groups = (long long)d.B * d.Hk;
+    if (attend_bf16_gate_fusable(d) || attend_f16_gate_fusable(d))
+        return groups >= 16 && (d.d > 32 ? groups <= sm_count && d.T >= 256 : groups <= sm_count / 2 && d.T >= 512);
+    return d.d > 32 || groups <= (d.d > 16 ? 5LL * sm_count / 2 : 5LL * sm_count / 4);
 }
 
 int check_attend_desc(const sentry_attend_desc* d) {
@@ -326,12 +342,15 @@ static int attend_body(sentry_ctx* ctx, const sentry_attend_desc* desc, const vo
     SENTRY_ON_DEVICE(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     a.active_out_user = active_out;
+    const bool fast = attend_bf16_supported(*desc) || attend_f16_supported(*desc);
+    const bool split = fast && ctx->attend_kernel == SENTRY_ATTEND_AUTO && ctx->long_select == SENTRY_LONG_SELECT_AUTO &&
+                       attend_split_faster(*desc, ctx->sm_count);
     if (gate_scores != nullptr) {
         // inside the attention launch where that saves a launch worth saving: up to a few waves of
         // CTAs (beyond, the selection repeated in every CTA costs more than one small launch: +5 %
         // on B = 4096)
-        const bool inside = ctx->attend_kernel != SENTRY_ATTEND_TCGEN05 &&
-                            (attend_bf16_gate_fusable(*desc) || attend_f16_gate_fusable(*desc)) &&
+        const bool inside = ctx->attend_kernel != SENTRY_ATTEND_TCGEN05 && desc->Hq <= 64 &&
+                            (split || attend_bf16_gate_fusable(*desc) || attend_f16_gate_fusable(*desc)) &&
                             (long long)desc->B * desc->Hk <= 8LL * ctx->sm_count;
         if (inside) {   // the fused attention kernel selects the heads itself
             a.gate_scores = gate_scores; a.gate_S = gate_S; a.kept_out = kept_heads;
@@ -348,6 +367,7 @@ static int attend_body(sentry_ctx* ctx, const sentry_attend_desc* desc, const vo
     // AUTO takes the kernel that measured faster for the shape: at present the warp-MMA kernels
     // on every shape they support (the tcgen05 kernel is within 10-20 % on T >= 512)
     if (ctx->attend_kernel == SENTRY_ATTEND_TCGEN05 && attend_tc_supported(*desc)) rc = launch_attend_tc(ctx, a, st);
+    else if (split) rc = desc->dtype == SENTRY_F16 ? launch_attend_split_f16(ctx, a, ws, st) : launch_attend_split(ctx, a, ws, st);
     else rc = attend_bf16_supported(*desc)  ? launch_attend_bf16(ctx, a, st)
               : attend_f16_supported(*desc) ? launch_attend_f16(ctx, a, st)
                                             : launch_attend_generic(ctx, a, st);

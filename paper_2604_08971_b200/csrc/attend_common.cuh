@@ -95,6 +95,14 @@ __device__ __forceinline__ void fma_bf16_pair(float& acc_lo, float& acc_hi, uint
         : "r"(a), "r"(b));
 }
 
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32." ATT_PTX_TYPE "." ATT_PTX_TYPE ".f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
 // s = q . k / sqrt(d) for NH heads against one key row in shared memory; updates max and sum.
 template <int D, int NH>
 __device__ __forceinline__ void score_one_key(const uint32_t (&qw)[NH][D / 2], uint32_t row_addr_base, int row,

@@ -377,6 +377,10 @@ int launch_attend_tc(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st);
 bool attend_bf16_supported(const sentry_attend_desc& d);
 bool attend_bf16_gate_fusable(const sentry_attend_desc& d);
 int launch_attend_bf16(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st);
+// the four-launch form (attend_split.cu); takes what attend_bf16_supported takes, scratch from ws
+size_t attend_split_ws_bytes(const sentry_attend_desc& d);
+int launch_attend_split(sentry_ctx* ctx, const AttendArgs& a, WsAlloc& ws, cudaStream_t st);
+int launch_attend_split_f16(sentry_ctx* ctx, const AttendArgs& a, WsAlloc& ws, cudaStream_t st);
 // the same kernels compiled for IEEE-half tensors (attend_f16.cu, attend_long_f16.cu)
 bool attend_long_select_f16_supported(const sentry_attend_desc& d);
 int launch_attend_long_select_f16(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st);

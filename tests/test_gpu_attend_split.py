@@ -1,0 +1,60 @@
+"""16-bit attention in four launches (few groups, or sequences whose K and V do not fit in shared memory) against the
+float64 oracle, and its selections against the CTA-per-group kernels bit for bit: every head width, one and many parts of
+the keys, lists around the tile edges, tied scores and a NaN row."""
+import pytest
+import torch
+
+import paper_2604_08971_b200 as sentry
+import synth
+from tests import parity
+from tests.parity import TOL
+
+pytestmark = pytest.mark.gpu
+
+
+def n_s_of(tv):
+    return sentry.num_active_queries(tv, 5)
+
+
+def _w(name, dtype, B, lengths, Hq, Hk, d, k_h, rule="cycle7"):
+    return synth.Workload(name, dtype, B, lengths, 64, Hq, Hk, d, 128, k_h, 64, rule, 11 + d)
+
+
+@pytest.mark.parametrize("w", [
+    _w("split_d16_one_present", "bf16", 16, (1, 510, 1), 4, 1, 16, 3),            # T_v = 1 and 2 in some samples
+    _w("split_d16_parts", "bf16", 9, (1400, 1300, 1396), 8, 2, 16, 5),            # T = 4096, 16 keys each lane to select from
+    _w("split_d32_tile_edges", "bf16", 8, (127, 257, 129), 6, 2, 32, 4),          # score blocks of 128 end at each list's edge
+    _w("split_d32_f16", "f16", 16, (384, 385, 255), 8, 2, 32, 8, "all"),          # every head kept
+    _w("split_d32_long", "bf16", 2, (3000, 2500, 2500), 4, 1, 32, 2, "all"),      # T = 8000: 16 parts
+    _w("split_d64_few", "f16", 8, (100, 99, 57), 8, 4, 64, 3),                    # T = 256: one part
+    _w("split_d64_wide", "bf16", 70, (300, 200, 203), 4, 2, 64, 2),               # a warp per head to select
+], ids=lambda w: w.name)
+def test_four_launch_attention(w):
+    sn = sentry.Sentry(0)
+    try:
+        inp = synth.generate(w, n_s_of)
+        kept_h, _ = parity.gate_lists(sn, inp)
+        for mode in (0, 1) if w.T <= 1024 else (0,):
+            err, _ = parity.attend_parity(sn, inp, kept_h, None if w.B < 20 else range(0, w.B, 9), mode, full_batch=True)
+            assert err <= TOL[w.dtype], (w.name, mode, err)
+        ids, masks = parity.dev(inp.ids), parity.masks_dev(inp.masks)
+        tbl, offs = parity.dev(inp.sample_table), parity.dev(inp.table_offsets)
+        Q, K, V = inp.Q.cuda(), inp.K.cuda(), inp.V.cuda()
+        Q[0, :, 7:40] = Q[0, :, 7:8]      # equal queries, and below equal keys: ties at the threshold
+        K[0, :, 3:] = K[0, :, 3:4]
+        Q[1, 0, 5] = float("nan")
+        args = (Q, K, V, kept_h, ids, masks, tbl, offs)
+        O, act = sn.attend_fwd(*args, c=w.c, return_active=True)
+        assert sn.last_launch_count() == 4
+        sn.set_attend_kernel(sentry.ATTEND_WARP_MMA)
+        O1, act1 = sn.attend_fwd(*args, c=w.c, return_active=True)
+        assert torch.equal(act, act1)
+        assert torch.equal(O.isnan(), O1.isnan())
+        a, b = torch.nan_to_num(O.float()), torch.nan_to_num(O1.float())
+        assert (a - b).abs().max().item() <= TOL[w.dtype] * b.abs().max().item()
+        # the same rows given by the caller
+        sn.set_attend_kernel(sentry.ATTEND_AUTO)
+        O2 = sn.attend_fwd(*args, c=w.c, active_in=act)
+        assert torch.equal(torch.nan_to_num(O2.float()), torch.nan_to_num(O.float()))
+    finally:
+        sn.close()
