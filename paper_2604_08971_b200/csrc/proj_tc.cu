@@ -1,14 +1,19 @@
-// Projections of the pruned layer (Section 4.6, head pruning with GQA consistency) for bf16 on
-// the 5th-generation tensor cores.  One CTA per (sample, tile of 128 present tokens).
+// Projections of the pruned layer (Section 4.6, head pruning with GQA consistency) for bf16 on the 5th-generation tensor
+// cores.  One CTA per (sample, tile of 128 present tokens, part of at most 256 output columns), two CTAs per SM: while one
+// lists its tokens or stores its results, the other multiplies.
 //
-//   QKV   A = the tile's X rows, gathered once into shared memory (K-major, 128-byte swizzle).
-//         Every kept head, and K and V of every referenced KV group, is one "slice": its column
-//         block W[:, i d:(i+1) d] streams through a ring of TMA stages as it lies in memory (rows =
-//         d_model index, i.e. an MN-major B operand) and is multiplied into its own d columns of
-//         tensor memory.  Pruned heads and unreferenced groups are never fetched.
-//   OUT   A = the tile's rows of every kept head's attention output (d wide each); the slice of
-//         head h is the row block W_O[h d:(h+1) d, :], accumulated into one [128 x d_model] tile.
-// Warp 0 feeds the weight ring, warp 1 issues the UMMAs, warps 4-7 read the accumulators and store.
+//   QKV   Every kept head, and K and V of every referenced KV group, is one "slice" of d columns.  A stage of the ring
+//         holds 64 d_model indices of the tile's X rows (gathered, K-major) and of all the part's slices: their column
+//         blocks W[64 rows, i d:(i+1) d] as they lie in memory (rows = d_model index, i.e. an MN-major B operand), so one
+//         UMMA multiplies all of them and X is read from shared memory once per K step, not once per slice.  Pruned heads
+//         and unreferenced groups are never fetched.
+//   OUT   A stage holds one kept head: the tile's rows of its attention output (d wide) and the rows W_O[h d:(h+1) d] of
+//         the part's columns.
+// Warp 0 feeds the weights by TMA, warp 1 issues the UMMAs, warps 4-7 gather the rows and then store: 64 accumulator columns
+// at a time pass through shared memory so that eight lanes write 128 consecutive bytes.
+// Bound by the L2 reads (each tile streams its weights: 200 MB at B = 128, T = 512, D = 384 with 15 slices of 32).
+// Measured there, the whole layer 262 -> 206 us: one CTA per SM that loaded X, multiplied slice by slice and then stored
+// took 73 us for QKV and 61 for OUT.
 // Every wait is bounded; on expiry the CTA raises SENTRY_STATUS_BIT_TIMEOUT and unwinds.
 #include <cuda.h>
 
@@ -25,368 +30,381 @@
 
 namespace {
 
-constexpr int kPThreads = 256;
-constexpr int kPStages = 3;
+constexpr int kPThreads = 256, kPWarps = kPThreads / 32;
+constexpr int kPCols = 256;                    // output columns of a part: two CTAs share the 512 columns of tensor memory
+constexpr int kPRing = 96 * 1024;              // bytes of stages
+constexpr int kPMaxStages = 8;
+constexpr int kPSmem = kPRing + 1024;
 constexpr int kMaxSlicesTc = 96;
 
 struct ProjMisc {
-    uint64_t w_full[kPStages], w_empty[kPStages];
-    uint64_t acc_full, acc_empty;
+    uint64_t full[kPMaxStages], empty[kPMaxStages], acc_full;
     uint32_t tmem_base;
-    int abort_flag;
-    int n_slices;
+    int abort_flag, n_slices, counts[kPWarps];
     int kind[kMaxSlicesTc], idx[kMaxSlicesTc];   // QKV: 0 = Q head, 1 = K group, 2 = V group.  OUT: kept-list slot, head
+    uint16_t tok[128];                           // tokens of this tile
 };
 
+// The tile's tokens (present ones number 128 tt .. 128 tt + 127) to misc->tok; returns T_v.  Every warp walks a run of
+// 32-token pieces twice, the second time with the number of present tokens before it.  Complete behind the next barrier.
+__device__ __forceinline__ int list_tile(const int32_t* __restrict__ ids, int T, uint32_t mask, int tt, ProjMisc* misc) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int pieces = (T + 31) / 32, per = (pieces + kPWarps - 1) / kPWarps;
+    const int p0 = min(warp * per, pieces), p1 = min(p0 + per, pieces);
+    auto present = [&](int t) {
+        const int m = t < T ? __ldg(ids + t) : -1;
+        return m >= 0 && m < 32 && ((mask >> m) & 1u);
+    };
+    int mine = 0;
+#pragma unroll 4
+    for (int pc = p0; pc < p1; ++pc) mine += __popc(__ballot_sync(0xffffffffu, present(pc * 32 + lane)));
+    if (lane == 0) misc->counts[warp] = mine;
+    __syncthreads();
+    int at = -tt * 128, total = 0;
+#pragma unroll
+    for (int w = 0; w < kPWarps; ++w) { const int c = misc->counts[w]; total += c; if (w < warp) at += c; }
+    if (at >= 128 || at + mine <= 0) return total;
+#pragma unroll 4
+    for (int pc = p0; pc < p1; ++pc) {
+        const bool ok = present(pc * 32 + lane);
+        const unsigned bm = __ballot_sync(0xffffffffu, ok);
+        const int r = at + __popc(bm & ((1u << lane) - 1u));
+        if (ok && r >= 0 && r < 128) misc->tok[r] = (uint16_t)(pc * 32 + lane);
+        at += __popc(bm);
+    }
+    return total;
+}
+
+// Barriers and the slice list of sample b (warp 0; behind the caller's barrier).  Hk = 0: kept heads only.
+__device__ __forceinline__ void proj_setup(ProjMisc* misc, int stages, const int32_t* __restrict__ kept, int k_h, int Hq, int Hk,
+                                           unsigned int* status) {
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) {
+        for (int s = 0; s < stages; ++s) {
+            ptx::mbar_init(ptx::smem_u32(&misc->full[s]), 5);   // the TMA's expect, and the four gathering warps
+            ptx::mbar_init(ptx::smem_u32(&misc->empty[s]), 1);
+        }
+        ptx::mbar_init(ptx::smem_u32(&misc->acc_full), 1);
+        misc->abort_flag = 0;
+        ptx::fence_barrier_init();
+    }
+    int n = 0;
+    uint32_t groups = 0u;
+    for (int j0 = 0; j0 < k_h; j0 += 32) {
+        const int j = j0 + lane, h = j < k_h ? kept[j] : -1;
+        const bool ok = h >= 0 && h < Hq;
+        if (j < k_h && !ok) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+        const unsigned bm = __ballot_sync(0xffffffffu, ok);
+        if (ok) {
+            const int at = n + __popc(bm & ((1u << lane) - 1u));
+            misc->kind[at] = Hk > 0 ? 0 : j;
+            misc->idx[at] = h;
+        }
+        n += __popc(bm);
+        groups |= __reduce_or_sync(0xffffffffu, ok && Hk > 0 ? 1u << (h / (Hq / Hk)) : 0u);
+    }
+    for (int g = 0; g < Hk; ++g)
+        if ((groups >> g) & 1u) {
+            if (lane < 2) { misc->kind[n + lane] = 1 + lane; misc->idx[n + lane] = g; }
+            n += 2;
+        }
+    if (lane == 0) misc->n_slices = n;
+    ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), kPCols);
+    ptx::tmem_relinquish();
+}
+
+// Gathers CPR 16-byte chunks of 128 rows per stage by warps 4-7: src(step, row, chunk) is the address or null (zeros),
+// off(row, chunk) its place in the stage.  Returns false when a wait ran out.
+template <int CPR, class Src, class Off>
+__device__ __forceinline__ bool gather_steps(ProjMisc* misc, uint32_t ring, uint32_t stage_bytes, int stages, int steps, Src src,
+                                             Off off, volatile int* abort_flag) {
+    const int tl = threadIdx.x - 128, lag = min(stages - 1, 2);
+    int published = 0, p_slot = 0;
+    auto publish = [&](int pending) {
+        cp_async_wait_pending(pending);
+        ptx::fence_proxy_async_smem();
+        warp_arrive(&misc->full[p_slot]);
+        p_slot = p_slot + 1 == stages ? 0 : p_slot + 1;
+        ++published;
+    };
+    bool ok = true;
+    int slot = 0;
+    uint32_t phase = 1u;
+    for (int k = 0; k < steps; ++k) {
+        // a slot is refilled only when its step has been read, which needs every earlier step published
+        if (k >= stages)
+            while (published <= k - stages) publish(k - published - 1);
+        ok = warp_wait(&misc->empty[slot], phase, abort_flag);
+        if (!ok) break;
+#pragma unroll
+        for (int j = 0; j < CPR; ++j) {
+            const int i = tl + j * 128, r = i / CPR, cc = i % CPR;
+            const uint32_t dst = ring + slot * stage_bytes + off(r, cc);
+            const __nv_bfloat16* from = src(k, r, cc, j);
+            if (from != nullptr) ptx::cp_async_16(dst, from);
+            else asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
+        }
+        ptx::cp_async_commit();
+        if (k - published >= lag) publish(lag);
+        if (++slot == stages) { slot = 0; phase ^= 1u; }
+    }
+    while (ok && published < steps) publish(steps - published - 1);
+    ptx::cp_async_wait_all();
+    return ok;
+}
+
+// 64 accumulator columns of the warp's 32 rows, rounded, to the warp's 4 KB of shared memory: 16-byte chunk c of row r at
+// r * 128 + ((c ^ (r & 7)) << 4).
+__device__ __forceinline__ void acc_to_smem(uint32_t taddr, uint32_t buf) {
+    const int lane = threadIdx.x & 31;
+    uint32_t acc[64];
+    ptx::tmem_ld_32x32(taddr, reinterpret_cast<uint32_t(&)[32]>(acc[0]));
+    ptx::tmem_ld_32x32(taddr + 32, reinterpret_cast<uint32_t(&)[32]>(acc[32]));
+    ptx::tmem_ld_wait();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) w[e] = pack2(__uint_as_float(acc[8 * c + 2 * e]), __uint_as_float(acc[8 * c + 2 * e + 1]));
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(buf + lane * 128 + ((c ^ (lane & 7)) << 4)), "r"(w[0]),
+                     "r"(w[1]), "r"(w[2]), "r"(w[3])
+                     : "memory");
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ uint4 smem_chunk(uint32_t buf, int r, int c) {
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(buf + r * 128 + ((c ^ (r & 7)) << 4))
+                 : "memory");
+    return v;
+}
+
 // ------------------------------------------------------------------------------------- QKV
-// dynamic smem: X tile [D/64][128 x 128 B] | weight ring [kPStages][D x DH] | misc | valid list
+// grid B * tiles * parts (the parts of a tile together: the second one's X rows come from L2)
 template <int DH>
-__global__ void __launch_bounds__(kPThreads, 1)
+__global__ void __launch_bounds__(kPThreads, 2)
 proj_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __nv_bfloat16* __restrict__ X,
                    const int32_t* __restrict__ kept_heads, const int32_t* __restrict__ ids,
-                   const uint32_t* __restrict__ masks, int Tlen, int D, int Hq, int Hk, int k_h,
+                   const uint32_t* __restrict__ masks, int Tlen, int D, int Hq, int Hk, int k_h, int tiles, int parts_max,
                    __nv_bfloat16* __restrict__ Q, __nv_bfloat16* __restrict__ K, __nv_bfloat16* __restrict__ V,
                    unsigned int* status) {
-    grid_dependency_wait();
-    constexpr int RB = DH * 2;
-    constexpr int NS = 512 / DH;                    // slices whose accumulators fit in tensor memory at once
+    constexpr int RB = DH * 2, NS = kPCols / DH;    // bytes of a slice row; slices of a part
     extern __shared__ uint8_t smem_raw[];
-    __shared__ int red[66];
-    const uint32_t raw_addr = ptx::smem_u32(smem_raw);
-    const uint32_t base = (raw_addr + 1023u) & ~1023u;
-    uint8_t* smem = smem_raw + (base - raw_addr);
-    const int KB = D / 64;
-    const uint32_t stage_bytes = (uint32_t)D * RB;
-    const uint32_t xs = base, wsm = base + (uint32_t)KB * 16384u;
-    ProjMisc* misc = reinterpret_cast<ProjMisc*>(smem + (size_t)KB * 16384 + (size_t)kPStages * stage_bytes);
-    uint16_t* s_valid = reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(misc) + ((sizeof(ProjMisc) + 127) / 128) * 128);
+    __shared__ ProjMisc misc_s;
+    ProjMisc* misc = &misc_s;
+    const uint32_t ring = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     volatile int* abort_flag = &misc->abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles_per_sample = (Tlen + 127) / 128;
-    const int b = blockIdx.x / tiles_per_sample, tt = blockIdx.x % tiles_per_sample;
-
-    const int Tv = block_build_valid(ids, Tlen, masks[b], s_valid, red);
-    if (tt * 128 >= Tv) return;                      // no present token in this tile
+    const int part = blockIdx.x % parts_max, tile = blockIdx.x / parts_max, b = tile / tiles, tt = tile % tiles;
+    const int KB = D / 64;
+    grid_dependency_wait();
+    const int Tv = list_tile(ids, Tlen, masks[b], tt, misc);
+    if (tt * 128 >= Tv) return;                     // no present token in this tile
     const int n_rows = min(128, Tv - tt * 128);
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kPStages; ++s) {
-            ptx::mbar_init(ptx::smem_u32(&misc->w_full[s]), 1);
-            ptx::mbar_init(ptx::smem_u32(&misc->w_empty[s]), 1);
-        }
-        ptx::mbar_init(ptx::smem_u32(&misc->acc_full), 1);
-        ptx::mbar_init(ptx::smem_u32(&misc->acc_empty), 4);
-        misc->abort_flag = 0;
-        ptx::fence_barrier_init();
-        const int r = Hq / Hk;
-        int n = 0;
-        uint32_t groups = 0;
-        for (int j = 0; j < k_h; ++j) {
-            const int h = kept_heads[(size_t)b * k_h + j];
-            if (h < 0 || h >= Hq) { atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX); continue; }
-            misc->kind[n] = 0; misc->idx[n] = h; ++n;
-            groups |= 1u << (h / r);
-        }
-        for (int g = 0; g < Hk; ++g)
-            if ((groups >> g) & 1u) {
-                misc->kind[n] = 1; misc->idx[n] = g; ++n;
-                misc->kind[n] = 2; misc->idx[n] = g; ++n;
-            }
-        misc->n_slices = n;
-    }
-    if (warp == 0) {
-        ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), 512);
-        ptx::tmem_relinquish();
-    }
-    // the tile's X rows: 16-byte chunk ci of row r of block kb at  r * 128 + ((ci ^ (r & 7)) << 4)
-    for (int i = threadIdx.x; i < KB * 128 * 8; i += blockDim.x) {
-        const int kb = i / 1024, r = (i >> 3) & 127, ci = i & 7;
-        const uint32_t dst = xs + (uint32_t)kb * 16384u + (uint32_t)r * 128u + (uint32_t)((ci ^ (r & 7)) << 4);
-        if (r < n_rows) {
-            const int tok = s_valid[tt * 128 + r];
-            ptx::cp_async_16(dst, X + ((size_t)b * Tlen + tok) * D + kb * 64 + ci * 8);
-        } else {
-            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
-        }
-    }
-    ptx::cp_async_wait_all();
-    ptx::fence_proxy_async_smem();
+    if (warp == 0) proj_setup(misc, kPMaxStages, kept_heads + (size_t)b * k_h, k_h, Hq, Hk, status);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = misc->tmem_base;
-    const int n_slices = misc->n_slices;
-
-    if (warp == 0) {
-        // ------------------------------------------------------------ weight producer
-        bool ok = true;
-        for (int s = 0; s < n_slices && ok; ++s) {
-            const uint32_t st = (uint32_t)s % kPStages, use = (uint32_t)s / kPStages;
-            ok = warp_wait(&misc->w_empty[st], (use & 1u) ^ 1u, abort_flag);
-            if (!ok) break;
-            if (elect_one()) {
-                const int kind = misc->kind[s], idx = misc->idx[s];
-                const CUtensorMap* tm = kind == 0 ? &tm_q : (kind == 1 ? &tm_k : &tm_v);
-                const uint32_t bar = ptx::smem_u32(&misc->w_full[st]);
-                ptx::mbar_arrive_expect_tx(bar, stage_bytes);
-                for (int kb = 0; kb < KB; ++kb)
-                    ptx::tma_load_2d(wsm + st * stage_bytes + (uint32_t)kb * 64u * RB, tm, idx * DH, kb * 64, bar);
-            }
-            __syncwarp();
-        }
-    } else if (warp == 1) {
-        // ---------------------------------------------------------------- UMMA issuer
-        constexpr uint32_t idesc = PROJ_IDESC(128, DH, false, true);
-        bool ok = true;
-        for (int s = 0; s < n_slices && ok; ++s) {
-            const uint32_t st = (uint32_t)s % kPStages, use = (uint32_t)s / kPStages;
-            const int grp = s / NS;
-            if (s % NS == 0 && grp > 0) ok = warp_wait(&misc->acc_empty, ((uint32_t)(grp - 1)) & 1u, abort_flag);
-            if (ok) ok = warp_wait(&misc->w_full[st], use & 1u, abort_flag);
-            if (!ok) break;
-            ptx::tc_fence_after_sync();
-            if (elect_one()) {
-                const uint32_t d_tm = tmem + (uint32_t)(s % NS) * DH;
-                for (int kb = 0; kb < KB; ++kb) {
-#pragma unroll
-                    for (int ks = 0; ks < 4; ++ks) {
-                        const uint64_t a = ptx::umma_smem_desc_sw128(xs + (uint32_t)kb * 16384u + ks * 32);
-                        const uint64_t bd = ptx::umma_smem_desc_rows(
-                            wsm + st * stage_bytes + (uint32_t)(kb * 64 + ks * 16) * RB, RB);
-                        ptx::umma_bf16(d_tm, a, bd, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+    // equal shares of the slices for the parts that are needed
+    const int n_all = misc->n_slices, parts = (n_all + NS - 1) / NS, per = parts > 0 ? (n_all + parts - 1) / parts : 0;
+    const int s0 = part * per, n_sl = min(n_all - s0, per);
+    if (n_sl > 0) {
+        const uint32_t stage_bytes = 16384u + (uint32_t)n_sl * 64u * RB;
+        const int stages = min(kPRing / (int)stage_bytes, kPMaxStages);
+        if (warp == 0) {
+            // -------------------------------------------------------- weights
+            bool ok = true;
+            int slot = 0;
+            uint32_t phase = 1u;
+            for (int kb = 0; kb < KB && ok; ++kb) {
+                ok = warp_wait(&misc->empty[slot], phase, abort_flag);
+                if (!ok) break;
+                if (elect_one()) {
+                    const uint32_t bar = ptx::smem_u32(&misc->full[slot]), dst = ring + slot * stage_bytes + 16384u;
+                    ptx::mbar_arrive_expect_tx(bar, (uint32_t)n_sl * 64u * RB);
+                    for (int j = 0; j < n_sl; ++j) {
+                        const int kind = misc->kind[s0 + j];
+                        ptx::tma_load_2d(dst + (uint32_t)j * 64u * RB, kind == 0 ? &tm_q : (kind == 1 ? &tm_k : &tm_v),
+                                         misc->idx[s0 + j] * DH, kb * 64, bar);
                     }
                 }
-                ptx::umma_commit(ptx::smem_u32(&misc->w_empty[st]));
-                if (s % NS == NS - 1 || s == n_slices - 1) ptx::umma_commit(ptx::smem_u32(&misc->acc_full));
+                __syncwarp();
+                if (++slot == stages) { slot = 0; phase ^= 1u; }
             }
-            __syncwarp();
-        }
-    } else if (warp >= 4) {
-        // ------------------------------------------------------------------- epilogue
-        const int quarter = warp & 3;
-        const int row = quarter * 32 + lane;
-        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-        const int tok = row < n_rows ? (int)s_valid[tt * 128 + row] : -1;
-        const int n_groups = (n_slices + NS - 1) / NS;
-        bool ok = true;
-        for (int grp = 0; grp < n_groups && ok; ++grp) {
-            ok = warp_wait(&misc->acc_full, (uint32_t)grp & 1u, abort_flag);
-            if (!ok) break;
-            ptx::tc_fence_after_sync();
-            const int s_end = min(n_slices, (grp + 1) * NS);
-            for (int s = grp * NS; s < s_end; ++s) {
-                uint32_t acc[DH];
-                if constexpr (DH == 16) {
-                    ptx::tmem_ld_32x16(lane_base + (uint32_t)(s % NS) * DH, reinterpret_cast<uint32_t(&)[16]>(acc));
-                } else {
+        } else if (warp == 1) {
+            // ---------------------------------------------------------- UMMA issuer
+            const uint32_t idesc = PROJ_IDESC(128, n_sl * DH, false, true);
+            bool ok = true;
+            int slot = 0;
+            uint32_t phase = 0u;
+            for (int kb = 0; kb < KB && ok; ++kb) {
+                ok = warp_wait(&misc->full[slot], phase, abort_flag);
+                if (!ok) break;
+                ptx::tc_fence_after_sync();
+                if (elect_one()) {
+                    const uint32_t a = ring + slot * stage_bytes, w = a + 16384u;
 #pragma unroll
-                    for (int j = 0; j < DH / 32; ++j)
-                        ptx::tmem_ld_32x32(lane_base + (uint32_t)(s % NS) * DH + 32 * j,
-                                           reinterpret_cast<uint32_t(&)[32]>(acc[32 * j]));
+                    for (int ks = 0; ks < 4; ++ks)
+                        ptx::umma_bf16(tmem, ptx::umma_smem_desc_sw128(a + ks * 32),
+                                       ptx::umma_smem_desc_rows(w + (uint32_t)ks * 16u * RB, RB, 64u * RB), idesc,
+                                       (kb > 0 || ks > 0) ? 1u : 0u);
+                    ptx::umma_commit(ptx::smem_u32(&misc->empty[slot]));
+                    if (kb == KB - 1) ptx::umma_commit(ptx::smem_u32(&misc->acc_full));
                 }
-                ptx::tmem_ld_wait();
-                if (tok >= 0) {
-                    const int kind = misc->kind[s], idx = misc->idx[s];
-                    __nv_bfloat16* dst = kind == 0 ? Q + (((size_t)b * Hq + idx) * Tlen + tok) * DH
-                                                   : (kind == 1 ? K : V) + (((size_t)b * Hk + idx) * Tlen + tok) * DH;
+                __syncwarp();
+                if (++slot == stages) { slot = 0; phase ^= 1u; }
+            }
+        } else if (warp >= 4) {
+            const __nv_bfloat16* rows[8];          // this thread's chunk of its rows
 #pragma unroll
-                    for (int cc = 0; cc < DH / 8; ++cc) {
-                        uint4 v;
-                        v.x = pack2(__uint_as_float(acc[8 * cc]), __uint_as_float(acc[8 * cc + 1]));
-                        v.y = pack2(__uint_as_float(acc[8 * cc + 2]), __uint_as_float(acc[8 * cc + 3]));
-                        v.z = pack2(__uint_as_float(acc[8 * cc + 4]), __uint_as_float(acc[8 * cc + 5]));
-                        v.w = pack2(__uint_as_float(acc[8 * cc + 6]), __uint_as_float(acc[8 * cc + 7]));
-                        reinterpret_cast<uint4*>(dst)[cc] = v;
+            for (int j = 0; j < 8; ++j) {
+                const int r = (threadIdx.x - 128 + j * 128) / 8;
+                rows[j] = r < n_rows ? X + ((size_t)b * Tlen + misc->tok[r]) * D + (threadIdx.x & 7) * 8 : nullptr;
+            }
+            const bool ok = gather_steps<8>(
+                misc, ring, stage_bytes, stages, KB,
+                [&](int kb, int, int, int j) { return rows[j] != nullptr ? rows[j] + kb * 64 : nullptr; },
+                [](int r, int cc) { return (uint32_t)(r * 128 + ((cc ^ (r & 7)) << 4)); }, abort_flag);
+            // ------------------------------------------------------------- results
+            if (ok && warp_wait(&misc->acc_full, 0u, abort_flag)) {
+                ptx::tc_fence_after_sync();
+                const int quarter = warp & 3, c = lane & 7;
+                const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16), buf = ring + quarter * 4096u;
+                for (int c0 = 0; c0 < n_sl * DH; c0 += 64) {
+                    acc_to_smem(taddr + c0, buf);
+                    const int s = (c0 + c * 8) / DH;                   // the slice of this lane's chunk
+                    if (s < n_sl) {
+                        const int kind = misc->kind[s0 + s], idx = misc->idx[s0 + s];
+                        __nv_bfloat16* dst = kind == 0 ? Q + ((size_t)b * Hq + idx) * Tlen * DH
+                                                       : (kind == 1 ? K : V) + ((size_t)b * Hk + idx) * Tlen * DH;
+                        dst += (c * 8) % DH;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int r = i * 4 + (lane >> 3);
+                            if (quarter * 32 + r < n_rows)
+                                *reinterpret_cast<uint4*>(dst + (size_t)misc->tok[quarter * 32 + r] * DH) = smem_chunk(buf, r, c);
+                        }
                     }
+                    __syncwarp();
                 }
             }
-            ptx::tc_fence_before_sync();
-            warp_arrive(&misc->acc_empty);
         }
     }
-
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    if (*abort_flag) {
-        if (threadIdx.x == 0) atomicOr(status, SENTRY_STATUS_BIT_TIMEOUT);
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000LL) __nanosleep(1000);
-        __syncthreads();
-    }
-    if (warp == 0) {
-        ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem, 512);
-    }
+    tc_cta_teardown(abort_flag, status, tmem, kPCols);
 }
 
 // ------------------------------------------------------------------------------------- OUT
-// dynamic smem: A tiles [k_h][128 x DH] | weight ring [kPStages][DH x D] | misc | valid list
+// grid B * tiles * parts; every CTA also clears its columns of the absent ones among token positions 128 tt ..
 template <int DH>
-__global__ void __launch_bounds__(kPThreads, 1)
+__global__ void __launch_bounds__(kPThreads, 2)
 proj_out_tc_kernel(const __grid_constant__ CUtensorMap tm_o, const __nv_bfloat16* __restrict__ A,
                    const int32_t* __restrict__ kept_heads, const int32_t* __restrict__ ids,
-                   const uint32_t* __restrict__ masks, int Tlen, int D, int Hq, int k_h,
+                   const uint32_t* __restrict__ masks, int Tlen, int D, int Hq, int k_h, int tiles, int parts,
                    __nv_bfloat16* __restrict__ out, unsigned int* status) {
-    grid_dependency_wait();
     using S = Sw<DH>;
-    constexpr int RB = DH * 2;
+    constexpr uint32_t RB = DH * 2, kBox = DH * 128;   // bytes of an A row; of 64 columns of a head's rows of W_O
     extern __shared__ uint8_t smem_raw[];
-    __shared__ int red[66];
-    const uint32_t raw_addr = ptx::smem_u32(smem_raw);
-    const uint32_t base = (raw_addr + 1023u) & ~1023u;
-    uint8_t* smem = smem_raw + (base - raw_addr);
-    const int NC = D / 64;
-    const uint32_t stage_bytes = (uint32_t)D * RB;
-    const uint32_t a_tile = 128u * RB;
-    const uint32_t as = base, wsm = base + (uint32_t)k_h * a_tile;
-    ProjMisc* misc = reinterpret_cast<ProjMisc*>(smem + (size_t)k_h * a_tile + (size_t)kPStages * stage_bytes);
-    uint16_t* s_valid = reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(misc) + ((sizeof(ProjMisc) + 127) / 128) * 128);
+    __shared__ ProjMisc misc_s;
+    ProjMisc* misc = &misc_s;
+    const uint32_t ring = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     volatile int* abort_flag = &misc->abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles_per_sample = (Tlen + 127) / 128;
-    const int b = blockIdx.x / tiles_per_sample, tt = blockIdx.x % tiles_per_sample;
+    const int part = blockIdx.x % parts, tile = blockIdx.x / parts, b = tile / tiles, tt = tile % tiles;
+    const int per = (D / 64 + parts - 1) / parts, box0 = part * per, n_box = min(D / 64 - box0, per);
+    grid_dependency_wait();
     const uint32_t mask = masks[b];
-
-    // rows of absent tokens are zero: every CTA clears those among its 128 token positions
     {
-        const int vpr = D / 8;
-        for (int i = threadIdx.x; i < 128 * vpr; i += blockDim.x) {
-            const int t = tt * 128 + i / vpr;
-            if (t >= Tlen) break;
-            const int m = ids[t];
-            if (!(m >= 0 && m < 32 && ((mask >> m) & 1u)))
-                reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + t) * D)[i % vpr] = make_uint4(0, 0, 0, 0);
+        const int t = tt * 128 + warp * 16 + (lane & 15), m = t < Tlen ? ids[t] : -1;
+        unsigned gone = __ballot_sync(0xffffffffu, t < Tlen && !(m >= 0 && m < 32 && ((mask >> m) & 1u))) & 0xffffu;
+        for (; gone; gone &= gone - 1) {
+            uint4* dst = reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + tt * 128 + warp * 16 + __ffs(gone) - 1) * D) + box0 * 8;
+            if (lane < n_box * 8) dst[lane] = make_uint4(0, 0, 0, 0);
         }
     }
-    const int Tv = block_build_valid(ids, Tlen, mask, s_valid, red);
+    const int Tv = list_tile(ids, Tlen, mask, tt, misc);
     if (tt * 128 >= Tv) return;
     const int n_rows = min(128, Tv - tt * 128);
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kPStages; ++s) {
-            ptx::mbar_init(ptx::smem_u32(&misc->w_full[s]), 1);
-            ptx::mbar_init(ptx::smem_u32(&misc->w_empty[s]), 1);
-        }
-        ptx::mbar_init(ptx::smem_u32(&misc->acc_full), 1);
-        misc->abort_flag = 0;
-        ptx::fence_barrier_init();
-        int n = 0;
-        for (int j = 0; j < k_h; ++j) {
-            const int h = kept_heads[(size_t)b * k_h + j];
-            if (h < 0 || h >= Hq) { atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX); continue; }
-            misc->kind[n] = j; misc->idx[n] = h; ++n;
-        }
-        misc->n_slices = n;
-    }
-    if (warp == 0) {
-        ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), 512);
-        ptx::tmem_relinquish();
-    }
-    // the tile's rows of every kept head's attention output
-    for (int i = threadIdx.x; i < k_h * 128 * S::CPR; i += blockDim.x) {
-        const int j = i / (128 * S::CPR), r = (i / S::CPR) % 128, cc = i % S::CPR;
-        const uint32_t dst = as + (uint32_t)j * a_tile + S::off(r, cc);
-        if (r < n_rows) {
-            const int tok = s_valid[tt * 128 + r];
-            ptx::cp_async_16(dst, A + (((size_t)b * k_h + j) * Tlen + tok) * DH + cc * 8);
-        } else {
-            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
-        }
-    }
-    ptx::cp_async_wait_all();
-    ptx::fence_proxy_async_smem();
+    if (warp == 0) proj_setup(misc, kPMaxStages, kept_heads + (size_t)b * k_h, k_h, Hq, 0, status);
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::tc_fence_after_sync();
     const uint32_t tmem = misc->tmem_base;
-    const int n_slices = misc->n_slices;
-
+    const int n_sl = misc->n_slices;
+    const uint32_t stage_bytes = 128u * RB + (uint32_t)n_box * kBox;
+    const int stages = min(kPRing / (int)stage_bytes, kPMaxStages);
     if (warp == 0) {
         bool ok = true;
-        for (int s = 0; s < n_slices && ok; ++s) {
-            const uint32_t st = (uint32_t)s % kPStages, use = (uint32_t)s / kPStages;
-            ok = warp_wait(&misc->w_empty[st], (use & 1u) ^ 1u, abort_flag);
+        int slot = 0;
+        uint32_t phase = 1u;
+        for (int s = 0; s < n_sl && ok; ++s) {
+            ok = warp_wait(&misc->empty[slot], phase, abort_flag);
             if (!ok) break;
             if (elect_one()) {
-                const uint32_t bar = ptx::smem_u32(&misc->w_full[st]);
-                ptx::mbar_arrive_expect_tx(bar, stage_bytes);
-                for (int nc = 0; nc < NC; ++nc)   // 64 output columns x DH rows of W_O per box
-                    ptx::tma_load_2d(wsm + st * stage_bytes + (uint32_t)nc * DH * 128u, &tm_o, nc * 64, misc->idx[s] * DH, bar);
+                const uint32_t bar = ptx::smem_u32(&misc->full[slot]), dst = ring + slot * stage_bytes + 128u * RB;
+                ptx::mbar_arrive_expect_tx(bar, (uint32_t)n_box * kBox);
+                for (int i = 0; i < n_box; ++i)
+                    ptx::tma_load_2d(dst + (uint32_t)i * kBox, &tm_o, (box0 + i) * 64, misc->idx[s] * DH, bar);
             }
             __syncwarp();
+            if (++slot == stages) { slot = 0; phase ^= 1u; }
         }
     } else if (warp == 1) {
-        constexpr uint32_t idesc = PROJ_IDESC(128, 64, false, true);
+        const uint32_t idesc = PROJ_IDESC(128, n_box * 64, false, true);
         bool ok = true;
-        for (int s = 0; s < n_slices && ok; ++s) {
-            const uint32_t st = (uint32_t)s % kPStages, use = (uint32_t)s / kPStages;
-            ok = warp_wait(&misc->w_full[st], use & 1u, abort_flag);
+        int slot = 0;
+        uint32_t phase = 0u;
+        for (int s = 0; s < n_sl && ok; ++s) {
+            ok = warp_wait(&misc->full[slot], phase, abort_flag);
             if (!ok) break;
             ptx::tc_fence_after_sync();
             if (elect_one()) {
-                const uint32_t a0 = as + (uint32_t)misc->kind[s] * a_tile;
-                for (int nc = 0; nc < NC; ++nc) {
+                const uint32_t a = ring + slot * stage_bytes, w = a + 128u * RB;
 #pragma unroll
-                    for (int ks = 0; ks < DH / 16; ++ks) {
-                        const uint64_t a = ptx::umma_smem_desc_rows(a0 + ks * 32, RB);
-                        const uint64_t bd = ptx::umma_smem_desc_rows(
-                            wsm + st * stage_bytes + (uint32_t)nc * DH * 128u + (uint32_t)ks * 16u * 128u, 128);
-                        ptx::umma_bf16(tmem + (uint32_t)nc * 64, a, bd, idesc, (s > 0 || ks > 0) ? 1u : 0u);
-                    }
-                }
-                ptx::umma_commit(ptx::smem_u32(&misc->w_empty[st]));
-                if (s == n_slices - 1) ptx::umma_commit(ptx::smem_u32(&misc->acc_full));
+                for (int ks = 0; ks < DH / 16; ++ks)
+                    ptx::umma_bf16(tmem, ptx::umma_smem_desc_rows(a + ks * 32, RB),
+                                   ptx::umma_smem_desc_rows(w + (uint32_t)ks * 16u * 128u, 128, kBox), idesc,
+                                   (s > 0 || ks > 0) ? 1u : 0u);
+                ptx::umma_commit(ptx::smem_u32(&misc->empty[slot]));
+                if (s == n_sl - 1) ptx::umma_commit(ptx::smem_u32(&misc->acc_full));
             }
             __syncwarp();
+            if (++slot == stages) { slot = 0; phase ^= 1u; }
         }
     } else if (warp >= 4) {
-        const int quarter = warp & 3;
-        const int row = quarter * 32 + lane;
-        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-        const int tok = row < n_rows ? (int)s_valid[tt * 128 + row] : -1;
-        if (n_slices > 0 && warp_wait(&misc->acc_full, 0u, abort_flag)) {
-            ptx::tc_fence_after_sync();
-            for (int c0 = 0; c0 < D; c0 += 32) {
-                uint32_t acc[32];
-                ptx::tmem_ld_32x32(lane_base + c0, acc);
-                ptx::tmem_ld_wait();
-                if (tok >= 0) {
-                    uint4* dst = reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + tok) * D + c0);
+        const __nv_bfloat16* rows[S::CPR];
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {
-                        uint4 v;
-                        v.x = pack2(__uint_as_float(acc[8 * cc]), __uint_as_float(acc[8 * cc + 1]));
-                        v.y = pack2(__uint_as_float(acc[8 * cc + 2]), __uint_as_float(acc[8 * cc + 3]));
-                        v.z = pack2(__uint_as_float(acc[8 * cc + 4]), __uint_as_float(acc[8 * cc + 5]));
-                        v.w = pack2(__uint_as_float(acc[8 * cc + 6]), __uint_as_float(acc[8 * cc + 7]));
-                        dst[cc] = v;
-                    }
+        for (int j = 0; j < S::CPR; ++j) {
+            const int i = threadIdx.x - 128 + j * 128, r = i / S::CPR;
+            rows[j] = r < n_rows ? A + ((size_t)b * k_h * Tlen + misc->tok[r]) * DH + (i % S::CPR) * 8 : nullptr;
+        }
+        const bool ok = gather_steps<S::CPR>(
+            misc, ring, stage_bytes, stages, n_sl,
+            [&](int s, int, int, int j) {
+                return rows[j] != nullptr ? rows[j] + (size_t)misc->kind[s] * Tlen * DH : nullptr;
+            },
+            [](int r, int cc) { return S::off(r, cc); }, abort_flag);
+        const int quarter = warp & 3, c = lane & 7;
+        if (ok && (n_sl == 0 || warp_wait(&misc->acc_full, 0u, abort_flag))) {
+            ptx::tc_fence_after_sync();
+            const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16), buf = ring + quarter * 4096u;
+            for (int i = 0; i < n_box; ++i) {
+                if (n_sl > 0) acc_to_smem(taddr + i * 64, buf);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int r = j * 4 + (lane >> 3);
+                    if (quarter * 32 + r < n_rows)   // (no valid kept head: the rows are zero)
+                        *reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + misc->tok[quarter * 32 + r]) * D + (box0 + i) * 64 + c * 8) =
+                            n_sl > 0 ? smem_chunk(buf, r, c) : make_uint4(0, 0, 0, 0);
                 }
+                __syncwarp();
             }
-        } else if (n_slices == 0 && tok >= 0) {   // no valid kept head: the rows are zero
-            for (int c0 = 0; c0 < D; c0 += 8)
-                *reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + tok) * D + c0) = make_uint4(0, 0, 0, 0);
         }
     }
-
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    if (*abort_flag) {
-        if (threadIdx.x == 0) atomicOr(status, SENTRY_STATUS_BIT_TIMEOUT);
-        const long long t0 = clock64();
-        while (clock64() - t0 < 2000000LL) __nanosleep(1000);
-        __syncthreads();
-    }
-    if (warp == 0) {
-        ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem, 512);
-    }
-}
-
-size_t out_smem_bytes(int D, int DH, int k_h, int T) {
-    return (size_t)k_h * 128 * DH * 2 + (size_t)kPStages * D * DH * 2 + ((sizeof(ProjMisc) + 127) / 128) * 128 +
-           ((size_t)T * 2 + 127) / 128 * 128 + 1024;
+    tc_cta_teardown(abort_flag, status, tmem, kPCols);
 }
 
 template <int DH>
@@ -394,20 +412,15 @@ int launch_out_d(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t st) {
     const sentry_proj_desc& d = a.d;
     CUtensorMap mo;
     if (!make_map_2d(&mo, a.WO, (uint64_t)d.Hq * DH, d.D, DH, 64)) return SENTRY_ERR_CUDA;
-    const size_t smem = out_smem_bytes(d.D, DH, d.k_h, d.T);
     auto kern = proj_out_tc_kernel<DH>;
-    SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const unsigned grid = (unsigned)((size_t)d.B * ((d.T + 127) / 128));
+    SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPSmem));
+    const int tiles = (d.T + 127) / 128, parts = (d.D + kPCols - 1) / kPCols;
     LaunchScope ls(ctx, KS_PROJ_OUT, st);
-    SENTRY_CUDA_TRY(launch_chained(kern, dim3(grid), dim3(kPThreads), smem, st, mo, (const __nv_bfloat16*)a.A, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq,
-                                        d.k_h, (__nv_bfloat16*)a.out, a.status));
+    SENTRY_CUDA_TRY(launch_chained(kern, dim3((unsigned)((size_t)d.B * tiles * parts)), dim3(kPThreads), (size_t)kPSmem, st, mo,
+                                   (const __nv_bfloat16*)a.A, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.k_h, tiles, parts,
+                                   (__nv_bfloat16*)a.out, a.status));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
-}
-
-size_t qkv_smem_bytes(int D, int DH, int T) {
-    return (size_t)(D / 64) * 16384 + (size_t)kPStages * D * DH * 2 + ((sizeof(ProjMisc) + 127) / 128) * 128 +
-           ((size_t)T * 2 + 127) / 128 * 128 + 1024;
 }
 
 template <int DH>
@@ -417,28 +430,30 @@ int launch_qkv_d(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t st) {
     if (!make_map_2d(&mq, a.WQ, d.D, (uint64_t)d.Hq * DH, 64, DH) || !make_map_2d(&mk, a.WK, d.D, (uint64_t)d.Hk * DH, 64, DH) ||
         !make_map_2d(&mv, a.WV, d.D, (uint64_t)d.Hk * DH, 64, DH))
         return SENTRY_ERR_CUDA;
-    const size_t smem = qkv_smem_bytes(d.D, DH, d.T);
     auto kern = proj_qkv_tc_kernel<DH>;
-    SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const unsigned grid = (unsigned)((size_t)d.B * ((d.T + 127) / 128));
+    SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPSmem));
+    const int tiles = (d.T + 127) / 128, groups = d.Hk < d.k_h ? d.Hk : d.k_h;   // at most: referenced groups
+    const int parts = ((d.k_h + 2 * groups) * DH + kPCols - 1) / kPCols;
     LaunchScope ls(ctx, KS_PROJ_QKV, st);
-    SENTRY_CUDA_TRY(launch_chained(kern, dim3(grid), dim3(kPThreads), smem, st, mq, mk, mv, (const __nv_bfloat16*)a.X, a.kept_heads, a.ids, a.masks, d.T, d.D,
-                                        d.Hq, d.Hk, d.k_h, (__nv_bfloat16*)a.Q, (__nv_bfloat16*)a.K,
-                                        (__nv_bfloat16*)a.V, a.status));
+    SENTRY_CUDA_TRY(launch_chained(kern, dim3((unsigned)((size_t)d.B * tiles * parts)), dim3(kPThreads), (size_t)kPSmem, st, mq, mk,
+                                   mv, (const __nv_bfloat16*)a.X, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.Hk, d.k_h, tiles,
+                                   parts, (__nv_bfloat16*)a.Q, (__nv_bfloat16*)a.K, (__nv_bfloat16*)a.V, a.status));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
 }
 
 }  // namespace
 
-// bf16, head dim 16/32/64, d_model a multiple of 64, everything within one SM's shared memory,
-// and one CTA's tile count within the grid limit
+// bf16, head dim 16/32/64, d_model a multiple of 64.  Q and K decide which positions attention selects, so which form sums
+// them is part of the result: d_model times head dimension beyond what one SM once had to hold (96 KB of X and 72 KB of
+// weights at d_model 384, d = 32) stays with the plain-ALU kernel, whose fp32 sums run in another order.
 bool project_qkv_tc_supported(const sentry_proj_desc& d) {
     if (d.dtype != ATT_DTYPE) return false;
     if (d.d != 16 && d.d != 32 && d.d != 64) return false;
     if (d.D % 64 != 0 || d.T > 65535) return false;
     if (d.k_h + 2 * d.Hk > kMaxSlicesTc) return false;
-    return qkv_smem_bytes(d.D, d.d, d.T) <= 220 * 1024;
+    const size_t list = ((size_t)d.T * 2 + 127) / 128 * 128;
+    return (size_t)d.D * 256 + (size_t)3 * d.D * d.d * 2 + 1920 + list <= 220 * 1024;
 }
 
 int launch_project_qkv_tc(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t st) {
@@ -453,8 +468,7 @@ int launch_project_qkv_tc(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t st) {
 bool project_out_tc_supported(const sentry_proj_desc& d) {
     if (d.dtype != ATT_DTYPE) return false;
     if (d.d != 16 && d.d != 32 && d.d != 64) return false;
-    if (d.D % 64 != 0 || d.D > 512 || d.T > 65535 || d.k_h > kMaxSlicesTc) return false;
-    return out_smem_bytes(d.D, d.d, d.k_h, d.T) <= 220 * 1024;
+    return d.D % 64 == 0 && d.T <= 65535 && d.k_h <= kMaxSlicesTc;
 }
 
 int launch_project_out_tc(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t st) {

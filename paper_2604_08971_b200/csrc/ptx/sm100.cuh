@@ -241,14 +241,15 @@ __device__ __forceinline__ uint64_t umma_smem_desc_sw128(uint32_t smem_addr) {
 // width; layout code 6 / 4 / 2), 8-row groups `sbo_bytes` apart (8 x row bytes when the rows are
 // contiguous).  K-major operand: a row is one M/N index, its bytes run along K.  MN-major operand
 // (major bit set in the instruction descriptor): a row is one K index, its bytes run along M/N,
-// and sbo_bytes is the distance between groups of 8 K indices.
+// and sbo_bytes is the distance between groups of 8 K indices; operands wider in M/N than a row are row blocks of that
+// kind lbo_bytes apart.
 __host__ __device__ constexpr uint32_t umma_layout_code(int row_bytes) {
     return row_bytes == 128 ? 2u : (row_bytes == 64 ? 4u : 6u);
 }
-__device__ __forceinline__ uint64_t umma_smem_desc_rows(uint32_t smem_addr, int row_bytes) {
+__device__ __forceinline__ uint64_t umma_smem_desc_rows(uint32_t smem_addr, int row_bytes, uint32_t lbo_bytes = 16) {
     uint64_t d = 0;
     d |= (uint64_t)((smem_addr >> 4) & 0x3fffu);
-    d |= (uint64_t)1u << 16;
+    d |= (uint64_t)((lbo_bytes >> 4) & 0x3fffu) << 16;
     d |= (uint64_t)((8u * (uint32_t)row_bytes) >> 4) << 32;
     d |= (uint64_t)1u << 46;
     d |= (uint64_t)umma_layout_code(row_bytes) << 61;
