@@ -1,6 +1,6 @@
 """Python binding of libsentry (C ABI in include/sentry.h).
 
-Argument marshalling only: every step of the pruned-layer path (gate selection,
+Argument marshalling only (csrc/binding.cpp for the calls a serving loop makes, ctypes for the rest): every step of the pruned-layer path (gate selection,
 sparse grouped-query attention, channel-compacted FFN) runs in the CUDA kernels
 of the shared library.  PyTorch is used for device memory and streams.  There is
 no CPU fallback: if the library is missing or no CUDA device is present, the
@@ -9,6 +9,7 @@ calls raise.
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
 from typing import Optional
 
@@ -69,6 +70,7 @@ class SentryError(RuntimeError):
 
 
 _lib = None
+_binding = None
 
 
 def load_library(path: Optional[str] = None) -> ctypes.CDLL:
@@ -136,6 +138,18 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     return lib
 
 
+def _load_binding():
+    """The native marshalling module, after the library it calls."""
+    global _binding
+    if _binding is None:
+        load_library()
+        if not os.path.exists(_build.BINDING):
+            raise FileNotFoundError("%s not found: build it with `python -m paper_2604_08971_b200.build`" % _build.BINDING)
+        _binding = importlib.import_module(__name__ + "._binding")
+        _binding.set_error(SentryError)
+    return _binding
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     return _build.build(force=force, verbose=verbose)
 
@@ -194,19 +208,22 @@ class Sentry:
         if not torch.cuda.is_available():
             raise RuntimeError("libsentry needs a CUDA device; there is no CPU fallback")
         self.lib = load_library()
+        _load_binding()
         self.device = int(device)
         h = ctypes.c_void_p()
         rc = self.lib.sentry_create(ctypes.byref(h), self.device)
         if rc != 0:
             raise SentryError(rc, "sentry_create")
         self.h = h
+        self._handle = h.value
         self._ws = None
+        self._ws_bytes = 0
         self.ensure_workspace(1 << 20)
 
     def close(self):
         if getattr(self, "h", None):
             self.lib.sentry_destroy(self.h)
-            self.h = None
+            self.h = self._handle = None
 
     def __del__(self):
         try:
@@ -221,6 +238,7 @@ class Sentry:
             rc = self.lib.sentry_set_workspace(self.h, self._ws.data_ptr(), self._ws.numel())
             if rc != 0:
                 raise SentryError(rc, "sentry_set_workspace")
+            self._ws_bytes = self._ws.numel()
 
     def workspace_bytes(self, attend: Optional[AttendDesc] = None, ffn: Optional[FfnDesc] = None) -> int:
         return int(self.lib.sentry_workspace_bytes(ctypes.byref(attend) if attend else None,
@@ -271,65 +289,39 @@ class Sentry:
                     heads_per_group: int = 0, kept: Optional[torch.Tensor] = None):
         """sentry_gate_select: scores [S,n] fp32, masks [n_masks] int32/uint32 bit patterns.
         Returns kept [n_masks,k] int32 (and the KV-group bitmaps if heads_per_group > 0)."""
-        S, n = scores.shape
-        n_masks = masks.shape[0]
-        assert scores.dtype == torch.float32 and masks.dtype in (torch.int32, torch.uint32)
         if kept is None:
-            kept = torch.empty((n_masks, k), dtype=torch.int32, device=scores.device)
-        groups = torch.empty((n_masks,), dtype=torch.int32, device=scores.device) \
-            if heads_per_group > 0 else None
-        self.ensure_workspace(max(1 << 20, S * k * 4 + S * 4 + 1024))
-        rc = self.lib.sentry_gate_select(self.h, _ptr(scores), S, n, _ptr(masks), n_masks, int(k),
-                                         _ptr(kept), _ptr(groups), int(heads_per_group), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_gate_select")
+            kept = torch.empty((masks.shape[0], k), dtype=torch.int32, device=scores.device)
+        groups = torch.empty((masks.shape[0],), dtype=torch.int32, device=scores.device) if heads_per_group > 0 else None
+        _binding.gate_select(self, self._handle, self._ws_bytes, scores, masks, k, kept, groups, heads_per_group)
         return (kept, groups) if heads_per_group > 0 else kept
 
     def gate_select_multi(self, sets):
         """sentry_gate_select_multi: several selections over the same mask values in one launch.
         `sets`: list of (scores [S,n] fp32, masks [n_masks], k, heads_per_group[, kept]) tuples.  Returns one
         entry per set: kept, or (kept, kv_groups) where heads_per_group > 0."""
-        arr = (GateSet * len(sets))()
-        outs = []
-        S = sets[0][0].shape[0]
-        need = 1024
-        for i, item in enumerate(sets):
+        outs, full = [], []
+        for item in sets:
             scores, masks, k, hpg = item[:4]
             kept = item[4] if len(item) > 4 else None
-            assert scores.shape[0] == S and scores.dtype == torch.float32
-            n_masks = masks.shape[0]
             if kept is None:
-                kept = torch.empty((n_masks, k), dtype=torch.int32, device=scores.device)
-            groups = torch.empty((n_masks,), dtype=torch.int32, device=scores.device) if hpg > 0 else None
-            arr[i] = GateSet(_ptr(scores), scores.shape[1], int(k), _ptr(masks), n_masks, _ptr(kept), _ptr(groups),
-                             int(hpg))
+                kept = torch.empty((masks.shape[0], k), dtype=torch.int32, device=scores.device)
+            groups = torch.empty((masks.shape[0],), dtype=torch.int32, device=scores.device) if hpg > 0 else None
+            full.append((scores, masks, k, hpg, kept, groups))
             outs.append((kept, groups) if hpg > 0 else kept)
-            need += S * k * 4 + S * 4 + 512
-        self.ensure_workspace(max(1 << 20, need))
-        rc = self.lib.sentry_gate_select_multi(self.h, S, arr, len(sets), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_gate_select_multi")
+        _binding.gate_select_multi(self, self._handle, self._ws_bytes, full)
         return outs
 
     def gate_attend_fwd(self, head_scores, k_h: int, Q, K, V, token_modality_ids, masks, sample_table=None,
                         sample_offsets=None, *, c: int = 5, score_mode: int = 0, O=None, kept_heads=None,
                         active_out=None):
         """sentry_gate_attend_fwd: head selection + attention.  Returns (O [B,k_h,T,d], kept_heads [B,k_h])."""
-        desc = self.attend_desc(Q, K, k_h, c, score_mode)
-        B, _, T, d = Q.shape
         if O is None:
+            B, _, T, d = Q.shape
             O = torch.empty((B, k_h, T, d), dtype=Q.dtype, device=Q.device)
         if kept_heads is None:
-            kept_heads = torch.empty((B, k_h), dtype=torch.int32, device=Q.device)
-        S = head_scores.shape[0]
-        self.ensure_workspace(max(self.workspace_bytes(attend=desc), S * k_h * 4 + S * 4 + 1024))
-        n_subsets = 0 if sample_offsets is None else sample_offsets.shape[0]
-        rc = self.lib.sentry_gate_attend_fwd(self.h, ctypes.byref(desc), _ptr(head_scores), S, _ptr(Q), _ptr(K), _ptr(V),
-                                             _ptr(token_modality_ids), _ptr(masks), _ptr(sample_table),
-                                             _ptr(sample_offsets), n_subsets, _ptr(O), _ptr(kept_heads),
-                                             _ptr(active_out), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_gate_attend_fwd")
+            kept_heads = torch.empty((Q.shape[0], k_h), dtype=torch.int32, device=Q.device)
+        _binding.gate_attend_fwd(self, self._handle, self._ws_bytes, head_scores, k_h, Q, K, V, token_modality_ids, masks,
+                                 sample_table, sample_offsets, c, score_mode, O, kept_heads, active_out)
         return O, kept_heads
 
     def sample_table_arrange(self, token_modality_ids, sample_table, sample_offsets, c: int = 5, out=None):
@@ -351,21 +343,14 @@ class Sentry:
                    sample_offsets=None, *, c: int = 5, score_mode: int = 0, O=None,
                    active_out=None, active_in=None, return_active: bool = False):
         """sentry_attend_fwd.  Returns O [B,k_h,T,d] (and the active lists when asked)."""
-        desc = self.attend_desc(Q, K, kept_heads.shape[1], c, score_mode)
-        assert K.shape == V.shape and K.dtype == Q.dtype and V.dtype == Q.dtype
         if O is None:
-            O = torch.empty((desc.B, desc.k_h, desc.T, desc.d), dtype=Q.dtype, device=Q.device)
+            B, _, T, d = Q.shape
+            O = torch.empty((B, kept_heads.shape[1], T, d), dtype=Q.dtype, device=Q.device)
         if return_active and active_out is None:
-            U_max = num_active_queries(desc.T, c)
-            active_out = torch.empty((desc.B, desc.k_h, U_max), dtype=torch.int32, device=Q.device)
-        self.ensure_workspace(self.workspace_bytes(attend=desc))
-        n_subsets = int(sample_offsets.shape[0]) if sample_offsets is not None else 0
-        rc = self.lib.sentry_attend_fwd(self.h, ctypes.byref(desc), _ptr(Q), _ptr(K), _ptr(V),
-                                        _ptr(kept_heads), _ptr(token_modality_ids), _ptr(masks),
-                                        _ptr(sample_table), _ptr(sample_offsets), n_subsets, _ptr(O),
-                                        _ptr(active_out), _ptr(active_in), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_attend_fwd")
+            U_max = num_active_queries(Q.shape[2], c)
+            active_out = torch.empty((Q.shape[0], kept_heads.shape[1], U_max), dtype=torch.int32, device=Q.device)
+        _binding.attend_fwd(self, self._handle, self._ws_bytes, Q, K, V, kept_heads, token_modality_ids, masks, sample_table,
+                            sample_offsets, c, score_mode, O, active_out, active_in)
         return (O, active_out) if return_active else O
 
     def ffn_desc(self, X, W1, kept_channels) -> FfnDesc:
@@ -376,35 +361,21 @@ class Sentry:
     def ffn_fwd(self, X, W1, W2, kept_channels, list_of_sample=None, token_modality_ids=None,
                 masks=None, Y=None):
         """sentry_ffn_fwd.  Returns Y [B,T,D]."""
-        if kept_channels.dim() == 1:
-            kept_channels = kept_channels[None, :]
-        desc = self.ffn_desc(X, W1, kept_channels)
-        assert W1.dtype == X.dtype and W2.dtype == X.dtype
         if Y is None:
             Y = torch.empty_like(X)
-        self.ensure_workspace(self.workspace_bytes(ffn=desc))
-        rc = self.lib.sentry_ffn_fwd(self.h, ctypes.byref(desc), _ptr(X), _ptr(W1), _ptr(W2),
-                                     _ptr(kept_channels), _ptr(list_of_sample),
-                                     _ptr(token_modality_ids), _ptr(masks), _ptr(Y), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_ffn_fwd")
+        _binding.ffn_fwd(self, self._handle, self._ws_bytes, X, W1, W2, kept_channels, list_of_sample, token_modality_ids,
+                         masks, Y)
         return Y
 
     def ffn_prepack(self, W1, W2, kept_channels, packed=None):
         """sentry_ffn_prepack: materialise W1[:, N], W2[N, :] of every kept list once.  Returns the
         packed buffer (a uint8 tensor) for ffn_fwd_packed."""
-        if kept_channels.dim() == 1:
-            kept_channels = kept_channels[None, :]
-        D, F = W1.shape
-        n_lists, k_c = kept_channels.shape
-        desc = FfnDesc(1, 1, D, F, k_c, n_lists, _dtype_code(W1))
-        nbytes = int(self.lib.sentry_ffn_packed_bytes(ctypes.byref(desc)))
         if packed is None:
-            packed = torch.empty((nbytes,), dtype=torch.uint8, device=W1.device)
-        rc = self.lib.sentry_ffn_prepack(self.h, ctypes.byref(desc), _ptr(W1), _ptr(W2), _ptr(kept_channels),
-                                         _ptr(packed), packed.numel(), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_ffn_prepack")
+            D, F = W1.shape
+            n_lists, k_c = kept_channels.shape if kept_channels.dim() == 2 else (1, kept_channels.shape[0])
+            desc = FfnDesc(1, 1, D, F, k_c, n_lists, _dtype_code(W1))
+            packed = torch.empty((int(self.lib.sentry_ffn_packed_bytes(ctypes.byref(desc))),), dtype=torch.uint8, device=W1.device)
+        _binding.ffn_prepack(self, self._handle, self._ws_bytes, W1, W2, kept_channels, packed)
         return packed
 
     def ffn_prepack_fp8(self, W1q, W2q, scale_w1: float, scale_w2: float, kept_channels, dtype=torch.bfloat16,
@@ -446,88 +417,53 @@ class Sentry:
     def ffn_fwd_fp8(self, Xq, packed, F: int, k_c: int, n_lists: int, scale_x: float, scale_w1: float, scale_w2: float,
                     scale_h: float, list_of_sample=None, token_modality_ids=None, masks=None, Y=None):
         """sentry_ffn_fwd_fp8: Xq [B,T,D] uint8 e4m3 codes, packed from ffn_prepack_e4m3.  Returns Y [B,T,D] bf16."""
-        B, T, D = Xq.shape
-        desc = FfnDesc(B, T, D, int(F), int(k_c), int(n_lists), SENTRY_FP8_E4M3)
         if Y is None:
-            Y = torch.empty((B, T, D), dtype=torch.bfloat16, device=Xq.device)
-        desc16 = FfnDesc(B, T, D, int(F), int(k_c), int(n_lists), SENTRY_BF16)
-        self.ensure_workspace(self.workspace_bytes(ffn=desc16))
-        rc = self.lib.sentry_ffn_fwd_fp8(self.h, ctypes.byref(desc), _ptr(Xq), _ptr(packed), _ptr(list_of_sample),
-                                         _ptr(token_modality_ids), _ptr(masks), float(scale_x), float(scale_w1),
-                                         float(scale_w2), float(scale_h), _ptr(Y), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_ffn_fwd_fp8")
+            Y = torch.empty(Xq.shape, dtype=torch.bfloat16, device=Xq.device)
+        _binding.ffn_fwd_fp8(self, self._handle, self._ws_bytes, Xq, packed, F, k_c, n_lists, scale_x, scale_w1, scale_w2,
+                             scale_h, list_of_sample, token_modality_ids, masks, Y)
         return Y
 
     def ffn_fwd_packed(self, X, packed, F: int, k_c: int, n_lists: int, list_of_sample=None,
                        token_modality_ids=None, masks=None, Y=None):
         """sentry_ffn_fwd_packed.  Returns Y [B,T,D]."""
-        B, T, D = X.shape
-        desc = FfnDesc(B, T, D, int(F), int(k_c), int(n_lists), _dtype_code(X))
         if Y is None:
             Y = torch.empty_like(X)
-        self.ensure_workspace(self.workspace_bytes(ffn=desc))
-        rc = self.lib.sentry_ffn_fwd_packed(self.h, ctypes.byref(desc), _ptr(X), _ptr(packed),
-                                            _ptr(list_of_sample), _ptr(token_modality_ids), _ptr(masks),
-                                            _ptr(Y), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_ffn_fwd_packed")
+        _binding.ffn_fwd_packed(self, self._handle, self._ws_bytes, X, packed, F, k_c, n_lists, list_of_sample,
+                                token_modality_ids, masks, Y)
         return Y
 
     def gate_eval(self, layer_offsets, zeta, gamma, W1, b1, w2, b2, return_gates: bool = False):
         """sentry_gate_eval: logits (and gates) [2^M, n_units] of SentryGate's per-unit MLP (Eq. 1)."""
-        n_units, hidden, M = W1.shape
-        n_layers = gamma.shape[0]
-        S = 1 << M
-        logits = torch.empty((S, n_units), dtype=torch.float32, device=W1.device)
+        n_units, _, M = W1.shape
+        logits = torch.empty((1 << M, n_units), dtype=torch.float32, device=W1.device)
         gates = torch.empty_like(logits) if return_gates else None
-        rc = self.lib.sentry_gate_eval(self.h, M, hidden, n_layers, _ptr(layer_offsets), n_units, _ptr(zeta),
-                                       _ptr(gamma), _ptr(W1), _ptr(b1), _ptr(w2), _ptr(b2), _ptr(logits),
-                                       _ptr(gates), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_gate_eval")
+        _binding.gate_eval(self, self._handle, self._ws_bytes, layer_offsets, zeta, gamma, W1, b1, w2, b2, logits, gates)
         return (logits, gates) if return_gates else logits
 
     def gate_layer_counts(self, kept, layer_offsets):
         """sentry_gate_layer_counts: kept [n_masks, k] ascending -> counts [n_masks, n_layers]."""
-        n_masks, k = kept.shape
-        n_layers = layer_offsets.shape[0] - 1
-        counts = torch.empty((n_masks, n_layers), dtype=torch.int32, device=kept.device)
-        rc = self.lib.sentry_gate_layer_counts(self.h, _ptr(kept), n_masks, k, _ptr(layer_offsets), n_layers,
-                                               _ptr(counts), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_gate_layer_counts")
+        counts = torch.empty((kept.shape[0], layer_offsets.shape[0] - 1), dtype=torch.int32, device=kept.device)
+        _binding.gate_layer_counts(self, self._handle, self._ws_bytes, kept, layer_offsets, counts)
         return counts
 
     def project_qkv(self, X, WQ, WK, WV, kept_heads, token_modality_ids, masks, Hq: int, Hk: int, d: int,
                     Q=None, K=None, V=None):
         """sentry_project_qkv.  Returns Q [B,Hq,T,d], K, V [B,Hk,T,d]; fresh outputs start at zero."""
-        B, T, D = X.shape
-        desc = ProjDesc(B, T, D, int(Hq), int(Hk), int(d), kept_heads.shape[1], _dtype_code(X))
         if Q is None:
-            Q = torch.zeros((B, Hq, T, d), dtype=X.dtype, device=X.device)
+            Q = torch.zeros((X.shape[0], Hq, X.shape[1], d), dtype=X.dtype, device=X.device)
         if K is None:
-            K = torch.zeros((B, Hk, T, d), dtype=X.dtype, device=X.device)
+            K = torch.zeros((X.shape[0], Hk, X.shape[1], d), dtype=X.dtype, device=X.device)
         if V is None:
-            V = torch.zeros((B, Hk, T, d), dtype=X.dtype, device=X.device)
-        rc = self.lib.sentry_project_qkv(self.h, ctypes.byref(desc), _ptr(X), _ptr(WQ), _ptr(WK), _ptr(WV),
-                                         _ptr(kept_heads), _ptr(token_modality_ids), _ptr(masks), _ptr(Q), _ptr(K),
-                                         _ptr(V), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_project_qkv")
+            V = torch.zeros((X.shape[0], Hk, X.shape[1], d), dtype=X.dtype, device=X.device)
+        _binding.project_qkv(self, self._handle, self._ws_bytes, X, WQ, WK, WV, kept_heads, token_modality_ids, masks, Hq, Hk,
+                             d, Q, K, V)
         return Q, K, V
 
     def project_out(self, A, WO, kept_heads, token_modality_ids, masks, Hq: int, out=None):
         """sentry_project_out.  A [B,k_h,T,d] -> out [B,T,D]."""
-        B, k_h, T, d = A.shape
-        D = WO.shape[1]
-        desc = ProjDesc(B, T, D, int(Hq), 1, d, k_h, _dtype_code(A))
         if out is None:
-            out = torch.empty((B, T, D), dtype=A.dtype, device=A.device)
-        rc = self.lib.sentry_project_out(self.h, ctypes.byref(desc), _ptr(A), _ptr(WO), _ptr(kept_heads),
-                                         _ptr(token_modality_ids), _ptr(masks), _ptr(out), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_project_out")
+            out = torch.empty((A.shape[0], A.shape[2], WO.shape[1]), dtype=A.dtype, device=A.device)
+        _binding.project_out(self, self._handle, self._ws_bytes, A, WO, kept_heads, token_modality_ids, masks, Hq, out)
         return out
 
     def moe_prepack(self, W1, W2, kept_channels, packed=None):
@@ -548,17 +484,11 @@ class Sentry:
                     F: Optional[int] = None, E: Optional[int] = None, k_c: Optional[int] = None, Y=None):
         """sentry_moe_ffn_fwd.  X [N,D]; expert_ids i32, expert_weights fp32 [N,top_k]; either W1 [E,D,F],
         W2 [E,F,D], kept_channels [E,k_c], or `packed` from moe_prepack with F, E, k_c.  Returns Y [N,D]."""
-        N, D = X.shape
         if packed is None:
             E, _, F = W1.shape
             k_c = kept_channels.shape[1]
-        desc = MoeDesc(N, D, int(F), int(E), expert_ids.shape[1], int(k_c), _dtype_code(X))
         if Y is None:
             Y = torch.empty_like(X)
-        self.ensure_workspace(int(self.lib.sentry_moe_workspace_bytes(ctypes.byref(desc))))
-        rc = self.lib.sentry_moe_ffn_fwd(self.h, ctypes.byref(desc), _ptr(X), _ptr(W1), _ptr(W2),
-                                         _ptr(kept_channels), _ptr(packed), _ptr(expert_ids), _ptr(expert_weights),
-                                         _ptr(Y), _stream())
-        if rc != 0:
-            raise SentryError(rc, "sentry_moe_ffn_fwd")
+        _binding.moe_ffn_fwd(self, self._handle, self._ws_bytes, X, expert_ids, expert_weights, W1, W2, kept_channels, packed,
+                             F, E, k_c, Y)
         return Y
