@@ -45,7 +45,8 @@ __device__ __forceinline__ void load_row(const T* __restrict__ p, float (&r)[D])
     }
 }
 
-// grid (ceil(T/threads), B*k_h).  mscore[(b*k_h+kh)*T + p] for p < T_v.
+// grid (B*k_h, ceil(T/threads)).  A thread per query; the rows of several sampled keys are on the way at once (a chain of
+// table entry, token and row loads otherwise).  mscore[(b*k_h+kh)*T + p] for p < T_v.
 template <typename T, int D>
 __global__ void __launch_bounds__(kScoreThreads)
 attend_score_kernel(const T* __restrict__ Q, const T* __restrict__ K,
@@ -56,6 +57,8 @@ attend_score_kernel(const T* __restrict__ Q, const T* __restrict__ K,
                     unsigned int* status) {
     extern __shared__ uint16_t s_valid[];
     __shared__ int red[66];
+    grid_dependents_start_if_small();
+    grid_dependency_wait();
     const int bh = blockIdx.x, b = bh / k_h;
     const uint32_t mask = masks[b];
     const int Tv = block_build_valid(ids, Tlen, mask, s_valid, red);
@@ -80,22 +83,43 @@ attend_score_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     if (p >= Tv) return;
     const T* Qh = Q + ((size_t)b * Hq + h) * Tlen * D;
     const T* Kg = K + ((size_t)b * Hk + g) * Tlen * D;
-    float q[D], kr[D];
+    constexpr int NB = 128 / D;
+    float q[D], kr[NB][D];
     load_row<T, D>(Qh + (size_t)s_valid[p] * D, q);
     const float scale = 1.0f / sqrtf((float)D);
     const int cnt = (score_mode != 1) ? n_s : Tv;
     float mx = -INFINITY, sum = 0.f;
-    for (int a = 0; a < cnt; ++a) {
-        int pj = (score_mode == 0) ? tbl[(size_t)p * n_s + a] : (score_mode == 2 ? tbl[(size_t)a * Tv + p] : a);
-        if (pj < 0 || pj >= Tv) { atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX); pj = 0; }
-        load_row<T, D>(Kg + (size_t)s_valid[pj] * D, kr);
-        float dot = 0.f;
+    bool bad = false;
+    int pj[NB], next[NB];
+    auto positions = [&](int a0, int (&out)[NB]) {
 #pragma unroll
-        for (int e = 0; e < D; ++e) dot = fmaf(q[e], kr[e], dot);
-        dot *= scale;
-        mx = fmaxf(mx, dot);
-        sum += dot;
+        for (int i = 0; i < NB; ++i) {
+            const int a = min(a0 + i, cnt - 1);
+            out[i] = (score_mode == 0) ? tbl[(size_t)p * n_s + a] : (score_mode == 2 ? tbl[(size_t)a * Tv + p] : a);
+        }
+    };
+    positions(0, next);
+    for (int a0 = 0; a0 < cnt; a0 += NB) {
+#pragma unroll
+        for (int i = 0; i < NB; ++i) pj[i] = next[i];
+        positions(a0 + NB, next);
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            if (pj[i] < 0 || pj[i] >= Tv) { bad = true; pj[i] = 0; }
+            load_row<T, D>(Kg + (size_t)s_valid[pj[i]] * D, kr[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            if (a0 + i >= cnt) break;
+            float dot = 0.f;
+#pragma unroll
+            for (int e = 0; e < D; ++e) dot = fmaf(q[e], kr[i][e], dot);
+            dot *= scale;
+            mx = fmaxf(mx, dot);
+            sum += dot;
+        }
     }
+    if (bad) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
     mscore[(size_t)bh * Tlen + p] = mx - sum / (float)cnt;
 }
 
@@ -108,6 +132,8 @@ attend_select_kernel(const float* __restrict__ mscore, const int32_t* __restrict
     __shared__ int red[66];
     uint16_t* s_valid = reinterpret_cast<uint16_t*>(s_raw);
     uint32_t* s_keys = reinterpret_cast<uint32_t*>(s_raw + (((size_t)Tlen * 2 + 15) / 16) * 16);
+    grid_dependents_start_if_small();
+    grid_dependency_wait();
     const int bh = blockIdx.x, b = bh / k_h;
     const int Tv = block_build_valid(ids, Tlen, masks[b], s_valid, red);
     int32_t* out = active + (size_t)bh * U_max;
@@ -123,7 +149,9 @@ attend_select_kernel(const float* __restrict__ mscore, const int32_t* __restrict
     block_select_topk(s_keys, Tv, U, out, s_valid, red);
 }
 
-// grid B*k_h.  O[bh, t, :] for every t.
+// grid (B*k_h, parts).  O[bh, t, :] for every t: part y takes every parts-th active row and a slice of the tokens to fill.
+// Parts, because a few samples' rows on one CTA each are a chain (5 rows one after the other per warp at U = 20).
+// 2 samples x 32 tokens, d = 16, 3 heads: 14 -> 6 us.
 template <typename T, int D>
 __global__ void __launch_bounds__(kCoreThreads)
 attend_core_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
@@ -133,16 +161,19 @@ attend_core_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __
                    unsigned int* status) {
     extern __shared__ uint8_t s_raw[];
     __shared__ int red[66];
-    __shared__ float s_ctx[D];
+    __shared__ float s_ctx[D], s_part[kCoreThreads];
     uint16_t* s_valid = reinterpret_cast<uint16_t*>(s_raw);
     // per token: 0 = absent modality, 1 = present & filled with the context vector, 2 = active
     uint8_t* s_kind = s_raw + (((size_t)Tlen * 2 + 15) / 16) * 16;
-    const int bh = blockIdx.x, b = bh / k_h;
+    grid_dependents_start_if_small();
+    grid_dependency_wait();
+    const int bh = blockIdx.x, b = bh / k_h, part = blockIdx.y, parts = gridDim.y;
+    const int t_begin = (int)((long long)Tlen * part / parts), t_end = (int)((long long)Tlen * (part + 1) / parts);
     const int Tv = block_build_valid(ids, Tlen, masks[b], s_valid, red);
     T* Oh = O + (size_t)bh * Tlen * D;
     const int h = kept_heads[bh];
     if (Tv == 0 || h < 0 || h >= Hq) {
-        for (size_t i = threadIdx.x; i < (size_t)Tlen * D; i += blockDim.x) Oh[i] = from_f32<T>(0.f);
+        for (int i = t_begin * D + threadIdx.x; i < t_end * D; i += blockDim.x) Oh[i] = from_f32<T>(0.f);
         if (threadIdx.x == 0)
             atomicOr(status, Tv == 0 ? SENTRY_STATUS_BIT_EMPTY_MASK : SENTRY_STATUS_BIT_BAD_INDEX);
         return;
@@ -162,10 +193,20 @@ attend_core_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __
         if (t >= Tlen || s_kind[t] == 0) { atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX); continue; }
         s_kind[t] = 2;
     }
-    // context vector: mean of V_g over present keys
-    if (threadIdx.x < D) {
+    // context vector: mean of V_g over present keys, every G-th key per group of D threads
+    constexpr int G = kCoreThreads / D;
+    {
+        const int gi = threadIdx.x / D, e = threadIdx.x % D;
         float acc = 0.f;
-        for (int pj = 0; pj < Tv; ++pj) acc += to_f32<T>(Vg[(size_t)s_valid[pj] * D + threadIdx.x]);
+#pragma unroll 8
+        for (int pj = gi; pj < Tv; pj += G) acc += to_f32<T>(Vg[(size_t)s_valid[pj] * D + e]);
+        s_part[threadIdx.x] = acc;
+    }
+    __syncthreads();
+    if (threadIdx.x < D) {
+        float acc = s_part[threadIdx.x];
+#pragma unroll
+        for (int gi = 1; gi < G; ++gi) acc += s_part[gi * D + threadIdx.x];
         s_ctx[threadIdx.x] = acc / (float)Tv;
     }
     __syncthreads();
@@ -174,7 +215,7 @@ attend_core_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __
     // merged across the warp at the end)
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const float scale = 1.0f / sqrtf((float)D);
-    for (int a = wid; a < U_max; a += nw) {
+    for (int a = part * nw + wid; a < U_max; a += nw * parts) {
         const int t = act[a];
         if (t < 0 || t >= Tlen || s_kind[t] != 2) continue;
         float q[D], kr[D], acc[D];
@@ -219,8 +260,8 @@ attend_core_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __
             if ((e & 31) == lane) Oh[(size_t)t * D + e] = from_f32<T>(acc[e]);
     }
     // fill rows and zero rows
-    for (size_t i = threadIdx.x; i < (size_t)Tlen * D; i += blockDim.x) {
-        const int t = (int)(i / D), e = (int)(i % D);
+    for (int i = t_begin * D + threadIdx.x; i < t_end * D; i += blockDim.x) {
+        const int t = i / D, e = i % D;
         const uint8_t kind = s_kind[t];
         if (kind == 2) continue;
         Oh[i] = from_f32<T>(kind == 1 ? s_ctx[e] : 0.f);
@@ -240,10 +281,9 @@ int launch_typed(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
                                                      (int)valid_bytes));
             dim3 grid(BH, (d.T + kScoreThreads - 1) / kScoreThreads);   // (sample, head) on x: no 65535 limit
             LaunchScope ls(ctx, KS_ATT_SCORE, st);
-            kern<<<grid, kScoreThreads, valid_bytes, st>>>(
-                (const T*)a.Q, (const T*)a.K, a.kept_heads, a.ids, a.masks, a.sample_table,
-                a.sample_offsets, a.n_subsets, d.T, d.Hq, d.Hk, d.k_h, d.c, d.score_mode, a.mscore,
-                a.status);
+            SENTRY_CUDA_TRY(launch_chained(kern, grid, dim3(kScoreThreads), valid_bytes, st, (const T*)a.Q, (const T*)a.K,
+                                           a.kept_heads, a.ids, a.masks, a.sample_table, a.sample_offsets, a.n_subsets, d.T,
+                                           d.Hq, d.Hk, d.k_h, d.c, d.score_mode, a.mscore, a.status));
         }
         SENTRY_CUDA_TRY(cudaGetLastError());
         {
@@ -253,8 +293,8 @@ int launch_typed(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
                                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)smem));
             LaunchScope ls(ctx, KS_ATT_SELECT, st);
-            attend_select_kernel<<<BH, 256, smem, st>>>(a.mscore, a.ids, a.masks, d.T, d.k_h, d.c,
-                                                         a.U_max, a.active, a.status);
+            SENTRY_CUDA_TRY(launch_chained(attend_select_kernel, dim3(BH), dim3(256), smem, st, a.mscore, a.ids, a.masks, d.T,
+                                           d.k_h, d.c, a.U_max, a.active, a.status));
         }
         SENTRY_CUDA_TRY(cudaGetLastError());
     }
@@ -265,9 +305,13 @@ int launch_typed(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
             SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem));
         LaunchScope ls(ctx, KS_ATT_CORE, st);
-        kern<<<BH, kCoreThreads, smem, st>>>((const T*)a.Q, (const T*)a.K, (const T*)a.V,
-                                              a.kept_heads, a.ids, a.masks, a.active, d.T, d.Hq,
-                                              d.Hk, d.k_h, d.c, a.U_max, (T*)a.O, a.status);
+        // about two CTAs per SM, no more than their warps have rows
+        int parts = (2 * ctx->sm_count + BH - 1) / BH;
+        const int most = (a.U_max + kCoreThreads / 32 - 1) / (kCoreThreads / 32);
+        if (parts > most) parts = most;
+        SENTRY_CUDA_TRY(launch_chained(kern, dim3(BH, parts), dim3(kCoreThreads), smem, st, (const T*)a.Q, (const T*)a.K,
+                                       (const T*)a.V, a.kept_heads, a.ids, a.masks, a.active, d.T, d.Hq, d.Hk, d.k_h, d.c,
+                                       a.U_max, (T*)a.O, a.status));
     }
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;

@@ -149,6 +149,10 @@ __host__ __device__ inline int sentry_num_active(int T_v, int c) {
 // The next kernel of the stream may be scheduled from here on (it waits for this one's end by itself).
 __device__ __forceinline__ void grid_dependents_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Every kernel before this one in the stream has completed and its writes are visible.
+// For kernels of any size: early where their blocks leave SMs free anyway.
+__device__ __forceinline__ void grid_dependents_start_if_small() {
+    if (gridDim.x * gridDim.y <= 128u) grid_dependents_start();
+}
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Order-preserving map float -> uint32 for "score descending" selection:

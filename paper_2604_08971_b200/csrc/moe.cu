@@ -298,8 +298,8 @@ struct MoeWs {
 
 sentry_ffn_desc as_ffn_desc(const sentry_moe_desc& m) {
     sentry_ffn_desc d;
-    d.B = 1;
-    d.T = 1;   // the row count of the plan is N * top_k; the fused-pair kernels read it from the plan
+    d.B = m.N;
+    d.T = m.top_k;   // the plan has N * top_k rows
     d.D = m.D; d.F = m.F; d.k_c = m.k_c; d.n_lists = m.E; d.dtype = m.dtype;
     return d;
 }

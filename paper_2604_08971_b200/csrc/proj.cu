@@ -20,6 +20,8 @@ project_qkv_kernel(const T* __restrict__ X, const T* __restrict__ WQ, const T* _
                    unsigned int* status) {
     extern __shared__ float s_x[];                 // [D]
     __shared__ int s_kind[kMaxSlices], s_idx[kMaxSlices], s_n;
+    grid_dependents_start_if_small();
+    grid_dependency_wait();
     const int b = blockIdx.x / Tlen, t = blockIdx.x % Tlen;
     const int m = ids[t];
     if (m < 0 || m >= 32 || !((masks[b] >> m) & 1u)) return;       // absent token: nothing is written
@@ -49,6 +51,7 @@ project_qkv_kernel(const T* __restrict__ X, const T* __restrict__ WQ, const T* _
         const int ld = (kind == 0 ? Hq : Hk) * d;
         const int col = idx * d + c;
         float acc = 0.f;
+#pragma unroll 16
         for (int e = 0; e < D; ++e) acc = fmaf(s_x[e], to_f32<T>(W[(size_t)e * ld + col]), acc);
         T* dst = kind == 0 ? Q + (((size_t)b * Hq + idx) * Tlen + t) * d
                            : (kind == 1 ? K : V) + (((size_t)b * Hk + idx) * Tlen + t) * d;
@@ -63,6 +66,8 @@ project_out_kernel(const T* __restrict__ A, const T* __restrict__ WO, const int3
                    int d, int k_h, T* __restrict__ out, unsigned int* status) {
     extern __shared__ float s_a[];                 // [k_h * d]
     __shared__ int s_h[64];
+    grid_dependents_start_if_small();
+    grid_dependency_wait();
     const int b = blockIdx.x / Tlen, t = blockIdx.x % Tlen;
     T* o = out + ((size_t)b * Tlen + t) * D;
     const int m = ids[t];
@@ -83,6 +88,7 @@ project_out_kernel(const T* __restrict__ A, const T* __restrict__ WO, const int3
         for (int j = 0; j < k_h; ++j) {
             const int h = s_h[j];
             if (h < 0) continue;
+#pragma unroll 16
             for (int c = 0; c < d; ++c) acc = fmaf(s_a[j * d + c], to_f32<T>(WO[(size_t)(h * d + c) * D + e]), acc);
         }
         o[e] = from_f32<T>(acc);
@@ -97,18 +103,15 @@ int launch_project_qkv_generic(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t 
     const size_t smem = (size_t)d.D * sizeof(float);
     LaunchScope ls(ctx, KS_PROJ_QKV, st);
     if (d.dtype == SENTRY_F32)
-        project_qkv_kernel<float><<<grid, kProjThreads, smem, st>>>(
-            (const float*)a.X, (const float*)a.WQ, (const float*)a.WK, (const float*)a.WV, a.kept_heads, a.ids, a.masks,
-            d.T, d.D, d.Hq, d.Hk, d.d, d.k_h, (float*)a.Q, (float*)a.K, (float*)a.V, a.status);
+        SENTRY_CUDA_TRY(launch_chained(project_qkv_kernel<float>, dim3(grid), dim3(kProjThreads), smem, st, (const float*)a.X, (const float*)a.WQ, (const float*)a.WK, (const float*)a.WV, a.kept_heads, a.ids, a.masks,
+            d.T, d.D, d.Hq, d.Hk, d.d, d.k_h, (float*)a.Q, (float*)a.K, (float*)a.V, a.status));
     else if (d.dtype == SENTRY_F16)
-        project_qkv_kernel<__half><<<grid, kProjThreads, smem, st>>>(
-            (const __half*)a.X, (const __half*)a.WQ, (const __half*)a.WK, (const __half*)a.WV, a.kept_heads, a.ids,
-            a.masks, d.T, d.D, d.Hq, d.Hk, d.d, d.k_h, (__half*)a.Q, (__half*)a.K, (__half*)a.V, a.status);
+        SENTRY_CUDA_TRY(launch_chained(project_qkv_kernel<__half>, dim3(grid), dim3(kProjThreads), smem, st, (const __half*)a.X, (const __half*)a.WQ, (const __half*)a.WK, (const __half*)a.WV, a.kept_heads, a.ids,
+            a.masks, d.T, d.D, d.Hq, d.Hk, d.d, d.k_h, (__half*)a.Q, (__half*)a.K, (__half*)a.V, a.status));
     else
-        project_qkv_kernel<__nv_bfloat16><<<grid, kProjThreads, smem, st>>>(
-            (const __nv_bfloat16*)a.X, (const __nv_bfloat16*)a.WQ, (const __nv_bfloat16*)a.WK,
+        SENTRY_CUDA_TRY(launch_chained(project_qkv_kernel<__nv_bfloat16>, dim3(grid), dim3(kProjThreads), smem, st, (const __nv_bfloat16*)a.X, (const __nv_bfloat16*)a.WQ, (const __nv_bfloat16*)a.WK,
             (const __nv_bfloat16*)a.WV, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.Hk, d.d, d.k_h,
-            (__nv_bfloat16*)a.Q, (__nv_bfloat16*)a.K, (__nv_bfloat16*)a.V, a.status);
+            (__nv_bfloat16*)a.Q, (__nv_bfloat16*)a.K, (__nv_bfloat16*)a.V, a.status));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
 }
@@ -119,17 +122,14 @@ int launch_project_out_generic(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t 
     const size_t smem = (size_t)d.k_h * d.d * sizeof(float);
     LaunchScope ls(ctx, KS_PROJ_OUT, st);
     if (d.dtype == SENTRY_F32)
-        project_out_kernel<float><<<grid, kProjThreads, smem, st>>>(
-            (const float*)a.A, (const float*)a.WO, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.d, d.k_h,
-            (float*)a.out, a.status);
+        SENTRY_CUDA_TRY(launch_chained(project_out_kernel<float>, dim3(grid), dim3(kProjThreads), smem, st, (const float*)a.A, (const float*)a.WO, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.d, d.k_h,
+            (float*)a.out, a.status));
     else if (d.dtype == SENTRY_F16)
-        project_out_kernel<__half><<<grid, kProjThreads, smem, st>>>(
-            (const __half*)a.A, (const __half*)a.WO, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.d, d.k_h,
-            (__half*)a.out, a.status);
+        SENTRY_CUDA_TRY(launch_chained(project_out_kernel<__half>, dim3(grid), dim3(kProjThreads), smem, st, (const __half*)a.A, (const __half*)a.WO, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.d, d.k_h,
+            (__half*)a.out, a.status));
     else
-        project_out_kernel<__nv_bfloat16><<<grid, kProjThreads, smem, st>>>(
-            (const __nv_bfloat16*)a.A, (const __nv_bfloat16*)a.WO, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.d,
-            d.k_h, (__nv_bfloat16*)a.out, a.status);
+        SENTRY_CUDA_TRY(launch_chained(project_out_kernel<__nv_bfloat16>, dim3(grid), dim3(kProjThreads), smem, st, (const __nv_bfloat16*)a.A, (const __nv_bfloat16*)a.WO, a.kept_heads, a.ids, a.masks, d.T, d.D, d.Hq, d.d,
+            d.k_h, (__nv_bfloat16*)a.out, a.status));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
 }
