@@ -599,7 +599,8 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
                          int n_subsets, const int32_t* __restrict__ active_in,
                          int32_t* __restrict__ active_out, int Tlen, int Hq, int Hk, int k_h, int c,
                          int score_mode, int U_max, __nv_bfloat16* __restrict__ O, unsigned int* status,
-                         const float* __restrict__ gate_scores, int gate_S, int32_t* __restrict__ kept_out) {
+                         const float* __restrict__ gate_scores, int gate_S, int32_t* __restrict__ kept_out,
+                         int order_batch) {
     grid_dependency_wait();
     using S = Sw<D>;
     constexpr int NT = D / 8;        // n-tiles of the output (8 dims each)
@@ -623,7 +624,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
     const uint32_t ks_addr = ptx::smem_u32(s_raw + o);          o += (size_t)Tpad * D * 2;
     const uint32_t vs_addr = ptx::smem_u32(s_raw + o);
 
-    // Samples with more modalities present take longer; in small batches the CTAs take them
+    // Samples with more modalities present take longer; in batches of a few waves the CTAs take them
     // heaviest first (every CTA finds the sample of its rank by itself with a counting sort on
     // the number of present modalities), so that the long ones do not end up alone in the tail
     // of the launch.
@@ -632,7 +633,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
     int b = blockIdx.x / Hk;
     const int g = blockIdx.x % Hk;
     const int Bn = gridDim.x / Hk;
-    if (Bn > 1 && Bn <= kOrderMaxBatch) {
+    if (order_batch) {
         __shared__ int s_cls[33];
         __shared__ int s_wcnt[16];
         __shared__ int s_pick[2];
@@ -1045,13 +1046,16 @@ int launch_d(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
         // one big CTA, or two per SM; short sequences get small CTAs (more of them per SM: their
         // phases are a few barrier-separated microseconds each, so concurrency is what helps)
         const int threads = fused_bytes > 100 * 1024 ? 512 : (d.T <= kSmallT ? 128 : 256);
+        // heaviest samples first only where there is more than one wave (128 registers a thread: 512 threads per SM):
+        // finding the sample of a rank takes 2900 cycles, of 32000 in a CTA of T = 192
+        const int order = d.B > 1 && d.B <= kOrderMaxBatch && (long long)d.B * d.Hk > (long long)ctx->sm_count * (512 / threads);
         LaunchScope ls(ctx, KS_ATT_CORE, st);
         SENTRY_CUDA_TRY(launch_chained(kern, dim3(d.B * d.Hk), dim3(threads), fused_bytes, st,
             (const __nv_bfloat16*)a.Q, (const __nv_bfloat16*)a.K, (const __nv_bfloat16*)a.V, a.kept_heads,
             a.ids, a.masks, a.sample_table, a.sample_offsets, a.n_subsets,
             a.selection_given ? a.active : nullptr, a.selection_given ? nullptr : a.active_out_user, d.T,
             d.Hq, d.Hk, d.k_h, d.c, d.score_mode, a.U_max, (__nv_bfloat16*)a.O, a.status, a.gate_scores, a.gate_S,
-            a.kept_out));
+            a.kept_out, order));
         SENTRY_CUDA_TRY(cudaGetLastError());
         return SENTRY_OK;
     }

@@ -211,37 +211,47 @@ __device__ inline void warp_select_topk_radix(const uint32_t* keys, int n, int k
     __syncwarp();
 }
 
-// Top-k of n <= 32 * KPL order keys by ONE warp with the keys in registers (lane l holds keys
-// l, l + 32, ...): the k-th largest key is built bit by bit from the top (a candidate bit stays
-// set if at least k keys are >= the candidate: 32 steps of KPL compares and one warp add), then
-// the entries above it and the first ties are compacted in ascending index order.  No shared-
-// memory histograms, no atomics and no block barriers.
+// Top-k of n <= 32 * KPL (up to 1023) order keys by ONE warp with the keys in registers (lane l holds keys l, l + 32, ...).
+// The threshold is found two bits per step -- three candidates counted in one warp-wide add -- from the first bit in which
+// the keys differ until exactly k keys lie from one on: 6 to 8 dependent adds, where one bit per step from the top took 32
+// (attention of 256 samples of T <= 192: 28.7 -> 27.8 us).  Then the entries above it and, where keys tie at it, the first
+// ties are compacted in ascending index order.  No shared-memory histograms, no atomics and no block barriers.
 template <int KPL>
 __device__ __forceinline__ void warp_select_topk_bits(const uint32_t* keys, int n, int k, int32_t* out,
                                                       const uint16_t* remap) {
     const int lane = threadIdx.x & 31;
-    uint32_t r[KPL];
+    uint32_t r[KPL], hi = 0u, lo = 0xffffffffu;
 #pragma unroll
     for (int j = 0; j < KPL; ++j) {
         const int i = j * 32 + lane;
         r[j] = i < n ? keys[i] : 0u;     // padding: below every candidate (candidates are >= 1)
+        hi = max(hi, r[j]);
+        if (i < n) lo = min(lo, r[j]);
     }
-    uint32_t t = 0;
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    bool cut = n == k;                                            // exactly k keys are >= t
+    int bit = hi != lo ? (31 - __clz((int)(hi ^ lo))) | 1 : -1;   // digits of two bits, aligned
+    uint32_t t = bit < 0 || cut ? lo : (bit == 31 ? 0u : hi & ~((2u << bit) - 1u));
 #pragma unroll 1
-    for (int b = 31; b >= 0; --b) {
-        const uint32_t cand = t | (1u << b);
-        int cnt = 0;
+    for (bit -= 1; bit >= 0 && !cut; bit -= 2) {
+        const uint32_t c1 = t + (1u << bit), c2 = t + (2u << bit), c3 = t + (3u << bit);
+        uint32_t cnt = 0u;                                        // from c1, c2, c3 on: ten bits each
 #pragma unroll
-        for (int j = 0; j < KPL; ++j) cnt += (r[j] >= cand) ? 1 : 0;
+        for (int j = 0; j < KPL; ++j) cnt += (r[j] >= c1 ? 1u : 0u) + (r[j] >= c2 ? 1u << 10 : 0u) + (r[j] >= c3 ? 1u << 20 : 0u);
         cnt = __reduce_add_sync(0xffffffffu, cnt);
-        if (cnt >= k) t = cand;
+        const int k1 = (int)(cnt & 1023u), k2 = (int)(cnt >> 10) & 1023, k3 = (int)(cnt >> 20);
+        if (k3 >= k) { t = c3; cut = k3 == k; }
+        else if (k2 >= k) { t = c2; cut = k2 == k; }
+        else if (k1 >= k) { t = c1; cut = k1 == k; }
     }
-    // t is the k-th largest key (0 only if fewer than k keys are non-zero: then every entry ties)
-    int gt = 0;
+    int need_eq = n;                     // cut: every key equal to t is wanted
+    if (!cut) {                          // t is the k-th largest key
+        int gt = 0;
 #pragma unroll
-    for (int j = 0; j < KPL; ++j) gt += (r[j] > t) ? 1 : 0;
-    gt = __reduce_add_sync(0xffffffffu, gt);
-    const int need_eq = k - gt;
+        for (int j = 0; j < KPL; ++j) gt += (r[j] > t) ? 1 : 0;
+        need_eq = k - __reduce_add_sync(0xffffffffu, gt);
+    }
     int base = 0, eq_seen = 0;
 #pragma unroll
     for (int j = 0; j < KPL; ++j) {
