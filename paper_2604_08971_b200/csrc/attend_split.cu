@@ -10,8 +10,8 @@
 // A CTA per (sample, group) does the same in attend_bf16.cu and attend_long.cu: ten phases with a barrier after each, of
 // which every one is a chain of latencies, on as many SMs as there are groups.  Taken apart, each phase runs with as many
 // warps as it has work: the form for long sequences and for few groups (attend_split_faster in api.cu has the line).
-// Measured on 16 x 4096 tokens, d = 32, 4 of 8 heads kept: 310 us before, 102 as four launches (score 53, select 15, rows
-// and fill 49 when timed one by one).
+// Measured on 16 x 4096 tokens, d = 32, 4 of 8 heads kept: 310 us before, 91 as four launches (100 with the parts of Eq. 6
+// merged by one warp per tile and the token list read twice).
 #include <math.h>
 #include <stddef.h>
 
@@ -22,6 +22,7 @@ namespace {
 constexpr int kSplitThreads = 256, kSplitWarps = kSplitThreads / 32;
 constexpr int kScoreBlock = 128;                 // query positions per score block
 constexpr int kRowTiles = kMaxRK * kMaxActive / 16;
+constexpr int kMaxParts = 16;                     // parts of the keys in the rows launch
 
 // ------------------------------------------------------------------------------------------ pieces
 __device__ __forceinline__ float max3(float a, float b, float c) {
@@ -70,21 +71,31 @@ __device__ __forceinline__ int list_present(const int32_t* __restrict__ ids, int
         const int m = t < T ? __ldg(ids + t) : -1;
         return m >= 0 && m < 32 && ((mask >> m) & 1u);
     };
+    constexpr int HELD = 8;       // ballots of the run's first pieces stay in registers (all of it up to T = 2048; 16 cost more)
+    unsigned bm[HELD];
     int mine = 0;
+    {
+        bool ok[HELD];
+#pragma unroll
+        for (int j = 0; j < HELD; ++j) ok[j] = p0 + j < p1 && present((p0 + j) * 32 + lane);   // all loads on the way at once
+#pragma unroll
+        for (int j = 0; j < HELD; ++j) { bm[j] = __ballot_sync(0xffffffffu, ok[j]); mine += __popc(bm[j]); }
+    }
 #pragma unroll 4
-    for (int pc = p0; pc < p1; ++pc) mine += __popc(__ballot_sync(0xffffffffu, present(pc * 32 + lane)));
+    for (int pc = p0 + HELD; pc < p1; ++pc) mine += __popc(__ballot_sync(0xffffffffu, present(pc * 32 + lane)));
     if (lane == 0) red[warp] = mine;
     __syncthreads();
     int base = 0, total = 0;
 #pragma unroll
     for (int w = 0; w < kSplitWarps; ++w) { const int c = red[w]; total += c; if (w < warp) base += c; }
+    auto put = [&](int pc, unsigned m) {
+        if ((m >> lane) & 1u) valid[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(pc * 32 + lane);
+        base += __popc(m);
+    };
+#pragma unroll
+    for (int j = 0; j < HELD; ++j) put(p0 + j, bm[j]);
 #pragma unroll 4
-    for (int pc = p0; pc < p1; ++pc) {
-        const bool ok = present(pc * 32 + lane);
-        const unsigned bm = __ballot_sync(0xffffffffu, ok);
-        if (ok) valid[base + __popc(bm & ((1u << lane) - 1u))] = (uint16_t)(pc * 32 + lane);
-        base += __popc(bm);
-    }
+    for (int pc = p0 + HELD; pc < p1; ++pc) put(pc, __ballot_sync(0xffffffffu, present(pc * 32 + lane)));
     return total;
 }
 
@@ -464,7 +475,16 @@ attend_split_select_kernel(const __grid_constant__ SplitArgs a) {
     const int i0 = (wi * 32 + lane) * KPT;
     uint32_t key[KPT], hi = 0u, lo = 0xffffffffu;
 #pragma unroll
-    for (int j = 0; j < KPT; ++j) key[j] = i0 + j < Tv ? sentry_order_key(__ldg(ms + i0 + j)) : 0u;
+    for (int j = 0; j < KPT; j += 4) {
+        if ((a.T & 3) == 0 && i0 + j + 4 <= Tv) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(ms + i0 + j));
+            key[j] = sentry_order_key(v.x); key[j + 1] = sentry_order_key(v.y);
+            key[j + 2] = sentry_order_key(v.z); key[j + 3] = sentry_order_key(v.w);
+        } else {
+#pragma unroll
+            for (int e = j; e < j + 4; ++e) key[e] = i0 + e < Tv ? sentry_order_key(__ldg(ms + i0 + e)) : 0u;
+        }
+    }
 #pragma unroll
     for (int j = 0; j < KPT; ++j)
         if (i0 + j < Tv) { hi = max(hi, key[j]); lo = min(lo, key[j]); }
@@ -669,6 +689,25 @@ attend_split_rows_kernel(const __grid_constant__ SplitArgs a) {
             for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
 #pragma unroll 1
         for (int kk = 0; kk < n_keys; kk += 32) {
+            // V of keys 2 tq, 2 tq + 1 and the two 8 further on (both halves of the step), dims gq * D/8 ..: on the way while
+            // the scores and their softmax are computed
+            uint32_t v[2][4][NT / 2];
+#pragma unroll
+            for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int key = min(kk + ks * 16 + 2 * tq + (i & 1) + (i >> 1) * 8, n_keys - 1);
+                    const __nv_bfloat16* src = Vg + (uint32_t)s_tok[key] * D;
+                    if constexpr (D == 16) {
+                        v[ks][i][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
+                    } else if constexpr (D == 32) {
+                        const uint2 x = __ldg(reinterpret_cast<const uint2*>(src));
+                        v[ks][i][0] = x.x; v[ks][i][1] = x.y;
+                    } else {
+                        const uint4 x = __ldg(reinterpret_cast<const uint4*>(src));
+                        v[ks][i][0] = x.x; v[ks][i][1] = x.y; v[ks][i][2] = x.z; v[ks][i][3] = x.w;
+                    }
+                }
             float s[4][4];
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt) {
@@ -727,26 +766,11 @@ attend_split_rows_kernel(const __grid_constant__ SplitArgs a) {
                 pb[3] = pack2_rem(s[2 * ks + 1][2], s[2 * ks + 1][3], pa[3]);
                 l_run[0] += (s[2 * ks][0] + s[2 * ks][1]) + (s[2 * ks + 1][0] + s[2 * ks + 1][1]);
                 l_run[1] += (s[2 * ks][2] + s[2 * ks][3]) + (s[2 * ks + 1][2] + s[2 * ks + 1][3]);
-                // V of keys 2 tq, 2 tq + 1 and the two 8 further on, dims gq * D/8 ..
-                uint32_t v[4][NT / 2];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int key = min(kk + ks * 16 + 2 * tq + (i & 1) + (i >> 1) * 8, n_keys - 1);
-                    const __nv_bfloat16* src = Vg + (uint32_t)s_tok[key] * D;
-                    if constexpr (D == 16) {
-                        v[i][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
-                    } else if constexpr (D == 32) {
-                        const uint2 x = __ldg(reinterpret_cast<const uint2*>(src));
-                        v[i][0] = x.x; v[i][1] = x.y;
-                    } else {
-                        const uint4 x = __ldg(reinterpret_cast<const uint4*>(src));
-                        v[i][0] = x.x; v[i][1] = x.y; v[i][2] = x.z; v[i][3] = x.w;
-                    }
-                }
 #pragma unroll
                 for (int j = 0; j < NT; ++j) {
                     const uint32_t sel = (j & 1) ? 0x7632u : 0x5410u;
-                    const uint32_t b0 = __byte_perm(v[0][j / 2], v[1][j / 2], sel), b1 = __byte_perm(v[2][j / 2], v[3][j / 2], sel);
+                    const uint32_t b0 = __byte_perm(v[ks][0][j / 2], v[ks][1][j / 2], sel),
+                                   b1 = __byte_perm(v[ks][2][j / 2], v[ks][3][j / 2], sel);
                     mma_bf16_16816(acc[j], pa, b0, b1);
                     mma_bf16_16816(acc[j], pb, b0, b1);
                 }
@@ -777,13 +801,16 @@ attend_split_rows_kernel(const __grid_constant__ SplitArgs a) {
 // grid (B * Hk, token slices).  Context rows (mean of V_g) on the present tokens that are not active, zeros on absent
 // ones, 16 bytes per store; with the keys in parts, the slices also share out the row tiles and merge their parts.
 // Bound by writing O.
-template <int D>
-__global__ void __launch_bounds__(kSplitThreads)
+// P: room for the parts (1: none to merge).  16 parts of loads in flight take 80 registers, 3 blocks per SM; fewer parts
+// leave more.
+template <int D, int P>
+__global__ void __launch_bounds__(kSplitThreads, P < 16 ? 4 : (D == 64 ? 2 : 3))
 attend_split_fill_kernel(const __grid_constant__ SplitArgs a) {
     constexpr int NT = D / 8, CPR = D / 8;
     extern __shared__ __align__(128) uint8_t s_raw[];   // active bits [kMaxRK][words of the slice]
     __shared__ int s_hs[kMaxRK], s_khs[kMaxRK], s_rk;
     __shared__ __align__(16) unsigned short s_mean[D];
+    __shared__ float s_acc[P > 1 ? D / 2 : 1][32];
     uint32_t* s_bits = reinterpret_cast<uint32_t*>(s_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gq = lane >> 2, tq = lane & 3;
     const int grp = blockIdx.x;
@@ -799,8 +826,13 @@ attend_split_fill_kernel(const __grid_constant__ SplitArgs a) {
             const int nb = (q.Tv + kScoreBlock - 1) / kScoreBlock;
             const float* vs = a.vsum + (size_t)grp * a.n_blk * D + threadIdx.x;
             float t = 0.f;
-#pragma unroll 4
-            for (int i = 0; i < nb; ++i) t += vs[i * D];
+            for (int i0 = 0; i0 < nb; i0 += 16) {   // 16 sums on the way at once, added in order
+                float v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] = i0 + i < nb ? vs[(i0 + i) * D] : 0.f;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) t += v[i];
+            }
             s_mean[threadIdx.x] = att_bits(t / (float)q.Tv);
         }
         for (int r = threadIdx.x; r < q.rk * q.Ue; r += kSplitThreads) {
@@ -810,6 +842,58 @@ attend_split_fill_kernel(const __grid_constant__ SplitArgs a) {
         }
     }
     __syncthreads();
+    if constexpr (P > 1) if (q.Tv > 0) {
+        // the parts of a row tile, by the whole block: a warp takes D/16 of the lanes' D/2 accumulator words, and all loads of
+        // all parts are on the way at once (one warp per tile, part after part, took 40 of the launch's 48 K cycles)
+        const float sl2 = rsqrtf((float)D) * 1.4426950408889634f;
+        const size_t step = (size_t)kRowTiles * part_words(D) * 32;
+        for (int tile = (int)blockIdx.y; tile < q.n_tiles; tile += (int)gridDim.y) {
+            const float* src = a.part + ((size_t)grp * a.nsplit * kRowTiles + tile) * part_words(D) * 32 + lane;
+            float w[2][P], v[D / 16][P];
+#pragma unroll
+            for (int sp = 0; sp < P; ++sp) {
+                const bool in = sp < a.nsplit;
+#pragma unroll
+                for (int h2 = 0; h2 < 2; ++h2) w[h2][sp] = in ? src[sp * step + (NT * 4 + h2) * 32] : -INFINITY;
+#pragma unroll
+                for (int k = 0; k < D / 16; ++k) v[k][sp] = in ? src[sp * step + (warp * (D / 16) + k) * 32] : 0.f;
+            }
+#pragma unroll
+            for (int h2 = 0; h2 < 2; ++h2) {
+                float m = w[h2][0];
+#pragma unroll
+                for (int sp = 1; sp < P; ++sp) m = fmaxf(m, w[h2][sp]);
+#pragma unroll
+                for (int sp = 0; sp < P; ++sp)
+                    w[h2][sp] = w[h2][sp] == -INFINITY ? 0.f : fast_exp2((w[h2][sp] - m) * sl2);   // (empty parts: 0)
+            }
+#pragma unroll
+            for (int k = 0; k < D / 16; ++k) {
+                const int h2 = ((warp * (D / 16) + k) >> 1) & 1;
+                float t = 0.f;
+#pragma unroll
+                for (int sp = 0; sp < P; ++sp) t = fmaf(v[k][sp], h2 ? w[1][sp] : w[0][sp], t);
+                s_acc[warp * (D / 16) + k][lane] = t;
+            }
+            __syncthreads();
+            if (warp < 2) {   // warp h2: rows gq + 8 h2 of the tile
+                float l = 0.f, acc[NT][4];
+#pragma unroll
+                for (int sp = 0; sp < P; ++sp)
+                    if (sp < a.nsplit) l = fmaf(src[sp * step + (NT * 4 + 2 + warp) * 32], warp ? w[1][sp] : w[0][sp], l);
+                l += __shfl_xor_sync(0xffffffffu, l, 1);
+                l += __shfl_xor_sync(0xffffffffu, l, 2);
+#pragma unroll
+                for (int n = 0; n < NT; ++n)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) acc[n][e] = s_acc[n * 4 + 2 * warp + e][lane];
+                int h, kh;
+                const int t = active_token(a, q, s_hs, s_khs, tile * 16 + gq + warp * 8, mask, h, kh);
+                if (t >= 0) store_cols<D>(a.O + (((size_t)q.b * a.k_h + kh) * a.T + t) * D + tq * (D / 4), acc, 0, 1.0f / l);
+            }
+            __syncthreads();
+        }
+    }
     const uint4* mean4 = reinterpret_cast<const uint4*>(s_mean);
     for (int hh = 0; hh < q.rk; ++hh) {
         uint4* dst = reinterpret_cast<uint4*>(a.O + ((size_t)q.b * a.k_h + s_khs[hh]) * a.T * D);
@@ -822,40 +906,6 @@ attend_split_fill_kernel(const __grid_constant__ SplitArgs a) {
             dst[i] = m >= 0 && m < 32 && ((mask >> m) & 1u) ? mean4[cc] : make_uint4(0, 0, 0, 0);
         }
     }
-    if (a.nsplit == 1 || q.Tv == 0) return;
-    const float sl2 = rsqrtf((float)D) * 1.4426950408889634f;
-    for (int tile = (int)blockIdx.y * kSplitWarps + warp; tile < q.n_tiles; tile += (int)gridDim.y * kSplitWarps) {
-        float acc[NT][4], m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
-#pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
-        for (int sp = 0; sp < a.nsplit; ++sp) {
-            const float* src = a.part + (((size_t)grp * a.nsplit + sp) * kRowTiles + tile) * part_words(D) * 32 + lane;
-            float ca[2], cb[2];
-#pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
-                const float mo = src[(NT * 4 + h2) * 32], m_new = fmaxf(m_run[h2], mo);
-                ca[h2] = m_run[h2] == -INFINITY ? 0.f : fast_exp2((m_run[h2] - m_new) * sl2);
-                cb[h2] = mo == -INFINITY ? 0.f : fast_exp2((mo - m_new) * sl2);   // an empty part
-                m_run[h2] = m_new;
-                l_run[h2] = l_run[h2] * ca[h2] + src[(NT * 4 + 2 + h2) * 32] * cb[h2];
-            }
-#pragma unroll
-            for (int n = 0; n < NT; ++n)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) acc[n][e] = acc[n][e] * ca[e >> 1] + src[(n * 4 + e) * 32] * cb[e >> 1];
-        }
-#pragma unroll
-        for (int h2 = 0; h2 < 2; ++h2) {
-            float l = l_run[h2];
-            l += __shfl_xor_sync(0xffffffffu, l, 1);
-            l += __shfl_xor_sync(0xffffffffu, l, 2);
-            int h, kh;
-            const int t = active_token(a, q, s_hs, s_khs, tile * 16 + gq + h2 * 8, mask, h, kh);
-            if (t >= 0) store_cols<D>(a.O + (((size_t)q.b * a.k_h + kh) * a.T + t) * D + tq * (D / 4), acc, h2, 1.0f / l);
-        }
-    }
 }
 
 // ------------------------------------------------------------------------------------------ launch
@@ -865,7 +915,7 @@ int split_parts(const sentry_attend_desc& d) {
     long long n = (444 + groups - 1) / groups;
     const long long most = (d.T + 255) / 256;
     if (n > most) n = most;
-    return (int)(n > 16 ? 16 : (n < 1 ? 1 : n));
+    return (int)(n > kMaxParts ? kMaxParts : (n < 1 ? 1 : n));
 }
 
 struct SplitWs { uint16_t* valid; int* tv; float *vsum, *part; };
@@ -926,12 +976,13 @@ int launch_d(sentry_ctx* ctx, const AttendArgs& a, const SplitWs& w, cudaStream_
     LaunchScope ls(ctx, KS_ATT_CORE, st, 2);
     SENTRY_CUDA_TRY(launch_chained(attend_split_rows_kernel<D>, dim3(groups * (unsigned)p.nsplit), dim3(kSplitThreads),
                                    list / p.nsplit + 128, st, p));
-    // slices of the tokens: about four blocks per SM, at least 64 tokens each
-    long long slices = (4LL * ctx->sm_count + groups - 1) / groups;
+    // slices of the tokens: three or four blocks per SM, at least 64 tokens each
+    long long slices = ((p.nsplit > 4 ? 3LL : 4LL) * ctx->sm_count + groups - 1) / groups;
     if (slices > (d.T + 63) / 64) slices = (d.T + 63) / 64;
     if (slices < 1) slices = 1;
     const size_t bits = (size_t)kMaxRK * (((d.T + slices - 1) / slices + 31) / 32) * 4;
-    SENTRY_CUDA_TRY(launch_chained(attend_split_fill_kernel<D>, dim3(groups, (unsigned)slices), dim3(kSplitThreads), bits, st, p));
+    auto fill = p.nsplit == 1 ? attend_split_fill_kernel<D, 1> : (p.nsplit <= 4 ? attend_split_fill_kernel<D, 4> : attend_split_fill_kernel<D, kMaxParts>);
+    SENTRY_CUDA_TRY(launch_chained(fill, dim3(groups, (unsigned)slices), dim3(kSplitThreads), bits, st, p));
     return SENTRY_OK;
 }
 

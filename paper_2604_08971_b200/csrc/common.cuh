@@ -132,9 +132,11 @@ __host__ __device__ inline int sentry_ceil_ln(int T) {
                                      22026u, 59874u, 162754u, 442413u, 1202604u, 3269017u,
                                      8886110u, 24154952u, 65659969u, 178482300u, 485165195u,
                                      1318815734u};
-    int k = 0;
-    while (k < 21 && (unsigned int)T > fl_exp[k]) ++k;
-    if ((unsigned int)T > fl_exp[21]) k = 22;
+    int k = 0;   // (counted, not searched: no branches and no table in local memory)
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int i = 0; i < 22; ++i) k += (unsigned int)T > fl_exp[i] ? 1 : 0;
     return k;
 }
 __host__ __device__ inline int sentry_num_active(int T_v, int c) {
@@ -148,11 +150,11 @@ __host__ __device__ inline int sentry_num_active(int T_v, int c) {
 #ifdef __CUDACC__
 // The next kernel of the stream may be scheduled from here on (it waits for this one's end by itself).
 __device__ __forceinline__ void grid_dependents_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// Every kernel before this one in the stream has completed and its writes are visible.
 // For kernels of any size: early where their blocks leave SMs free anyway.
 __device__ __forceinline__ void grid_dependents_start_if_small() {
     if (gridDim.x * gridDim.y <= 128u) grid_dependents_start();
 }
+// Every kernel before this one in the stream has completed and its writes are visible.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Order-preserving map float -> uint32 for "score descending" selection:
