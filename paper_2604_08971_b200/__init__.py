@@ -289,10 +289,8 @@ class Sentry:
                     heads_per_group: int = 0, kept: Optional[torch.Tensor] = None):
         """sentry_gate_select: scores [S,n] fp32, masks [n_masks] int32/uint32 bit patterns.
         Returns kept [n_masks,k] int32 (and the KV-group bitmaps if heads_per_group > 0)."""
-        if kept is None:
-            kept = torch.empty((masks.shape[0], k), dtype=torch.int32, device=scores.device)
         groups = torch.empty((masks.shape[0],), dtype=torch.int32, device=scores.device) if heads_per_group > 0 else None
-        _binding.gate_select(self, self._handle, self._ws_bytes, scores, masks, k, kept, groups, heads_per_group)
+        kept = _binding.gate_select(self, self._handle, self._ws_bytes, scores, masks, k, kept, groups, heads_per_group)
         return (kept, groups) if heads_per_group > 0 else kept
 
     def gate_select_multi(self, sets):
@@ -370,13 +368,7 @@ class Sentry:
     def ffn_prepack(self, W1, W2, kept_channels, packed=None):
         """sentry_ffn_prepack: materialise W1[:, N], W2[N, :] of every kept list once.  Returns the
         packed buffer (a uint8 tensor) for ffn_fwd_packed."""
-        if packed is None:
-            D, F = W1.shape
-            n_lists, k_c = kept_channels.shape if kept_channels.dim() == 2 else (1, kept_channels.shape[0])
-            desc = FfnDesc(1, 1, D, F, k_c, n_lists, _dtype_code(W1))
-            packed = torch.empty((int(self.lib.sentry_ffn_packed_bytes(ctypes.byref(desc))),), dtype=torch.uint8, device=W1.device)
-        _binding.ffn_prepack(self, self._handle, self._ws_bytes, W1, W2, kept_channels, packed)
-        return packed
+        return _binding.ffn_prepack(self, self._handle, self._ws_bytes, W1, W2, kept_channels, packed)
 
     def ffn_prepack_fp8(self, W1q, W2q, scale_w1: float, scale_w2: float, kept_channels, dtype=torch.bfloat16,
                         packed=None):
@@ -434,17 +426,13 @@ class Sentry:
 
     def gate_eval(self, layer_offsets, zeta, gamma, W1, b1, w2, b2, return_gates: bool = False):
         """sentry_gate_eval: logits (and gates) [2^M, n_units] of SentryGate's per-unit MLP (Eq. 1)."""
-        n_units, _, M = W1.shape
-        logits = torch.empty((1 << M, n_units), dtype=torch.float32, device=W1.device)
-        gates = torch.empty_like(logits) if return_gates else None
-        _binding.gate_eval(self, self._handle, self._ws_bytes, layer_offsets, zeta, gamma, W1, b1, w2, b2, logits, gates)
+        gates = torch.empty((1 << W1.shape[2], W1.shape[0]), dtype=torch.float32, device=W1.device) if return_gates else None
+        logits = _binding.gate_eval(self, self._handle, self._ws_bytes, layer_offsets, zeta, gamma, W1, b1, w2, b2, None, gates)
         return (logits, gates) if return_gates else logits
 
     def gate_layer_counts(self, kept, layer_offsets):
         """sentry_gate_layer_counts: kept [n_masks, k] ascending -> counts [n_masks, n_layers]."""
-        counts = torch.empty((kept.shape[0], layer_offsets.shape[0] - 1), dtype=torch.int32, device=kept.device)
-        _binding.gate_layer_counts(self, self._handle, self._ws_bytes, kept, layer_offsets, counts)
-        return counts
+        return _binding.gate_layer_counts(self, self._handle, self._ws_bytes, kept, layer_offsets, None)
 
     def project_qkv(self, X, WQ, WK, WV, kept_heads, token_modality_ids, masks, Hq: int, Hk: int, d: int,
                     Q=None, K=None, V=None):

@@ -10,11 +10,13 @@
 // needs more than the given size.  The GIL is released around the library call.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
+#include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 
 #include "../../include/sentry.h"
 
@@ -52,12 +54,18 @@ const at::Tensor& tensor(PyObject* o, int dims) {
 }
 // Device address of a contiguous device tensor; None is a null pointer.
 template <typename T = void>
-T* ptr(PyObject* o) {
-    if (o == Py_None) return nullptr;
-    const at::Tensor& t = tensor(o);
+T* ptr(const at::Tensor& t) {
     if (!t.is_cuda()) raise(PyExc_ValueError, "libsentry takes device tensors (got a " + t.device().str() + " tensor)");
     if (!t.is_contiguous()) raise(PyExc_ValueError, "libsentry takes contiguous tensors");
     return (T*)t.data_ptr();
+}
+template <typename T = void>
+T* ptr(PyObject* o) {
+    return o == Py_None ? nullptr : ptr<T>(tensor(o));
+}
+// The caller's output, or a fresh one beside `like` (from native code: half the time of torch.empty).
+at::Tensor output(PyObject* o, at::IntArrayRef shape, at::ScalarType type, const at::Tensor& like) {
+    return o != Py_None ? tensor(o) : at::empty(shape, like.options().dtype(type));
 }
 int dtype_code(const at::Tensor& t) {
     switch (t.scalar_type()) {
@@ -111,8 +119,12 @@ template <typename F>
 PyObject* guarded(PyObject* const* args, Py_ssize_t n, Py_ssize_t want, F body) {
     try {
         Call c(args, n, want);
-        body(c);
-        Py_RETURN_NONE;
+        if constexpr (std::is_void_v<decltype(body(c))>) {
+            body(c);
+            Py_RETURN_NONE;
+        } else {
+            return THPVariable_Wrap(body(c));   // the output
+        }
     } catch (const Raised&) {
     } catch (const std::exception& e) {
         if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
@@ -132,7 +144,7 @@ void invoke(const char* what, F f) {
 
 // ------------------------------------------------------------------------------------------ gate
 METHOD(gate_select) {   // scores, masks, k, kept, groups, heads_per_group
-    return guarded(args, n, 6, [](Call& c) {
+    return guarded(args, n, 6, [](Call& c) -> at::Tensor {
         const at::Tensor& scores = tensor(c.a[0], 2);
         const at::Tensor& masks = tensor(c.a[1]);
         require(scores.scalar_type() == at::kFloat && (masks.scalar_type() == at::kInt || masks.scalar_type() == at::kUInt32),
@@ -141,11 +153,13 @@ METHOD(gate_select) {   // scores, masks, k, kept, groups, heads_per_group
         c.workspace(std::max<size_t>(1u << 20, (size_t)S * std::max(k, 0) * 4 + (size_t)S * 4 + 1024));
         const float* sc = ptr<float>(c.a[0]);
         const uint32_t* m = ptr<uint32_t>(c.a[1]);
-        int32_t* kept = ptr<int32_t>(c.a[3]);
+        at::Tensor out = output(c.a[3], {n_masks, k}, at::kInt, scores);
+        int32_t* kept = ptr<int32_t>(out);
         uint32_t* groups = ptr<uint32_t>(c.a[4]);
         const int hpg = small(c.a[5]);
         void* st = stream();
         invoke("sentry_gate_select", [&] { return sentry_gate_select(c.ctx, sc, S, units, m, n_masks, k, kept, groups, hpg, st); });
+        return out;
     });
 }
 METHOD(gate_select_multi) {   // list of (scores, masks, k, heads_per_group, kept, groups)
@@ -179,27 +193,31 @@ METHOD(gate_select_multi) {   // list of (scores, masks, k, heads_per_group, kep
     });
 }
 METHOD(gate_eval) {   // layer_offsets, zeta, gamma, W1, b1, w2, b2, logits, gates
-    return guarded(args, n, 9, [](Call& c) {
+    return guarded(args, n, 9, [](Call& c) -> at::Tensor {
         const at::Tensor& W1 = tensor(c.a[3], 3);
         const int units = (int)W1.size(0), hidden = (int)W1.size(1), M = (int)W1.size(2), layers = (int)tensor(c.a[2]).size(0);
         const int32_t* off = ptr<int32_t>(c.a[0]);
         const float *zeta = ptr<float>(c.a[1]), *gamma = ptr<float>(c.a[2]), *w1 = ptr<float>(c.a[3]), *b1 = ptr<float>(c.a[4]),
                     *w2 = ptr<float>(c.a[5]), *b2 = ptr<float>(c.a[6]);
-        float *logits = ptr<float>(c.a[7]), *gates = ptr<float>(c.a[8]);
+        at::Tensor out = output(c.a[7], {(int64_t)1 << std::min(M, 30), units}, at::kFloat, W1);
+        float *logits = ptr<float>(out), *gates = ptr<float>(c.a[8]);
         void* st = stream();
         invoke("sentry_gate_eval", [&] {
             return sentry_gate_eval(c.ctx, M, hidden, layers, off, units, zeta, gamma, w1, b1, w2, b2, logits, gates, st);
         });
+        return out;
     });
 }
 METHOD(gate_layer_counts) {   // kept, layer_offsets, counts
-    return guarded(args, n, 3, [](Call& c) {
+    return guarded(args, n, 3, [](Call& c) -> at::Tensor {
         const at::Tensor& kept = tensor(c.a[0], 2);
         const int n_masks = (int)kept.size(0), k = (int)kept.size(1), layers = (int)tensor(c.a[1]).size(0) - 1;
         const int32_t *kp = ptr<int32_t>(c.a[0]), *off = ptr<int32_t>(c.a[1]);
-        int32_t* counts = ptr<int32_t>(c.a[2]);
+        at::Tensor out = output(c.a[2], {n_masks, layers}, at::kInt, kept);
+        int32_t* counts = ptr<int32_t>(out);
         void* st = stream();
         invoke("sentry_gate_layer_counts", [&] { return sentry_gate_layer_counts(c.ctx, kp, n_masks, k, off, layers, counts, st); });
+        return out;
     });
 }
 
@@ -332,16 +350,18 @@ METHOD(ffn_fwd_fp8) {   // Xq, packed, F, k_c, n_lists, scale_x, scale_w1, scale
     });
 }
 METHOD(ffn_prepack) {   // W1, W2, kept_channels, packed
-    return guarded(args, n, 4, [](Call& c) {
+    return guarded(args, n, 4, [](Call& c) -> at::Tensor {
         const at::Tensor& W1 = tensor(c.a[0], 2);
         sentry_ffn_desc d;
         d.B = d.T = 1; d.D = (int)W1.size(0); d.F = (int)W1.size(1); d.dtype = dtype_code(W1);
         list_shape(tensor(c.a[2]), d.n_lists, d.k_c);
-        void *w1 = ptr(c.a[0]), *w2 = ptr(c.a[1]), *packed = ptr(c.a[3]);
+        at::Tensor out = c.a[3] != Py_None ? tensor(c.a[3]) : output(c.a[3], {(int64_t)sentry_ffn_packed_bytes(&d)}, at::kByte, W1);
+        void *w1 = ptr(c.a[0]), *w2 = ptr(c.a[1]), *packed = ptr(out);
         const int32_t* kept = ptr<int32_t>(c.a[2]);
-        const size_t bytes = (size_t)tensor(c.a[3]).numel();
+        const size_t bytes = (size_t)out.numel();
         void* st = stream();
         invoke("sentry_ffn_prepack", [&] { return sentry_ffn_prepack(c.ctx, &d, w1, w2, kept, packed, bytes, st); });
+        return out;
     });
 }
 METHOD(moe_ffn_fwd) {   // X, expert_ids, expert_weights, W1, W2, kept_channels, packed, F, E, k_c, Y
