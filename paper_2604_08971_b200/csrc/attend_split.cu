@@ -1,8 +1,8 @@
 // SentryAttend (Section 4.4, Eq. 6) for 16-bit tensors in four launches, each of which spreads over the whole GPU:
 //
-//   score   a warp scores batches of 8 query positions of one (sample, KV group) for all kept heads on the warp MMA, the
-//           sampled key rows gathered straight from global memory (they stay in L1: no staging, no barriers); the block
-//           also lists the sample's present tokens and sums V over its positions
+//   score   a warp scores batches of 8 query positions of one (sample, KV group) for all kept heads, with the arithmetic of
+//           the one-launch form (fused_score_pass), the sampled key rows copied to shared memory a few steps ahead; the
+//           block also lists the sample's present tokens and sums V over its positions
 //   select  the U best positions per head, a warp (T <= 1024) or a block each
 //   rows    Eq. 6 on tiles of 16 active rows, a warp per tile and part of the keys, K and V fragments from global memory
 //   fill    context and zero rows, and the merge of the key parts
@@ -10,17 +10,19 @@
 // A CTA per (sample, group) does the same in attend_bf16.cu and attend_long.cu: ten phases with a barrier after each, of
 // which every one is a chain of latencies, on as many SMs as there are groups.  Taken apart, each phase runs with as many
 // warps as it has work: the form for long sequences and for few groups (attend_split_faster in api.cu has the line).
-// Measured on 16 x 4096 tokens, d = 32, 4 of 8 heads kept: 310 us before, 91 as four launches (100 with the parts of Eq. 6
-// merged by one warp per tile and the token list read twice).
+// Measured on 16 x 4096 tokens, d = 32, 4 of 8 heads kept, one to three of three modalities present: 310 us in one CTA per
+// group, 81 as four launches.
 #include <math.h>
 #include <stddef.h>
+
+#include <type_traits>
 
 #include "attend_common.cuh"
 
 namespace {
 
 constexpr int kSplitThreads = 256, kSplitWarps = kSplitThreads / 32;
-constexpr int kScoreBlock = 128;                 // query positions per score block
+constexpr int kScoreBlock = 128;                 // query positions per score block (or two blocks with half of them each)
 constexpr int kRowTiles = kMaxRK * kMaxActive / 16;
 constexpr int kMaxParts = 16;                     // parts of the keys in the rows launch
 
@@ -47,55 +49,58 @@ __device__ __forceinline__ void ld_row_frag(uint32_t (&w)[D / 8], const __nv_bfl
         }
     }
 }
-// c0, c1 = rows 0..7 of the 16 x 8 x D product (rows 8..15 of A are zero and their results dropped)
-template <int D>
-__device__ __forceinline__ void mma_rows8(float& c0, float& c1, const uint32_t (&q)[D / 8], const uint32_t (&k)[D / 8]) {
-    float c2, c3;
-    asm("mma.sync.aligned.m16n8k16.row.col.f32." ATT_PTX_TYPE "." ATT_PTX_TYPE ".f32 {%0, %1, %2, %3}, {%4, %6, %5, %6}, "
-        "{%7, %8}, {%9, %9, %9, %9};"
-        : "=f"(c0), "=f"(c1), "=f"(c2), "=f"(c3) : "r"(q[0]), "r"(q[1]), "r"(0), "r"(k[0]), "r"(k[1]), "f"(0.f));
-#pragma unroll
-    for (int ks = 1; ks < D / 16; ++ks)
-        asm("mma.sync.aligned.m16n8k16.row.col.f32." ATT_PTX_TYPE "." ATT_PTX_TYPE ".f32 {%0, %1, %2, %3}, {%4, %6, %5, %6}, "
-            "{%7, %8}, {%0, %1, %2, %3};"
-            : "+f"(c0), "+f"(c1), "+f"(c2), "+f"(c3) : "r"(q[2 * ks]), "r"(q[2 * ks + 1]), "r"(0), "r"(k[2 * ks]), "r"(k[2 * ks + 1]));
-}
 
-// Present-token list of a sample, ascending, by 256 threads: every warp a run of 32-token pieces, after one count of what
-// comes before it.  red: kSplitWarps ints.  Returns T_v; the list is complete behind the caller's next barrier.
-__device__ __forceinline__ int list_present(const int32_t* __restrict__ ids, int T, uint32_t mask, uint16_t* valid, int* red) {
+// Present-token list of a sample, ascending, by 256 threads: every warp a run of 128-token pieces, four tokens to a lane and
+// all its loads on the way at once.  red: kSplitWarps ints.  Returns T_v; the list is complete behind the caller's next
+// barrier -- where T_v is above needed_from: there is nothing to do with the list otherwise.
+__device__ __forceinline__ int list_present(const int32_t* __restrict__ ids, int T, uint32_t mask, uint16_t* valid, int* red,
+                                            int needed_from) {
+    constexpr int MOST = 8192 / (128 * kSplitWarps);   // pieces of a warp's run (attend_bf16_supported: T <= 8192)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int pieces = (T + 31) / 32, per = (pieces + kSplitWarps - 1) / kSplitWarps;
-    const int p0 = min(warp * per, pieces), p1 = min(p0 + per, pieces);
-    auto present = [&](int t) {
-        const int m = t < T ? __ldg(ids + t) : -1;
-        return m >= 0 && m < 32 && ((mask >> m) & 1u);
-    };
-    constexpr int HELD = 8;       // ballots of the run's first pieces stay in registers (all of it up to T = 2048; 16 cost more)
-    unsigned bm[HELD];
-    int mine = 0;
-    {
-        bool ok[HELD];
+    const int per = ((T + 127) / 128 + kSplitWarps - 1) / kSplitWarps, t0 = warp * per * 128 + lane * 4;
+    const bool wide = ((uintptr_t)ids & 15) == 0;
+    int4 id[MOST];
 #pragma unroll
-        for (int j = 0; j < HELD; ++j) ok[j] = p0 + j < p1 && present((p0 + j) * 32 + lane);   // all loads on the way at once
-#pragma unroll
-        for (int j = 0; j < HELD; ++j) { bm[j] = __ballot_sync(0xffffffffu, ok[j]); mine += __popc(bm[j]); }
+    for (int j = 0; j < MOST; ++j) {
+        const int t = t0 + j * 128;
+        id[j] = make_int4(-1, -1, -1, -1);
+        if (j >= per || t >= T) continue;
+        if (wide && t + 4 <= T) {
+            id[j] = __ldg(reinterpret_cast<const int4*>(ids + t));
+        } else {
+            id[j].x = __ldg(ids + t);
+            if (t + 1 < T) id[j].y = __ldg(ids + t + 1);
+            if (t + 2 < T) id[j].z = __ldg(ids + t + 2);
+            if (t + 3 < T) id[j].w = __ldg(ids + t + 3);
+        }
     }
-#pragma unroll 4
-    for (int pc = p0 + HELD; pc < p1; ++pc) mine += __popc(__ballot_sync(0xffffffffu, present(pc * 32 + lane)));
+    auto present = [&](int m) { return m >= 0 && m < 32 ? (mask >> m) & 1u : 0u; };
+    uint32_t bits = 0u;                            // four per piece
+#pragma unroll
+    for (int j = 0; j < MOST; ++j)
+        bits |= (present(id[j].x) | present(id[j].y) << 1 | present(id[j].z) << 2 | present(id[j].w) << 3) << (4 * j);
+    const int mine = __reduce_add_sync(0xffffffffu, __popc(bits));
     if (lane == 0) red[warp] = mine;
     __syncthreads();
     int base = 0, total = 0;
 #pragma unroll
     for (int w = 0; w < kSplitWarps; ++w) { const int c = red[w]; total += c; if (w < warp) base += c; }
-    auto put = [&](int pc, unsigned m) {
-        if ((m >> lane) & 1u) valid[base + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(pc * 32 + lane);
-        base += __popc(m);
-    };
+    if (total <= needed_from) return total;
 #pragma unroll
-    for (int j = 0; j < HELD; ++j) put(p0 + j, bm[j]);
-#pragma unroll 4
-    for (int pc = p0 + HELD; pc < p1; ++pc) put(pc, __ballot_sync(0xffffffffu, present(pc * 32 + lane)));
+    for (int j = 0; j < MOST; ++j) {
+        if (j >= per) break;
+        const uint32_t b4 = bits >> (4 * j) & 15u, lt = (1u << lane) - 1u;
+        int at = base;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t bm = __ballot_sync(0xffffffffu, (b4 >> k) & 1u);
+            at += __popc(bm & lt);
+            base += __popc(bm);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if ((b4 >> k) & 1u) valid[at++] = (uint16_t)(t0 + j * 128 + k);
+    }
     return total;
 }
 
@@ -116,17 +121,6 @@ __device__ __forceinline__ int warp_group_heads(const int32_t* kept_row, int k_h
     }
     return min(rk, kMaxRK);
 }
-
-// Where the sampled key positions of a query come from.
-struct SampleSrc {
-    const int32_t* tbl;   // table of the sample's subset (null in score_mode 1)
-    int n_s;              // sampled keys per query
-    int cnt;              // keys a query is scored on: n_s, or T_v in score_mode 1
-    int score_mode;
-    __device__ __forceinline__ int at(int p, int a, int Tv) const {
-        return score_mode == 1 ? a : __ldg(tbl + (score_mode == 2 ? (size_t)a * Tv + p : (size_t)p * n_s + a));
-    }
-};
 
 struct SplitArgs {
     const __nv_bfloat16 *Q, *K, *V;
@@ -151,117 +145,233 @@ struct SplitArgs {
 };
 
 // ------------------------------------------------------------------------------------------ score
-// Max and sum of the scores of the lane's row over NT tiles of 8 sampled keys; idx: this lane's first staged token.
-// tail: valid columns of the last tile counted from this lane's first.
-template <int D, int NT>
-__device__ __forceinline__ void score_query(const uint32_t (&qf)[D / 8], const __nv_bfloat16* Kg, const uint16_t* idx, int tq,
-                                            int tail, float& mx, float& sm) {
-    mx = -INFINITY;
-    float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-        uint32_t kf[D / 8];
-        ld_row_frag<D>(kf, Kg + (uint32_t)idx[t * 8] * D, tq);
-        float c0, c1;
-        mma_rows8<D>(c0, c1, qf, kf);
-        mx = max3(mx, c0, c1);
-        if (t == NT - 1) {
-            c0 = tail > 0 ? c0 : 0.f;
-            c1 = tail > 1 ? c1 : 0.f;
-        }
-        s0 += c0;
-        s1 += c1;
-    }
-    sm = s0 + s1;
-}
-
-// The rows of several queries sit in the A operand together (8 / kept heads of them): a tile of sampled keys belongs to
-// one of them, the lanes of the other rows drop theirs, and the query fragment and the reduction across lanes are paid
-// once per set.  NT = key tiles per query (0: every present key, no table).
-template <int D, int NT>
-__device__ __forceinline__ void score_batches(const __nv_bfloat16* __restrict__ qh, const __nv_bfloat16* __restrict__ Kg,
-                                              float* __restrict__ out, bool mine, int lh, const uint16_t* s_valid,
-                                              uint16_t* s_idx, int Tv, int p_begin, int p_end, const SampleSrc& src, int warp,
-                                              unsigned int* status) {
-    constexpr int W = D / 8;
-    const int lane = threadIdx.x & 31, gq = lane >> 2, tq = lane & 3;
-    const int my_j = gq >> lh, QP = 8 >> lh;
-    const float scale = rsqrtf((float)D), inv_cnt = 1.0f / (float)src.cnt;
-    for (int p0 = p_begin + warp * 8; p0 < p_end; p0 += kSplitWarps * 8) {
-        if constexpr (NT > 0) {
-            // 8 queries x 8 NT sampled positions -> tokens; entries past the count repeat the last one
-            const int q = lane & 7, a4 = lane >> 3, p = min(p0 + q, Tv - 1);
-            const int first = src.score_mode == 2 ? p : p * src.n_s, es = src.score_mode == 2 ? Tv : 1;
-            int e[2 * NT];
-#pragma unroll
-            for (int i = 0; i < 2 * NT; ++i) {
-                const int at = i < 2 * NT - 2 ? 4 * i + a4 : min(4 * i + a4, src.cnt - 1);
-                e[i] = __ldg(src.tbl + (first + at * es));
-            }
-            bool bad = false;
-#pragma unroll
-            for (int i = 0; i < 2 * NT; ++i) {
-                if ((unsigned)e[i] >= (unsigned)Tv) { bad = true; e[i] = 0; }
-                s_idx[q * NT * 8 + 4 * i + a4] = s_valid[e[i]];
-            }
-            if (bad) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
-            __syncwarp();
-        }
-#pragma unroll 1
-        for (int j0 = 0; j0 < 8 && p0 + j0 < p_end; j0 += QP) {
-            uint32_t qf[W];
-#pragma unroll
-            for (int i = 0; i < W; ++i) qf[i] = 0u;
-            const int pq = p0 + j0 + my_j;
-            if (mine && pq < p_end) ld_row_frag<D>(qf, qh + (uint32_t)s_valid[pq] * D, tq);
-            float M = -INFINITY, Sm = 0.f;
-            if constexpr (NT > 0) {
-                const int nq = min(QP, p_end - p0 - j0);
-                const uint16_t* my_idx = s_idx + j0 * NT * 8 + gq;
-                const int tail = src.cnt - (NT - 1) * 8 - 2 * tq;
-#pragma unroll 1
-                for (int j = 0; j < nq; ++j, my_idx += NT * 8) {
-                    float mx, sm;
-                    score_query<D, NT>(qf, Kg, my_idx, tq, tail, mx, sm);
-                    if (my_j == j) { M = mx; Sm = sm; }
-                }
-            } else {
-                // all present keys: the same key tiles for every query row, so one walk serves the whole set
-                for (int t = 0; t * 8 < Tv; ++t) {
-                    uint32_t kf[W];
-                    ld_row_frag<D>(kf, Kg + (uint32_t)s_valid[min(t * 8 + gq, Tv - 1)] * D, tq);
-                    float c0, c1;
-                    mma_rows8<D>(c0, c1, qf, kf);
-                    M = max3(M, c0, t * 8 + 2 * tq + 1 < Tv ? c1 : c0);
-                    if (t * 8 + 2 * tq < Tv) Sm += c0;
-                    if (t * 8 + 2 * tq + 1 < Tv) Sm += c1;
-                }
-            }
-#pragma unroll
-            for (int o = 1; o < 4; o <<= 1) {
-                M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-                Sm += __shfl_xor_sync(0xffffffffu, Sm, o);
-            }
-            if (mine && tq == 0 && pq < p_end) out[pq] = (M - Sm * inv_cnt) * scale;
-        }
-        __syncwarp();   // the staged positions are free for the next batch
-    }
-}
-
-// grid B * Hk * n_blk (blocks of a group together).  Dynamic smem: valid[T] u16 | staged tokens of the warps' batches.
-// Bound by the L1's gathers of key rows, 16 bytes a lane: with four lanes to a 64-byte row they take 6 cycles a warp.  128
-// query positions per block: a batch of 8 for every warp twice, which leaves 4 blocks per SM at 16 x 4096.
+// A warp scores batches of 8 query positions; the four lanes of a quad take four keys of one of them.  Shared memory of a
+// block: per warp a ring of copied key rows (a step's 32, one per lane) and the tokens of its batches' sampled keys, then
+// the sample's present-token list.
+constexpr int kBatch = 8;                         // query positions of a batch
+constexpr int kBatches = kScoreBlock / (kBatch * kSplitWarps);   // of a warp
+constexpr int kTokPitch = kMaxActive + 2;
 template <int D>
-__global__ void __launch_bounds__(kSplitThreads, 4)
-attend_split_score_kernel(const __grid_constant__ SplitArgs a) {
+struct ScoreSmem {
+    static constexpr int STAGES = 3;
+    static constexpr int STAGE_BYTES = 32 * D * 2;
+    static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
+    static constexpr int TOK_AT = kSplitWarps * RING_BYTES;
+    static constexpr int VALID_AT = TOK_AT + kSplitWarps * kBatches * kBatch * kTokPitch * 2;
+};
+
+// Tokens of the sampled keys of a warp's batches: s_tok[(batch * kBatch + q) * kTokPitch + a].  Positions outside the list are
+// flagged and count as position 0; entries from n_s on (to a multiple of 4) repeat the last one, queries past the list those
+// of the last.
+__device__ __forceinline__ void stage_tokens(const int32_t* __restrict__ tbl, int score_mode, int n_s, int p0, int batches, int Tv,
+                                             const uint16_t* s_valid, uint16_t* s_tok, unsigned int* status) {
+    constexpr int PER = kMaxActive / 4;            // table entries of a lane and batch, all on the way at once
+    const int lane = threadIdx.x & 31, q = lane & 7, a4 = lane >> 3, n4 = (n_s + 3) & ~3;
+    const size_t es = score_mode == 2 ? (size_t)Tv : 1;
+    int e[kBatches][PER];
+#pragma unroll
+    for (int b = 0; b < kBatches; ++b) {
+        const int p = min(p0 + b * kBatch * kSplitWarps + q, Tv - 1);
+        const int32_t* src = tbl + (score_mode == 2 ? (size_t)p : (size_t)p * n_s);
+#pragma unroll
+        for (int i = 0; i < PER; ++i) e[b][i] = b < batches && 4 * i < n4 ? __ldg(src + (size_t)min(4 * i + a4, n_s - 1) * es) : 0;
+    }
+    bool bad = false;
+#pragma unroll
+    for (int b = 0; b < kBatches; ++b) {
+        if (b >= batches) break;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            if (4 * i >= n4) break;
+            if ((unsigned)e[b][i] >= (unsigned)Tv) { bad = true; e[b][i] = 0; }
+            s_tok[(b * kBatch + q) * kTokPitch + 4 * i + a4] = s_valid[e[b][i]];
+        }
+    }
+    if (bad) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+}
+
+// The query rows of a token, as they are stored.
+template <int D, int NH>
+__device__ __forceinline__ void load_queries(uint32_t (&q)[NH][D / 2], const __nv_bfloat16* const (&qh)[NH], uint32_t tok) {
+#pragma unroll
+    for (int h = 0; h < NH; ++h)
+#pragma unroll
+        for (int c = 0; c < D / 8; ++c) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(qh[h] + tok * D) + c);
+            q[h][4 * c] = v.x; q[h][4 * c + 1] = v.y; q[h][4 * c + 2] = v.z; q[h][4 * c + 3] = v.w;
+        }
+}
+// Dot products of NH query rows with a key row, chunk by chunk (8 elements) from `chunk`, each in the four accumulators and
+// the order of the one-launch form (fused_score_pass), so that the two forms round alike.
+template <int D, int NH, typename Chunk>
+__device__ __forceinline__ void dot_rows(const uint32_t (&q)[NH][D / 2], Chunk chunk, float scale, float (&sc)[NH]) {
+    float acc[NH][4];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) acc[h][0] = acc[h][1] = acc[h][2] = acc[h][3] = 0.f;
+#pragma unroll
+    for (int c = 0; c < D / 8; ++c) {
+        const uint4 v = chunk(c);
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            fma_bf16_pair(acc[h][0], acc[h][1], q[h][4 * c], v.x);
+            fma_bf16_pair(acc[h][2], acc[h][3], q[h][4 * c + 1], v.y);
+            fma_bf16_pair(acc[h][0], acc[h][1], q[h][4 * c + 2], v.z);
+            fma_bf16_pair(acc[h][2], acc[h][3], q[h][4 * c + 3], v.w);
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < NH; ++h) sc[h] = __fmul_rn((acc[h][0] + acc[h][1]) + (acc[h][2] + acc[h][3]), scale);
+}
+
+// Scores M = max_j s_j - mean_j s_j of NH heads for the warp's batches of query positions (p: the quad's in the first one)
+// over their sampled keys, in table order.  The rows come through the warp's ring, STAGES - 1 steps ahead, copied with D/8
+// lanes to a row, so that a copy instruction touches few lines, and read back as a whole row per lane without bank
+// conflicts (Sw).  Every lane of the quad adds the quad's four scores in key order.
+template <int D, int NH>
+__device__ __forceinline__ void score_sampled(const __nv_bfloat16* const (&qh)[NH], const __nv_bfloat16* __restrict__ Kg,
+                                              float* const (&out)[NH], const uint16_t* s_valid, const uint16_t* s_tok,
+                                              uint32_t ring, int n_s, int p, int batches, int Tv) {
+    using S = Sw<D>;
+    using M = ScoreSmem<D>;
+    constexpr int RPC = 32 / S::CPR;                // rows of a copy instruction
+    const int lane = threadIdx.x & 31, tq = lane & 3, row0 = lane / S::CPR, cc = lane % S::CPR;
+    const float scale = rsqrtf((float)D), inv_cnt = 1.0f / (float)n_s;
+    const int steps = (n_s + 3) / 4;                // of a batch
+    const __nv_bfloat16* Kc = Kg + cc * 8;
+    const uint32_t copy_to = ring + S::off(row0, cc), row_at = ring + S::off(lane, 0);
+    const uint16_t* tp = s_tok + (row0 >> 2) * kTokPitch + (row0 & 3);
+    int f_left = batches * steps, f_step = 0;       // what is still to be fetched
+    auto fetch = [&](uint32_t stage) {              // stage: byte offset in the ring
+        if (f_left > 0) {
+#pragma unroll
+            for (int i = 0; i < S::CPR; ++i) {
+                // (row i * RPC + row0 is swizzled as row0 is; d = 64: with bit 2 of the row in every other i)
+                const uint32_t to = (D == 64 ? copy_to ^ ((i & 1) << 6) : copy_to) + stage + i * RPC * S::RB;
+                ptx::cp_async_16(to, Kc + (uint32_t)tp[i * (RPC / 4) * kTokPitch + f_step * 4] * D);
+            }
+            --f_left;
+            if (++f_step == steps) { f_step = 0; tp += kBatch * kTokPitch; }
+        }
+        ptx::cp_async_commit();
+    };
+    __syncwarp();                                   // the ring is free, the tokens are there
+#pragma unroll
+    for (int s = 0; s < M::STAGES - 1; ++s) fetch(s * M::STAGE_BYTES);
+    uint32_t stage = 0, ahead = M::RING_BYTES - M::STAGE_BYTES;
+#pragma unroll 1
+    for (int batch = 0; batch < batches; ++batch, p += kBatch * kSplitWarps) {
+        uint32_t q[NH][D / 2];
+        load_queries<D, NH>(q, qh, s_valid[min(p, Tv - 1)]);
+        float mx[NH], sum[NH], sc[NH];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) { mx[h] = -INFINITY; sum[h] = 0.f; }
+        auto take = [&](int n) {                    // the quad's four scores, of which n count
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                float v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = __shfl_sync(0xffffffffu, sc[h], j, 4);
+                if (n >= 4) {
+                    mx[h] = fmaxf(mx[h], sc[h]);
+                    sum[h] = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(sum[h], v[0]), v[1]), v[2]), v[3]);
+                } else {
+                    if (tq < n) mx[h] = fmaxf(mx[h], sc[h]);
+#pragma unroll
+                    for (int j = 0; j < 3; ++j)
+                        if (j < n) sum[h] = __fadd_rn(sum[h], v[j]);
+                }
+            }
+        };
+#pragma unroll 1
+        for (int step = 0; step < steps; ++step) {
+            ptx::cp_async_wait_group<M::STAGES - 2>();
+            __syncwarp();                           // every lane's copies of this step are there, the stage before is free
+            fetch(ahead);
+            const uint32_t addr = row_at + stage;
+            constexpr int EARLY = S::CPR <= 4 ? S::CPR : 2;   // under way while the step before is taken in
+            uint4 v[EARLY];
+#pragma unroll
+            for (int c = 0; c < EARLY; ++c) v[c] = lds128(addr ^ (c << 4));
+            if (step > 0) take(4);
+            dot_rows<D, NH>(q, [&](int c) { return c < EARLY ? v[c] : lds128(addr ^ (c << 4)); }, scale, sc);
+            ahead = stage;
+            stage = stage == M::RING_BYTES - M::STAGE_BYTES ? 0 : stage + M::STAGE_BYTES;
+        }
+        take(n_s - (steps - 1) * 4);
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
+            mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
+            if (tq == 0 && p < Tv) out[h][p] = __fmaf_rn(-sum[h], inv_cnt, mx[h]);
+        }
+    }
+}
+
+// The same for 32 positions, p the lane's, over every present key (score_mode 1): all lanes take the same row.
+template <int D, int NH>
+__device__ __forceinline__ void score_all(const __nv_bfloat16* const (&qh)[NH], const __nv_bfloat16* __restrict__ Kg,
+                                          float* const (&out)[NH], const uint16_t* s_valid, uint32_t ring, int p, int p_end,
+                                          int Tv) {
+    using S = Sw<D>;
+    using M = ScoreSmem<D>;
+    const int lane = threadIdx.x & 31, row0 = lane / S::CPR, cc = lane % S::CPR;
+    const float scale = rsqrtf((float)D), inv_cnt = 1.0f / (float)Tv;
+    const int steps = (Tv + 31) / 32;
+    auto fetch = [&](int step, uint32_t stage) {
+        if (step < steps) {
+#pragma unroll
+            for (int i = 0; i < S::CPR; ++i) {
+                const int r = i * (32 / S::CPR) + row0;
+                ptx::cp_async_16(ring + stage + S::off(r, cc), Kg + (size_t)s_valid[min(step * 32 + r, Tv - 1)] * D + cc * 8);
+            }
+        }
+        ptx::cp_async_commit();
+    };
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < M::STAGES - 1; ++s) fetch(s, s * M::STAGE_BYTES);
+    uint32_t q[NH][D / 2], stage = 0, ahead = M::RING_BYTES - M::STAGE_BYTES;
+    load_queries<D, NH>(q, qh, s_valid[min(p, Tv - 1)]);
+    float mx[NH], sum[NH];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) { mx[h] = -INFINITY; sum[h] = 0.f; }
+#pragma unroll 1
+    for (int step = 0; step < steps; ++step) {
+        ptx::cp_async_wait_group<M::STAGES - 2>();
+        __syncwarp();
+        fetch(step + M::STAGES - 1, ahead);
+        const int n = min(32, Tv - step * 32);
+#pragma unroll 2
+        for (int j = 0; j < n; ++j) score_one_key<D, NH>(q, ring + stage, j, scale, mx, sum);
+        ahead = stage;
+        stage = stage == M::RING_BYTES - M::STAGE_BYTES ? 0 : stage + M::STAGE_BYTES;
+    }
+#pragma unroll
+    for (int h = 0; h < NH; ++h)
+        if (p < p_end) out[h][p] = __fmaf_rn(-sum[h], inv_cnt, mx[h]);
+}
+
+// grid B * Hk * n_blk * subs (blocks of a group together).  Dynamic smem: ScoreSmem.
+//
+// The scores decide which rows are active, so they are rounded as the one-launch form rounds them, whatever the data: fp32
+// FMAs, four accumulators per dot product, the mean's sum in table order.  On the warp MMA the dot products take a tenth of
+// the instructions, but they round in another order; ranking those and scoring the contested entries again is either not
+// exact for keys with a large common part (a margin taken from the scores) or has contested entries in every other head (a
+// margin proved from the rows' norms: the selection 15 -> 25 us) and thousands where scores tie.  Bound by the issue of 200
+// instructions per 32 keys and two heads (0.57 per cycle and scheduler at 16 warps per SM) and by the shared-memory pipe
+// (half busy).  Whole calls on the MMA with a margin / here, us: 16 x 4096 tokens, d = 32: 82 / 81; 8 x 648, d = 64: 44 / 42;
+// 1 x 4096, d = 32: 51 / 36; 64 x 2048: 170 / 182; 16 x 2048, d = 64: 89 / 124; every key (score_mode 1), 32 x 1024: 133 / 185.
+template <int D, bool SAMPLED>
+__global__ void __launch_bounds__(kSplitThreads, 2)
+attend_split_score_kernel(const __grid_constant__ SplitArgs a, int subs) {
     extern __shared__ __align__(128) uint8_t s_raw[];
     __shared__ int red[kSplitWarps], s_hs[kMaxRK], s_khs[kMaxRK], s_rk;
     __shared__ int32_t s_kept[64];
     __shared__ float s_vs[kSplitWarps][D];
-    uint16_t* s_valid = reinterpret_cast<uint16_t*>(s_raw);
+    using M = ScoreSmem<D>;
+    uint16_t* s_valid = reinterpret_cast<uint16_t*>(s_raw + M::VALID_AT);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint16_t* s_idx = s_valid + ((a.T + 63) & ~63) + warp * 8 * kMaxActive;
-    const int grp = blockIdx.x / a.n_blk, blk = blockIdx.x % a.n_blk;
+    const int grp = blockIdx.x / (a.n_blk * subs), sub = blockIdx.x % subs, blk = blockIdx.x / subs % a.n_blk;
     const int b = grp / a.Hk, g = grp % a.Hk;
     grid_dependency_wait();
     const uint32_t mask = a.masks[b];
@@ -288,7 +398,7 @@ attend_split_score_kernel(const __grid_constant__ SplitArgs a) {
             if (keep0) s_kept[__popc(b0 & lt)] = lane;
             if (keep1) s_kept[__popc(b0) + __popc(b1 & lt)] = lane + 32;
             __syncwarp();
-            if (g == 0 && blk == 0)
+            if (g == 0 && blk == 0 && sub == 0)
                 for (int i = lane; i < a.k_h; i += 32) a.kept_out[(size_t)b * a.k_h + i] = s_kept[i];
             kept_row = s_kept;
         }
@@ -297,18 +407,18 @@ attend_split_score_kernel(const __grid_constant__ SplitArgs a) {
         if (bad && blk == 0) atomicOr(a.status, SENTRY_STATUS_BIT_BAD_INDEX);
         if (lane == 0) s_rk = n;
     }
-    const int Tv = list_present(a.ids, a.T, mask, s_valid, red);
+    const int Tv = list_present(a.ids, a.T, mask, s_valid, red, blk * kScoreBlock);
     __syncthreads();
     const int rk = s_rk;
     const int p_begin = blk * kScoreBlock, p_end = min(Tv, p_begin + kScoreBlock);
-    if (g == 0) {   // the list for the launches that follow
+    if (g == 0 && sub == 0) {   // the list for the launches that follow
         for (int p = p_begin + threadIdx.x; p < p_end; p += kSplitThreads) a.valid[(size_t)b * a.T + p] = s_valid[p];
         if (blk == 0 && threadIdx.x == 0) a.tv[b] = Tv;
     }
     if (rk == 0) return;
     if (Tv == 0 && blk == 0 && threadIdx.x == 0) atomicOr(a.status, SENTRY_STATUS_BIT_EMPTY_MASK);
     if (p_begin >= Tv) return;
-    {   // column sums of V over this block's positions: 16 bytes of a row per lane
+    if (sub == 0) {   // column sums of V over the positions: 16 bytes of a row per lane
         constexpr int CPR = D / 8, RPW = 32 / CPR;
         const __nv_bfloat16* Vg = a.V + (size_t)grp * a.T * D;
         const int cc = lane % CPR;
@@ -331,7 +441,7 @@ attend_split_score_kernel(const __grid_constant__ SplitArgs a) {
         }
     }
     __syncthreads();
-    if (threadIdx.x < D) {
+    if (sub == 0 && threadIdx.x < D) {
         float t = 0.f;
 #pragma unroll
         for (int w = 0; w < kSplitWarps; ++w) t += s_vs[w][threadIdx.x];
@@ -339,88 +449,55 @@ attend_split_score_kernel(const __grid_constant__ SplitArgs a) {
     }
     if (a.given) return;
 
-    const int lh = rk == 1 ? 0 : (rk == 2 ? 1 : 2);   // log2 of the padded head count
-    const int my_h = (lane >> 2) & ((1 << lh) - 1);
-    const bool mine = my_h < rk;
-    const int hq = s_hs[min(my_h, rk - 1)], kh = s_khs[min(my_h, rk - 1)];
-    const __nv_bfloat16* qh = a.Q + ((size_t)b * a.Hq + hq) * a.T * D;
+    // positions of this block to score
+    const int p_share = kScoreBlock / subs, p_from = p_begin + sub * p_share, p_to = min(p_end, p_from + p_share);
+    const int n_s = sentry_num_active(Tv, a.c);
+    if (SAMPLED && (mask >= (uint32_t)a.n_subsets || a.offsets[mask] < 0)) {   // no table: every score ties
+        if (threadIdx.x == 0) atomicOr(a.status, SENTRY_STATUS_BIT_BAD_INDEX);
+        for (int h = 0; h < rk; ++h)
+            for (int p = p_from + threadIdx.x; p < p_to; p += kSplitThreads)
+                a.mscore[((size_t)b * a.k_h + s_khs[h]) * a.T + p] = 0.f;
+        return;
+    }
+    uint16_t* s_tok = reinterpret_cast<uint16_t*>(s_raw + M::TOK_AT) + warp * kBatches * kBatch * kTokPitch;
+    const uint32_t ring = ptx::smem_u32(s_raw) + warp * M::RING_BYTES;
     const __nv_bfloat16* Kg = a.K + (size_t)grp * a.T * D;
-    float* out = a.mscore + ((size_t)b * a.k_h + kh) * a.T;
-    SampleSrc src;
-    src.score_mode = a.score_mode;
-    src.n_s = sentry_num_active(Tv, a.c);
-    src.cnt = a.score_mode != 1 ? src.n_s : Tv;
-    src.tbl = nullptr;
-    if (a.score_mode != 1) {
-        if (mask >= (uint32_t)a.n_subsets || a.offsets[mask] < 0) {   // no table: every score ties
-            if (threadIdx.x == 0) atomicOr(a.status, SENTRY_STATUS_BIT_BAD_INDEX);
-            for (int h = 0; h < rk; ++h)
-                for (int p = p_begin + threadIdx.x; p < p_end; p += kSplitThreads)
-                    a.mscore[((size_t)b * a.k_h + s_khs[h]) * a.T + p] = 0.f;
-            return;
+    // sampled: a warp takes every eighth batch of the positions for all heads; all keys: 32 positions and a part of the heads
+    int p0 = p_from + warp * kBatch, batches = (p_to - p0 + kBatch * kSplitWarps - 1) / (kBatch * kSplitWarps), h_begin = 0, h_end = rk;
+    if constexpr (!SAMPLED) {
+        const int chunks = p_share / 32, part = warp / chunks, per = (rk * chunks + kSplitWarps - 1) / kSplitWarps;
+        p0 = p_from + warp % chunks * 32;
+        h_begin = part * per;
+        h_end = min(rk, h_begin + per);
+    }
+    if (p0 >= p_to) return;
+    if constexpr (SAMPLED) stage_tokens(a.table + a.offsets[mask], a.score_mode, n_s, p0, batches, Tv, s_valid, s_tok, a.status);
+    auto pass = [&](auto heads, int h0) {
+        constexpr int NH = decltype(heads)::value;
+        const __nv_bfloat16* qh[NH];
+        float* out[NH];
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+            qh[h] = a.Q + ((size_t)b * a.Hq + s_hs[h0 + h]) * a.T * D;
+            out[h] = a.mscore + ((size_t)b * a.k_h + s_khs[h0 + h]) * a.T;
         }
-        src.tbl = a.table + a.offsets[mask];
+        if constexpr (SAMPLED) score_sampled<D, NH>(qh, Kg, out, s_valid, s_tok, ring, n_s, p0 + (lane >> 2), batches, Tv);
+        else score_all<D, NH>(qh, Kg, out, s_valid, ring, p0 + lane, p_to, Tv);
+    };
+    constexpr int HPP = D == 64 ? 2 : 4;            // heads per pass: their query rows live in registers
+#pragma unroll 1
+    for (int h0 = h_begin; h0 < h_end; h0 += HPP) {
+        const int nh = min(HPP, h_end - h0);
+        if (nh == 1) pass(std::integral_constant<int, 1>(), h0);
+        else if (nh == 2) pass(std::integral_constant<int, 2>(), h0);
+        else if constexpr (HPP == 4) {
+            if (nh == 3) pass(std::integral_constant<int, 3>(), h0);
+            else pass(std::integral_constant<int, 4>(), h0);
+        }
     }
-#define SCORE_CASE(N) score_batches<D, N>(qh, Kg, out, mine, lh, s_valid, s_idx, Tv, p_begin, p_end, src, warp, a.status)
-    switch (a.score_mode == 1 ? 0 : (src.cnt + 7) >> 3) {
-        case 0: SCORE_CASE(0); break;
-        case 1: SCORE_CASE(1); break;
-        case 2: SCORE_CASE(2); break;
-        case 3: SCORE_CASE(3); break;
-        case 4: SCORE_CASE(4); break;
-        case 5: SCORE_CASE(5); break;
-        default: SCORE_CASE(6); break;
-    }
-#undef SCORE_CASE
 }
 
 // ------------------------------------------------------------------------------------------ select
-// The MMA sums in its own order, so a score may differ from an fp32 loop's over the table row by rounding.  The selection
-// takes the scores as approximate: entries within a margin of the U-th score are scored again in the loop's order and
-// ranked on that, so that what is selected does not depend on which kernel computed the scores.  Most heads have no
-// contested entry.
-//
-// The score of one query position in the order of the loop, by a whole warp: every lane takes one sampled key, the sum
-// then runs over the lanes in table order.
-template <int D>
-__device__ __noinline__ uint32_t exact_score_key(const __nv_bfloat16* qrow, const __nv_bfloat16* Kg, const uint16_t* valid,
-                                                 int Tv, SampleSrc src, int p) {
-    const int lane = threadIdx.x & 31;
-    const float scale = rsqrtf((float)D);
-    float mx = -INFINITY, sum = 0.f;
-    for (int a0 = 0; a0 < src.cnt; a0 += 32) {
-        const int at = min(a0 + lane, src.cnt - 1);
-        int pj = src.at(p, at, Tv);
-        if (pj < 0 || pj >= Tv) pj = 0;
-        const uint4* kr = reinterpret_cast<const uint4*>(Kg + (size_t)valid[pj] * D);
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int cc = 0; cc < D / 8; ++cc) {
-            const uint4 q = __ldg(reinterpret_cast<const uint4*>(qrow) + cc), v = __ldg(kr + cc);
-            fma_bf16_pair(acc[0], acc[1], q.x, v.x);
-            fma_bf16_pair(acc[2], acc[3], q.y, v.y);
-            fma_bf16_pair(acc[0], acc[1], q.z, v.z);
-            fma_bf16_pair(acc[2], acc[3], q.w, v.w);
-        }
-        const float sc = ((acc[0] + acc[1]) + (acc[2] + acc[3])) * scale;
-        const int n = min(32, src.cnt - a0);
-        for (int j = 0; j < n; ++j) {
-            const float v = __shfl_sync(0xffffffffu, sc, j);
-            mx = fmaxf(mx, v);
-            sum += v;
-        }
-    }
-    return sentry_order_key(mx - sum * (1.0f / (float)src.cnt));
-}
-
-__device__ __forceinline__ float order_key_value(uint32_t key) {   // inverse of sentry_order_key (not for NaN's 0)
-    return __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
-}
-// Margin within which two approximate scores are not taken to be in order, as a fraction of the head's largest |M|.
-// The fp32 loop and the MMA each round to about 1e-6 of sum |q_i k_i| / sqrt d, which is 1 to 3 times the largest score for
-// data without systematic cancellation; measured differences are a tenth of that.
-constexpr float kScoreMargin = 1.0f / 262144.0f;
-
 // Sum, max or min of a value over the NW warps that share a head (NW = 1: over the lanes).  buf: which of two exchange
 // buffers in turn -- the barrier of one exchange also frees the buffer of the one before.
 template <int NW>
@@ -456,7 +533,7 @@ struct HeadReduce {
 // lane in registers, NW warps per head (1: eight heads per block, 8: a block per head).  The threshold is found two bits
 // per step -- three candidates counted at once -- from the first bit in which the keys differ until exactly U keys lie
 // above one: 6 to 8 steps.  Bound by latency: a warp-wide reduction takes 56 cycles, a block-wide round 300.
-template <int D, int KPT, int NW>
+template <int KPT, int NW>
 __global__ void __launch_bounds__(kSplitThreads)
 attend_split_select_kernel(const __grid_constant__ SplitArgs a) {
     __shared__ uint32_t s_x[2][3][8];
@@ -490,72 +567,23 @@ attend_split_select_kernel(const __grid_constant__ SplitArgs a) {
         if (i0 + j < Tv) { hi = max(hi, key[j]); lo = min(lo, key[j]); }
     HeadReduce<NW> R{s_x, 0, lane, warp};
     R.max_min(hi, lo);
-    uint32_t t = lo;
     bool cut = Tv == U;            // exactly U keys are >= t
+    int bit = hi != lo ? (31 - __clz((int)(hi ^ lo))) | 1 : -1;   // digits of two bits, aligned
+    uint32_t t = bit < 0 || cut ? lo : (bit == 31 ? 0u : hi & ~((2u << bit) - 1u));
 #pragma unroll 1
-    for (bool settled = false; !cut; settled = true) {
-        int bit = hi != lo ? (31 - __clz((int)(hi ^ lo))) | 1 : -1;   // digits of two bits, aligned
-        t = bit < 0 ? lo : (bit == 31 ? 0u : hi & ~((2u << bit) - 1u));
-#pragma unroll 1
-        for (bit -= 1; bit >= 0 && !cut; bit -= 2) {
-            const uint32_t c1 = t + (1u << bit), c2 = t + (2u << bit), c3 = t + (3u << bit);
-            uint32_t n12 = 0u, n3 = 0u;                    // counts above c1 (low half), c2 (high half) and c3
-#pragma unroll
-            for (int j = 0; j < KPT; ++j) {
-                n12 += (key[j] >= c1 ? 1u : 0u) + (key[j] >= c2 ? 65536u : 0u);
-                n3 += key[j] >= c3 ? 1u : 0u;
-            }
-            R.sum3(n12, n3);
-            const int k1 = (int)(n12 & 0xffffu), k2 = (int)(n12 >> 16), k3 = (int)n3;
-            if (k3 >= U) { t = c3; cut = k3 == U; }
-            else if (k2 >= U) { t = c2; cut = k2 == U; }
-            else if (k1 >= U) { t = c1; cut = k1 == U; }
-        }
-        if (settled) break;        // (not cut: ties of exact keys at t)
-        uint32_t u = 0u, m = 0xffffffffu;   // the largest key not kept, the U-th key (ties: the same)
+    for (bit -= 1; bit >= 0 && !cut; bit -= 2) {
+        const uint32_t c1 = t + (1u << bit), c2 = t + (2u << bit), c3 = t + (3u << bit);
+        uint32_t n12 = 0u, n3 = 0u;                    // counts above c1 (low half), c2 (high half) and c3
 #pragma unroll
         for (int j = 0; j < KPT; ++j) {
-            if (i0 + j >= Tv) continue;
-            if (key[j] >= t) m = min(m, key[j]);
-            else u = max(u, key[j]);
+            n12 += (key[j] >= c1 ? 1u : 0u) + (key[j] >= c2 ? 65536u : 0u);
+            n3 += key[j] >= c3 ? 1u : 0u;
         }
-        R.max_min(u, m);
-        const bool finite = lo > 0x007fffffu && hi < 0xff800000u;
-        uint32_t k_up = 0xffffffffu, k_dn = 0u;            // NaN or infinite scores: everything is contested
-        if (finite) {
-            const float margin = 2.0f * kScoreMargin * fmaxf(fabsf(order_key_value(hi)), fabsf(order_key_value(lo)));
-            if (cut && order_key_value(m) - order_key_value(u) > margin) break;
-            k_up = sentry_order_key(order_key_value(m) + margin);
-            k_dn = sentry_order_key(order_key_value(m) - margin);
-        }
-        // surely active entries get the top key, hopeless ones zero, contested ones their exact key
-        const uint32_t mask = a.masks[b];
-        SampleSrc src;
-        src.score_mode = a.score_mode;
-        src.n_s = U;
-        src.cnt = a.score_mode != 1 ? U : Tv;
-        src.tbl = nullptr;
-        if (a.score_mode != 1 && mask < (uint32_t)a.n_subsets && a.offsets[mask] >= 0) src.tbl = a.table + a.offsets[mask];
-        const bool scored = src.tbl != nullptr || a.score_mode == 1;
-        const __nv_bfloat16* qh = a.Q + ((size_t)b * a.Hq + h) * a.T * D;
-        const __nv_bfloat16* Kg = a.K + ((size_t)b * a.Hk + h / (a.Hq / a.Hk)) * a.T * D;
-#pragma unroll
-        for (int j = 0; j < KPT; ++j) {
-            const bool in = i0 + j < Tv, open = in && key[j] >= k_dn && key[j] <= k_up;
-            unsigned todo = __ballot_sync(0xffffffffu, open);
-            uint32_t nk = in && key[j] > k_up ? 0xffffffffu : 0u;
-            while (todo) {
-                const int sl = __ffs(todo) - 1;
-                todo &= todo - 1;
-                const int p = (wi * 32 + sl) * KPT + j;
-                const uint32_t e = scored ? exact_score_key<D>(qh + (size_t)valid[p] * D, Kg, valid, Tv, src, p) : 1u;
-                if (lane == sl) nk = min(max(e, 1u), 0xfffffffeu);
-            }
-            key[j] = nk;
-        }
-        hi = 0xffffffffu;
-        lo = 0u;
-        cut = false;
+        R.sum3(n12, n3);
+        const int k1 = (int)(n12 & 0xffffu), k2 = (int)(n12 >> 16), k3 = (int)n3;
+        if (k3 >= U) { t = c3; cut = k3 == U; }
+        else if (k2 >= U) { t = c2; cut = k2 == U; }
+        else if (k1 >= U) { t = c1; cut = k1 == U; }
     }
     // ordered compaction: everything above t and, in index order, as many of the entries equal to t as are wanted
     uint32_t mine = 0u;            // above t: low half, equal to t: high half
@@ -930,11 +958,10 @@ SplitWs split_carve(const sentry_attend_desc& d, WsAlloc& w) {
     return s;
 }
 
-template <int D>
 int launch_select(sentry_ctx* ctx, const SplitArgs& p, cudaStream_t st) {
     const unsigned heads = (unsigned)p.B * p.k_h, packs = (heads + kSplitWarps - 1) / kSplitWarps;
     LaunchScope ls(ctx, KS_ATT_SELECT, st);
-#define SELECT(KPT, NW, GRID) SENTRY_CUDA_TRY(launch_chained(attend_split_select_kernel<D, KPT, NW>, dim3(GRID), dim3(kSplitThreads), 0, st, p))
+#define SELECT(KPT, NW, GRID) SENTRY_CUDA_TRY(launch_chained(attend_split_select_kernel<KPT, NW>, dim3(GRID), dim3(kSplitThreads), 0, st, p))
     // a warp per head where there are enough heads to fill the GPU that way, or the list is short anyway
     if (p.T <= 256) SELECT(8, 1, packs);
     else if (p.T <= 512 && packs >= 64) SELECT(16, 1, packs);
@@ -965,12 +992,17 @@ int launch_d(sentry_ctx* ctx, const AttendArgs& a, const SplitWs& w, cudaStream_
     const unsigned groups = (unsigned)d.B * d.Hk;
     const size_t list = (size_t)((d.T + 63) & ~63) * 2;
     {
+        // half the positions to a block while the blocks fit the GPU at once (two to an SM)
+        const int subs = !p.given && (long long)groups * p.n_blk <= 2LL * ctx->sm_count ? 2 : 1;
+        auto kern = d.score_mode != 1 ? attend_split_score_kernel<D, true> : attend_split_score_kernel<D, false>;
+        const size_t smem = (size_t)ScoreSmem<D>::VALID_AT + list;
+        if (smem > 46 * 1024)   // (beside the static arrays)
+            SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         LaunchScope ls(ctx, KS_ATT_SCORE, st);
-        SENTRY_CUDA_TRY(launch_chained(attend_split_score_kernel<D>, dim3(groups * (unsigned)p.n_blk), dim3(kSplitThreads),
-                                       list + (size_t)kSplitWarps * 8 * kMaxActive * 2, st, p));
+        SENTRY_CUDA_TRY(launch_chained(kern, dim3(groups * (unsigned)(p.n_blk * subs)), dim3(kSplitThreads), smem, st, p, subs));
     }
     if (!p.given) {
-        const int rc = launch_select<D>(ctx, p, st);
+        const int rc = launch_select(ctx, p, st);
         if (rc != SENTRY_OK) return rc;
     }
     LaunchScope ls(ctx, KS_ATT_CORE, st, 2);

@@ -58,3 +58,65 @@ def test_four_launch_attention(w):
         assert torch.equal(torch.nan_to_num(O2.float()), torch.nan_to_num(O.float()))
     finally:
         sn.close()
+
+
+@pytest.mark.parametrize("w", [
+    _w("split_common_d16", "bf16", 30, (342, 341, 341), 8, 2, 16, 8, "all"),
+    _w("split_common_d32", "bf16", 16, (342, 341, 341), 8, 2, 32, 4, "all"),
+    _w("split_common_d32_f16", "f16", 16, (342, 341, 341), 8, 2, 32, 8, "all"),
+    _w("split_common_d64", "bf16", 16, (100, 100, 100), 8, 2, 64, 8, "all"),
+], ids=lambda w: w.name)
+def test_selection_does_not_depend_on_the_form(w):
+    """Keys with a large common part: the raw scores are 2^10 times what is ranked, and so is their rounding.  The lists are
+    those of the one-launch form's fp32 loop all the same."""
+    sn = sentry.Sentry(0)
+    try:
+        inp = synth.generate(w, n_s_of)
+        kept_h, _ = parity.gate_lists(sn, inp)
+        ids, masks = parity.dev(inp.ids), parity.masks_dev(inp.masks)
+        tbl, offs = parity.dev(inp.sample_table), parity.dev(inp.table_offsets)
+        Q, V = inp.Q.cuda(), inp.V.cuda()
+        for power in (8, 13, 15):
+            K = inp.K.cuda()
+            K[..., 0] = 2.0 ** power
+            for mode in (0, 1):
+                act = []
+                for kernel, launches in ((sentry.ATTEND_AUTO, 4), (sentry.ATTEND_WARP_MMA, 1)):
+                    sn.set_attend_kernel(kernel)
+                    act.append(sn.attend_fwd(Q, K, V, kept_h, ids, masks, tbl, offs, c=w.c, score_mode=mode, return_active=True)[1])
+                    assert sn.last_launch_count() == launches
+                assert torch.equal(act[0], act[1]), (w.name, power, mode)
+    finally:
+        sn.close()
+
+
+def test_tied_scores_take_no_longer():
+    """Zero queries (a padded window): every score of a list ties.  The time of a call does not depend on the values; the bound
+    is twice the time of normal data, where a path for ties that scores entries one by one takes nine times as long."""
+    w = _w("split_tied", "bf16", 16, (1366, 1365, 1365), 8, 2, 32, 4, "all")
+    sn = sentry.Sentry(0)
+    try:
+        inp = synth.generate(w, n_s_of)
+        kept_h, _ = parity.gate_lists(sn, inp)
+        args = (kept_h, parity.dev(inp.ids), parity.masks_dev(inp.masks), parity.dev(inp.sample_table), parity.dev(inp.table_offsets))
+        Q, K, V = inp.Q.cuda(), inp.K.cuda(), inp.V.cuda()
+        O = torch.empty((w.B, w.k_h, w.T, w.d), dtype=Q.dtype, device="cuda")
+
+        def best_ms(q):
+            best = float("inf")
+            for _ in range(5):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                for _ in range(10):
+                    sn.attend_fwd(q, K, V, *args, c=w.c, O=O)
+                b.record()
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(b))
+            return best
+        zero = torch.zeros_like(Q)
+        act = sn.attend_fwd(zero, K, V, *args, c=w.c, return_active=True)[1]
+        assert sn.last_launch_count() == 4
+        assert torch.equal(act.cpu(), torch.arange(n_s_of(w.T)).int().expand_as(act))   # ties: the first U
+        assert best_ms(zero) <= 2 * best_ms(Q)
+    finally:
+        sn.close()
