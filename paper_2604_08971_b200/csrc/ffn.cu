@@ -178,7 +178,6 @@ ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__
                    const int32_t* __restrict__ kept, int n_lists, int D, int F, int k_c, int kc_pad,
                    int layout, size_t w_stride, T* __restrict__ out1, T* __restrict__ out2,
                    unsigned int* status) {
-    grid_dependents_start();
     grid_dependency_wait();
     // w_stride: elements between the weight matrices of consecutive lists (0: every list gathers
     // from the same W1, W2; D*F: list l has its own, as the experts of a Sparse-MoE block do)

@@ -35,7 +35,6 @@ constexpr int kGateMaxRegUnits = 8192;
 template <int KPT>
 __global__ void __launch_bounds__(1024)
 gate_select_kernel(const __grid_constant__ GateSetsDev sets, int S, unsigned int* status) {
-    grid_dependents_start();
     grid_dependency_wait();
     extern __shared__ int32_t s_list[];            // [k] kept units, ascending
     __shared__ uint32_t s_red[2][3][32];           // per-warp partial results of a counting step, two steps in turn
