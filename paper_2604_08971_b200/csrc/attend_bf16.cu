@@ -1120,16 +1120,19 @@ bool attend_bf16_supported(const sentry_attend_desc& d) {
     return d.d == 16 || d.d == 32 || d.d == 64;
 }
 
-// Whether the head selection can ride inside the attention launch: the fused kernel (K and V of a
-// group resident in shared memory) with at most 64 heads.
-bool attend_bf16_gate_fusable(const sentry_attend_desc& d) {
-    if (!attend_bf16_supported(d) || d.Hq > 64 || d.k_h > 64) return false;
+// Whether K and V of a group fit in shared memory together, as the fused kernel holds them (16-bit elements of either type).
+bool attend_bf16_resident(const sentry_attend_desc& d) {
     switch (d.d) {
         case 16: return fused_smem_bytes<16>(d.T) <= 200 * 1024;
         case 32: return fused_smem_bytes<32>(d.T) <= 200 * 1024;
         case 64: return fused_smem_bytes<64>(d.T) <= 200 * 1024;
         default: return false;
     }
+}
+
+// Whether the head selection can ride inside the attention launch: the fused kernel with at most 64 heads.
+bool attend_bf16_gate_fusable(const sentry_attend_desc& d) {
+    return attend_bf16_supported(d) && d.Hq <= 64 && d.k_h <= 64 && attend_bf16_resident(d);
 }
 
 int launch_attend_bf16(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {

@@ -5,6 +5,7 @@
 #define SENTRY_ATT_F16 1
 #define attend_bf16_supported attend_f16_supported
 #define attend_bf16_gate_fusable attend_f16_gate_fusable
+#define attend_bf16_resident attend_f16_resident
 #define launch_attend_bf16 launch_attend_f16
 #define attend_long_select_supported attend_long_select_f16_supported
 #define launch_attend_long_select launch_attend_long_select_f16

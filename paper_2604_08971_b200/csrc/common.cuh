@@ -386,6 +386,7 @@ int launch_attend_long_select(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t
 int launch_attend_tc(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st);
 bool attend_bf16_supported(const sentry_attend_desc& d);
 bool attend_bf16_gate_fusable(const sentry_attend_desc& d);
+bool attend_bf16_resident(const sentry_attend_desc& d);   // K and V of a group fit in shared memory (either 16-bit type)
 int launch_attend_bf16(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st);
 // the four-launch form (attend_split.cu); takes what attend_bf16_supported takes, scratch from ws
 size_t attend_split_ws_bytes(const sentry_attend_desc& d);

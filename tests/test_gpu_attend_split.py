@@ -120,3 +120,20 @@ def test_tied_scores_take_no_longer():
         assert best_ms(zero) <= 2 * best_ms(Q)
     finally:
         sn.close()
+
+
+@pytest.mark.parametrize("w, launches", [
+    (_w("form_96_heads_d32", "bf16", 4, (86, 85, 85), 96, 24, 32, 48), 1),     # 96 groups whose K and V fit: one launch
+    (_w("form_96_heads_d16", "f16", 8, (171, 171, 170), 96, 24, 16, 40), 1),
+    (_w("form_96_heads_few", "bf16", 1, (171, 171, 170), 96, 24, 32, 48, "all"), 4),
+], ids=lambda v: v.name if hasattr(v, "name") else str(v))
+def test_the_form_does_not_depend_on_the_number_of_heads(w, launches):
+    sn = sentry.Sentry(0)
+    try:
+        inp = synth.generate(w, n_s_of)
+        kept_h, _ = parity.gate_lists(sn, inp)
+        err, _ = parity.attend_parity(sn, inp, kept_h, None, 0, full_batch=True)
+        assert sn.last_launch_count() == launches
+        assert err <= TOL[w.dtype]
+    finally:
+        sn.close()
