@@ -90,31 +90,36 @@ gate_eval_kernel(const float* __restrict__ zeta, const float* __restrict__ gamma
 
 // kept [n_masks, k] ascending unit indices -> counts [n_masks, n_layers].  A block per list; a warp finds the first
 // position not below a layer's offset by a 32-way search (three rounds of memory latency up to 32 K entries where a
-// binary search takes up to 15), the counts are the differences.
+// binary search takes up to 15), the counts are the differences.  Layers go through shared memory kCountLayers at a time.
+constexpr int kCountLayers = 8192;
 __global__ void __launch_bounds__(256)
 layer_count_kernel(const int32_t* __restrict__ kept, int n_masks, int k, const int32_t* __restrict__ layer_offsets,
                    int n_layers, int32_t* __restrict__ counts) {
     grid_dependents_start();
     grid_dependency_wait();
-    extern __shared__ int s_pos[];                 // [n_layers + 1]
+    extern __shared__ int s_pos[];                 // [min(n_layers, kCountLayers) + 1]
     const int m = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t* row = kept + (size_t)m * k;
-    for (int l = warp; l <= n_layers; l += 8) {
-        const int bound = layer_offsets[l];
-        int lo = 0, hi = k;                        // row[lo - 1] < bound <= row[hi]
-        while (lo < hi) {
-            const int step = (hi - lo + 31) / 32;
-            const int at = lo + step * (lane + 1) - 1;
-            const bool below = at < hi && row[at] < bound;
-            const int n = __popc(__ballot_sync(0xffffffffu, below));   // probes below the bound: the first n lanes
-            hi = min(hi, lo + step * (n + 1) - 1);
-            lo += step * n;
-            hi = max(hi, lo);
+    for (int l0 = 0; l0 < n_layers; l0 += kCountLayers) {
+        const int nl = min(n_layers - l0, kCountLayers);
+        for (int l = warp; l <= nl; l += 8) {
+            const int bound = layer_offsets[l0 + l];
+            int lo = 0, hi = k;                    // row[lo - 1] < bound <= row[hi]
+            while (lo < hi) {
+                const int step = (hi - lo + 31) / 32;
+                const int at = lo + step * (lane + 1) - 1;
+                const bool below = at < hi && row[at] < bound;
+                const int n = __popc(__ballot_sync(0xffffffffu, below));   // probes below the bound: the first n lanes
+                hi = min(hi, lo + step * (n + 1) - 1);
+                lo += step * n;
+                hi = max(hi, lo);
+            }
+            if (lane == 0) s_pos[l] = lo;
         }
-        if (lane == 0) s_pos[l] = lo;
+        __syncthreads();
+        for (int l = threadIdx.x; l < nl; l += blockDim.x) counts[(size_t)m * n_layers + l0 + l] = s_pos[l + 1] - s_pos[l];
+        __syncthreads();
     }
-    __syncthreads();
-    for (int l = threadIdx.x; l < n_layers; l += blockDim.x) counts[(size_t)m * n_layers + l] = s_pos[l + 1] - s_pos[l];
 }
 
 }  // namespace
@@ -137,11 +142,7 @@ int launch_gate_eval(sentry_ctx* ctx, const float* zeta, const float* gamma, con
 int launch_layer_counts(sentry_ctx* ctx, const int32_t* kept, int n_masks, int k, const int32_t* layer_offsets,
                         int n_layers, int32_t* counts, cudaStream_t st) {
     LaunchScope ls(ctx, KS_GATE_EVAL, st);
-    const size_t smem = ((size_t)n_layers + 1) * sizeof(int);
-    if (smem > 48 * 1024) {
-        if (smem > 220 * 1024) return SENTRY_ERR_UNSUPPORTED;
-        SENTRY_CUDA_TRY(cudaFuncSetAttribute(layer_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
+    const size_t smem = ((size_t)(n_layers < kCountLayers ? n_layers : kCountLayers) + 1) * sizeof(int);
     SENTRY_CUDA_TRY(launch_chained(layer_count_kernel, dim3(n_masks), dim3(256), smem, st, kept, n_masks, k, layer_offsets, n_layers, counts));
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;

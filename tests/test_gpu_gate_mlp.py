@@ -51,3 +51,20 @@ def test_gate_eval_global_threshold_and_layer_counts(units, hidden, M):
         assert sn.last_status() == 0
     finally:
         sn.close()
+
+
+@pytest.mark.parametrize("n_layers", [1, 8191, 8192, 8193, 70000])
+def test_layer_counts_of_any_number_of_layers(n_layers):
+    g = np.random.default_rng(n_layers)
+    N = 3 * n_layers + 5
+    lo = np.concatenate([[0], np.sort(g.integers(0, N + 1, n_layers - 1)), [N]]).astype(np.int32)   # some layers are empty
+    kept = np.sort(g.permutation(N)[:N // 2 + 1]).astype(np.int32)[None].repeat(2, 0)
+    kept[1] = np.arange(kept.shape[1])
+    sn = sentry.Sentry(0)
+    try:
+        counts = sn.gate_layer_counts(torch.as_tensor(kept).cuda(), torch.as_tensor(lo).cuda()).cpu().numpy()
+        for r in range(2):
+            np.testing.assert_array_equal(counts[r], np.diff(np.searchsorted(kept[r], lo)))
+        assert sn.last_status() == 0
+    finally:
+        sn.close()
