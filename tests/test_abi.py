@@ -2,6 +2,7 @@
 exports every function the header declares, and its host-only helpers agree
 with the oracle.  No kernel is launched here."""
 import ctypes
+import importlib
 import os
 import re
 
@@ -75,3 +76,23 @@ def test_create_without_device_fails_loudly(lib):
     assert lib.sentry_create(ctypes.byref(h), 0) == -5 and not h.value
     with pytest.raises(RuntimeError):
         sentry.Sentry(0)
+
+
+def test_a_binding_of_another_torch_is_rebuilt(lib, monkeypatch):
+    """The binding is compiled against torch's headers: with another torch it would fail where it is loaded."""
+    build = importlib.import_module("paper_2604_08971_b200.build")
+    compiled = []
+    monkeypatch.setattr(build, "_compile", lambda cmd, target: compiled.append(target) or "")
+    build.build()
+    assert compiled == []
+    monkeypatch.setattr(build.metadata, "version", lambda name: "0.0.1")
+    monkeypatch.setattr(build, "BINDING_STAMP", build.BINDING_STAMP + ".test")   # (not the real binding's)
+    with open(build.BINDING_STAMP, "w") as f:
+        f.write("torch 0.0.0 python x")
+    try:
+        assert build.needs_build()
+        build.build()
+        assert compiled == [build.BINDING]
+        assert not build.needs_build()
+    finally:
+        os.remove(build.BINDING_STAMP)
