@@ -940,7 +940,7 @@ attend_split_fill_kernel(const __grid_constant__ SplitArgs a) {
 // Parts of the keys in the rows launch: about three blocks per SM, at least 256 keys a part, at most 16 parts.
 int split_parts(const sentry_attend_desc& d) {
     const long long groups = (long long)d.B * d.Hk;
-    long long n = (444 + groups - 1) / groups;
+    long long n = (3 * kSmCount + groups - 1) / groups;
     const long long most = (d.T + 255) / 256;
     if (n > most) n = most;
     return (int)(n > kMaxParts ? kMaxParts : (n < 1 ? 1 : n));

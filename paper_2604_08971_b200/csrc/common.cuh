@@ -11,6 +11,10 @@
 
 #include "../../include/sentry.h"
 
+// SMs of a B200, for sizes that a workspace query (which has no context) and the launch must agree on; what a launch decides
+// for itself asks the context's sm_count.
+constexpr int kSmCount = 148;
+
 // Kernel slots for launch accounting and optional per-kernel timing.
 enum KernelSlot {
     KS_GATE_ROWS = 0, KS_GATE_EXPAND, KS_ATT_SCORE, KS_ATT_SELECT, KS_ATT_CORE,

@@ -467,7 +467,7 @@ bool k_major(const sentry_ffn_desc& d) { return ffn_tc_supported(d) || ffn_wide_
 int tile_rows_for(const sentry_ffn_desc& d) {
     if (k_major(d)) return kTcTileRows;
     // tiles of 4 while they leave an SM to each: shorter chains, and the weights they read more often come from L2
-    return (long long)d.B * d.T <= 4 * 148 ? kGenericFewRows : kGenericTileRows;
+    return (long long)d.B * d.T <= kGenericFewRows * kSmCount ? kGenericFewRows : kGenericTileRows;
 }
 
 template <typename T>
