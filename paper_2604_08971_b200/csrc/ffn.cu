@@ -296,9 +296,7 @@ ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__
     const int32_t* N = kept + (size_t)l * k_c;
     if (which == 0) {
         // W1: destination-major index so that writes coalesce
-        int n, e;
-        if (layout == 0) { e = (int)(i / kc_pad); n = (int)(i % kc_pad); }
-        else             { n = (int)(i / D);      e = (int)(i % D); }
+        const int e = (int)(i / kc_pad), n = (int)(i % kc_pad);
         T v = from_f32<T>(0.f);
         if (n < k_c) {
             const int ch = N[n];
@@ -307,9 +305,7 @@ ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__
         }
         out1[(size_t)l * per + i] = v;
     } else {
-        int n, e;
-        if (layout == 0) { n = (int)(i / D);      e = (int)(i % D); }
-        else             { e = (int)(i / kc_pad); n = (int)(i % kc_pad); }
+        const int n = (int)(i / D), e = (int)(i % D);
         T v = from_f32<T>(0.f);
         if (n < k_c) {
             const int ch = N[n];
