@@ -22,26 +22,20 @@ size_t attend_workspace_bytes(const sentry_attend_desc& d) {
 }
 
 // Which form 16-bit attention takes: a CTA per (sample, KV head) group, or four launches spread over all SMs.  Measured, the
-// CTA per group against the four launches, us per call, every token present:
+// CTA per group against the four launches, us per call, every token present unless said otherwise:
 //   K and V of a group fit in shared memory (asked of the shape alone: the number of heads does not matter): 64 groups of
-//     T = 512, d = 32: 56 / 47, T = 768: 53 / 55, T = 1024: 78 / 61; 128 groups 56 / 62, 53 / 83 and 78 / 98; d = 64: 64
-//     groups of T = 256 62 / 43, T = 512: 88 / 67, 128 groups 63 / 56 and 88 / 99 (one to three of three modalities present:
-//     148 groups of T = 512 89 / 91, T = 640 107 / 94).  Few groups: 8 of T = 768, d = 32 52 / 28; a single sample of one
-//     modality in three 23 / 23, which one launch does with less work for the host.
-//   longer sequences, K of a group in one piece beside the scores (up to about 180 KB): T = 2048, d = 32: 128 groups 292 / 182,
-//     256 groups 333 / 356; d = 64, T = 1400: 192 groups 456 / 387, 256 groups 444 / 519; T = 4096, d = 16: 128 groups
-//     416 / 300, 192 groups 391 / 451.
-//   K in two pieces: d = 32, T = 4096: 384 groups 1167 / 1104; d = 64, T = 2048: 256 groups 801 / 757, 512 groups 1373 / 1467.
-//   K in more: d = 64, T = 4096: 512 groups 4128 / 3259.
-//   Every key scored, K not in shared memory: multiply-adds bound both, T = 4096, d = 32: 16 groups 1528 / 1096, 64 groups
-//     3827 / 3846, 128 groups 6728 / 7575.
+//     T = 512, d = 32: 56 / 45, T = 768: 53 / 51, T = 1024: 78 / 59; 128 groups 56 / 60, 53 / 80 and 79 / 94; d = 64: 64
+//     groups of T = 256 62 / 40, T = 512: 88 / 60; 128 groups 63 / 51 and 88 / 88; 192 groups 73 / 72.  Few groups: 8 of
+//     T = 768, d = 32 52 / 28; a single sample of one modality in three 23 / 23, which one launch does with less host work.
+//   longer sequences: d = 64: 512 groups of T = 768 432 / 388, T = 2048: 1370 / 1036, 800 groups of T = 1400 704 / 724;
+//     d = 32, T = 2048: 256 groups 333 / 344, 400 groups 348 / 375 (one to three of three modalities present: 183 / 165 and
+//     242 / 243), T = 4096: 400 groups 884 / 794, 512 groups 952 / 1018; d = 16, T = 4096: 128 groups 416 / 301, 192 groups
+//     392 / 454 (one to three modalities: 160 groups 187 / 174).
 bool attend_split_faster(const sentry_attend_desc& d, int sm_count) {
     const long long groups = (long long)d.B * d.Hk;
     if (attend_bf16_resident(d))
         return groups >= 8 && (d.d > 32 ? groups <= sm_count && d.T >= 256 : groups <= sm_count / 2 && d.T >= 512);
-    if (d.score_mode == 1) return groups <= sm_count / 2;
-    const long long k_kb = (long long)d.T * d.d * 2 / 1024;
-    return k_kb > 360 || groups <= (k_kb > 180 ? 5LL * sm_count / 2 : 5LL * sm_count / 4);
+    return d.d > 32 || groups <= (d.d > 16 ? 5LL * sm_count / 2 : 5LL * sm_count / 4);
 }
 
 int check_attend_desc(const sentry_attend_desc* d) {

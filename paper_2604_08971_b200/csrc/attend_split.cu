@@ -11,7 +11,7 @@
 // which every one is a chain of latencies, on as many SMs as there are groups.  Taken apart, each phase runs with as many
 // warps as it has work: the form for long sequences and for few groups (attend_split_faster in api.cu has the line).
 // Measured on 16 x 4096 tokens, d = 32, 4 of 8 heads kept, one to three of three modalities present: 310 us in one CTA per
-// group, 81 as four launches.
+// group, 80 as four launches.
 #include <math.h>
 #include <stddef.h>
 
@@ -150,44 +150,63 @@ struct SplitArgs {
 // the sample's present-token list.
 constexpr int kBatch = 8;                         // query positions of a batch
 constexpr int kBatches = kScoreBlock / (kBatch * kSplitWarps);   // of a warp
-constexpr int kTokPitch = kMaxActive + 2;
+constexpr int kBatchSteps = kMaxActive / 4;       // steps of a batch: a key for each lane of a quad
 template <int D>
 struct ScoreSmem {
-    static constexpr int STAGES = 3;
+    static constexpr int STAGES = D == 64 ? 2 : 3;   // two blocks fit an SM at every T
     static constexpr int STAGE_BYTES = 32 * D * 2;
     static constexpr int RING_BYTES = STAGES * STAGE_BYTES;
     static constexpr int TOK_AT = kSplitWarps * RING_BYTES;
-    static constexpr int VALID_AT = TOK_AT + kSplitWarps * kBatches * kBatch * kTokPitch * 2;
+    static constexpr int VALID_AT = TOK_AT + kSplitWarps * kBatches * kBatchSteps * 32 * 2;
 };
 
-// Tokens of the sampled keys of a warp's batches: s_tok[(batch * kBatch + q) * kTokPitch + a].  Positions outside the list are
-// flagged and count as position 0; entries from n_s on (to a multiple of 4) repeat the last one, queries past the list those
-// of the last.
+// Tokens of the sampled keys of a warp's batches, 32 per step.  Row r = 4 q + a of a step (query q, key a of its four) is at
+// (r % RPC) CPR + r / RPC: the CPR tokens that a lane copies chunks of are then one word of shared memory.  Positions outside
+// the list are flagged and count as position 0; keys from n_s on (to a multiple of 4) repeat the last one, queries past the
+// list those of the last.
+template <int CPR>
 __device__ __forceinline__ void stage_tokens(const int32_t* __restrict__ tbl, int score_mode, int n_s, int p0, int batches, int Tv,
                                              const uint16_t* s_valid, uint16_t* s_tok, unsigned int* status) {
-    constexpr int PER = kMaxActive / 4;            // table entries of a lane and batch, all on the way at once
-    const int lane = threadIdx.x & 31, q = lane & 7, a4 = lane >> 3, n4 = (n_s + 3) & ~3;
+    constexpr int RPC = 32 / CPR;
+    const int lane = threadIdx.x & 31, q = lane & 7, a4 = lane >> 3, n4 = (n_s + 3) & ~3, r = 4 * q + a4;
     const size_t es = score_mode == 2 ? (size_t)Tv : 1;
-    int e[kBatches][PER];
+    int e[kBatches][kBatchSteps];                  // all of a lane's table entries on the way at once
 #pragma unroll
     for (int b = 0; b < kBatches; ++b) {
         const int p = min(p0 + b * kBatch * kSplitWarps + q, Tv - 1);
         const int32_t* src = tbl + (score_mode == 2 ? (size_t)p : (size_t)p * n_s);
 #pragma unroll
-        for (int i = 0; i < PER; ++i) e[b][i] = b < batches && 4 * i < n4 ? __ldg(src + (size_t)min(4 * i + a4, n_s - 1) * es) : 0;
+        for (int i = 0; i < kBatchSteps; ++i)
+            e[b][i] = b < batches && 4 * i < n4 ? __ldg(src + (size_t)min(4 * i + a4, n_s - 1) * es) : 0;
     }
     bool bad = false;
 #pragma unroll
     for (int b = 0; b < kBatches; ++b) {
         if (b >= batches) break;
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
+        for (int i = 0; i < kBatchSteps; ++i) {
             if (4 * i >= n4) break;
             if ((unsigned)e[b][i] >= (unsigned)Tv) { bad = true; e[b][i] = 0; }
-            s_tok[(b * kBatch + q) * kTokPitch + 4 * i + a4] = s_valid[e[b][i]];
+            s_tok[(b * kBatchSteps + i) * 32 + r % RPC * CPR + r / RPC] = s_valid[e[b][i]];
         }
     }
     if (bad) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+}
+// N tokens from shared memory in one load.
+template <int N>
+__device__ __forceinline__ void load_tokens(uint32_t (&t)[N], const uint16_t* s) {
+    uint32_t w[N / 2];
+    if constexpr (N == 2) {
+        w[0] = *reinterpret_cast<const uint32_t*>(s);
+    } else if constexpr (N == 4) {
+        const uint2 v = *reinterpret_cast<const uint2*>(s);
+        w[0] = v.x; w[1] = v.y;
+    } else {
+        const uint4 v = *reinterpret_cast<const uint4*>(s);
+        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) t[i] = (i & 1) ? w[i / 2] >> 16 : w[i / 2] & 0xffffu;
 }
 
 // The query rows of a token, as they are stored.
@@ -239,18 +258,20 @@ __device__ __forceinline__ void score_sampled(const __nv_bfloat16* const (&qh)[N
     const int steps = (n_s + 3) / 4;                // of a batch
     const __nv_bfloat16* Kc = Kg + cc * 8;
     const uint32_t copy_to = ring + S::off(row0, cc), row_at = ring + S::off(lane, 0);
-    const uint16_t* tp = s_tok + (row0 >> 2) * kTokPitch + (row0 & 3);
+    const uint16_t* tp = s_tok + row0 * S::CPR;
     int f_left = batches * steps, f_step = 0;       // what is still to be fetched
     auto fetch = [&](uint32_t stage) {              // stage: byte offset in the ring
         if (f_left > 0) {
+            uint32_t t[S::CPR];
+            load_tokens(t, tp + f_step * 32);
 #pragma unroll
             for (int i = 0; i < S::CPR; ++i) {
                 // (row i * RPC + row0 is swizzled as row0 is; d = 64: with bit 2 of the row in every other i)
                 const uint32_t to = (D == 64 ? copy_to ^ ((i & 1) << 6) : copy_to) + stage + i * RPC * S::RB;
-                ptx::cp_async_16(to, Kc + (uint32_t)tp[i * (RPC / 4) * kTokPitch + f_step * 4] * D);
+                ptx::cp_async_16(to, Kc + t[i] * D);
             }
             --f_left;
-            if (++f_step == steps) { f_step = 0; tp += kBatch * kTokPitch; }
+            if (++f_step == steps) { f_step = 0; tp += kBatchSteps * 32; }
         }
         ptx::cp_async_commit();
     };
@@ -286,12 +307,12 @@ __device__ __forceinline__ void score_sampled(const __nv_bfloat16* const (&qh)[N
         for (int step = 0; step < steps; ++step) {
             ptx::cp_async_wait_group<M::STAGES - 2>();
             __syncwarp();                           // every lane's copies of this step are there, the stage before is free
-            fetch(ahead);
             const uint32_t addr = row_at + stage;
             constexpr int EARLY = S::CPR <= 4 ? S::CPR : 2;   // under way while the step before is taken in
             uint4 v[EARLY];
 #pragma unroll
             for (int c = 0; c < EARLY; ++c) v[c] = lds128(addr ^ (c << 4));
+            fetch(ahead);
             if (step > 0) take(4);
             dot_rows<D, NH>(q, [&](int c) { return c < EARLY ? v[c] : lds128(addr ^ (c << 4)); }, scale, sc);
             ahead = stage;
@@ -359,8 +380,9 @@ __device__ __forceinline__ void score_all(const __nv_bfloat16* const (&qh)[NH], 
 // exact for keys with a large common part (a margin taken from the scores) or has contested entries in every other head (a
 // margin proved from the rows' norms: the selection 15 -> 25 us) and thousands where scores tie.  Bound by the issue of 200
 // instructions per 32 keys and two heads (0.57 per cycle and scheduler at 16 warps per SM) and by the shared-memory pipe
-// (half busy).  Whole calls on the MMA with a margin / here, us: 16 x 4096 tokens, d = 32: 82 / 81; 8 x 648, d = 64: 44 / 42;
-// 1 x 4096, d = 32: 51 / 36; 64 x 2048: 170 / 182; 16 x 2048, d = 64: 89 / 124; every key (score_mode 1), 32 x 1024: 133 / 185.
+// (half busy): the tokens of a lane's copies come in one load (CPR loads: 2 to 7 % of the call more).  Whole calls on the MMA
+// with a margin / here, us: 16 x 4096 tokens, d = 32: 82 / 80; 8 x 648, d = 64: 44 / 39; 1 x 4096, d = 32: 51 / 36; 64 x 2048:
+// 170 / 175; 64 x 1024, d = 64: 130 / 140; 16 x 2048: 89 / 100; every key (score_mode 1), 32 x 1024, d = 32: 133 / 185.
 template <int D, bool SAMPLED>
 __global__ void __launch_bounds__(kSplitThreads, 2)
 attend_split_score_kernel(const __grid_constant__ SplitArgs a, int subs) {
@@ -459,7 +481,7 @@ attend_split_score_kernel(const __grid_constant__ SplitArgs a, int subs) {
                 a.mscore[((size_t)b * a.k_h + s_khs[h]) * a.T + p] = 0.f;
         return;
     }
-    uint16_t* s_tok = reinterpret_cast<uint16_t*>(s_raw + M::TOK_AT) + warp * kBatches * kBatch * kTokPitch;
+    uint16_t* s_tok = reinterpret_cast<uint16_t*>(s_raw + M::TOK_AT) + warp * kBatches * kBatchSteps * 32;
     const uint32_t ring = ptx::smem_u32(s_raw) + warp * M::RING_BYTES;
     const __nv_bfloat16* Kg = a.K + (size_t)grp * a.T * D;
     // sampled: a warp takes every eighth batch of the positions for all heads; all keys: 32 positions and a part of the heads
@@ -471,7 +493,7 @@ attend_split_score_kernel(const __grid_constant__ SplitArgs a, int subs) {
         h_end = min(rk, h_begin + per);
     }
     if (p0 >= p_to) return;
-    if constexpr (SAMPLED) stage_tokens(a.table + a.offsets[mask], a.score_mode, n_s, p0, batches, Tv, s_valid, s_tok, a.status);
+    if constexpr (SAMPLED) stage_tokens<D / 8>(a.table + a.offsets[mask], a.score_mode, n_s, p0, batches, Tv, s_valid, s_tok, a.status);
     auto pass = [&](auto heads, int h0) {
         constexpr int NH = decltype(heads)::value;
         const __nv_bfloat16* qh[NH];
