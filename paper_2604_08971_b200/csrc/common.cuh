@@ -94,7 +94,7 @@ struct DeviceGuard {
 // of everything before it.  Small kernels also call grid_dependents_start() at their top.  Kernels that fill the GPU do
 // not: blocks of the next kernels that sit on their SMs waiting cost them more than the earlier start gains (64 windows x
 // 1024 tokens: 129 -> 122 us a step without it, 256 x 192 tokens: 57.5 -> 54).  Nor do small kernels whose successor fills
-// the GPU, the channel selection and the weight gather: the gather's hundreds of blocks, waiting for a selection of a few,
+// the GPU, the channel selection and the weight gather before a large FFN: the gather's hundreds of blocks, waiting for a selection of a few,
 // hold registers on the SMs that another stream's attention CTAs need in full (two of them take an SM's register file).
 // With attention and FFN branches forked on two streams, 128 x 512 tokens at d_model 384: 125 us a step with the early
 // start, 117 without; 4 layers' selections and one gather on one stream: 32 and 27; one window of 64 tokens: 31.0 and 31.7.
