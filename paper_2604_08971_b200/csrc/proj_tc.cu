@@ -444,9 +444,11 @@ int launch_qkv_d(sentry_ctx* ctx, const ProjArgs& a, cudaStream_t st) {
 
 }  // namespace
 
-// bf16, head dim 16/32/64, d_model a multiple of 64.  Q and K decide which positions attention selects, so which form sums
-// them is part of the result: d_model times head dimension beyond what one SM once had to hold (96 KB of X and 72 KB of
-// weights at d_model 384, d = 32) stays with the plain-ALU kernel, whose fp32 sums run in another order.
+// bf16, head dim 16/32/64, d_model a multiple of 64.  The size clause describes no limit of this kernel: it is where an
+// earlier one ended (96 KB of X and 72 KB of weights at d_model 384, d = 32), and it stays because Q and K decide which
+// positions attention selects: beyond it the plain-ALU kernel's fp32 sums, in another order, are the result so far.  What
+// that costs: 128 x 512 tokens at d_model 384 take 49 us here with 12 heads of 32, and 3690 us there with 6 heads of 64 (a
+// CTA per token, which reads all kept weight columns).
 bool project_qkv_tc_supported(const sentry_proj_desc& d) {
     if (d.dtype != ATT_DTYPE) return false;
     if (d.d != 16 && d.d != 32 && d.d != 64) return false;
