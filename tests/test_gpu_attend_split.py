@@ -137,3 +137,43 @@ def test_the_form_does_not_depend_on_the_number_of_heads(w, launches):
         assert err <= TOL[w.dtype]
     finally:
         sn.close()
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_odd_inputs_are_treated_as_in_one_launch(mode):
+    """Token ids that start off a 16-byte boundary and name modalities out of range, a sample without any modality, a subset
+    without a table, sampled positions outside the list: the lists, the zero rows and the status word of the other form."""
+    w = _w("split_odd", "bf16", 16, (172, 170, 173), 8, 2, 32, 5)
+    sn = sentry.Sentry(0)
+    try:
+        inp = synth.generate(w, n_s_of)
+        kept_h, _ = parity.gate_lists(sn, inp)
+        ids = torch.empty(w.T + 1, dtype=torch.int32, device="cuda")[1:]
+        ids.copy_(parity.dev(inp.ids))
+        masks = parity.masks_dev(inp.masks)
+        tv = [int(sum(n for j, n in enumerate(w.lengths) if (int(m) >> j) & 1)) for m in inp.masks]
+        masks[3] = 0
+        offs = parity.dev(inp.table_offsets).clone()
+        table = parity.dev(inp.sample_table).clone()
+        if mode == 0:
+            table[int(offs[int(inp.masks[6])]) + 77] = w.T      # one entry beyond the list, one before it
+            table[int(offs[int(inp.masks[5])]) + 5] = -1
+        if mode == 2:
+            table = parity.dev(synth.entry_major_tables(w, inp.sample_table, inp.table_offsets, n_s_of))
+            offs[int(inp.masks[1])] = -1
+        if mode == 1:
+            ids[10], ids[w.T - 1] = 40, -7                       # present in no sample
+        out = []
+        for kernel, launches in ((sentry.ATTEND_AUTO, 4), (sentry.ATTEND_WARP_MMA, 1)):
+            sn.set_attend_kernel(kernel)
+            O, act = sn.attend_fwd(inp.Q.cuda(), inp.K.cuda(), inp.V.cuda(), kept_h, ids, masks, table, offs, c=w.c,
+                                   score_mode=mode, return_active=True)
+            assert sn.last_launch_count() == launches
+            out.append((O.float(), act, sn.last_status()))
+        (O, act, status), (O1, act1, status1) = out
+        assert torch.equal(act, act1) and status == status1 != 0
+        assert O[3].abs().max().item() == 0 and (act[3] == -1).all()
+        assert (O - O1).abs().max().item() <= TOL[w.dtype] * O1.abs().max().item()
+        assert tv[6] == w.T
+    finally:
+        sn.close()
