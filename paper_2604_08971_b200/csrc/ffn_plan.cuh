@@ -31,6 +31,10 @@ bool ffn_tc_supported(const sentry_ffn_desc& d);
 int ffn_tc_kc_pad(int D, int k_c);
 int launch_ffn_tc(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c, int kc_pad, int max_tiles,
                   cudaStream_t st);
+// ffn_tmem.cu: the fused form that launch_ffn_tc takes for 16-bit operands at d_model 128 and 256
+bool ffn_tmem_supported(const sentry_ffn_desc& d);
+int launch_ffn_tmem(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c, int kc_pad, int max_tiles,
+                    cudaStream_t st);
 bool ffn_wide_supported(const sentry_ffn_desc& d);
 int ffn_wide_kc_pad(int k_c);
 size_t ffn_wide_hidden_bytes(int kc_pad, long long max_tiles);

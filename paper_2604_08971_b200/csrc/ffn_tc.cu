@@ -1,8 +1,10 @@
 // Channel-compacted FFN on the 5th-generation tensor cores (Section 4.6):
 //   Y = gelu(X . W1[:, N]) . W2[N, :]   for the present rows of every sample.
+// With the hidden tile in shared memory: 16-bit operands at d_model 384, FP8 at 128, 256 and 384 (16-bit operands at 128 and 256
+// keep it in tensor memory, ffn_tmem.cu, which launch_ffn_tc hands them to).
 //
 // One persistent CTA per SM walks tiles of 128 present rows (row table in ffn_plan.cuh).
-// Per tile and per chunk of CH kept channels (CH = 256, or 128 when d_model = 384):
+// Per tile and per chunk of CH kept channels (CH = 256 with FP8, or 128 when d_model = 384):
 //   GEMM1  H[128 x CH] = X_tile[128 x D] . W1c_chunk^T            (tcgen05, fp32 in TMEM)
 //   epilogue  H -> gelu -> bf16 -> shared memory (K-major, 128-byte swizzle)
 //   GEMM2  Y[128 x D] += H[128 x CH] . W2c_chunk                  (tcgen05, fp32 in TMEM)
@@ -33,20 +35,11 @@
 
 #include "common.cuh"
 #include "ffn_plan.cuh"
+#include "ffn_tc_common.cuh"
 #include "tc_common.cuh"
 #include "ptx/sm100.cuh"
 
 namespace {
-
-constexpr int kTileRows = 128;
-constexpr int kBlockBytes = 128 * 128;   // 128 rows x 64 bf16: one X block, one hidden block
-constexpr int kStageBytes = 2 * kBlockBytes;
-constexpr int kStages = 3;
-constexpr int kThreads = 512;
-constexpr int kLoaderWarp0 = 3, kLoaderWarps = 4, kLoaderThreads = kLoaderWarps * 32;
-constexpr int kEpiWarp0 = 7, kEpiWarps = 8;
-constexpr int kZeroWarp = 15, kZeroBytes = 1024;   // zeros at the end of the misc block
-constexpr int kTmemCols = 512;
 
 // FP8: X, the weights and the hidden activations are e4m3 bytes (a 128-byte operand row then
 // holds 128 elements instead of 64), the accumulators stay fp32, Y is stored as bf16.
@@ -84,49 +77,7 @@ struct Misc {
 };
 static_assert(sizeof(Misc) <= 2048 - kZeroBytes, "misc block too large");
 
-// ---- lean forms for the single-thread roles -------------------------------------------------
-// A warp that walks a chain of dependent scalar instructions with shared-memory round trips in
-// it (an mbarrier probe, a flag poll, a vote) advances at 8 to 15 cycles per instruction here,
-// so what the producers and issuers execute per stage is counted in instructions: barrier
-// addresses are one add from a base, descriptors are a 32-bit add and a register pair, all the
-// probes of a stage are issued back to back and voted on once.
 #define MISC_BAR(base, field) ((base) + (uint32_t)offsetof(Misc, field))
-constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);   // upper word of umma_smem_desc_sw128
-__device__ __forceinline__ uint32_t desc_lo(uint32_t smem_addr) { return ((smem_addr >> 4) & 0x3fffu) | (1u << 16); }
-// D (+)= A . B^T for one 128-byte K block = four 32-byte K steps (K = 16 16-bit or 32 8-bit elements);
-// descriptors from their low words
-#define SENTRY_MMA_KBLOCK(KIND)                                                                                       \
-    asm volatile(                                                                                                     \
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t.reg .b32 ta, tb;\n\t"                                            \
-        "setp.ne.b32 p, %5, 0;\n\t"                                                                                   \
-        "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t"                                                          \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%0], da, db, %3, p;\n\t"                                             \
-        "setp.ne.b32 p, 1, 0;\n\t"                                                                                    \
-        "add.u32 ta, %1, 2;\n\tadd.u32 tb, %2, 2;\n\tmov.b64 da, {ta, %4};\n\tmov.b64 db, {tb, %4};\n\t"              \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%0], da, db, %3, p;\n\t"                                             \
-        "add.u32 ta, %1, 4;\n\tadd.u32 tb, %2, 4;\n\tmov.b64 da, {ta, %4};\n\tmov.b64 db, {tb, %4};\n\t"              \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%0], da, db, %3, p;\n\t"                                             \
-        "add.u32 ta, %1, 6;\n\tadd.u32 tb, %2, 6;\n\tmov.b64 da, {ta, %4};\n\tmov.b64 db, {tb, %4};\n\t"              \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%0], da, db, %3, p;\n\t}"                                            \
-        :                                                                                                             \
-        : "r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(kDescHi), "r"(accumulate_first)                          \
-        : "memory")
-template <bool FP8>
-__device__ __forceinline__ void mma_kblock(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
-                                           uint32_t accumulate_first) {
-    if constexpr (FP8) SENTRY_MMA_KBLOCK("f8f6f4");
-    else SENTRY_MMA_KBLOCK("f16");
-}
-// Slow path of a stage's combined wait: the barriers one after the other, bounded (0 = none).
-static __device__ __noinline__ bool wait_each_slow(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1, uint32_t b2,
-                                                   uint32_t p2, uint32_t b3, uint32_t p3, volatile int* abort_flag) {
-    bool ok = ptx::mbar_wait(b0, p0, abort_flag);
-    if (ok && b1 != 0u) ok = ptx::mbar_wait(b1, p1, abort_flag);
-    if (ok && b2 != 0u) ok = ptx::mbar_wait(b2, p2, abort_flag);
-    if (ok && b3 != 0u) ok = ptx::mbar_wait(b3, p3, abort_flag);
-    return ok;
-}
-
 // F16: X, W and Y are IEEE half instead of bf16.  FP8: X and the weights are e4m3 bytes with
 // per-tensor scales, the hidden activations are requantised to e4m3 (gelu(acc * a_scale) * h_inv),
 // Y = acc * y_scale is stored as bf16.
@@ -640,45 +591,7 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__
         }
         if (ok && ti > 0) drain_y(ti - 1, my_row, my_third);
     } else if (warp == kZeroWarp && plan.zero_ids != nullptr) {
-        // ------------------------------------------------- zero rows of Y for absent tokens
-        // The CTAs share the rows out evenly; runs of absent rows are written by bulk copies from a block of zeros, an
-        // instruction per kilobyte.  As blocks of the prepare launch these stores were a pass of their own over the absent
-        // part of Y (65 of 85 us at 4096 x 256 tokens, 3/7 absent); here they run beside the arithmetic.
-        const uint32_t zsm = ptx::smem_u32(misc) + 2048u - kZeroBytes;
-        for (int i = lane; i < kZeroBytes / 16; i += 32)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(zsm + i * 16), "r"(0) : "memory");
-        ptx::fence_proxy_async_smem();
-        __syncwarp();
-        const int per = (plan.n_rows + (int)gridDim.x - 1) / (int)gridDim.x;
-        const int r1 = min(plan.n_rows, ((int)blockIdx.x + 1) * per);
-        for (int r0 = (int)blockIdx.x * per; r0 < r1; r0 += 128) {
-            // 128 rows at a time: their ids and masks are requested together (a round trip per 32 rows made this warp
-            // the last to finish)
-            int m[4];
-            uint32_t mask[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int r = min(r0 + u * 32 + lane, plan.n_rows - 1), bb = r / plan.Tlen;
-                m[u] = __ldg(plan.zero_ids + (r - bb * plan.Tlen));
-                mask[u] = __ldg(plan.zero_masks + bb);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool absent = r0 + u * 32 + lane < r1 && !(m[u] >= 0 && m[u] < 32 && ((mask[u] >> m[u]) & 1u));
-                unsigned todo = __ballot_sync(0xffffffffu, absent);
-                while (todo) {   // runs of absent rows: contiguous in Y, kZeroBytes per lane (32 rows are at most 24 KB)
-                    const int first = __ffs(todo) - 1;
-                    const unsigned rest = ~(todo >> first);
-                    const int len = rest ? min(__ffs(rest) - 1, 32 - first) : 32 - first;
-                    todo &= ~((len == 32 ? 0xffffffffu : (1u << len) - 1u) << first);
-                    const int off = lane * kZeroBytes, bytes = min(len * D * 2 - off, kZeroBytes);
-                    if (bytes > 0)
-                        ptx::bulk_store(reinterpret_cast<uint8_t*>(Y) + (size_t)(r0 + u * 32 + first) * D * 2 + off, zsm,
-                                        (uint32_t)bytes);
-                }
-            }
-        }
-        ptx::bulk_store_wait();   // the zeros have been read (and the rows are written before the grid ends)
+        ffn_zero_rows<D>(plan, Y, ptx::smem_u32(misc) + 2048u - kZeroBytes);
     }
 
     tc_cta_teardown(abort_flag, status, tmem, kTmemCols);
@@ -789,16 +702,12 @@ int launch_ffn_tc(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* 
         SENTRY_CUDA_TRY(cudaGetLastError());
         return SENTRY_OK;
     }
+    // 16-bit operands: d_model 128 and 256 keep the hidden tile in tensor memory; at 384 Y leaves no room for that
     const bool f16 = a.d.dtype == SENTRY_F16;
-    switch (a.d.D) {
-        case 128: rc = f16 ? launch_d<128, true>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
-                           : launch_d<128, false>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st); break;
-        case 256: rc = f16 ? launch_d<256, true>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
-                           : launch_d<256, false>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st); break;
-        case 384: rc = f16 ? launch_d<384, true>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
-                           : launch_d<384, false>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st); break;
-        default: return SENTRY_ERR_UNSUPPORTED;
-    }
+    if (ffn_tmem_supported(a.d)) rc = launch_ffn_tmem(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
+    else if (a.d.D != 384) return SENTRY_ERR_UNSUPPORTED;
+    else rc = f16 ? launch_d<384, true>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
+                  : launch_d<384, false>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
     if (rc != SENTRY_OK) return rc;
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;

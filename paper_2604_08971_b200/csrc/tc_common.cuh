@@ -125,6 +125,8 @@ __device__ __forceinline__ bool elect_one() {
 
 // End of a CTA: if any wait ran out, raise the status bit and give copies and UMMAs that may
 // still be in flight time to land before shared memory and TMEM go away; then free the TMEM.
+// P: 2 for a pair of CTAs that allocated together.
+template <int P = 1>
 __device__ __forceinline__ void tc_cta_teardown(volatile int* abort_flag, unsigned int* status, uint32_t tmem,
                                              uint32_t tmem_cols) {
     ptx::tc_fence_before_sync();
@@ -137,7 +139,8 @@ __device__ __forceinline__ void tc_cta_teardown(volatile int* abort_flag, unsign
     }
     if ((threadIdx.x >> 5) == 0) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem, tmem_cols);
+        if constexpr (P == 2) ptx::tmem_dealloc_pair(tmem, tmem_cols);
+        else ptx::tmem_dealloc(tmem, tmem_cols);
     }
 }
 
