@@ -1,17 +1,20 @@
 // Channel-compacted FFN (Section 4.6) for the d_model that the fused kernel of ffn_tc.cu does not take (its Y accumulator
 // and an X tile must fit one SM beside the hidden tile: 128, 256, 384): any other multiple of 64 up to 1024, bf16 or fp16.
 //
-// Two tcgen05 GEMMs over the row plan, 128 x 128 tiles of one CTA each:
-//   1  H = gelu(X[rows] . W1c^T)   X rows gathered by 16-byte async copies, W1c by TMA; exact erf
+// Two tcgen05 GEMMs over the row plan, a CTA per tile of 128 rows and BN columns:
+//   1  H = gelu(X[rows] . W1c^T)   X rows gathered by 16-byte async copies, W1c by TMA; erf form
 //   2  Y[rows] = H . W2c^T         both operands by TMA
 // The hidden activations pass through a buffer of kWideTiles row tiles that stays in L2 (84 MB at 1280 channels); more
 // rows than that go in turns.  They are stored as a 16-bit head plus a 16-bit remainder (h = hi + lo to 2^-17), and
 // GEMM 2 multiplies both: what the plain-ALU kernel keeps in fp32 is not rounded to 16 bits here either.
 //
-// Tensor-bound in principle (6 D k_c operations per row with the remainder's product).  Measured on 3.7 k rows of
-// d_model 768, 1229 channels in seven lists (33 row tiles): 32 + 25 us, 380 TFLOP/s of these operations, where the
-// plain-ALU kernel (16 rows per CTA, one weight load per 16 multiply-adds) took 1065 us.
-// Three 32 KB or two 48 KB stages let two CTAs share an SM, so that one's epilogue runs beside the other's arithmetic.
+// What bounds them: GEMM 1 its epilogue (two special-function and thirteen other instructions per element, by all eight warps;
+// with the library's erff and four warps 6 us of 13 a tile) and its row gather, GEMM 2 the shared memory that serves the UMMAs'
+// operands and the copies (128 bytes a cycle).  The column tile follows the number of row tiles, which only the device
+// knows: small calls spread over more SMs, large ones read A less often.
+// Measured, a call with its row plan on materialised weights, before (128 x 128 tiles, erff, four epilogue warps that stored row
+// by row) and now: 3.7 k rows of d_model 768, 1229 channels in seven lists 55.1 -> 47.0 us; 524 rows, 765 channels 29.0 -> 23.9;
+// 46 rows, 967 channels 30.2 -> 25.0; 233 rows of d_model 192, 340 channels 19.0 -> 15.3; 5.6 k rows, 384 channels 21.6 -> 18.6.
 #include <cuda.h>
 #include <math.h>
 
@@ -28,14 +31,17 @@ constexpr int kWideTiles = 128;         // row tiles the hidden buffer holds
 
 template <bool FIRST>
 struct WideCfg {
-    static constexpr int BLOCKS = FIRST ? 2 : 3;            // operand blocks per stage: A, B or A head, A remainder, B
-    static constexpr int STAGES = FIRST ? 3 : 2;
-    static constexpr int STAGE_BYTES = BLOCKS * kWBlock;
+    static constexpr int A_BLOCKS = FIRST ? 1 : 2;          // A, or A's head and remainder
+    static constexpr int BN_MAX = FIRST ? 160 : 192;        // columns of a tile: a multiple of 32, 64 to this
+    static constexpr int CTAS = FIRST ? 2 : 1;              // per SM
+    static constexpr int STAGES = FIRST ? 3 : 4;
+    static constexpr int STAGE_BYTES = A_BLOCKS * kWBlock + BN_MAX * 128;
+    static constexpr int TMEM_COLS = 256;
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* misc */ + 1024 /* alignment */;
 };
 
 struct WideMisc {
-    uint64_t full[3], empty[3], acc_full;
+    uint64_t full[4], empty[4], acc_full;
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -50,16 +56,46 @@ __device__ __forceinline__ float hi_of(uint32_t w) {
     if constexpr (F16) return __half2float(__ushort_as_half((unsigned short)(w >> 16)));
     else return __uint_as_float(w & 0xffff0000u);
 }
-__device__ __forceinline__ float gelu_exact(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752440f)); }
+// gelu(z) = z Phi(z) = max(z, 0) - |z| Q(|z|) with Q(a) = exp(-a^2/2) R(1 / (1 + a/4)), the tail of the normal distribution: own
+// minimax fit of R (degree 7, 9e-9 of the value at the worst a, weighted by exp(-a^2/2) down to 1e-2).  In fp32 it is off by
+// at most 2.4e-7 |z|, where 0.5 z (1 + erff(z / sqrt 2)) is by 1.1e-7 |z| and the buffer's head and remainder by 2^-17 |h|:
+// 15 instructions, about a third of the library form's.  NaN stays NaN, and +inf and -inf give inf and NaN as that form does.
+__device__ __forceinline__ float gelu_tail(float z) {
+    const float a = fabsf(z), c = fminf(a, 16.f);           // (the tail is 0 from 14 on)
+    float t, e;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.25f, c, 1.f)));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(c * c * -0.72134752f));
+    float r = fmaf(-0.0961182937f, t, 0.363730848f);
+    r = fmaf(r, t, -0.312237799f);
+    r = fmaf(r, t, 0.331047446f);
+    r = fmaf(r, t, -0.00703657651f);
+    r = fmaf(r, t, 0.123881109f);
+    r = fmaf(r, t, 0.0965574905f);
+    r = fmaf(r, t, 0.000175767025f);
+    return fmaf(0.5f, z + a, -c * (r * e));
+}
 
-// grid (N tiles, row tiles of this turn).  FIRST: tm_b = W1c [lists * kc_pad, D], out_h / out_l = the hidden buffer's two
-// planes.  Otherwise tm_a_hi / tm_a_lo = those planes, tm_b = W2c [lists * D, kc_pad], Y the result.
+// Columns of a tile where R row tiles have `cols` columns and `slots` CTAs run at once: the rounds times what a K block costs
+// in shared-memory traffic, which is that of A and the columns of B (in units of B's).
+template <bool FIRST>
+__device__ __forceinline__ int wide_bn(int R, int cols, int slots) {
+    int best = 64, best_cost = 0x7fffffff;
+    for (int bn = 64; bn <= WideCfg<FIRST>::BN_MAX; bn += 32) {
+        const int items = R * ((cols + bn - 1) / bn), cost = (items + slots - 1) / slots * ((FIRST ? 128 : 170) + bn);
+        if (cost < best_cost) { best = bn; best_cost = cost; }
+    }
+    return best;
+}
+
+// grid (column tiles of 64, row tiles of this turn); a CTA beyond the tiles that there are at the width taken has nothing to do.
+// FIRST: tm_b = W1c [lists * kc_pad, D], out_h / out_l = the hidden buffer's two planes.  Otherwise tm_a_hi / tm_a_lo = those
+// planes, tm_b = W2c [lists * D, kc_pad], Y the result.
 template <bool FIRST, bool F16>
-__global__ void __launch_bounds__(kWThreads, 2)
+__global__ void __launch_bounds__(kWThreads, WideCfg<FIRST>::CTAS)
 ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_constant__ CUtensorMap tm_a_lo,
                 const __grid_constant__ CUtensorMap tm_b, const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ out_h,
-                __nv_bfloat16* __restrict__ out_l, __nv_bfloat16* __restrict__ Y, FfnPlan plan, int n_lists, int tile0, int D,
-                int kc_pad, unsigned int* status) {
+                __nv_bfloat16* __restrict__ out_l, __nv_bfloat16* __restrict__ Y, FfnPlan plan, int n_lists, int tile0, int turn,
+                int D, int k_c, int kc_pad, int sm_count, unsigned int* status) {
     using C = WideCfg<FIRST>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = ptx::smem_u32(smem_raw);
@@ -70,8 +106,13 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
     grid_dependency_wait();
     int l, row0, n_rows;
     if (!ffn_tile_lookup(plan, n_lists, tile0 + (int)blockIdx.y, 128, l, row0, n_rows)) return;
-    const int n0 = blockIdx.x * 128;                       // first output column
-    const int KB = (FIRST ? D : kc_pad) / 64;              // 64-element K blocks
+    const int kc = (k_c + 63) / 64 * 64;                   // channels that are computed (padded ones carry zero weights)
+    const int cols = FIRST ? kc : D;
+    const int bn = wide_bn<FIRST>(min(plan.tile_start[n_lists] - tile0, turn), cols, sm_count * C::CTAS);
+    const int n0 = blockIdx.x * bn;                        // first output column
+    if (n0 >= cols) return;
+    const int n_cols = min(bn, cols - n0);                 // a multiple of 32
+    const int KB = (FIRST ? D : kc) / 64;                  // 64-element K blocks
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::STAGES; ++s) {
@@ -83,7 +124,7 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
         ptx::fence_barrier_init();
     }
     if (warp == 0) {
-        ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), 128);
+        ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), C::TMEM_COLS);
         ptx::tmem_relinquish();
     }
     ptx::tc_fence_before_sync();
@@ -100,18 +141,19 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
             if (!ok) break;
             if (elect_one()) {
                 const uint32_t bar = ptx::smem_u32(&misc->full[s]), dst = base + s * C::STAGE_BYTES;
-                ptx::mbar_arrive_expect_tx(bar, FIRST ? kWBlock : 3 * kWBlock);
+                ptx::mbar_arrive_expect_tx(bar, (FIRST ? 0 : 2 * kWBlock) + n_cols * 128);
                 if constexpr (!FIRST) {
                     ptx::tma_load_2d(dst, &tm_a_hi, kb * 64, (int)blockIdx.y * 128, bar);
                     ptx::tma_load_2d(dst + kWBlock, &tm_a_lo, kb * 64, (int)blockIdx.y * 128, bar);
                 }
-                ptx::tma_load_2d(dst + (C::BLOCKS - 1) * kWBlock, &tm_b, kb * 64, l * (FIRST ? kc_pad : D) + n0, bar);
+                for (int c = 0; c < n_cols; c += 32)
+                    ptx::tma_load_2d(dst + C::A_BLOCKS * kWBlock + c * 128, &tm_b, kb * 64, l * (FIRST ? kc_pad : D) + n0 + c, bar);
             }
             __syncwarp();
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- UMMA issuer
-        constexpr uint32_t idesc = F16 ? ptx::umma_idesc_f16(128, 128) : ptx::umma_idesc_bf16(128, 128);
+        const uint32_t idesc = F16 ? ptx::umma_idesc_f16(128, n_cols) : ptx::umma_idesc_bf16(128, n_cols);
         bool ok = true;
         for (int kb = 0; kb < KB && ok; ++kb) {
             const int s = kb % C::STAGES, use = kb / C::STAGES;
@@ -119,9 +161,9 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
             if (!ok) break;
             ptx::tc_fence_after_sync();
             if (elect_one()) {
-                const uint32_t a = base + s * C::STAGE_BYTES, b = a + (C::BLOCKS - 1) * kWBlock;
+                const uint32_t a = base + s * C::STAGE_BYTES, b = a + C::A_BLOCKS * kWBlock;
 #pragma unroll
-                for (int part = 0; part < C::BLOCKS - 1; ++part)
+                for (int part = 0; part < C::A_BLOCKS; ++part)
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
                         ptx::umma_bf16(tmem, ptx::umma_smem_desc_sw128(a + part * kWBlock + ks * 32),
@@ -131,86 +173,98 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
             }
             __syncwarp();
         }
-    } else if (warp >= 4) {
+    } else if (FIRST && warp >= 4) {
+        // ---------------------------------------------------------------- X row gather
         bool ok = true;
-        if constexpr (FIRST) {
-            // ------------------------------------------------------------ X row gather
-            const int tl = threadIdx.x - 128;
-            int32_t rows[8];
+        const int tl = threadIdx.x - 128;
+        int32_t rows[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int r = (tl + j * 128) >> 3;
+            rows[j] = r < n_rows ? plan.rowidx[row0 + r] : -1;
+        }
+        int published = 0;
+        auto publish = [&](int pending) {
+            cp_async_wait_pending(pending);
+            ptx::fence_proxy_async_smem();
+            warp_arrive(&misc->full[published % C::STAGES]);
+            ++published;
+        };
+        for (int kb = 0; kb < KB && ok; ++kb) {
+            const int s = kb % C::STAGES, use = kb / C::STAGES;
+            // a slot is refilled only when its block has been read, which needs every earlier block published
+            if (kb >= C::STAGES)
+                while (published <= kb - C::STAGES) publish(kb - published - 1);
+            ok = warp_wait(&misc->empty[s], (use & 1) ^ 1, abort_flag);
+            if (!ok) break;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const int r = (tl + j * 128) >> 3;
-                rows[j] = r < n_rows ? plan.rowidx[row0 + r] : -1;
+                const int r = (tl + j * 128) >> 3, ci = tl & 7;
+                const uint32_t dst = base + s * C::STAGE_BYTES + r * 128 + ((ci ^ (r & 7)) << 4);
+                if (rows[j] >= 0) ptx::cp_async_16(dst, X + (size_t)rows[j] * D + kb * 64 + ci * 8);
+                else asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
             }
-            int published = 0;
-            auto publish = [&](int pending) {
-                cp_async_wait_pending(pending);
-                ptx::fence_proxy_async_smem();
-                warp_arrive(&misc->full[published % C::STAGES]);
-                ++published;
-            };
-            for (int kb = 0; kb < KB && ok; ++kb) {
-                const int s = kb % C::STAGES, use = kb / C::STAGES;
-                // a slot is refilled only when its block has been read, which needs every earlier block published
-                if (kb >= C::STAGES)
-                    while (published <= kb - C::STAGES) publish(kb - published - 1);
-                ok = warp_wait(&misc->empty[s], (use & 1) ^ 1, abort_flag);
-                if (!ok) break;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int r = (tl + j * 128) >> 3, ci = tl & 7;
-                    const uint32_t dst = base + s * C::STAGE_BYTES + r * 128 + ((ci ^ (r & 7)) << 4);
-                    if (rows[j] >= 0) ptx::cp_async_16(dst, X + (size_t)rows[j] * D + kb * 64 + ci * 8);
-                    else asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
-                }
-                ptx::cp_async_commit();
-                if (kb - published >= 2) publish(2);
-            }
-            while (ok && published < KB) publish(KB - published - 1);
-            ptx::cp_async_wait_all();
+            ptx::cp_async_commit();
+            if (kb - published >= 2) publish(2);
         }
-        // -------------------------------------------------------------------- epilogue
-        const int quarter = warp & 3, row = quarter * 32 + lane;
-        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-        const int n_cols = min(128, (FIRST ? kc_pad : D) - n0);
-        int32_t yrow = -1;
-        if (!FIRST && row < n_rows) yrow = (plan.rowout ? plan.rowout : plan.rowidx)[row0 + row];
-        if (ok && warp_wait(&misc->acc_full, 0u, abort_flag)) {
-            ptx::tc_fence_after_sync();
-            const size_t hrow = ((size_t)blockIdx.y * 128 + row) * kc_pad + n0;
+        while (ok && published < KB) publish(KB - published - 1);
+        ptx::cp_async_wait_all();
+    }
+    // -------------------------------------------------------------------- epilogue: all warps, two to a row, every other 32 columns
+    // 32 columns at a time through 2 KB of the warp's own in the first stage (every UMMA has read it), so that a store writes
+    // 64 consecutive bytes of eight rows.
+    const int quarter = warp & 3, row = quarter * 32 + lane, half = warp >> 2;
+    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+    if (warp_wait(&misc->acc_full, 0u, abort_flag)) {
+        ptx::tc_fence_after_sync();
+        const uint32_t stg = base + (uint32_t)warp * 2048u;
+        const uint32_t wr = stg + lane * 64, rd = stg + (lane >> 2) * 64;
+        const uint32_t wx = (lane >> 1) & 3, rx = ((lane & 3) ^ ((lane >> 3) & 3)) << 4;
+        int32_t grs[4];                                    // where the rows go that this lane stores pieces of
+        {
+            int32_t mine = -1;
+            if (row < n_rows) mine = FIRST ? (int)blockIdx.y * 128 + row : (plan.rowout ? plan.rowout : plan.rowidx)[row0 + row];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) grs[i] = __shfl_sync(0xffffffffu, mine, i * 8 + (lane >> 2));
+        }
+        auto store32 = [&](const uint32_t (&w)[16], __nv_bfloat16* dst, int ld) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(wr + ((i ^ wx) << 4)), "r"(w[4 * i]), "r"(w[4 * i + 1]),
+                             "r"(w[4 * i + 2]), "r"(w[4 * i + 3])
+                             : "memory");
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint4 v;
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(rd + i * 512 + rx));
+                if (grs[i] >= 0) *reinterpret_cast<uint4*>(dst + (size_t)grs[i] * ld + (lane & 3) * 8) = v;
+            }
+            __syncwarp();
+        };
 #pragma unroll 1
-            for (int c0 = 0; c0 < n_cols; c0 += 32) {
-                uint32_t r[32];
-                ptx::tmem_ld_32x32(lane_base + c0, r);
-                ptx::tmem_ld_wait();
-                if constexpr (FIRST) {
+        for (int c0 = half * 32; c0 < n_cols; c0 += 64) {
+            uint32_t r[32], w[16];
+            ptx::tmem_ld_32x32(lane_base + c0, r);
+            ptx::tmem_ld_wait();
+            if constexpr (FIRST) {
+                uint32_t q[16];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        uint32_t h[4], q[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float g0 = gelu_exact(__uint_as_float(r[8 * i + 2 * e])), g1 = gelu_exact(__uint_as_float(r[8 * i + 2 * e + 1]));
-                            h[e] = pack_16x2<F16>(g0, g1);
-                            q[e] = pack_16x2<F16>(g0 - lo_of<F16>(h[e]), g1 - hi_of<F16>(h[e]));
-                        }
-                        if (row < n_rows) {
-                            *reinterpret_cast<uint4*>(out_h + hrow + c0 + 8 * i) = make_uint4(h[0], h[1], h[2], h[3]);
-                            *reinterpret_cast<uint4*>(out_l + hrow + c0 + 8 * i) = make_uint4(q[0], q[1], q[2], q[3]);
-                        }
-                    }
-                } else if (yrow >= 0) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        *reinterpret_cast<uint4*>(Y + (size_t)yrow * D + n0 + c0 + 8 * i) =
-                            make_uint4(pack_16x2<F16>(__uint_as_float(r[8 * i]), __uint_as_float(r[8 * i + 1])),
-                                       pack_16x2<F16>(__uint_as_float(r[8 * i + 2]), __uint_as_float(r[8 * i + 3])),
-                                       pack_16x2<F16>(__uint_as_float(r[8 * i + 4]), __uint_as_float(r[8 * i + 5])),
-                                       pack_16x2<F16>(__uint_as_float(r[8 * i + 6]), __uint_as_float(r[8 * i + 7])));
+                for (int i = 0; i < 16; ++i) {
+                    const float g0 = gelu_tail(__uint_as_float(r[2 * i])), g1 = gelu_tail(__uint_as_float(r[2 * i + 1]));
+                    w[i] = pack_16x2<F16>(g0, g1);
+                    q[i] = pack_16x2<F16>(g0 - lo_of<F16>(w[i]), g1 - hi_of<F16>(w[i]));
                 }
+                store32(w, out_h + n0 + c0, kc_pad);
+                store32(q, out_l + n0 + c0, kc_pad);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) w[i] = pack_16x2<F16>(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
+                store32(w, Y + n0 + c0, D);
             }
         }
     }
-    tc_cta_teardown(abort_flag, status, tmem, 128);
+    tc_cta_teardown(abort_flag, status, tmem, C::TMEM_COLS);
 }
 
 template <bool F16>
@@ -221,8 +275,8 @@ int launch_wide(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1
     __nv_bfloat16* hh = (__nv_bfloat16*)hidden;
     __nv_bfloat16* hl = hh + (size_t)turn * 128 * kc_pad;
     CUtensorMap m1, m2, ah, al;
-    if (!make_weight_map(&m1, w1c, (uint64_t)d.n_lists * kc_pad, d.D, 128) ||
-        !make_weight_map(&m2, w2c, (uint64_t)d.n_lists * d.D, kc_pad, 128) ||
+    if (!make_weight_map(&m1, w1c, (uint64_t)d.n_lists * kc_pad, d.D, 32) ||
+        !make_weight_map(&m2, w2c, (uint64_t)d.n_lists * d.D, kc_pad, 32) ||
         !make_weight_map(&ah, hh, (uint64_t)turn * 128, kc_pad, 128) || !make_weight_map(&al, hl, (uint64_t)turn * 128, kc_pad, 128))
         return SENTRY_ERR_CUDA;
     auto k1 = ffn_wide_kernel<true, F16>;
@@ -232,12 +286,12 @@ int launch_wide(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1
     for (int t0 = 0; t0 < max_tiles; t0 += turn) {
         const unsigned nt = (unsigned)(max_tiles - t0 < turn ? max_tiles - t0 : turn);
         LaunchScope ls(ctx, KS_FFN_MAIN, st, 2);
-        SENTRY_CUDA_TRY(launch_chained(k1, dim3((unsigned)(kc_pad / 128), nt), dim3(kWThreads), (size_t)WideCfg<true>::SMEM_BYTES,
-                                       st, ah, al, m1, (const __nv_bfloat16*)a.X, hh, hl, nullptr, plan, d.n_lists, t0, d.D,
-                                       kc_pad, a.status));
-        SENTRY_CUDA_TRY(launch_chained(k2, dim3((unsigned)((d.D + 127) / 128), nt), dim3(kWThreads),
-                                       (size_t)WideCfg<false>::SMEM_BYTES, st, ah, al, m2, nullptr, nullptr, nullptr,
-                                       (__nv_bfloat16*)a.Y, plan, d.n_lists, t0, d.D, kc_pad, a.status));
+        SENTRY_CUDA_TRY(launch_chained(k1, dim3((unsigned)((d.k_c + 63) / 64), nt), dim3(kWThreads), (size_t)WideCfg<true>::SMEM_BYTES,
+                                       st, ah, al, m1, (const __nv_bfloat16*)a.X, hh, hl, nullptr, plan, d.n_lists, t0, (int)nt, d.D,
+                                       d.k_c, kc_pad, ctx->sm_count, a.status));
+        SENTRY_CUDA_TRY(launch_chained(k2, dim3((unsigned)(d.D / 64), nt), dim3(kWThreads), (size_t)WideCfg<false>::SMEM_BYTES, st, ah,
+                                       al, m2, nullptr, nullptr, nullptr, (__nv_bfloat16*)a.Y, plan, d.n_lists, t0, (int)nt, d.D,
+                                       d.k_c, kc_pad, ctx->sm_count, a.status));
     }
     return SENTRY_OK;
 }
