@@ -44,26 +44,47 @@ __device__ __forceinline__ void plan_block(const int32_t* __restrict__ ids, cons
     if (first_block)
         for (int l = threadIdx.x; l < min(n_lists, kPlanListsSmem); l += blockDim.x) s_rows[l] = 0;
     __syncthreads();
+    // the first sample of this thread's share and the block's own ones, requested before the token counts are there
+    const int bb_first = threadIdx.x;
+    int l_first = 0, own_l[G];
+    uint32_t mask_first = 0u, own_mask[G];
+    if (bb_first < B) {
+        if (list_of_sample != nullptr) l_first = list_of_sample[bb_first];
+        if (ids != nullptr) mask_first = masks[bb_first];
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        own_l[g] = b0 + g < B && list_of_sample != nullptr ? list_of_sample[b0 + g] : 0;
+        own_mask[g] = b0 + g < B && ids != nullptr ? masks[b0 + g] : 0xffffffffu;
+    }
     if (ids != nullptr) {
-        for (int t0 = 0; t0 < Tlen; t0 += blockDim.x) {
-            const int t = t0 + threadIdx.x;
-            const int m = t < Tlen ? ids[t] : -1;
-            if (t < Tlen && (m < 0 || m >= 32) && first_block) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
-            // tokens of a modality lie together: one shared-memory atomic per warp and modality
-            const unsigned peers = __match_any_sync(0xffffffffu, m);
-            if (m >= 0 && m < 32 && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[m], __popc(peers));
+        // eight of a thread's tokens on the way at once (with one, 16 round trips at 4096 tokens: 15 us of this kernel, now 7)
+        for (int t0 = 0; t0 < Tlen; t0 += 8 * blockDim.x) {
+            int m[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int t = t0 + u * blockDim.x + threadIdx.x;
+                m[u] = t < Tlen ? ids[t] : -1;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int t = t0 + u * blockDim.x + threadIdx.x;
+                if (t0 + u * (int)blockDim.x >= Tlen) break;
+                if (t < Tlen && (m[u] < 0 || m[u] >= 32) && first_block) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+                // tokens of a modality lie together: one shared-memory atomic per warp and modality
+                const unsigned peers = __match_any_sync(0xffffffffu, m[u]);
+                if (m[u] >= 0 && m[u] < 32 && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[m[u]], __popc(peers));
+            }
         }
         __syncthreads();
     }
-    auto present_rows = [&](int bb) {
+    auto present_rows = [&](uint32_t mask) {
         if (ids == nullptr) return Tlen;
-        uint32_t mask = masks[bb];
         int n = 0;
         while (mask) { const int m = __ffs(mask) - 1; n += s_cnt[m]; mask &= mask - 1; }
         return n;
     };
-    auto list_of = [&](int bb) {
-        int l = list_of_sample ? list_of_sample[bb] : 0;
+    auto checked = [&](int l) {
         if (l < 0 || l >= n_lists) {
             if (first_block) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
             l = 0;
@@ -73,9 +94,11 @@ __device__ __forceinline__ void plan_block(const int32_t* __restrict__ ids, cons
     // rows of all samples in earlier lists, and of earlier samples in the sample's list
     int my_list[G], before[G];
 #pragma unroll
-    for (int g = 0; g < G; ++g) { my_list[g] = b0 + g < B ? list_of(b0 + g) : -1; before[g] = 0; }
+    for (int g = 0; g < G; ++g) { my_list[g] = b0 + g < B ? checked(own_l[g]) : -1; before[g] = 0; }
     for (int bb = threadIdx.x; bb < B; bb += blockDim.x) {
-        const int l = list_of(bb), r = present_rows(bb);
+        const bool have = bb == bb_first;
+        const int l = checked(have ? l_first : (list_of_sample ? list_of_sample[bb] : 0));
+        const int r = present_rows(have ? mask_first : (ids != nullptr ? masks[bb] : 0u));
 #pragma unroll
         for (int g = 0; g < G; ++g)
             if (l < my_list[g] || (l == my_list[g] && bb < b0 + g)) before[g] += r;
@@ -115,7 +138,7 @@ __device__ __forceinline__ void plan_block(const int32_t* __restrict__ ids, cons
             for (int l = 0; l < n_lists; ++l) {
                 int rows = 0;
                 for (int bb = threadIdx.x; bb < B; bb += blockDim.x)
-                    if (list_of(bb) == l) rows += present_rows(bb);
+                    if (checked(list_of_sample ? list_of_sample[bb] : 0) == l) rows += present_rows(ids != nullptr ? masks[bb] : 0u);
                 rows = block_sum_int(rows, red);
                 if (threadIdx.x == 0) { p.list_row0[l] = row0; p.tile_start[l] = tile0; }
                 row0 += rows;
@@ -124,13 +147,25 @@ __device__ __forceinline__ void plan_block(const int32_t* __restrict__ ids, cons
             if (threadIdx.x == 0) { p.list_row0[n_lists] = row0; p.tile_start[n_lists] = tile0; }
         }
     }
-    // present tokens of the samples, ascending -> row table
-    auto present = [&](int t, uint32_t mask) {
-        if (t >= Tlen) return false;
-        if (ids == nullptr) return true;
-        const int m = ids[t];
-        return m >= 0 && m < 32 && ((mask >> m) & 1u);
+    // present tokens of the samples, ascending -> row table; eight pieces of 32 tokens at a time
+    auto pieces = [&](int pc, int p1, uint32_t mask, unsigned (&bm)[8]) {
+        int m[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int t = (pc + u) * 32 + lane;
+            m[u] = pc + u < p1 && t < Tlen ? (ids != nullptr ? ids[t] : 0) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) bm[u] = __ballot_sync(0xffffffffu, m[u] >= 0 && m[u] < 32 && ((mask >> m[u]) & 1u));
     };
+    auto put = [&](int b, int pc, const unsigned (&bm)[8], int& base) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if ((bm[u] >> lane) & 1u) p.rowidx[base + __popc(bm[u] & ((1u << lane) - 1u))] = b * Tlen + (pc + u) * 32 + lane;
+            base += __popc(bm[u]);
+        }
+    };
+    const int n_pieces = (Tlen + 31) / 32;
     if constexpr (G > 1) {   // a warp per sample
         static_assert(G <= 8, "one warp per sample of the group");
         const int b = b0 + wid;
@@ -139,11 +174,10 @@ __device__ __forceinline__ void plan_block(const int32_t* __restrict__ ids, cons
             for (int w = 0; w < nw; ++w) base += s_before[wid][w];
             if (lane == 0) p.sample_row0[b] = base;
             const uint32_t mask = ids != nullptr ? masks[b] : 0xffffffffu;
-            for (int t0 = 0; t0 < Tlen; t0 += 32) {
-                const bool ok = present(t0 + lane, mask);
-                const unsigned bm = __ballot_sync(0xffffffffu, ok);
-                if (ok) p.rowidx[base + __popc(bm & ((1u << lane) - 1u))] = b * Tlen + t0 + lane;
-                base += __popc(bm);
+            for (int pc = 0; pc < n_pieces; pc += 8) {
+                unsigned bm[8];
+                pieces(pc, n_pieces, mask, bm);
+                put(b, pc, bm, base);
             }
         }
     } else {                 // the whole block: every warp a run of 32-token pieces, after one count of what comes before
@@ -151,20 +185,21 @@ __device__ __forceinline__ void plan_block(const int32_t* __restrict__ ids, cons
         int base = 0;
         for (int w = 0; w < nw; ++w) base += s_before[0][w];
         if (threadIdx.x == 0) p.sample_row0[b] = base;
-        const uint32_t mask = ids != nullptr ? masks[b] : 0xffffffffu;
-        const int per = ((Tlen + 31) / 32 + nw - 1) / nw;
-        const int p0 = wid * per, p1 = min(p0 + per, (Tlen + 31) / 32);
+        const int per = (n_pieces + nw - 1) / nw;
+        const int p0 = wid * per, p1 = min(p0 + per, n_pieces);
+        unsigned bm[8];
         int mine = 0;
-        for (int pc = p0; pc < p1; ++pc) mine += __popc(__ballot_sync(0xffffffffu, present(pc * 32 + lane, mask)));
+        for (int pc = p0; pc < p1; pc += 8) {
+            pieces(pc, p1, own_mask[0], bm);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) mine += __popc(bm[u]);
+        }
         if (lane == 0) red[wid] = mine;
         __syncthreads();
         for (int w = 0; w < wid; ++w) base += red[w];
-        for (int pc = p0; pc < p1; ++pc) {
-            const int t = pc * 32 + lane;
-            const bool ok = present(t, mask);
-            const unsigned bm = __ballot_sync(0xffffffffu, ok);
-            if (ok) p.rowidx[base + __popc(bm & ((1u << lane) - 1u))] = b * Tlen + t;
-            base += __popc(bm);
+        for (int pc = p0; pc < p1; pc += 8) {
+            if (per > 8) pieces(pc, p1, own_mask[0], bm);   // (with one run of eight they are still there)
+            put(b, pc, bm, base);
         }
     }
 }
@@ -209,82 +244,149 @@ ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__
     pb -= zero_blocks;
     if (layout == 1) {
         // K-major copies for the tensor-core kernels, one tile of 64 channels x 64 columns per block, transposed through
-        // shared memory:  W1c[l][n][e] = W1[e][N[n]],  W2c[l][e][n] = W2[N[n]][e].  Bound by latency (a few MB in all), so
-        // a thread has all its loads in flight at once: 16 single elements of W1 (kept columns are scattered), 16-byte
-        // pieces of W2's rows; both copies are written 16 bytes at a time.
-        constexpr int VEC = 16 / (int)sizeof(T);           // elements of a 16-byte piece
-        constexpr int PITCH = 64 + (sizeof(T) == 1 ? 4 : 2);   // elements; odd number of words
-        __shared__ __align__(16) T s_tile[64 * PITCH];
-        __shared__ int s_ch[64];
-        const int tiles_n = kc_pad / 64, tiles_e = D / 64;
-        const size_t per_list = (size_t)tiles_n * tiles_e;
-        const int which = (int)(pb / (per_list * n_lists));
-        pb -= (size_t)which * per_list * n_lists;
-        const int l = (int)(pb / per_list);
-        const int tn = (int)((pb % per_list) / tiles_e), te = (int)(pb % tiles_e);
-        const int n0 = tn * 64, e0 = te * 64;
-        const T* W1l = W1 + (size_t)l * w_stride;
-        const T* W2l = W2 + (size_t)l * w_stride;
-        if (threadIdx.x < 64) {
-            const int n = n0 + threadIdx.x;
-            int ch = -1;
-            if (n < k_c) {
-                ch = kept[(size_t)l * k_c + n];
-                if (ch < 0 || ch >= F) {
-                    if (which == 0 && te == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
-                    ch = -1;
+        // shared memory:  W1c[l][n][e] = W1[e][N[n]],  W2c[l][e][n] = W2[N[n]][e].  A thread has all its loads in flight at once.
+        if constexpr (sizeof(T) == 2) {
+            // A thread turns 16-bit elements into whole 16-byte pieces in its registers; the pieces pass through shared memory
+            // (swizzled, no bank conflicts) so that eight lanes write a row's 128 bytes.  Bound by latency for one list, by L2
+            // beyond (26 MB of copies at d_model 768, 1229 channels, seven lists: 24 us with element-wise shared memory and 16-byte
+            // stores of 32 different rows, which L2 saw as 100 MB of sectors).
+            __shared__ __align__(16) uint4 s_piece[64 * 8];
+            const int tiles_n = kc_pad / 64, tiles_e = D / 64;
+            const size_t per_list = (size_t)tiles_n * tiles_e;
+            const int which = (int)(pb / (per_list * n_lists));
+            pb -= (size_t)which * per_list * n_lists;
+            const int l = (int)(pb / per_list);
+            const int tn = (int)((pb % per_list) / tiles_e), te = (int)(pb % tiles_e);
+            const int n0 = tn * 64, e0 = te * 64, tid = threadIdx.x;
+            auto channel = [&](int n) {
+                if (n >= k_c) return -1;
+                const int ch = kept[(size_t)l * k_c + n];
+                if (ch >= 0 && ch < F) return ch;
+                if (which == 0 && te == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+                return -1;
+            };
+            T* dst;
+            size_t ld;
+            int swz;      // pieces of row r sit at c ^ ((r >> swz) & 7)
+            if (which == 0) {
+                // thread: channel tid & 63, columns 16 (tid >> 6) ..
+                const int n = tid & 63, c0 = 2 * (tid >> 6);
+                const int ch = channel(n0 + n);
+                const uint16_t* src = reinterpret_cast<const uint16_t*>(W1 + (size_t)l * w_stride) + (size_t)(e0 + 8 * c0) * F + ch;
+                uint32_t v[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] = ch >= 0 ? src[(size_t)i * F] : 0u;
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    s_piece[n * 8 + ((c0 + h) ^ (n & 7))] = make_uint4(v[8 * h] | v[8 * h + 1] << 16, v[8 * h + 2] | v[8 * h + 3] << 16,
+                                                                       v[8 * h + 4] | v[8 * h + 5] << 16, v[8 * h + 6] | v[8 * h + 7] << 16);
+                dst = out1 + ((size_t)l * kc_pad + n0) * D + e0;
+                ld = D;
+                swz = 0;
+            } else {
+                // warp: channels 8 wid .., lane: columns 2 lane, 2 lane + 1
+                const int lane = tid & 31, wid = tid >> 5;
+                const int mine = lane < 8 ? channel(n0 + 8 * wid + lane) : -1;
+                uint32_t v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int ch = __shfl_sync(0xffffffffu, mine, i);
+                    v[i] = ch >= 0 ? *reinterpret_cast<const uint32_t*>(W2 + (size_t)l * w_stride + (size_t)ch * D + e0 + 2 * lane) : 0u;
                 }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t sel = h == 0 ? 0x5410u : 0x7632u;
+                    s_piece[(2 * lane + h) * 8 + (wid ^ (lane & 7))] =
+                        make_uint4(__byte_perm(v[0], v[1], sel), __byte_perm(v[2], v[3], sel), __byte_perm(v[4], v[5], sel),
+                                   __byte_perm(v[6], v[7], sel));
+                }
+                dst = out2 + ((size_t)l * D + e0) * kc_pad + n0;
+                ld = kc_pad;
+                swz = 1;
             }
-            s_ch[threadIdx.x] = ch;
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int r = (tid >> 3) + 32 * j, c = tid & 7;
+                *reinterpret_cast<uint4*>(dst + (size_t)r * ld + c * 8) = s_piece[r * 8 + (c ^ ((r >> swz) & 7))];
+            }
         }
-        __syncthreads();
-        const T zero = from_f32<T>(0.f);
-        T* dst;
-        size_t ld;
-        if (which == 0) {
-            // s_tile[e][n]
-            const int tx = threadIdx.x & 31, wy = threadIdx.x >> 5;   // 8 warps
-            const int c0 = s_ch[tx], c1 = s_ch[tx + 32];
-            T v0[8], v1[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const T* row = W1l + (size_t)(e0 + wy + 8 * i) * F;
-                v0[i] = c0 >= 0 ? row[c0] : zero;
-                v1[i] = c1 >= 0 ? row[c1] : zero;
+        if constexpr (sizeof(T) == 1) {   // element by element
+            constexpr int VEC = 16;           // elements of a 16-byte piece
+            constexpr int PITCH = 64 + 4;     // elements; odd number of words
+            __shared__ __align__(16) T s_tile[64 * PITCH];
+            __shared__ int s_ch[64];
+            const int tiles_n = kc_pad / 64, tiles_e = D / 64;
+            const size_t per_list = (size_t)tiles_n * tiles_e;
+            const int which = (int)(pb / (per_list * n_lists));
+            pb -= (size_t)which * per_list * n_lists;
+            const int l = (int)(pb / per_list);
+            const int tn = (int)((pb % per_list) / tiles_e), te = (int)(pb % tiles_e);
+            const int n0 = tn * 64, e0 = te * 64;
+            const T* W1l = W1 + (size_t)l * w_stride;
+            const T* W2l = W2 + (size_t)l * w_stride;
+            if (threadIdx.x < 64) {
+                const int n = n0 + threadIdx.x;
+                int ch = -1;
+                if (n < k_c) {
+                    ch = kept[(size_t)l * k_c + n];
+                    if (ch < 0 || ch >= F) {
+                        if (which == 0 && te == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+                        ch = -1;
+                    }
+                }
+                s_ch[threadIdx.x] = ch;
             }
+            __syncthreads();
+            const T zero = from_f32<T>(0.f);
+            T* dst;
+            size_t ld;
+            if (which == 0) {
+                // s_tile[e][n]
+                const int tx = threadIdx.x & 31, wy = threadIdx.x >> 5;   // 8 warps
+                const int c0 = s_ch[tx], c1 = s_ch[tx + 32];
+                T v0[8], v1[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                s_tile[(wy + 8 * i) * PITCH + tx] = v0[i];
-                s_tile[(wy + 8 * i) * PITCH + tx + 32] = v1[i];
+                for (int i = 0; i < 8; ++i) {
+                    const T* row = W1l + (size_t)(e0 + wy + 8 * i) * F;
+                    v0[i] = c0 >= 0 ? row[c0] : zero;
+                    v1[i] = c1 >= 0 ? row[c1] : zero;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    s_tile[(wy + 8 * i) * PITCH + tx] = v0[i];
+                    s_tile[(wy + 8 * i) * PITCH + tx + 32] = v1[i];
+                }
+                dst = out1 + ((size_t)l * kc_pad + n0) * D + e0;
+                ld = D;
+            } else {
+                // s_tile[n][e]
+                for (int i = threadIdx.x; i < 64 * 64 / VEC; i += 256) {
+                    const int nn = i / (64 / VEC), c = i % (64 / VEC);
+                    const int ch = s_ch[nn];
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (ch >= 0) {
+                        const T* src = W2l + (size_t)ch * D + e0 + c * VEC;
+                        v = *reinterpret_cast<const uint4*>(src);
+                    }
+                    const T* p8 = reinterpret_cast<const T*>(&v);
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) s_tile[nn * PITCH + c * VEC + e] = p8[e];
+                }
+                dst = out2 + ((size_t)l * D + e0) * kc_pad + n0;
+                ld = kc_pad;
             }
-            dst = out1 + ((size_t)l * kc_pad + n0) * D + e0;
-            ld = D;
-        } else {
-            // s_tile[n][e]
+            __syncthreads();
+            // column r of s_tile -> row r of the copy
             for (int i = threadIdx.x; i < 64 * 64 / VEC; i += 256) {
-                const int nn = i / (64 / VEC), c = i % (64 / VEC);
-                const int ch = s_ch[nn];
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (ch >= 0) {
-                    const T* src = W2l + (size_t)ch * D + e0 + c * VEC;
-                    v = *reinterpret_cast<const uint4*>(src);
-                }
-                const T* p8 = reinterpret_cast<const T*>(&v);
+                const int r = i % 64, c = i / 64;
+                uint4 v;
+                T* p8 = reinterpret_cast<T*>(&v);
 #pragma unroll
-                for (int e = 0; e < VEC; ++e) s_tile[nn * PITCH + c * VEC + e] = p8[e];
+                for (int e = 0; e < VEC; ++e) p8[e] = s_tile[(c * VEC + e) * PITCH + r];
+                *reinterpret_cast<uint4*>(dst + (size_t)r * ld + c * VEC) = v;
             }
-            dst = out2 + ((size_t)l * D + e0) * kc_pad + n0;
-            ld = kc_pad;
-        }
-        __syncthreads();
-        // column r of s_tile -> row r of the copy
-        for (int i = threadIdx.x; i < 64 * 64 / VEC; i += 256) {
-            const int r = i % 64, c = i / 64;
-            uint4 v;
-            T* p8 = reinterpret_cast<T*>(&v);
-#pragma unroll
-            for (int e = 0; e < VEC; ++e) p8[e] = s_tile[(c * VEC + e) * PITCH + r];
-            *reinterpret_cast<uint4*>(dst + (size_t)r * ld + c * VEC) = v;
+            return;
         }
         return;
     }
