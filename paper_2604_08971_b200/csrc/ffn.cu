@@ -250,65 +250,52 @@ ffn_prepare_kernel(const int32_t* __restrict__ ids, const uint32_t* __restrict__
             // (swizzled, no bank conflicts) so that eight lanes write a row's 128 bytes.  Bound by latency for one list, by L2
             // beyond (26 MB of copies at d_model 768, 1229 channels, seven lists: 24 us with element-wise shared memory and 16-byte
             // stores of 32 different rows, which L2 saw as 100 MB of sectors).
-            __shared__ __align__(16) uint4 s_piece[64 * 8];
+            // A block has the tile of both copies, for the same channels and columns: one set of channel numbers, twice the loads on
+            // the way (19.6 -> 16.5 us there).
+            __shared__ __align__(16) uint4 s_piece[2][64 * 8];
             const int tiles_n = kc_pad / 64, tiles_e = D / 64;
             const size_t per_list = (size_t)tiles_n * tiles_e;
-            const int which = (int)(pb / (per_list * n_lists));
-            pb -= (size_t)which * per_list * n_lists;
             const int l = (int)(pb / per_list);
             const int tn = (int)((pb % per_list) / tiles_e), te = (int)(pb % tiles_e);
-            const int n0 = tn * 64, e0 = te * 64, tid = threadIdx.x;
+            const int n0 = tn * 64, e0 = te * 64, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
             auto channel = [&](int n) {
                 if (n >= k_c) return -1;
                 const int ch = kept[(size_t)l * k_c + n];
                 if (ch >= 0 && ch < F) return ch;
-                if (which == 0 && te == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+                if (te == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
                 return -1;
             };
-            T* dst;
-            size_t ld;
-            int swz;      // pieces of row r sit at c ^ ((r >> swz) & 7)
-            if (which == 0) {
-                // thread: channel tid & 63, columns 16 (tid >> 6) ..
-                const int n = tid & 63, c0 = 2 * (tid >> 6);
-                const int ch = channel(n0 + n);
-                const uint16_t* src = reinterpret_cast<const uint16_t*>(W1 + (size_t)l * w_stride) + (size_t)(e0 + 8 * c0) * F + ch;
-                uint32_t v[16];
+            // W1: thread = channel tid & 63, columns 16 (tid >> 6) ..;  W2: warp = channels 8 wid .., lane = columns 2 lane, 2 lane + 1
+            const int n = tid & 63, c0 = 2 * (tid >> 6);
+            const int ch1 = channel(n0 + n), mine = lane < 8 ? channel(n0 + 8 * wid + lane) : -1;
+            const uint16_t* src1 = reinterpret_cast<const uint16_t*>(W1 + (size_t)l * w_stride) + (size_t)(e0 + 8 * c0) * F + ch1;
+            uint32_t v[16], w[8];
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = ch >= 0 ? src[(size_t)i * F] : 0u;
+            for (int i = 0; i < 16; ++i) v[i] = ch1 >= 0 ? src1[(size_t)i * F] : 0u;
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    s_piece[n * 8 + ((c0 + h) ^ (n & 7))] = make_uint4(v[8 * h] | v[8 * h + 1] << 16, v[8 * h + 2] | v[8 * h + 3] << 16,
-                                                                       v[8 * h + 4] | v[8 * h + 5] << 16, v[8 * h + 6] | v[8 * h + 7] << 16);
-                dst = out1 + ((size_t)l * kc_pad + n0) * D + e0;
-                ld = D;
-                swz = 0;
-            } else {
-                // warp: channels 8 wid .., lane: columns 2 lane, 2 lane + 1
-                const int lane = tid & 31, wid = tid >> 5;
-                const int mine = lane < 8 ? channel(n0 + 8 * wid + lane) : -1;
-                uint32_t v[8];
+            for (int i = 0; i < 8; ++i) {
+                const int ch = __shfl_sync(0xffffffffu, mine, i);
+                w[i] = ch >= 0 ? *reinterpret_cast<const uint32_t*>(W2 + (size_t)l * w_stride + (size_t)ch * D + e0 + 2 * lane) : 0u;
+            }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int ch = __shfl_sync(0xffffffffu, mine, i);
-                    v[i] = ch >= 0 ? *reinterpret_cast<const uint32_t*>(W2 + (size_t)l * w_stride + (size_t)ch * D + e0 + 2 * lane) : 0u;
-                }
+            for (int h = 0; h < 2; ++h)
+                s_piece[0][n * 8 + ((c0 + h) ^ (n & 7))] = make_uint4(v[8 * h] | v[8 * h + 1] << 16, v[8 * h + 2] | v[8 * h + 3] << 16,
+                                                                      v[8 * h + 4] | v[8 * h + 5] << 16, v[8 * h + 6] | v[8 * h + 7] << 16);
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t sel = h == 0 ? 0x5410u : 0x7632u;
-                    s_piece[(2 * lane + h) * 8 + (wid ^ (lane & 7))] =
-                        make_uint4(__byte_perm(v[0], v[1], sel), __byte_perm(v[2], v[3], sel), __byte_perm(v[4], v[5], sel),
-                                   __byte_perm(v[6], v[7], sel));
-                }
-                dst = out2 + ((size_t)l * D + e0) * kc_pad + n0;
-                ld = kc_pad;
-                swz = 1;
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t sel = h == 0 ? 0x5410u : 0x7632u;
+                s_piece[1][(2 * lane + h) * 8 + (wid ^ (lane & 7))] =
+                    make_uint4(__byte_perm(w[0], w[1], sel), __byte_perm(w[2], w[3], sel), __byte_perm(w[4], w[5], sel),
+                               __byte_perm(w[6], w[7], sel));
             }
             __syncthreads();
+            T* dst1 = out1 + ((size_t)l * kc_pad + n0) * D + e0;
+            T* dst2 = out2 + ((size_t)l * D + e0) * kc_pad + n0;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int r = (tid >> 3) + 32 * j, c = tid & 7;
-                *reinterpret_cast<uint4*>(dst + (size_t)r * ld + c * 8) = s_piece[r * 8 + (c ^ ((r >> swz) & 7))];
+                *reinterpret_cast<uint4*>(dst1 + (size_t)r * D + c * 8) = s_piece[0][r * 8 + (c ^ (r & 7))];
+                *reinterpret_cast<uint4*>(dst2 + (size_t)r * kc_pad + c * 8) = s_piece[1][r * 8 + (c ^ ((r >> 1) & 7))];
             }
         }
         if constexpr (sizeof(T) == 1) {   // element by element
@@ -622,6 +609,11 @@ FfnWs carve(const sentry_ffn_desc& d, int kc_pad, void* ws, size_t bytes, bool w
     return w;
 }
 
+// Blocks of the K-major gather: a 64 x 64 tile of both copies each (8-bit: of one).
+size_t k_major_blocks(const sentry_ffn_desc& d, int kc_pad) {
+    return (d.dtype == SENTRY_FP8_E4M3 ? 2 : 1) * (size_t)d.n_lists * (kc_pad / 64) * (d.D / 64);
+}
+
 int kc_pad_for(const sentry_ffn_desc& d) {
     if (ffn_tc_supported(d)) return ffn_tc_kc_pad(d.D, d.k_c);
     if (ffn_wide_supported(d)) return ffn_wide_kc_pad(d.k_c);
@@ -654,8 +646,7 @@ int launch_ffn_prepack(sentry_ctx* ctx, const FfnArgs& a, void* packed, cudaStre
     const bool tc = k_major(d);
     const int kc_pad = kc_pad_for(d);
     const size_t per = (size_t)kc_pad * d.D;
-    const size_t pack_blocks = tc ? 2 * (size_t)d.n_lists * (kc_pad / 64) * (d.D / 64)
-                                  : 2 * (size_t)d.n_lists * ((per + 255) / 256);
+    const size_t pack_blocks = tc ? k_major_blocks(d, kc_pad) : 2 * (size_t)d.n_lists * ((per + 255) / 256);
     uint8_t* w1p = (uint8_t*)packed;
     uint8_t* w2p = w1p + packed_half_bytes(d, kc_pad);
     FfnPlan none = {};
@@ -757,8 +748,7 @@ int launch_ffn(sentry_ctx* ctx, const FfnArgs& a, void* ws, size_t ws_bytes, con
         if (!fused && zsplit < 1) zsplit = 1;
         if (zsplit > 32) zsplit = 32;
         const size_t pack_blocks = packed != nullptr ? 0
-                                   : (tc ? 2 * (size_t)d.n_lists * (kc_pad / 64) * (d.D / 64)
-                                         : 2 * (size_t)d.n_lists * ((per + 255) / 256));
+                                   : (tc ? k_major_blocks(d, kc_pad) : 2 * (size_t)d.n_lists * ((per + 255) / 256));
         // the next kernel starts early where it leaves half of the SMs free: one window of 64 tokens 31.7 -> 31.3 us a step; on
         // 64 windows x 1024 tokens, whose FFN has a CTA for every SM, 116 -> 119
         const long long next = tiles_bound(d) * (ffn_wide_supported(d) ? kc_pad / 128 : 1);
