@@ -95,6 +95,15 @@ __device__ __forceinline__ void fma_bf16_pair(float& acc_lo, float& acc_hi, uint
         : "r"(a), "r"(b));
 }
 
+// The first product of a sum: fma onto zero.
+__device__ __forceinline__ void mul_bf16_pair(float& lo, float& hi, uint32_t a, uint32_t b) {
+    asm("{\n\t.reg .b16 al, ah, bl, bh;\n\t"
+        "mov.b32 {al, ah}, %2;\n\tmov.b32 {bl, bh}, %3;\n\t"
+        "fma.rn.f32." ATT_PTX_TYPE " %0, al, bl, 0f00000000;\n\tfma.rn.f32." ATT_PTX_TYPE " %1, ah, bh, 0f00000000;\n\t}"
+        : "=f"(lo), "=f"(hi)
+        : "r"(a), "r"(b));
+}
+
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32." ATT_PTX_TYPE "." ATT_PTX_TYPE ".f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
