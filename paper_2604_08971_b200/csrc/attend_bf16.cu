@@ -398,29 +398,34 @@ attend_core_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16
                 }
             }
             // online softmax over this tile (rows gq and gq+8), base-2 exponent
+            if (key0 + kKeyTile > Tv) {   // the last, partial tile: keys past the end drop out
+#pragma unroll
+                for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (key0 + nt * 8 + tq * 2 + (e & 1) >= Tv) s[nt][e] = -INFINITY;
+            }
             float mt[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int key = key0 + nt * 8 + tq * 2 + (e & 1);
-                    s[nt][e] = key < Tv ? s[nt][e] * sl2 : -INFINITY;
-                    mt[e >> 1] = fmaxf(mt[e >> 1], s[nt][e]);
-                }
-            float corr[2];
+            for (int nt = 0; nt < 8; ++nt) {
+                mt[0] = max3(mt[0], s[nt][0], s[nt][1]);
+                mt[1] = max3(mt[1], s[nt][2], s[nt][3]);
+            }
+            float corr[2], ms[2];
 #pragma unroll
             for (int h2 = 0; h2 < 2; ++h2) {
                 mt[h2] = fmaxf(mt[h2], __shfl_xor_sync(0xffffffffu, mt[h2], 1));
                 mt[h2] = fmaxf(mt[h2], __shfl_xor_sync(0xffffffffu, mt[h2], 2));
                 const float m_new = fmaxf(m_run[j][h2], mt[h2]);
-                corr[h2] = fast_exp2(m_run[j][h2] - m_new);   // 0 on the first tile
+                corr[h2] = fast_exp2((m_run[j][h2] - m_new) * sl2);   // 0 on the first tile
                 m_run[j][h2] = m_new;
+                ms[h2] = m_new * sl2;
                 l_run[j][h2] *= corr[h2];
             }
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) s[nt][e] = fast_exp2(s[nt][e] - m_run[j][e >> 1]);
+                for (int e = 0; e < 4; ++e) s[nt][e] = fast_exp2(fmaf(s[nt][e], sl2, -ms[e >> 1]));
 #pragma unroll
             for (int n = 0; n < NT; ++n) {
                 acc[j][n][0] *= corr[0]; acc[j][n][1] *= corr[0];
@@ -515,7 +520,7 @@ attend_core_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16
 // memory.  The order keys of the scores go to keys_out[h][p].  The query rows stay in
 // registers as packed bf16 (D/2 words per head), so all kept heads of a group fit in one pass
 // and a sampled key row is fetched once per group.
-template <int D, int NH>
+template <int D, int NH, bool TIGHT>
 __device__ __forceinline__ void fused_score_pass(const __nv_bfloat16* __restrict__ Q,
                                                  const size_t* q_base, const uint16_t* s_valid,
                                                  uint32_t ks_addr, int Tv,
@@ -541,9 +546,9 @@ __device__ __forceinline__ void fused_score_pass(const __nv_bfloat16* __restrict
 #pragma unroll
         for (int h = 0; h < NH; ++h) { mx[h] = -INFINITY; sum[h] = 0.f; }
         // The sampled positions are requested four ahead: a thread walks its own table row, and with most of the L1 given to
-        // shared memory the row's lines do not survive from one use to the next.  Four keys a round without a branch among
-        // them, the rest after the loop: with a test of position and count per key a round of 512 queries took 595 cycles a
-        // key for two heads (774 for three, 1086 for four) on a table without bank conflicts, now 520 (690, 880).
+        // shared memory the row's lines do not survive from one use to the next.  The keys of a round come without a branch among
+        // them: with a test of position and count per key a round of 512 queries took 595 cycles a key for two heads (774 for
+        // three, 1086 for four) on a table without bank conflicts, now 520 (690, 880).
         // query-major table: entry a of row p at p * n_s + a; entry-major (score_mode 2): a * Tv + p
         const bool all = score_mode == 1;      // every key in turn
         const int es = score_mode == 2 ? Tv : 1;
@@ -580,22 +585,37 @@ __device__ __forceinline__ void fused_score_pass(const __nv_bfloat16* __restrict
         int nxt[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) nxt[u] = all ? u : __ldg(row + min(u, cnt - 1) * es);
-        int a0 = 0;
+        if constexpr (TIGHT) {
 #pragma unroll 1
-        for (; a0 + 4 <= cnt; a0 += 4) {
-            int cur[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int an = a0 + 4 + u;
-                cur[u] = nxt[u];
-                if (an < cnt) nxt[u] = all ? an : __ldg(row + an * es);
+            for (int a0 = 0; a0 < cnt; a0 += 2) {
+                const int k0 = nxt[0], k1 = nxt[1], an = a0 + 4;
+                nxt[0] = nxt[2];
+                nxt[1] = nxt[3];
+                if (an < cnt) nxt[2] = all ? an : __ldg(row + an * es);
+                if (an + 1 < cnt) nxt[3] = all ? an + 1 : __ldg(row + (an + 1) * es);
+                one_key(k0);
+                if (a0 + 1 < cnt) one_key(k1);
             }
+        } else {
+            int a0 = 0;
+#pragma unroll 1
+            for (; a0 + 4 <= cnt; a0 += 4) {
+                int cur[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) one_key(cur[u]);
+                for (int u = 0; u < 4; ++u) {
+                    const int an = a0 + 4 + u;
+                    cur[u] = nxt[u];
+                    if (an < cnt) nxt[u] = all ? an : __ldg(row + an * es);
+                }
+#pragma unroll 1
+                for (int u = 0; u < 4; u += 2) {
+                    one_key(u ? cur[2] : cur[0]);
+                    one_key(u ? cur[3] : cur[1]);
+                }
+            }
+#pragma unroll 1
+            for (int u = 0; a0 + u < cnt; ++u) one_key(u == 0 ? nxt[0] : (u == 1 ? nxt[1] : nxt[2]));
         }
-#pragma unroll
-        for (int u = 0; u < 3; ++u)
-            if (a0 + u < cnt) one_key(nxt[u]);
         if (bad) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
 #pragma unroll
         for (int h = 0; h < NH; ++h) keys_out[h][p] = sentry_order_key(mx[h] - sum[h] * inv_cnt);
@@ -604,7 +624,13 @@ __device__ __forceinline__ void fused_score_pass(const __nv_bfloat16* __restrict
 
 // grid B*Hk, 256 or 512 threads.  Dynamic smem: valid[T] u16 | kind[T] u8 | actbits[4][T/32] u32 |
 // keys[4][T] u32 | hist[4][256] | K[Tpad][D] | V[Tpad][D]   (Tpad = T rounded up to 64).
-template <int D>
+// TIGHT (128-thread CTAs, four to an SM, T <= kSmallT): CTAs of an SM are in different phases, and the instructions of all phases
+// together are what an SM's instruction cache has to hold.  The score loop is then a body of two keys, and loops that are not hot
+// are not unrolled: attention of 4096 x 256 tokens took 560 us with bodies of four keys and three for the rest, 456 with two and
+// one, 427 with two alone, 422 with the other loops rolled.  Larger CTAs do not gain by the last steps (256 x 1024: 124 us with
+// bodies of two and one, 128 with TIGHT).  FOUR false: four heads of d = 32 go in two passes, and the other bodies keep more
+// registers: 408 us; a single wave of CTAs, which waits for the slowest, takes the one pass (256 x 192 tokens 31 us, 37 with two).
+template <int D, bool TIGHT, bool FOUR>
 __global__ void __launch_bounds__(512, 1)
 attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K,
                          const __nv_bfloat16* __restrict__ V, const int32_t* __restrict__ kept_heads,
@@ -624,7 +650,8 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
     __shared__ int red[66];
     __shared__ int32_t s_kept[64];
     __shared__ int32_t s_act[kMaxRK][kMaxActive];
-    __shared__ float s_vpart[512 / (D / 2)][D];
+    __shared__ float s_vpart[512 / (D / 2)][D];            // (until the column sums of V: scratch of the selection)
+    static_assert(kSelectScratch <= 512 / (D / 2) * D, "scratch of the selection");
     __shared__ __align__(16) __nv_bfloat16 s_mean[D];
 
     const int words = (Tlen + 31) / 32;
@@ -642,6 +669,9 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
     // heaviest first (every CTA finds the sample of its rank by itself with a counting sort on
     // the number of present modalities), so that the long ones do not end up alone in the tail
     // of the launch.
+    int id[4];
+    prefetch_ids(ids, Tlen, id);
+    uint32_t mask = masks[blockIdx.x / Hk];   // (of the sample in natural order)
     __shared__ int s_fill_next;
     if (threadIdx.x == 0) s_fill_next = 0;
     int b = blockIdx.x / Hk;
@@ -655,6 +685,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
         if (threadIdx.x < 33) s_cls[threadIdx.x] = 0;
         __syncthreads();
         // samples per class (number of present modalities): one shared-memory atomic per warp and class
+#pragma unroll (TIGHT ? 1 : 4)
         for (int b0 = 0; b0 < Bn; b0 += blockDim.x) {
             const int bb = b0 + threadIdx.x;
             const int c = bb < Bn ? __popc(masks[bb]) : -1;
@@ -680,6 +711,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
             cls = hit ? 32 - src : 0;
             need = hit ? b - above_src : b - incl_src;   // the need-th sample of that class, in index order
         }
+#pragma unroll (TIGHT ? 1 : 4)
         for (int b0 = 0; b0 < Bn; b0 += blockDim.x) {
             const int bb = b0 + threadIdx.x;
             const bool hit = bb < Bn && __popc(masks[bb]) == cls;
@@ -694,26 +726,37 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
             need -= tot;
         }
         b = s_pick[0];
+        mask = masks[b];
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    const uint32_t mask = masks[b];
-    const int Tv = block_build_valid(ids, Tlen, mask, s_valid, red);
+    int kept0 = gate_scores == nullptr && lane < k_h ? kept_heads[(size_t)b * k_h + lane] : 0;
+    // SentryGate's head selection for this sample's mask, done here instead of by a launch of its own: the k_h best of the
+    // Hq <= 64 scores of row `mask` (score descending, equal scores -> lower index, NaN below every number), ascending.  Every
+    // CTA of the sample computes the same list, its first warp while the token list is made; the CTA of group 0 leaves it in
+    // kept_out.
+    float g0 = 0.f, g1 = 0.f;
+    if (gate_scores != nullptr && warp == 0) {
+        uint32_t row = mask;
+        if (row >= (uint32_t)gate_S) { if (lane == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX); row = 0; }
+        const float* sr = gate_scores + (size_t)row * Hq;
+        if (lane < Hq) g0 = sr[lane];
+        if (lane + 32 < Hq) g1 = sr[lane + 32];
+    }
+    const int Tv = block_list_present(ids, Tlen, mask, id, s_valid, s_kind, red);
     const int32_t* kept_row = kept_heads + (size_t)b * k_h;
     if (gate_scores != nullptr) {
-        // SentryGate's head selection for this sample's mask, done here instead of by a launch of
-        // its own: the k_h best of the Hq <= 64 scores of row `mask` (score descending, equal
-        // scores -> lower index, NaN below every number), ascending.  Every CTA of the sample
-        // computes the same list; the CTA of group 0 leaves it in kept_out.
         if (warp == 0) {
-            uint32_t row = mask;
-            if (row >= (uint32_t)gate_S) { if (lane == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX); row = 0; }
-            const float* sr = gate_scores + (size_t)row * Hq;
-            const uint32_t k0 = lane < Hq ? sentry_order_key(sr[lane]) : 0u;
-            const uint32_t k1 = lane + 32 < Hq ? sentry_order_key(sr[lane + 32]) : 0u;
+            const uint32_t k0 = lane < Hq ? sentry_order_key(g0) : 0u;
+            const uint32_t k1 = lane + 32 < Hq ? sentry_order_key(g1) : 0u;
             int r0 = 0, r1 = 0;
-            for (int j = 0; j < Hq; ++j) {
-                const uint32_t kj = __shfl_sync(0xffffffffu, j < 32 ? k0 : k1, j & 31);
+            for (int j = 0; j < min(Hq, 32); ++j) {
+                const uint32_t kj = __shfl_sync(0xffffffffu, k0, j);
                 r0 += (kj > k0 || (kj == k0 && j < lane)) ? 1 : 0;
+                r1 += kj >= k1 ? 1 : 0;
+            }
+            for (int j = 32; j < Hq; ++j) {
+                const uint32_t kj = __shfl_sync(0xffffffffu, k1, j - 32);
+                r0 += kj > k0 ? 1 : 0;
                 r1 += (kj > k1 || (kj == k1 && j < lane + 32)) ? 1 : 0;
             }
             const bool keep0 = lane < Hq && r0 < k_h, keep1 = lane + 32 < Hq && r1 < k_h;
@@ -725,13 +768,15 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
         __syncthreads();
         if (g == 0 && kept_out != nullptr && (int)threadIdx.x < k_h) kept_out[(size_t)b * k_h + threadIdx.x] = s_kept[threadIdx.x];
         kept_row = s_kept;
+        kept0 = lane < k_h ? s_kept[lane] : 0;
     }
-    int hs[kMaxRK], khs[kMaxRK];
+    __shared__ int hs[kMaxRK], khs[kMaxRK];
     bool bad;
-    const int rk = group_heads(kept_row, k_h, Hq / Hk, g, Hq, hs, khs, bad);
+    const int rk = warp_heads(kept0, kept_row, k_h, Hq / Hk, g, Hq, hs, khs, bad);
     if (bad && threadIdx.x == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
     if (rk == 0) return;
     if (Tv == 0) {  // no modality present: zero rows, flag
+        __syncthreads();
         for (int hh = 0; hh < rk; ++hh) {
             uint4* dst = reinterpret_cast<uint4*>(O + ((size_t)b * k_h + khs[hh]) * Tlen * D);
             for (int i = threadIdx.x; i < Tlen * S::CPR; i += blockDim.x) dst[i] = make_uint4(0, 0, 0, 0);
@@ -749,12 +794,14 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
     const __nv_bfloat16* Vg = V + ((size_t)b * Hk + g) * Tlen * D;
     const int n_kt = (Tv + kKeyTile - 1) / kKeyTile;
     const int rows_staged = n_kt * kKeyTile;
+#pragma unroll (TIGHT ? 2 : 4)
     for (int i = threadIdx.x; i < rows_staged * S::CPR; i += blockDim.x) {
         const int row = i / S::CPR, cc = i % S::CPR;
         if (row < Tv) ptx::cp_async_16(ks_addr + S::off(row, cc), Kg + (size_t)s_valid[row] * D + cc * 8);
         else asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(ks_addr + S::off(row, cc)), "r"(0) : "memory");
     }
     ptx::cp_async_commit();
+#pragma unroll (TIGHT ? 2 : 4)
     for (int i = threadIdx.x; i < rows_staged * S::CPR; i += blockDim.x) {
         const int row = i / S::CPR, cc = i % S::CPR;
         if (row < Tv) ptx::cp_async_16(vs_addr + S::off(row, cc), Vg + (size_t)s_valid[row] * D + cc * 8);
@@ -762,11 +809,10 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
     }
     ptx::cp_async_commit();
 
-    for (int t = threadIdx.x; t < Tlen; t += blockDim.x) s_kind[t] = 0;
+#pragma unroll (TIGHT ? 1 : 4)
     for (int i = threadIdx.x; i < kMaxRK * words; i += blockDim.x) s_abits[i] = 0u;
+#pragma unroll (TIGHT ? 1 : 4)
     for (int i = threadIdx.x; i < kMaxRK * kMaxActive; i += blockDim.x) (&s_act[0][0])[i] = -1;
-    __syncthreads();
-    for (int p = threadIdx.x; p < Tv; p += blockDim.x) s_kind[s_valid[p]] = 1;
 
     if (active_in == nullptr) {
         // ---- sparsity scores (Section 4.4) from the resident K rows
@@ -782,8 +828,9 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
         __syncthreads();
         if (table_ok) {
             constexpr int HPP = (D == 64) ? 2 : 4;   // heads per pass: packed q rows live in registers
-            for (int h0 = 0; h0 < rk; h0 += HPP) {
-                const int nh = min(HPP, rk - h0);
+            const int step = !FOUR && HPP == 4 && rk == 4 ? 2 : HPP;
+            for (int h0 = 0; h0 < rk; h0 += step) {
+                const int nh = min(step, rk - h0);
                 size_t q_base[4];
                 uint32_t* keys_out[4];
                 for (int j = 0; j < 4; ++j) {
@@ -791,31 +838,35 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
                     q_base[j] = ((size_t)b * Hq + hs[hh]) * Tlen * D;
                     keys_out[j] = s_keys + (size_t)hh * Tlen;
                 }
-                if (nh == 1) fused_score_pass<D, 1>(Q, q_base, s_valid, ks_addr, Tv, tbl, n_s, cnt, score_mode, keys_out, status);
-                else if (nh == 2) fused_score_pass<D, 2>(Q, q_base, s_valid, ks_addr, Tv, tbl, n_s, cnt, score_mode, keys_out, status);
+                if (nh == 1) fused_score_pass<D, 1, TIGHT>(Q, q_base, s_valid, ks_addr, Tv, tbl, n_s, cnt, score_mode, keys_out, status);
+                else if (nh == 2) fused_score_pass<D, 2, TIGHT>(Q, q_base, s_valid, ks_addr, Tv, tbl, n_s, cnt, score_mode, keys_out, status);
                 else if constexpr (HPP == 4) {
-                    if (nh == 3) fused_score_pass<D, 3>(Q, q_base, s_valid, ks_addr, Tv, tbl, n_s, cnt, score_mode, keys_out, status);
-                    else fused_score_pass<D, 4>(Q, q_base, s_valid, ks_addr, Tv, tbl, n_s, cnt, score_mode, keys_out, status);
+                    if (nh == 3) fused_score_pass<D, 3, TIGHT>(Q, q_base, s_valid, ks_addr, Tv, tbl, n_s, cnt, score_mode, keys_out, status);
+                    else if constexpr (FOUR) fused_score_pass<D, 4, TIGHT>(Q, q_base, s_valid, ks_addr, Tv, tbl, n_s, cnt, score_mode, keys_out, status);
                 }
             }
         } else {
             if (threadIdx.x == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+#pragma unroll (TIGHT ? 1 : 4)
             for (int i = threadIdx.x; i < rk * Tlen; i += blockDim.x) s_keys[i] = 0u;
         }
         __syncthreads();
         // ---- the U present queries with the largest score are active
-        // short lists: one warp per head with the keys in registers; longer ones: digit counting
-        // by the whole block (measured: the warp form wins up to 256 keys, loses from 1024 on)
-        if (Tv <= 256) warps_select_topk_heads(s_keys, Tlen, Tv, U, rk, s_act, s_valid);
-        else block_select_topk_heads(s_keys, Tlen, Tv, U, rk, s_act, s_valid, s_hist);
+        // short lists: one warp per head with the keys in registers; longer ones: digit counting by the whole block (which on
+        // short ones is the slower way: 35.8 us for 31.1 on 256 x 192 tokens)
+        static_assert(!TIGHT || kSmallT <= 256, "the selection of 128-thread CTAs");
+        if (TIGHT || Tv <= 256) warps_select_topk_heads(s_keys, Tlen, Tv, U, rk, s_act, s_valid);
+        else block_select_topk_heads(s_keys, Tlen, Tv, U, rk, s_act, s_valid, s_hist, reinterpret_cast<int*>(&s_vpart[0][0]));
         __syncthreads();
         if (active_out != nullptr)
+#pragma unroll (TIGHT ? 1 : 4)
             for (int i = threadIdx.x; i < rk * U_max; i += blockDim.x) {
                 const int hh = i / U_max, a = i % U_max;
                 active_out[((size_t)b * k_h + khs[hh]) * U_max + a] = a < U ? s_act[hh][a] : -1;
             }
     } else {
         __syncthreads();
+#pragma unroll (TIGHT ? 1 : 4)
         for (int i = threadIdx.x; i < rk * kMaxActive; i += blockDim.x) {
             const int hh = i / kMaxActive, a = i % kMaxActive;
             int t = a < U_max ? active_in[((size_t)b * k_h + khs[hh]) * U_max + a] : -1;
@@ -824,6 +875,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
         }
         __syncthreads();
     }
+#pragma unroll (TIGHT ? 1 : 4)
     for (int i = threadIdx.x; i < rk * kMaxActive; i += blockDim.x) {
         const int hh = i / kMaxActive, t = s_act[hh][i % kMaxActive];
         if (t >= 0) atomicOr(&s_abits[hh * words + (t >> 5)], 1u << (t & 31));
@@ -837,6 +889,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
         const int vs_dp = threadIdx.x % DP, vs_k0 = threadIdx.x / DP;
         const int stride = blockDim.x / DP;
         float v0 = 0.f, v1 = 0.f;
+#pragma unroll (TIGHT ? 2 : 4)
         for (int row = vs_k0; row < rows_staged; row += stride) {
             uint32_t w;
             asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(vs_addr + S::off(row, vs_dp >> 2) + (vs_dp & 3) * 4));
@@ -848,6 +901,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
         __syncthreads();
         if (threadIdx.x < D) {
             float t = 0.f;
+#pragma unroll (TIGHT ? 1 : 4)
             for (int i = 0; i < stride; ++i) t += s_vpart[i][threadIdx.x];
             reinterpret_cast<unsigned short*>(s_mean)[threadIdx.x] = att_bits(t / (float)Tv);
         }
@@ -874,13 +928,9 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
                 hh = r / Ue;
                 t = s_act[hh][r - hh * Ue];
             }
-            int h_sel = hs[0], kh_sel = khs[0];
-#pragma unroll
-            for (int j = 1; j < kMaxRK; ++j)
-                if (hh == j) { h_sel = hs[j]; kh_sel = khs[j]; }
             row_t[half] = t;
-            row_kh[half] = kh_sel;
-            row_q[half] = Q + ((size_t)b * Hq + h_sel) * Tlen * D;
+            row_kh[half] = khs[hh];
+            row_q[half] = Q + ((size_t)b * Hq + hs[hh]) * Tlen * D;
         }
         uint32_t qf[KS][4];
         float acc[NT][4];
@@ -934,29 +984,34 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
                     mma_bf16_16816(sc[nt], qf[3], bfr[2], bfr[3]);
                 }
             }
+            if (key0 + kKeyTile > Tv) {   // the last, partial tile: keys past the end drop out
+#pragma unroll
+                for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (key0 + nt * 8 + tq * 2 + (e & 1) >= Tv) sc[nt][e] = -INFINITY;
+            }
             float mt[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int key = key0 + nt * 8 + tq * 2 + (e & 1);
-                    sc[nt][e] = key < Tv ? sc[nt][e] * sl2 : -INFINITY;
-                    mt[e >> 1] = fmaxf(mt[e >> 1], sc[nt][e]);
-                }
-            float corr[2];
+            for (int nt = 0; nt < 8; ++nt) {
+                mt[0] = max3(mt[0], sc[nt][0], sc[nt][1]);
+                mt[1] = max3(mt[1], sc[nt][2], sc[nt][3]);
+            }
+            float corr[2], ms[2];
 #pragma unroll
             for (int h2 = 0; h2 < 2; ++h2) {
                 mt[h2] = fmaxf(mt[h2], __shfl_xor_sync(0xffffffffu, mt[h2], 1));
                 mt[h2] = fmaxf(mt[h2], __shfl_xor_sync(0xffffffffu, mt[h2], 2));
                 const float m_new = fmaxf(m_run[h2], mt[h2]);
-                corr[h2] = fast_exp2(m_run[h2] - m_new);   // 0 on the first tile
+                corr[h2] = fast_exp2((m_run[h2] - m_new) * sl2);   // 0 on the first tile
                 m_run[h2] = m_new;
+                ms[h2] = m_new * sl2;
                 l_run[h2] *= corr[h2];
             }
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) sc[nt][e] = fast_exp2(sc[nt][e] - m_run[e >> 1]);
+                for (int e = 0; e < 4; ++e) sc[nt][e] = fast_exp2(fmaf(sc[nt][e], sl2, -ms[e >> 1]));
 #pragma unroll
             for (int n = 0; n < NT; ++n) {
                 acc[n][0] *= corr[0]; acc[n][1] *= corr[0];
@@ -1012,6 +1067,7 @@ attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat1
         for (int hh = 0; hh < rk; ++hh) {
             uint4* dst = reinterpret_cast<uint4*>(O + ((size_t)b * k_h + khs[hh]) * Tlen * D);
             const uint32_t* bits = s_abits + hh * words;
+#pragma unroll (TIGHT ? 1 : 4)
             for (int i = threadIdx.x; i < Tlen * S::CPR; i += blockDim.x) {
                 const int t = i / S::CPR, cc = i % S::CPR;
                 if ((bits[t >> 5] >> (t & 31)) & 1u) continue;
@@ -1055,11 +1111,14 @@ int launch_d(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
     const size_t fused_bytes = fused_smem_bytes<D>(d.T);
     if (fused_bytes <= 200 * 1024) {
         // the group's K and V fit in shared memory: one kernel does everything
-        auto kern = attend_fused_bf16_kernel<D>;
-        SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_bytes));
         // one big CTA, or two per SM; short sequences get small CTAs (more of them per SM: their
         // phases are a few barrier-separated microseconds each, so concurrency is what helps)
         const int threads = fused_bytes > 100 * 1024 ? 512 : (d.T <= kSmallT ? 128 : 256);
+        const long long waves = (long long)d.B * d.Hk / ((long long)ctx->sm_count * (512 / threads));
+        auto kern = threads != 128 ? attend_fused_bf16_kernel<D, false, true>
+                    : (D == 32 && waves >= 4) ? attend_fused_bf16_kernel<D, true, D != 32>
+                                              : attend_fused_bf16_kernel<D, true, true>;
+        SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_bytes));
         // heaviest samples first only where there is more than one wave (128 registers a thread: 512 threads per SM):
         // finding the sample of a rank takes 2900 cycles, of 32000 in a CTA of T = 192
         const int order = d.B > 1 && d.B <= kOrderMaxBatch && (long long)d.B * d.Hk > (long long)ctx->sm_count * (512 / threads);

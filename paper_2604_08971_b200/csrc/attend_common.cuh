@@ -83,6 +83,85 @@ __device__ __forceinline__ int group_heads(const int32_t* kept, int k_h, int r, 
     return rk;
 }
 
+// The same by every warp for itself, a list entry to a lane (kept: shared or global memory; first: entry `lane`, 0 past the
+// end).  The count is returned to all; the
+// block's first warp leaves ids and slots in hs, khs (shared, complete behind the caller's next barrier): held in registers
+// through the score pass they cost it 4 % at four CTAs per SM.
+__device__ __forceinline__ int warp_heads(int first, const int32_t* kept, int k_h, int r, int g, int Hq, int* hs, int* khs,
+                                          bool& bad) {
+    const int lane = threadIdx.x & 31;
+    int rk = 0;
+    bad = false;
+    for (int j0 = 0; j0 < k_h; j0 += 32) {
+        const int h = j0 == 0 ? first : (j0 + lane < k_h ? kept[j0 + lane] : 0);
+        const bool valid = h >= 0 && h < Hq, mine = j0 + lane < k_h && valid && h / r == g;
+        bad |= __any_sync(0xffffffffu, !valid);
+        const unsigned im = __ballot_sync(0xffffffffu, mine);
+        const int at = rk + __popc(im & ((1u << lane) - 1u));
+        if (threadIdx.x < 32 && mine && at < kMaxRK) { hs[at] = h; khs[at] = j0 + lane; }
+        rk += __popc(im);
+    }
+    return min(rk, kMaxRK);
+}
+
+// The first four of a thread's tokens (positions u * blockDim + thread), requested before the sample's mask is known.
+__device__ __forceinline__ void prefetch_ids(const int32_t* __restrict__ ids, int T, int (&id)[4]) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int t = u * blockDim.x + threadIdx.x;
+        id[u] = ids == nullptr ? 0 : (t < T ? __ldg(ids + t) : -1);
+    }
+}
+// Present-token list of a sample, valid[p] = p-th present token, and kind[t] = present: four of a thread's tokens per round of
+// counts (a round per blockDim tokens, with two barriers and a request each, took 6300 cycles of a CTA's 71000 at T = 1024,
+// head selection included).  red: 64 ints; up to 16 warps.  Returns T_v.
+__device__ __forceinline__ int block_list_present(const int32_t* __restrict__ ids, int T, uint32_t mask, int (&id)[4],
+                                                  uint16_t* valid, uint8_t* kind, int* red) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int total = 0;
+    for (int t0 = 0; t0 < T; t0 += 4 * blockDim.x) {
+        if (t0 > 0) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int t = t0 + u * blockDim.x + threadIdx.x;
+                id[u] = ids == nullptr ? 0 : (t < T ? __ldg(ids + t) : -1);
+            }
+            __syncthreads();                         // the counts of the round before have been read
+        }
+        const int rounds = min(4, (T - t0 + (int)blockDim.x - 1) / (int)blockDim.x);
+        unsigned bm[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = t0 + u * blockDim.x + threadIdx.x;
+            const bool ok = t < T && (ids == nullptr || (id[u] >= 0 && id[u] < 32 && ((mask >> id[u]) & 1u)));
+            bm[u] = __ballot_sync(0xffffffffu, ok);
+            if (t < T) kind[t] = ok;
+            if (lane == 0 && u < rounds) red[u * nw + wid] = __popc(bm[u]);
+        }
+        __syncthreads();
+        // counts in token order: entry u * nw + warp; a lane scans entries lane and lane + 32
+        const int n = rounds * nw, c0 = lane < n ? red[lane] : 0, c1 = lane + 32 < n ? red[lane + 32] : 0;
+        int s0 = c0, s1 = c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int a = __shfl_up_sync(0xffffffffu, s0, o), b = __shfl_up_sync(0xffffffffu, s1, o);
+            if (lane >= o) { s0 += a; s1 += b; }
+        }
+        const int half = __shfl_sync(0xffffffffu, s0, 31);
+        const int e0 = total + s0 - c0, e1 = total + half + s1 - c1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = u * nw + wid;
+            const int base = e < 32 ? __shfl_sync(0xffffffffu, e0, e & 31) : __shfl_sync(0xffffffffu, e1, e & 31);
+            if (u < rounds && ((bm[u] >> lane) & 1u))
+                valid[base + __popc(bm[u] & ((1u << lane) - 1u))] = (uint16_t)(t0 + u * blockDim.x + threadIdx.x);
+        }
+        total += half + __shfl_sync(0xffffffffu, s1, 31);
+    }
+    __syncthreads();
+    return total;
+}
+
 // ------------------------------------------------------------------------------------ score
 // acc_lo += a.lo * b.lo, acc_hi += a.hi * b.hi for two bf16 pairs, in fp32: the mixed-precision
 // FMA of sm_100 takes the bf16 operands as they are (exact products, fp32 accumulate), so
@@ -139,6 +218,11 @@ __device__ __forceinline__ void score_one_key(const uint32_t (&qw)[NH][D / 2], u
     }
 }
 
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -282,63 +366,114 @@ __device__ __forceinline__ void warps_select_topk_heads(const uint32_t* keys, in
     const int warp = threadIdx.x >> 5;
     if (warp < rk) warp_select_topk_bits<8>(keys + (size_t)warp * stride, n, k, out[warp], remap);
 }
-// The same selection for the rk <= kMaxRK heads of a group at once, by the whole block: all
-// threads count digits for every head (the long part), warp hh then picks head hh's digit, and
-// at the end compacts head hh's selection.  keys: [rk][stride] order keys, n per head;
-// hist: kMaxRK * 256 ints of shared memory.
+// The same selection for the rk <= kMaxRK heads of a group at once, by the whole block: the threshold by counting digits of
+// eight bits from the first bit in which a head's keys differ, until exactly k keys lie from it on (two counts as a rule; from
+// the top bit, where most keys share a digit and the counters serialise, it took four, and a warp per head then went through
+// all keys to put the selection in order: 10300 cycles of a CTA's 71000 at T = 1024, now 8000).  What lies from the threshold on is
+// collected and put in order by rank; where keys tie at the threshold and not all of them are taken, a warp goes through the
+// head's keys.  keys: [rk][stride] order keys, n per head; shared memory: hist kMaxRK * 256 ints, scratch kSelectScratch.
+constexpr int kSelectScratch = 2 * kMaxRK * 32 + kMaxRK * kMaxActive + 5 * kMaxRK;
 __device__ inline void block_select_topk_heads(const uint32_t* keys, int stride, int n, int k, int rk,
-                                               int32_t (*out)[kMaxActive], const uint16_t* remap, int* hist) {
-    __shared__ uint32_t s_sel[2 * kMaxRK];   // per head: fixed key prefix, entries still wanted
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x < rk) { s_sel[2 * threadIdx.x] = 0u; s_sel[2 * threadIdx.x + 1] = (uint32_t)k; }
-    uint32_t fixed = 0;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int i = threadIdx.x; i < rk * 256; i += blockDim.x) hist[i] = 0;
-        __syncthreads();
+                                               int32_t (*out)[kMaxActive], const uint16_t* remap, int* hist, int* scratch) {
+    uint32_t (*s_mm)[kMaxRK][32] = reinterpret_cast<uint32_t (*)[kMaxRK][32]>(scratch);   // [2] per warp: largest and smallest key
+    int (*s_list)[kMaxActive] = reinterpret_cast<int (*)[kMaxActive]>(scratch + 2 * kMaxRK * 32);
+    int* s_state = scratch + 2 * kMaxRK * 32 + kMaxRK * kMaxActive;
+    uint32_t* s_prefix = reinterpret_cast<uint32_t*>(s_state);        // threshold: the bits that are known
+    int *s_nb = s_state + kMaxRK, *s_want = s_nb + kMaxRK;            // bits that are not, keys still wanted among them
+    int *s_done = s_want + kMaxRK, *s_n = s_done + kMaxRK;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i = threadIdx.x; i < rk * 256; i += blockDim.x) hist[i] = 0;
+    for (int hh = 0; hh < rk; ++hh) {
+        uint32_t hi = 0u, lo = 0xffffffffu;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            const uint32_t key = keys[(size_t)hh * stride + i];
+            hi = max(hi, key);
+            lo = min(lo, key);
+        }
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        if (lane == 0) { s_mm[0][hh][warp] = hi; s_mm[1][hh][warp] = lo; }
+    }
+    __syncthreads();
+    if (warp < rk) {
+        const uint32_t hi = __reduce_max_sync(0xffffffffu, lane < nw ? s_mm[0][warp][lane] : 0u);
+        const uint32_t lo = __reduce_min_sync(0xffffffffu, lane < nw ? s_mm[1][warp][lane] : 0xffffffffu);
+        if (lane == 0) {
+            const int nb = hi != lo ? 32 - __clz((int)(hi ^ lo)) : 0;
+            s_prefix[warp] = n == k || nb == 32 ? 0u : hi >> nb << nb;
+            s_nb[warp] = nb;
+            s_want[warp] = k;
+            s_n[warp] = 0;
+            s_done[warp] = n == k ? 1 : (nb == 0 ? 2 : 0);   // 1: all keys from the threshold on, 2: ties at it are split
+        }
+    }
+    __syncthreads();
+    for (;;) {
+        bool more = false;
         for (int hh = 0; hh < rk; ++hh) {
-            const uint32_t prefix = s_sel[2 * hh];
-            const uint32_t* kh = keys + (size_t)hh * stride;
-            int* hh_hist = hist + hh * 256;
+            if (s_done[hh]) continue;
+            more = true;
+            const uint32_t prefix = s_prefix[hh];
+            const int nb = s_nb[hh], shift = max(nb - 8, 0);
+            const uint32_t known = nb == 32 ? 0u : ~0u << nb, digit = (1u << (nb - shift)) - 1u;
             for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const uint32_t key = kh[i];
-                if ((key & fixed) == prefix) atomicAdd(&hh_hist[(key >> shift) & 255u], 1);
+                const uint32_t key = keys[(size_t)hh * stride + i];
+                if ((key & known) == prefix) atomicAdd(&hist[hh * 256 + ((key >> shift) & digit)], 1);
             }
         }
+        if (!more) break;
         __syncthreads();
-        if (warp < rk) {
-            const int* h = hist + warp * 256;
-            const int want = (int)s_sel[2 * warp + 1];
+        if (warp < rk && !s_done[warp]) {
+            int* h = hist + warp * 256;
+            const int want = s_want[warp], shift = max(s_nb[warp] - 8, 0);
             const int top = 255 - 8 * lane;      // this lane's digits, descending
-            int mine = 0;
+            int c[8], mine = 0;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) mine += h[top - j];
+            for (int j = 0; j < 8; ++j) { c[j] = h[top - j]; mine += c[j]; }
             int incl = mine;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int v = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += v;
             }
-            const int above = incl - mine;
-            if (above < want && want <= incl) {   // exactly one lane
-                int acc = above;
+            int acc = incl - mine;
+            if (acc < want && want <= incl) {    // exactly one lane
+                int at = 0, cnt = 0;
+                bool found = false;
+#pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const int cdig = h[top - j];
-                    if (want <= acc + cdig) {
-                        s_sel[2 * warp] |= (uint32_t)(top - j) << shift;
-                        s_sel[2 * warp + 1] = (uint32_t)(want - acc);
-                        break;
-                    }
-                    acc += cdig;
+                    if (!found && want <= acc + c[j]) { found = true; at = j; cnt = c[j]; }
+                    if (!found) acc += c[j];
                 }
+                s_prefix[warp] |= (uint32_t)(top - at) << shift;
+                s_nb[warp] = shift;
+                s_want[warp] = want - acc;
+                s_done[warp] = cnt == want - acc ? 1 : (shift == 0 ? 2 : 0);
             }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) h[top - j] = 0;
         }
-        fixed |= 255u << shift;
         __syncthreads();
     }
-    if (warp < rk) {
+    for (int hh = 0; hh < rk; ++hh) {
+        if (s_done[hh] != 1) continue;
+        const uint32_t t = s_prefix[hh];
+        for (int i = threadIdx.x; i < n; i += blockDim.x)
+            if (keys[(size_t)hh * stride + i] >= t) s_list[hh][atomicAdd(&s_n[hh], 1)] = i;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < rk * 64; e += blockDim.x) {
+        const int hh = e >> 6, a = e & 63;
+        if (a >= k || s_done[hh] != 1) continue;
+        const int mine = s_list[hh][a];
+        int pos = 0;
+        for (int b = 0; b < k; ++b) pos += s_list[hh][b] < mine ? 1 : 0;
+        out[hh][pos] = (int32_t)remap[mine];
+    }
+    if (warp < rk && s_done[warp] == 2) {
         const uint32_t* kh = keys + (size_t)warp * stride;
-        const uint32_t t = s_sel[2 * warp];
-        const int need_eq = (int)s_sel[2 * warp + 1];
+        const uint32_t t = s_prefix[warp];
+        const int need_eq = s_want[warp];
         int base = 0, eq_seen = 0;
         for (int i0 = 0; i0 < n; i0 += 32) {
             const int i = i0 + lane;

@@ -179,8 +179,9 @@ attend_long_select_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat
     }
     __syncthreads();
     // ---- the U present queries with the largest score are active (ties -> lower index)
+    __shared__ int s_sel[kSelectScratch];
     if (Tv <= 256) warps_select_topk_heads(s_keys, Tv, Tv, U, rk, s_act, s_valid);
-    else block_select_topk_heads(s_keys, Tv, Tv, U, rk, s_act, s_valid, s_hist);
+    else block_select_topk_heads(s_keys, Tv, Tv, U, rk, s_act, s_valid, s_hist, s_sel);
     __syncthreads();
     for (int i = threadIdx.x; i < rk * U_max; i += blockDim.x) {
         const int hh = i / U_max, a = i % U_max;

@@ -27,11 +27,6 @@ constexpr int kRowTiles = kMaxRK * kMaxActive / 16;
 constexpr int kMaxParts = 16;                     // parts of the keys in the rows launch
 
 // ------------------------------------------------------------------------------------------ pieces
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
 // The D/8 words of a row that lane quarter tq holds as an MMA operand, straight from global memory: the K index of the
 // MMA is permuted so that they are contiguous (d = 16: 8 bytes, 32: 16 bytes, 64: pieces tq and tq + 4 of 16 bytes); key and
 // query fragments use the same order.

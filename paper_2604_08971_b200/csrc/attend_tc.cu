@@ -86,11 +86,6 @@ struct AttSmem {
 __device__ __forceinline__ void bar_sync_group(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
-__device__ __forceinline__ float max3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
 // valid-key bits of the 32 keys starting at r0 (keys are the present tokens 0 .. Tv-1)
 __device__ __forceinline__ uint32_t key_bits(int r0, int Tv) {
     return r0 + 32 <= Tv ? 0xffffffffu : (r0 < Tv ? (1u << (Tv - r0)) - 1u : 0u);
@@ -443,8 +438,9 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap tm_k64, const __grid_consta
     if (ok && active_in == nullptr) {
         // ---- the U present queries with the largest score are active
         int* s_hist = reinterpret_cast<int*>(scratch);
+        __shared__ int s_sel[kSelectScratch];
         if (Tv <= 256) warps_select_topk_heads(s_keys, Tlen, Tv, U, rk, s_act, s_valid);
-        else block_select_topk_heads(s_keys, Tlen, Tv, U, rk, s_act, s_valid, s_hist);
+        else block_select_topk_heads(s_keys, Tlen, Tv, U, rk, s_act, s_valid, s_hist, s_sel);
         __syncthreads();
         if (active_out != nullptr)
             for (int i = threadIdx.x; i < rk * U_max; i += blockDim.x) {
