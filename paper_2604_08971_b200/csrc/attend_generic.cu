@@ -60,12 +60,14 @@ attend_score_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     grid_dependents_start_if_small();
     grid_dependency_wait();
     const int bh = blockIdx.x, b = bh / k_h;
+    // (what does not depend on the token list is requested before it is made: each is a round trip of the chain)
     const uint32_t mask = masks[b];
+    const int h = kept_heads[bh];
+    const int64_t offset = score_mode != 1 && mask < (uint32_t)n_subsets ? offsets[mask] : -1;
     const int Tv = block_build_valid(ids, Tlen, mask, s_valid, red);
     if (Tv == 0) return;
     const int p = blockIdx.y * blockDim.x + threadIdx.x;
     if (blockIdx.y * blockDim.x >= Tv) return;
-    const int h = kept_heads[bh];
     if (h < 0 || h >= Hq) {
         if (threadIdx.x == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
         return;
@@ -74,11 +76,11 @@ attend_score_kernel(const T* __restrict__ Q, const T* __restrict__ K,
     const int n_s = sentry_num_active(Tv, c);
     const int32_t* tbl = nullptr;
     if (score_mode != 1) {
-        if (mask >= (uint32_t)n_subsets || offsets[mask] < 0) {
+        if (offset < 0) {
             if (threadIdx.x == 0) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
             return;
         }
-        tbl = table + offsets[mask];
+        tbl = table + offset;
     }
     if (p >= Tv) return;
     const T* Qh = Q + ((size_t)b * Hq + h) * Tlen * D;
@@ -135,6 +137,8 @@ attend_select_kernel(const float* __restrict__ mscore, const int32_t* __restrict
     grid_dependents_start_if_small();
     grid_dependency_wait();
     const int bh = blockIdx.x, b = bh / k_h;
+    const int p0 = threadIdx.x;
+    const float m0 = p0 < Tlen ? mscore[(size_t)bh * Tlen + p0] : 0.f;   // requested before T_v is known
     const int Tv = block_build_valid(ids, Tlen, masks[b], s_valid, red);
     int32_t* out = active + (size_t)bh * U_max;
     const int U = sentry_num_active(Tv, c);
@@ -144,7 +148,7 @@ attend_select_kernel(const float* __restrict__ mscore, const int32_t* __restrict
         return;
     }
     for (int p = threadIdx.x; p < Tv; p += blockDim.x)
-        s_keys[p] = sentry_order_key(mscore[(size_t)bh * Tlen + p]);
+        s_keys[p] = sentry_order_key(p == p0 ? m0 : mscore[(size_t)bh * Tlen + p]);
     __syncthreads();
     block_select_topk(s_keys, Tv, U, out, s_valid, red);
 }
@@ -169,9 +173,9 @@ attend_core_kernel(const T* __restrict__ Q, const T* __restrict__ K, const T* __
     grid_dependency_wait();
     const int bh = blockIdx.x, b = bh / k_h, part = blockIdx.y, parts = gridDim.y;
     const int t_begin = (int)((long long)Tlen * part / parts), t_end = (int)((long long)Tlen * (part + 1) / parts);
+    const int h = kept_heads[bh];
     const int Tv = block_build_valid(ids, Tlen, masks[b], s_valid, red);
     T* Oh = O + (size_t)bh * Tlen * D;
-    const int h = kept_heads[bh];
     if (Tv == 0 || h < 0 || h >= Hq) {
         for (int i = t_begin * D + threadIdx.x; i < t_end * D; i += blockDim.x) Oh[i] = from_f32<T>(0.f);
         if (threadIdx.x == 0)

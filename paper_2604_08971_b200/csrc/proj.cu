@@ -9,7 +9,7 @@
 namespace {
 
 constexpr int kProjThreads = 256;
-constexpr int kMaxSlices = 96;   // kept heads + 2 x referenced groups
+constexpr int kMaxSlices = 128;  // kept heads (at most 64) + 2 x referenced groups (at most 32)
 
 template <typename T>
 __global__ void __launch_bounds__(kProjThreads)
@@ -23,25 +23,36 @@ project_qkv_kernel(const T* __restrict__ X, const T* __restrict__ WQ, const T* _
     grid_dependents_start_if_small();
     grid_dependency_wait();
     const int b = blockIdx.x / Tlen, t = blockIdx.x % Tlen;
+    // the list entry and the row are requested together with what tells whether the token is there
+    const int lane = threadIdx.x & 31;
+    const int h_mine = threadIdx.x < 32 && lane < k_h ? kept_heads[(size_t)b * k_h + lane] : 0;
+    const T* x = X + ((size_t)b * Tlen + t) * D;
+    const float x_mine = (int)threadIdx.x < D ? to_f32<T>(x[threadIdx.x]) : 0.f;
     const int m = ids[t];
     if (m < 0 || m >= 32 || !((masks[b] >> m) & 1u)) return;       // absent token: nothing is written
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
         // slices: one per kept head (Q), one K and one V per referenced group
         const int r = Hq / Hk;
         int n = 0;
         uint32_t groups = 0;
-        for (int j = 0; j < k_h; ++j) {
-            const int h = kept_heads[(size_t)b * k_h + j];
-            if (h < 0 || h >= Hq) { atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX); continue; }
-            s_kind[n] = 0; s_idx[n] = h; ++n;
-            groups |= 1u << (h / r);
+        for (int j0 = 0; j0 < k_h; j0 += 32) {
+            const int j = j0 + lane, h = j0 == 0 ? h_mine : (j < k_h ? kept_heads[(size_t)b * k_h + j] : 0);
+            const bool valid = h >= 0 && h < Hq, in = j < k_h && valid;
+            if (j < k_h && !valid) atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX);
+            const unsigned im = __ballot_sync(0xffffffffu, in);
+            if (in) { const int at = n + __popc(im & ((1u << lane) - 1u)); s_kind[at] = 0; s_idx[at] = h; }
+            n += __popc(im);
+            groups |= __reduce_or_sync(0xffffffffu, in ? 1u << (h / r) : 0u);
         }
-        for (int g = 0; g < Hk; ++g)
-            if ((groups >> g) & 1u) { s_kind[n] = 1; s_idx[n] = g; ++n; s_kind[n] = 2; s_idx[n] = g; ++n; }
-        s_n = n;
+        const bool in = lane < Hk && ((groups >> lane) & 1u);
+        if (in) {
+            const int at = n + 2 * __popc(groups & ((1u << lane) - 1u));
+            s_kind[at] = 1; s_idx[at] = lane;
+            s_kind[at + 1] = 2; s_idx[at + 1] = lane;
+        }
+        if (lane == 0) s_n = n + 2 * __popc(groups);
     }
-    const T* x = X + ((size_t)b * Tlen + t) * D;
-    for (int e = threadIdx.x; e < D; e += blockDim.x) s_x[e] = to_f32<T>(x[e]);
+    for (int e = threadIdx.x; e < D; e += blockDim.x) s_x[e] = e == (int)threadIdx.x ? x_mine : to_f32<T>(x[e]);
     __syncthreads();
     const int total = s_n * d;
     for (int o = threadIdx.x; o < total; o += blockDim.x) {
@@ -70,6 +81,8 @@ project_out_kernel(const T* __restrict__ A, const T* __restrict__ WO, const int3
     grid_dependency_wait();
     const int b = blockIdx.x / Tlen, t = blockIdx.x % Tlen;
     T* o = out + ((size_t)b * Tlen + t) * D;
+    const int n_a = k_h * d, i_mine = min((int)threadIdx.x, n_a - 1);   // (requested with the mask; of an absent token, not used)
+    const float a_mine = to_f32<T>(A[(((size_t)b * k_h + i_mine / d) * Tlen + t) * d + i_mine % d]);
     const int m = ids[t];
     if (m < 0 || m >= 32 || !((masks[b] >> m) & 1u)) {             // absent token: zero row
         for (int e = threadIdx.x; e < D; e += blockDim.x) o[e] = from_f32<T>(0.f);
@@ -80,8 +93,8 @@ project_out_kernel(const T* __restrict__ A, const T* __restrict__ WO, const int3
         if (h < 0 || h >= Hq) { atomicOr(status, SENTRY_STATUS_BIT_BAD_INDEX); h = -1; }
         s_h[j] = h;
     }
-    for (int i = threadIdx.x; i < k_h * d; i += blockDim.x)
-        s_a[i] = to_f32<T>(A[(((size_t)b * k_h + i / d) * Tlen + t) * d + i % d]);
+    for (int i = threadIdx.x; i < n_a; i += blockDim.x)
+        s_a[i] = i == (int)threadIdx.x ? a_mine : to_f32<T>(A[(((size_t)b * k_h + i / d) * Tlen + t) * d + i % d]);
     __syncthreads();
     for (int e = threadIdx.x; e < D; e += blockDim.x) {
         float acc = 0.f;
