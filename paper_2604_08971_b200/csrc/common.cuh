@@ -98,6 +98,7 @@ struct DeviceGuard {
 // hold registers on the SMs that another stream's attention CTAs need in full (two of them take an SM's register file).
 // With attention and FFN branches forked on two streams, 128 x 512 tokens at d_model 384: 125 us a step with the early
 // start, 117 without; 4 layers' selections and one gather on one stream: 32 and 27; one window of 64 tokens: 31.0 and 31.7.
+// cluster: CTAs of a cluster (1: none); the grid is a multiple of it.
 template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_chained_clusters(int cluster, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
                                                   cudaStream_t st, Args... args) {

@@ -1,7 +1,7 @@
 // Channel-compacted FFN (Section 4.6): y = gelu(x W1[:, N]) W2[N, :].
 // This file holds the row plan, the weight gather ("materialising" W1', W2')
-// and the plain-ALU fp32-accumulate kernel; the tensor-core kernel for bf16
-// lives in ffn_tc.cu and shares the plan.
+// and the plain-ALU fp32-accumulate kernel; the tensor-core kernels live
+// in ffn_tmem.cu, ffn_tc.cu and ffn_wide.cu and share the plan.
 #include <math.h>
 
 #include "common.cuh"
@@ -58,7 +58,7 @@ __device__ __forceinline__ void plan_block(const int32_t* __restrict__ ids, cons
         own_mask[g] = b0 + g < B && ids != nullptr ? masks[b0 + g] : 0xffffffffu;
     }
     if (ids != nullptr) {
-        // eight of a thread's tokens on the way at once (with one, 16 round trips at 4096 tokens: 15 us of this kernel, now 7)
+        // eight of a thread's tokens on the way at once (with one, 16 round trips at 4096 tokens: 15 us of this kernel, now 10)
         for (int t0 = 0; t0 < Tlen; t0 += 8 * blockDim.x) {
             int m[8];
 #pragma unroll
