@@ -9,9 +9,15 @@
 //         and unreferenced groups are never fetched.
 //   OUT   A stage holds one kept head: the tile's rows of its attention output (d wide) and the rows W_O[h d:(h+1) d] of
 //         the part's columns.
-// Warp 0 feeds the weights by TMA, warp 1 issues the UMMAs, warps 4-7 gather the rows and then store: 64 accumulator columns
-// at a time pass through shared memory so that eight lanes write 128 consecutive bytes.
-// Bound by the L2 reads (each tile streams its weights: 200 MB at B = 128, T = 512, D = 384 with 15 slices of 32).
+// Before the stages warp 0 allocates tensor memory, warp 1 sets up barriers and slices and warps 2-7 list the tile's tokens, at
+// once.  Then warp 0 feeds the weights by TMA, warp 1 issues the UMMAs, warps 4-7 gather the rows, and all eight store: 64
+// accumulator columns at a time pass through shared memory so that eight lanes write 128 consecutive bytes.
+// Bound by what a CTA does one after the other (19 K cycles at B = 128, T = 512, D = 384 with 15 slices of 32: 3.4 K to the first
+// copy, 4.5 K until X and weights of the first stage are there, 7.5 K for six stages of 48 KB, two in flight, 3.5 K to store), which
+// two CTAs per SM overlap in part.  One after the other with four storing warps, list and set-up took 2 and 3 K cycles:
+// 128 x 512 tokens, 9 of 12 heads, QKV 63.4 -> 61.5 us, OUT 40.9 -> 37.7; 16 x 4096 at D = 256 46.5 -> 42.4 and 26.4 -> 20.9; 256 x 256 36.6 -> 35.4
+// and 22.9 -> 17.9.  Slower: two row tiles to a CTA that share the weights, one CTA per SM (63 -> 74 and 41 -> 53), three CTAs per SM with
+// 128 columns (65 and 42; 46 -> 65 on 16 x 4096); without effect: box coordinates kept in registers (issue of a stage 1.2 -> 0.7 K cycles).
 // Measured there, the whole layer 262 -> 206 us: one CTA per SM that loaded X, multiplied slice by slice and then stored
 // took 73 us for QKV and 61 for OUT.
 // Every wait is bounded; on expiry the CTA raises SENTRY_STATUS_BIT_TIMEOUT and unwinds.
@@ -45,49 +51,83 @@ struct ProjMisc {
     uint16_t tok[128];                           // tokens of this tile
 };
 
-// The tile's tokens (present ones number 128 tt .. 128 tt + 127) to misc->tok; returns T_v.  Every warp walks a run of
-// 32-token pieces twice, the second time with the number of present tokens before it.  Complete behind the next barrier.
-__device__ __forceinline__ int list_tile(const int32_t* __restrict__ ids, int T, uint32_t mask, int tt, ProjMisc* misc) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int pieces = (T + 31) / 32, per = (pieces + kPWarps - 1) / kPWarps;
-    const int p0 = min(warp * per, pieces), p1 = min(p0 + per, pieces);
-    auto present = [&](int t) {
-        const int m = t < T ? __ldg(ids + t) : -1;
-        return m >= 0 && m < 32 && ((mask >> m) & 1u);
-    };
-    int mine = 0;
-#pragma unroll 4
-    for (int pc = p0; pc < p1; ++pc) mine += __popc(__ballot_sync(0xffffffffu, present(pc * 32 + lane)));
-    if (lane == 0) misc->counts[warp] = mine;
-    __syncthreads();
-    int at = -tt * 128, total = 0;
+// The tile's tokens (present ones number 128 tt .. 128 tt + 127), by warps 2 to 7.  Every warp counts the present tokens of a run of
+// 32-token pieces, eight of them requested at once; behind the CTA's barrier it writes the tokens of its run that are the
+// tile's.  A run of at most eight pieces keeps its bits and is not read again.
+constexpr int kListWarp0 = 2, kListWarps = kPWarps - kListWarp0;
+struct TileList {
+    int p0, p1, mine;
+    unsigned bits[8];                            // of the pieces read last
+    __device__ __forceinline__ void read(const int32_t* __restrict__ ids, int T, uint32_t mask, int pc) {
+        const int lane = threadIdx.x & 31;
+        int m[8];
 #pragma unroll
-    for (int w = 0; w < kPWarps; ++w) { const int c = misc->counts[w]; total += c; if (w < warp) at += c; }
-    if (at >= 128 || at + mine <= 0) return total;
-#pragma unroll 4
-    for (int pc = p0; pc < p1; ++pc) {
-        const bool ok = present(pc * 32 + lane);
-        const unsigned bm = __ballot_sync(0xffffffffu, ok);
-        const int r = at + __popc(bm & ((1u << lane) - 1u));
-        if (ok && r >= 0 && r < 128) misc->tok[r] = (uint16_t)(pc * 32 + lane);
-        at += __popc(bm);
+        for (int u = 0; u < 8; ++u) {
+            const int t = (pc + u) * 32 + lane;
+            m[u] = pc + u < p1 && t < T ? __ldg(ids + t) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) bits[u] = __ballot_sync(0xffffffffu, m[u] >= 0 && m[u] < 32 && ((mask >> (m[u] & 31)) & 1u));
     }
+    __device__ __forceinline__ void count(const int32_t* __restrict__ ids, int T, uint32_t mask, ProjMisc* misc) {
+        const int w = (threadIdx.x >> 5) - kListWarp0, pieces = (T + 31) / 32, per = (pieces + kListWarps - 1) / kListWarps;
+        p0 = min(w * per, pieces), p1 = min(p0 + per, pieces), mine = 0;
+        for (int pc = p0; pc < p1; pc += 8) {
+            read(ids, T, mask, pc);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) mine += __popc(bits[u]);
+        }
+        if ((threadIdx.x & 31) == 0) misc->counts[w] = mine;
+    }
+    __device__ __forceinline__ void fill(const int32_t* __restrict__ ids, int T, uint32_t mask, int tt, ProjMisc* misc) {
+        const int lane = threadIdx.x & 31, w = (threadIdx.x >> 5) - kListWarp0;
+        int at = -tt * 128;
+#pragma unroll
+        for (int v = 0; v < kListWarps; ++v)
+            if (v < w) at += misc->counts[v];
+        if (at >= 128 || at + mine <= 0) return;
+        for (int pc = p0; pc < p1; pc += 8) {
+            if (p1 - p0 > 8) read(ids, T, mask, pc);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int r = at + __popc(bits[u] & ((1u << lane) - 1u));
+                if (((bits[u] >> lane) & 1u) && r >= 0 && r < 128) misc->tok[r] = (uint16_t)((pc + u) * 32 + lane);
+                at += __popc(bits[u]);
+            }
+        }
+    }
+};
+// T_v of the sample, behind the barrier that follows TileList::count
+__device__ __forceinline__ int present_tokens(const ProjMisc* misc) {
+    int total = 0;
+#pragma unroll
+    for (int v = 0; v < kListWarps; ++v) total += misc->counts[v];
     return total;
 }
+// misc->tok is complete: among the warps that list (they gather next), and for warps 0 and 1, which read it with the results
+__device__ __forceinline__ void list_done() {
+    __syncwarp();
+    asm volatile("bar.arrive 2, %0;" ::"n"(kPThreads) : "memory");
+    asm volatile("bar.sync 1, %0;" ::"n"(kListWarps * 32) : "memory");
+}
+__device__ __forceinline__ void list_wait() {
+    __syncwarp();
+    asm volatile("bar.sync 2, %0;" ::"n"(kPThreads) : "memory");
+}
 
-// Barriers and the slice list of sample b (warp 0; behind the caller's barrier).  Hk = 0: kept heads only.
+// Barriers and the slice list of sample b (one warp; complete behind the caller's barrier).  Hk = 0: kept heads only.
 __device__ __forceinline__ void proj_setup(ProjMisc* misc, int stages, const int32_t* __restrict__ kept, int k_h, int Hq, int Hk,
                                            unsigned int* status) {
     const int lane = threadIdx.x & 31;
+    if (lane < stages) {
+        ptx::mbar_init(ptx::smem_u32(&misc->full[lane]), 5);   // the TMA's expect, and the four gathering warps
+        ptx::mbar_init(ptx::smem_u32(&misc->empty[lane]), 1);
+    }
     if (lane == 0) {
-        for (int s = 0; s < stages; ++s) {
-            ptx::mbar_init(ptx::smem_u32(&misc->full[s]), 5);   // the TMA's expect, and the four gathering warps
-            ptx::mbar_init(ptx::smem_u32(&misc->empty[s]), 1);
-        }
         ptx::mbar_init(ptx::smem_u32(&misc->acc_full), 1);
         misc->abort_flag = 0;
-        ptx::fence_barrier_init();
     }
+    ptx::fence_barrier_init();
     int n = 0;
     uint32_t groups = 0u;
     for (int j0 = 0; j0 < k_h; j0 += 32) {
@@ -103,14 +143,33 @@ __device__ __forceinline__ void proj_setup(ProjMisc* misc, int stages, const int
         n += __popc(bm);
         groups |= __reduce_or_sync(0xffffffffu, ok && Hk > 0 ? 1u << (h / (Hq / Hk)) : 0u);
     }
-    for (int g = 0; g < Hk; ++g)
-        if ((groups >> g) & 1u) {
-            if (lane < 2) { misc->kind[n + lane] = 1 + lane; misc->idx[n + lane] = g; }
-            n += 2;
-        }
+    if ((groups >> lane) & 1u) {                 // (Hk is at most 32)
+        const int at = n + 2 * __popc(groups & ((1u << lane) - 1u));
+        misc->kind[at] = 1;
+        misc->kind[at + 1] = 2;
+        misc->idx[at] = misc->idx[at + 1] = lane;
+    }
+    n += 2 * __popc(groups);
     if (lane == 0) misc->n_slices = n;
-    ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), kPCols);
-    ptx::tmem_relinquish();
+}
+
+// What a CTA does before its stages, at once: tensor memory (warp 0), barriers and slices (warp 1), the tokens counted (the rest).
+// Returns T_v.
+__device__ __forceinline__ int proj_prologue(ProjMisc* misc, TileList& list, const int32_t* __restrict__ kept, int k_h, int Hq, int Hk,
+                                             const int32_t* __restrict__ ids, int T, uint32_t mask, unsigned int* status) {
+    const int warp = threadIdx.x >> 5;
+    if (warp == 0) {
+        ptx::tmem_alloc(ptx::smem_u32(&misc->tmem_base), kPCols);
+        ptx::tmem_relinquish();
+    } else if (warp == 1) {
+        proj_setup(misc, kPMaxStages, kept, k_h, Hq, Hk, status);
+    } else {
+        list.count(ids, T, mask, misc);
+    }
+    ptx::tc_fence_before_sync();
+    __syncthreads();
+    ptx::tc_fence_after_sync();
+    return present_tokens(misc);
 }
 
 // Gathers CPR 16-byte chunks of 128 rows per stage by warps 4-7: src(step, row, chunk) is the address or null (zeros),
@@ -200,21 +259,28 @@ proj_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int part = blockIdx.x % parts_max, tile = blockIdx.x / parts_max, b = tile / tiles, tt = tile % tiles;
     const int KB = D / 64;
+    if (warp == 0 && elect_one()) {
+        ptx::prefetch_tensormap(&tm_q);
+        ptx::prefetch_tensormap(&tm_k);
+        ptx::prefetch_tensormap(&tm_v);
+    }
     grid_dependency_wait();
-    const int Tv = list_tile(ids, Tlen, masks[b], tt, misc);
-    if (tt * 128 >= Tv) return;                     // no present token in this tile
-    const int n_rows = min(128, Tv - tt * 128);
-    if (warp == 0) proj_setup(misc, kPMaxStages, kept_heads + (size_t)b * k_h, k_h, Hq, Hk, status);
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
+    const uint32_t mask = masks[b];
+    TileList list;
+    const int Tv = proj_prologue(misc, list, kept_heads + (size_t)b * k_h, k_h, Hq, Hk, ids, Tlen, mask, status);
     const uint32_t tmem = misc->tmem_base;
+    if (tt * 128 >= Tv) {                           // no present token in this tile
+        tc_cta_teardown(abort_flag, status, tmem, kPCols);
+        return;
+    }
+    const int n_rows = min(128, Tv - tt * 128);
     // equal shares of the slices for the parts that are needed
     const int n_all = misc->n_slices, parts = (n_all + NS - 1) / NS, per = parts > 0 ? (n_all + parts - 1) / parts : 0;
     const int s0 = part * per, n_sl = min(n_all - s0, per);
     if (n_sl > 0) {
         const uint32_t stage_bytes = 16384u + (uint32_t)n_sl * 64u * RB;
         const int stages = min(kPRing / (int)stage_bytes, kPMaxStages);
+        bool ready = true;                          // this warp's part before the results went through
         if (warp == 0) {
             // -------------------------------------------------------- weights
             bool ok = true;
@@ -258,39 +324,44 @@ proj_qkv_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                 __syncwarp();
                 if (++slot == stages) { slot = 0; phase ^= 1u; }
             }
-        } else if (warp >= 4) {
+        } else {
+            list.fill(ids, Tlen, mask, tt, misc);
+            list_done();
+        }
+        if (warp < kListWarp0) list_wait();
+        if (warp >= 4) {
             const __nv_bfloat16* rows[8];          // this thread's chunk of its rows
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int r = (threadIdx.x - 128 + j * 128) / 8;
                 rows[j] = r < n_rows ? X + ((size_t)b * Tlen + misc->tok[r]) * D + (threadIdx.x & 7) * 8 : nullptr;
             }
-            const bool ok = gather_steps<8>(
+            ready = gather_steps<8>(
                 misc, ring, stage_bytes, stages, KB,
                 [&](int kb, int, int, int j) { return rows[j] != nullptr ? rows[j] + kb * 64 : nullptr; },
                 [](int r, int cc) { return (uint32_t)(r * 128 + ((cc ^ (r & 7)) << 4)); }, abort_flag);
-            // ------------------------------------------------------------- results
-            if (ok && warp_wait(&misc->acc_full, 0u, abort_flag)) {
-                ptx::tc_fence_after_sync();
-                const int quarter = warp & 3, c = lane & 7;
-                const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16), buf = ring + quarter * 4096u;
-                for (int c0 = 0; c0 < n_sl * DH; c0 += 64) {
-                    acc_to_smem(taddr + c0, buf);
-                    const int s = (c0 + c * 8) / DH;                   // the slice of this lane's chunk
-                    if (s < n_sl) {
-                        const int kind = misc->kind[s0 + s], idx = misc->idx[s0 + s];
-                        __nv_bfloat16* dst = kind == 0 ? Q + ((size_t)b * Hq + idx) * Tlen * DH
-                                                       : (kind == 1 ? K : V) + ((size_t)b * Hk + idx) * Tlen * DH;
-                        dst += (c * 8) % DH;
+        }
+        // ----------------------------------------------------------------- results: two warps per 32 rows, blocks of 64 columns in turn
+        if (ready && warp_wait(&misc->acc_full, 0u, abort_flag)) {
+            ptx::tc_fence_after_sync();
+            const int quarter = warp & 3, c = lane & 7;
+            const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16), buf = ring + warp * 4096u;
+            for (int c0 = (warp >> 2) * 64; c0 < n_sl * DH; c0 += 128) {
+                acc_to_smem(taddr + c0, buf);
+                const int s = (c0 + c * 8) / DH;                   // the slice of this lane's chunk
+                if (s < n_sl) {
+                    const int kind = misc->kind[s0 + s], idx = misc->idx[s0 + s];
+                    __nv_bfloat16* dst = kind == 0 ? Q + ((size_t)b * Hq + idx) * Tlen * DH
+                                                   : (kind == 1 ? K : V) + ((size_t)b * Hk + idx) * Tlen * DH;
+                    dst += (c * 8) % DH;
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int r = i * 4 + (lane >> 3);
-                            if (quarter * 32 + r < n_rows)
-                                *reinterpret_cast<uint4*>(dst + (size_t)misc->tok[quarter * 32 + r] * DH) = smem_chunk(buf, r, c);
-                        }
+                    for (int i = 0; i < 8; ++i) {
+                        const int r = i * 4 + (lane >> 3);
+                        if (quarter * 32 + r < n_rows)
+                            *reinterpret_cast<uint4*>(dst + (size_t)misc->tok[quarter * 32 + r] * DH) = smem_chunk(buf, r, c);
                     }
-                    __syncwarp();
                 }
+                __syncwarp();
             }
         }
     }
@@ -315,27 +386,33 @@ proj_out_tc_kernel(const __grid_constant__ CUtensorMap tm_o, const __nv_bfloat16
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int part = blockIdx.x % parts, tile = blockIdx.x / parts, b = tile / tiles, tt = tile % tiles;
     const int per = (D / 64 + parts - 1) / parts, box0 = part * per, n_box = min(D / 64 - box0, per);
+    if (warp == 0 && elect_one()) ptx::prefetch_tensormap(&tm_o);
     grid_dependency_wait();
     const uint32_t mask = masks[b];
-    {
-        const int t = tt * 128 + warp * 16 + (lane & 15), m = t < Tlen ? ids[t] : -1;
-        unsigned gone = __ballot_sync(0xffffffffu, t < Tlen && !(m >= 0 && m < 32 && ((mask >> m) & 1u))) & 0xffffu;
-        for (; gone; gone &= gone - 1) {
-            uint4* dst = reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + tt * 128 + warp * 16 + __ffs(gone) - 1) * D) + box0 * 8;
-            if (lane < n_box * 8) dst[lane] = make_uint4(0, 0, 0, 0);
+    // its columns of the absent ones among token positions 128 tt .., by nw warps
+    auto clear_absent = [&](int w, int nw) {
+        for (int p = tt * 128 + w * 32; p < tt * 128 + 128; p += nw * 32) {
+            const int t = p + lane, m = t < Tlen ? ids[t] : -1;
+            unsigned gone = __ballot_sync(0xffffffffu, t < Tlen && !(m >= 0 && m < 32 && ((mask >> m) & 1u)));
+            for (; gone; gone &= gone - 1) {
+                uint4* dst = reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + p + __ffs(gone) - 1) * D) + box0 * 8;
+                if (lane < n_box * 8) dst[lane] = make_uint4(0, 0, 0, 0);
+            }
         }
-    }
-    const int Tv = list_tile(ids, Tlen, mask, tt, misc);
-    if (tt * 128 >= Tv) return;
-    const int n_rows = min(128, Tv - tt * 128);
-    if (warp == 0) proj_setup(misc, kPMaxStages, kept_heads + (size_t)b * k_h, k_h, Hq, 0, status);
-    ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::tc_fence_after_sync();
+    };
+    TileList list;
+    const int Tv = proj_prologue(misc, list, kept_heads + (size_t)b * k_h, k_h, Hq, 0, ids, Tlen, mask, status);
     const uint32_t tmem = misc->tmem_base;
+    if (tt * 128 >= Tv) {
+        clear_absent(warp, kPWarps);
+        tc_cta_teardown(abort_flag, status, tmem, kPCols);
+        return;
+    }
+    const int n_rows = min(128, Tv - tt * 128);
     const int n_sl = misc->n_slices;
     const uint32_t stage_bytes = 128u * RB + (uint32_t)n_box * kBox;
     const int stages = min(kPRing / (int)stage_bytes, kPMaxStages);
+    bool ready = true;                              // this warp's part before the results went through
     if (warp == 0) {
         bool ok = true;
         int slot = 0;
@@ -374,34 +451,41 @@ proj_out_tc_kernel(const __grid_constant__ CUtensorMap tm_o, const __nv_bfloat16
             __syncwarp();
             if (++slot == stages) { slot = 0; phase ^= 1u; }
         }
-    } else if (warp >= 4) {
+    } else {
+        list.fill(ids, Tlen, mask, tt, misc);
+        list_done();
+        if (warp < 4) clear_absent(warp - kListWarp0, 4 - kListWarp0);
+    }
+    if (warp < kListWarp0) list_wait();
+    if (warp >= 4) {
         const __nv_bfloat16* rows[S::CPR];
 #pragma unroll
         for (int j = 0; j < S::CPR; ++j) {
             const int i = threadIdx.x - 128 + j * 128, r = i / S::CPR;
             rows[j] = r < n_rows ? A + ((size_t)b * k_h * Tlen + misc->tok[r]) * DH + (i % S::CPR) * 8 : nullptr;
         }
-        const bool ok = gather_steps<S::CPR>(
+        ready = gather_steps<S::CPR>(
             misc, ring, stage_bytes, stages, n_sl,
             [&](int s, int, int, int j) {
                 return rows[j] != nullptr ? rows[j] + (size_t)misc->kind[s] * Tlen * DH : nullptr;
             },
             [](int r, int cc) { return S::off(r, cc); }, abort_flag);
+    }
+    // results: two warps per 32 rows, boxes in turn
+    if (ready && (n_sl == 0 || warp_wait(&misc->acc_full, 0u, abort_flag))) {
+        ptx::tc_fence_after_sync();
         const int quarter = warp & 3, c = lane & 7;
-        if (ok && (n_sl == 0 || warp_wait(&misc->acc_full, 0u, abort_flag))) {
-            ptx::tc_fence_after_sync();
-            const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16), buf = ring + quarter * 4096u;
-            for (int i = 0; i < n_box; ++i) {
-                if (n_sl > 0) acc_to_smem(taddr + i * 64, buf);
+        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16), buf = ring + warp * 4096u;
+        for (int i = warp >> 2; i < n_box; i += 2) {
+            if (n_sl > 0) acc_to_smem(taddr + i * 64, buf);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int r = j * 4 + (lane >> 3);
-                    if (quarter * 32 + r < n_rows)   // (no valid kept head: the rows are zero)
-                        *reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + misc->tok[quarter * 32 + r]) * D + (box0 + i) * 64 + c * 8) =
-                            n_sl > 0 ? smem_chunk(buf, r, c) : make_uint4(0, 0, 0, 0);
-                }
-                __syncwarp();
+            for (int j = 0; j < 8; ++j) {
+                const int r = j * 4 + (lane >> 3);
+                if (quarter * 32 + r < n_rows)   // (no valid kept head: the rows are zero)
+                    *reinterpret_cast<uint4*>(out + ((size_t)b * Tlen + misc->tok[quarter * 32 + r]) * D + (box0 + i) * 64 + c * 8) =
+                        n_sl > 0 ? smem_chunk(buf, r, c) : make_uint4(0, 0, 0, 0);
             }
+            __syncwarp();
         }
     }
     tc_cta_teardown(abort_flag, status, tmem, kPCols);

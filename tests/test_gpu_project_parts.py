@@ -28,6 +28,7 @@ def _w(name, dtype, B, lengths, D, Hq, Hk, d, k_h, rule="cycle7"):
     _w("parts_d32_3_parts", "f16", 7, (127, 2, 129), 256, 16, 8, 32, 9),          # 9 + up to 16 slices: up to four parts
     _w("parts_d64_5_slices", "bf16", 5, (40, 128, 88), 128, 6, 2, 64, 3),         # parts of 3 and 2 or 4 and 3 slices
     _w("parts_d64_wide_out", "bf16", 4, (200, 97, 90), 768, 12, 4, 64, 7, "all"),    # output in three parts; plain-ALU Q, K, V
+    _w("parts_d16_2000_tokens", "bf16", 7, (1500, 37, 460), 64, 4, 2, 16, 3),     # a warp's run of token pieces above eight; empty tiles
     _w("plain_f32_128_slices", "f32", 2, (5, 6, 7), 64, 64, 32, 16, 64),          # 64 heads, K and V of 32 groups
     _w("plain_f32_40_of_48", "f32", 3, (5, 6, 7), 320, 48, 12, 16, 40),           # list entries beyond a warp's first 32
     _w("parts_d32_wide_out", "f16", 4, (30, 97, 90), 320, 12, 4, 32, 12),         # five column boxes in parts of 3 and 2
