@@ -20,7 +20,7 @@
 // both: 2300 cycles a chunk.  Per call with the row plan, hidden tile in shared memory / P = 1 / P = 2: 149 k rows, d_model 256,
 // 512 channels 80 / 79 / 72 us; 599 k rows 303 / 298 / 270; 65 k rows 38.6 / 37.4 / 36.1; 37 k rows 26.2 / 24.4 / 25.5; 2.2 k rows
 // 15.4 / 14.4 / 15.1; 35 k rows of d_model 128, 256 channels 16.7 / 14.1 / 16.0.  So pairs from three rounds of tiles on at d_model
-// 256, where the weights are what is moved, and single CTAs otherwise.
+// 256 (six where absent tokens are not yet counted), where the weights are what is moved, and single CTAs otherwise.
 //
 // Warp roles (512 threads): warp 0 = weight TMA producer (owns TMEM), warp 1 = UMMA issuer, warps 3-6 = X row gather, warps 7-14 = epilogue (two warps per TMEM lane quarter), warp 15 = zero rows of absent tokens.  Every wait is
 // bounded; on expiry the CTA raises SENTRY_STATUS_BIT_TIMEOUT and unwinds.
@@ -524,8 +524,11 @@ int launch_ffn_tmem(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void
     const bool f16 = a.d.dtype == SENTRY_F16;
     if (a.d.D == 128) return f16 ? launch_d<128, true, 1>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
                                  : launch_d<128, false, 1>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
-    // pairs: see above; a list with an odd number of tiles leaves half of a pair idle, and every thread adds up the lists
-    if (max_tiles >= 3 * ctx->sm_count && a.d.n_lists <= 64)
+    // pairs: see above; a list with an odd number of tiles leaves half of a pair idle, and every thread adds up the lists.  With
+    // masks max_tiles is what there is when every token is present: twice as many then, so that half of the tokens still
+    // make three rounds (65 k tokens of seven lists, 37 k present: two full rounds of single CTAs 29 us, of pairs a third one, 33)
+    const int rounds = a.ids == nullptr ? 3 : 6;
+    if (max_tiles >= rounds * ctx->sm_count && a.d.n_lists <= 64)
         return f16 ? launch_d<256, true, 2>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
                    : launch_d<256, false, 2>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
     return f16 ? launch_d<256, true, 1>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)

@@ -48,7 +48,7 @@ def test_one_row(D):
 def test_pairs_equal_single_ctas(k_c, n_lists):
     """A large call (pairs of CTAs) against the same samples in small calls (single CTAs): equal bits, and equal again."""
     gen = torch.Generator(device="cuda").manual_seed(k_c)
-    B, T, D, F = 640, 100, 256, 512
+    B, T, D, F = 1280, 100, 256, 512
     X = torch.randn((B, T, D), generator=gen, device="cuda").bfloat16()
     W1 = torch.randn((D, F), generator=gen, device="cuda").mul_(0.05).bfloat16()
     W2 = torch.randn((F, D), generator=gen, device="cuda").mul_(0.05).bfloat16()
