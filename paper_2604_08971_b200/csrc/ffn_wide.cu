@@ -59,7 +59,8 @@ __device__ __forceinline__ float hi_of(uint32_t w) {
 // gelu(z) = z Phi(z) = max(z, 0) - |z| Q(|z|) with Q(a) = exp(-a^2/2) R(1 / (1 + a/4)), the tail of the normal distribution: own
 // minimax fit of R (degree 7, 9e-9 of the value at the worst a, weighted by exp(-a^2/2) down to 1e-2).  In fp32 it is off by
 // at most 2.4e-7 |z|, where 0.5 z (1 + erff(z / sqrt 2)) is by 1.1e-7 |z| and the buffer's head and remainder by 2^-17 |h|:
-// 15 instructions, about a third of the library form's.  NaN stays NaN, and +inf and -inf give inf and NaN as that form does.
+// 15 instructions, about a third of the library form's.  max(z, 0) is z/2 + |z|/2, exact for every finite z (z + |z| is inf from half of
+// the largest float on, and the remainder of an infinite head NaN).  NaN stays NaN, and +inf and -inf give inf and NaN as that form does.
 __device__ __forceinline__ float gelu_tail(float z) {
     const float a = fabsf(z), c = fminf(a, 16.f);           // (the tail is 0 from 14 on)
     float t, e;
@@ -72,7 +73,7 @@ __device__ __forceinline__ float gelu_tail(float z) {
     r = fmaf(r, t, 0.123881109f);
     r = fmaf(r, t, 0.0965574905f);
     r = fmaf(r, t, 0.000175767025f);
-    return fmaf(0.5f, z + a, -c * (r * e));
+    return fmaf(0.5f, z, 0.5f * a) - c * (r * e);
 }
 
 // Columns of a tile where R row tiles have `cols` columns and `slots` CTAs run at once: the rounds times what a K block costs

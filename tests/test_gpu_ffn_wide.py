@@ -46,6 +46,32 @@ def test_wide_ffn_matches_oracle(w):
         sn.close()
 
 
+@pytest.mark.parametrize("dtype,large", [("bf16", (2.0e38, -2.0e38, 3.38e38, -3.38e38, 1.0e30)), ("f16", (60000.0, -60000.0, 40000.0))])
+def test_wide_ffn_extreme_values(dtype, large):
+    """One channel a column (W1, W2 the identity), so that a pre-activation is X's value: large finite ones come back
+    (gelu(z) = z, or 0 below), an infinite or NaN one spoils its own row and no other."""
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float16
+    D, T = 64, 130
+    X = torch.randn((1, T, D), generator=torch.Generator().manual_seed(1)).to(dt)
+    special = {}
+    for i, v in enumerate(large + (float("inf"), float("-inf"), float("nan"))):
+        X[0, 7 * i + 3, i] = v
+        special[7 * i + 3] = v
+    eye, kept = torch.eye(D).to(dt), torch.arange(D, dtype=torch.int32).reshape(1, D)
+    sn = sentry.Sentry(0)
+    try:
+        Y = sn.ffn_fwd(X.cuda(), eye.cuda(), eye.cuda(), kept.cuda(), torch.zeros(1, dtype=torch.int32).cuda()).cpu()[0]
+        want = torch.nn.functional.gelu(X[0].double())
+        for r in range(T):
+            if np.isfinite(special.get(r, 0.0)):   # (the two roundings of a stored value, and fp32 sums)
+                assert torch.allclose(Y[r].double(), want[r], rtol=2.0 ** (-8 if dtype == "bf16" else -11) * 1.01, atol=1e-6), r
+            else:
+                assert not torch.isfinite(Y[r]).all(), r
+        assert sn.last_status() == 0
+    finally:
+        sn.close()
+
+
 def test_wide_moe_matches_oracle():
     m = synth.generate_moe(300, 512, 256, 5, 2, 100, "bf16", seed=3, skew=1.0)
     sn = sentry.Sentry(0)
