@@ -8,18 +8,21 @@
 // rows than that go in turns.  They are stored as a 16-bit head plus a 16-bit remainder (h = hi + lo to 2^-17), and
 // GEMM 2 multiplies both: what the plain-ALU kernel keeps in fp32 is not rounded to 16 bits here either.
 //
-// What bounds them: GEMM 1 its epilogue (two special-function and thirteen other instructions per element, by all eight warps;
-// with the library's erff and four warps 6 us of 13 a tile) and its row gather, GEMM 2 the shared memory that serves the UMMAs'
+// What bounds them: GEMM 1 its epilogue (two special-function and twenty other instructions per element, ffn_wide_math.cuh, by all
+// eight warps; with the library's erff and four warps 6 us of 13 a tile) and its row gather, GEMM 2 the shared memory that serves the UMMAs'
 // operands and the copies (128 bytes a cycle).  The column tile follows the number of row tiles, which only the device
 // knows: small calls spread over more SMs, large ones read A less often.
 // Measured, a call with its row plan on materialised weights, before (128 x 128 tiles, erff, four epilogue warps that stored row
-// by row) and now: 3.7 k rows of d_model 768, 1229 channels in seven lists 55.1 -> 47.0 us; 524 rows, 765 channels 29.0 -> 23.9;
-// 46 rows, 967 channels 30.2 -> 25.0; 233 rows of d_model 192, 340 channels 19.0 -> 15.3; 5.6 k rows, 384 channels 21.6 -> 18.6.
+// by row) and now: 3.7 k rows of d_model 768, 1229 channels in seven lists 55.1 -> 47.1 us; 524 rows, 765 channels 29.0 -> 23.8;
+// 46 rows, 967 channels 30.2 -> 24.8; 233 rows of d_model 192, 340 channels 19.0 -> 15.1; 5.6 k rows, 384 channels 21.6 -> 18.4.
+// The GELU alone, as the erff form / the tail form without the polynomial / both parts: 3.7 k rows 47.9 / 46.3 / 47.1; 30.7 k rows of
+// d_model 512, 1024 channels 191.4 / 182.7 / 187.5; 46 rows 24.9 / 24.6 / 24.8.
 #include <cuda.h>
 #include <math.h>
 
 #include "common.cuh"
 #include "ffn_plan.cuh"
+#include "ffn_wide_math.cuh"
 #include "tc_common.cuh"
 #include "ptx/sm100.cuh"
 
@@ -56,24 +59,19 @@ __device__ __forceinline__ float hi_of(uint32_t w) {
     if constexpr (F16) return __half2float(__ushort_as_half((unsigned short)(w >> 16)));
     else return __uint_as_float(w & 0xffff0000u);
 }
-// gelu(z) = z Phi(z) = max(z, 0) - |z| Q(|z|) with Q(a) = exp(-a^2/2) R(1 / (1 + a/4)), the tail of the normal distribution: own
-// minimax fit of R (degree 7, 9e-9 of the value at the worst a, weighted by exp(-a^2/2) down to 1e-2).  In fp32 it is off by
-// at most 2.4e-7 |z|, where 0.5 z (1 + erff(z / sqrt 2)) is by 1.1e-7 |z| and the buffer's head and remainder by 2^-17 |h|:
-// 15 instructions, about a third of the library form's.  max(z, 0) is z/2 + |z|/2, exact for every finite z (z + |z| is inf from half of
-// the largest float on, and the remainder of an infinite head NaN).  NaN stays NaN, and +inf and -inf give inf and NaN as that form does.
-__device__ __forceinline__ float gelu_tail(float z) {
-    const float a = fabsf(z), c = fminf(a, 16.f);           // (the tail is 0 from 14 on)
-    float t, e;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.25f, c, 1.f)));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(c * c * -0.72134752f));
-    float r = fmaf(-0.0961182937f, t, 0.363730848f);
-    r = fmaf(r, t, -0.312237799f);
-    r = fmaf(r, t, 0.331047446f);
-    r = fmaf(r, t, -0.00703657651f);
-    r = fmaf(r, t, 0.123881109f);
-    r = fmaf(r, t, 0.0965574905f);
-    r = fmaf(r, t, 0.000175767025f);
-    return fmaf(0.5f, z, 0.5f * a) - c * (r * e);
+__device__ __forceinline__ float gelu_wide(float z) {
+    return gelu_two_part(
+        z,
+        [](float x) {
+            float y;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+            return y;
+        },
+        [](float x) {
+            float y;
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+            return y;
+        });
 }
 
 // Columns of a tile where R row tiles have `cols` columns and `slots` CTAs run at once: the rounds times what a K block costs
@@ -252,7 +250,7 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
                 uint32_t q[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    const float g0 = gelu_tail(__uint_as_float(r[2 * i])), g1 = gelu_tail(__uint_as_float(r[2 * i + 1]));
+                    const float g0 = gelu_wide(__uint_as_float(r[2 * i])), g1 = gelu_wide(__uint_as_float(r[2 * i + 1]));
                     w[i] = pack_16x2<F16>(g0, g1);
                     q[i] = pack_16x2<F16>(g0 - lo_of<F16>(w[i]), g1 - hi_of<F16>(w[i]));
                 }
