@@ -59,6 +59,15 @@ __device__ __forceinline__ float hi_of(uint32_t w) {
     if constexpr (F16) return __half2float(__ushort_as_half((unsigned short)(w >> 16)));
     else return __uint_as_float(w & 0xffff0000u);
 }
+// Heads of a pair: the nearest values of the storage type, its largest one instead of inf.  A hidden value of up to twice that keeps a
+// finite head and a remainder that makes up for it (an infinite head's remainder would be inf - inf).
+template <bool F16>
+__device__ __forceinline__ uint32_t pack_heads(float a, float b) {
+    uint32_t v;
+    if constexpr (F16) asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(v) : "f"(b), "f"(a));
+    else asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(v) : "f"(b), "f"(a));
+    return v;
+}
 __device__ __forceinline__ float gelu_wide(float z) {
     return gelu_two_part(
         z,
@@ -251,7 +260,7 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
                     const float g0 = gelu_wide(__uint_as_float(r[2 * i])), g1 = gelu_wide(__uint_as_float(r[2 * i + 1]));
-                    w[i] = pack_16x2<F16>(g0, g1);
+                    w[i] = pack_heads<F16>(g0, g1);
                     q[i] = pack_16x2<F16>(g0 - lo_of<F16>(w[i]), g1 - hi_of<F16>(w[i]));
                 }
                 store32(w, out_h + n0 + c0, kc_pad);

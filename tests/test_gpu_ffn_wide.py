@@ -72,6 +72,25 @@ def test_wide_ffn_extreme_values(dtype, large):
         sn.close()
 
 
+@pytest.mark.parametrize("dtype,x,scale", [("f16", 60000.0, 2.0), ("f16", -60000.0, 2.0), ("f16", 65504.0, 1.0), ("bf16", 3.38e38, 1.0078125)])
+def test_wide_ffn_hidden_value_beyond_the_storage_type(dtype, x, scale):
+    """A hidden value above the largest 16-bit one (below twice it) reaches a result that is in range."""
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float16
+    D = 64
+    X = torch.randn((1, 3, D), generator=torch.Generator().manual_seed(2)).to(dt)
+    X[0, 1, 5] = x
+    W1, W2 = (torch.eye(D) * scale).to(dt), (torch.eye(D) * 0.25).to(dt)
+    z = X[0].double() * float(W1[0, 0])
+    sn = sentry.Sentry(0)
+    try:
+        Y = sn.ffn_fwd(X.cuda(), W1.cuda(), W2.cuda(), torch.arange(D, dtype=torch.int32).reshape(1, D).cuda(),
+                       torch.zeros(1, dtype=torch.int32).cuda()).cpu()[0]
+        want = torch.nn.functional.gelu(z) * 0.25
+        assert torch.allclose(Y.double(), want, rtol=2.0 ** (-8 if dtype == "bf16" else -11) * 1.01, atol=1e-6)
+    finally:
+        sn.close()
+
+
 def test_wide_moe_matches_oracle():
     m = synth.generate_moe(300, 512, 256, 5, 2, 100, "bf16", seed=3, skew=1.0)
     sn = sentry.Sentry(0)
