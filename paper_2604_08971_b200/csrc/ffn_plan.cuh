@@ -37,6 +37,7 @@ int launch_ffn_tmem(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void
                     cudaStream_t st);
 bool ffn_wide_supported(const sentry_ffn_desc& d);
 int ffn_wide_kc_pad(int k_c);
+long long ffn_wide_first_ctas(int k_c, long long max_tiles);
 size_t ffn_wide_hidden_bytes(int kc_pad, long long max_tiles);
 int launch_ffn_wide(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c, int kc_pad, int max_tiles,
                     void* hidden, cudaStream_t st);

@@ -35,8 +35,8 @@ constexpr int kWideTiles = 128;         // row tiles the hidden buffer holds
 template <bool FIRST>
 struct WideCfg {
     static constexpr int A_BLOCKS = FIRST ? 1 : 2;          // A, or A's head and remainder
-    static constexpr int BN_MAX = FIRST ? 160 : 192;        // columns of a tile: a multiple of 32, 64 to this
-    static constexpr int CTAS = FIRST ? 2 : 1;              // per SM
+    static constexpr int BN_MAX = wide_bn_max(FIRST);
+    static constexpr int CTAS = wide_ctas(FIRST);           // per SM
     static constexpr int STAGES = FIRST ? 3 : 4;
     static constexpr int STAGE_BYTES = A_BLOCKS * kWBlock + BN_MAX * 128;
     static constexpr int TMEM_COLS = 256;
@@ -83,18 +83,6 @@ __device__ __forceinline__ float gelu_wide(float z) {
         });
 }
 
-// Columns of a tile where R row tiles have `cols` columns and `slots` CTAs run at once: the rounds times what a K block costs
-// in shared-memory traffic, which is that of A and the columns of B (in units of B's).
-template <bool FIRST>
-__device__ __forceinline__ int wide_bn(int R, int cols, int slots) {
-    int best = 64, best_cost = 0x7fffffff;
-    for (int bn = 64; bn <= WideCfg<FIRST>::BN_MAX; bn += 32) {
-        const int items = R * ((cols + bn - 1) / bn), cost = (items + slots - 1) / slots * ((FIRST ? 128 : 170) + bn);
-        if (cost < best_cost) { best = bn; best_cost = cost; }
-    }
-    return best;
-}
-
 // grid (column tiles of 64, row tiles of this turn); a CTA beyond the tiles that there are at the width taken has nothing to do.
 // FIRST: tm_b = W1c [lists * kc_pad, D], out_h / out_l = the hidden buffer's two planes.  Otherwise tm_a_hi / tm_a_lo = those
 // planes, tm_b = W2c [lists * D, kc_pad], Y the result.
@@ -116,7 +104,7 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
     if (!ffn_tile_lookup(plan, n_lists, tile0 + (int)blockIdx.y, 128, l, row0, n_rows)) return;
     const int kc = (k_c + 63) / 64 * 64;                   // channels that are computed (padded ones carry zero weights)
     const int cols = FIRST ? kc : D;
-    const int bn = wide_bn<FIRST>(min(plan.tile_start[n_lists] - tile0, turn), cols, sm_count * C::CTAS);
+    const int bn = wide_bn(FIRST, min(plan.tile_start[n_lists] - tile0, turn), cols, sm_count);
     const int n0 = blockIdx.x * bn;                        // first output column
     if (n0 >= cols) return;
     const int n_cols = min(bn, cols - n0);                 // a multiple of 32
@@ -294,10 +282,10 @@ int launch_wide(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1
     for (int t0 = 0; t0 < max_tiles; t0 += turn) {
         const unsigned nt = (unsigned)(max_tiles - t0 < turn ? max_tiles - t0 : turn);
         LaunchScope ls(ctx, KS_FFN_MAIN, st, 2);
-        SENTRY_CUDA_TRY(launch_chained(k1, dim3((unsigned)((d.k_c + 63) / 64), nt), dim3(kWThreads), (size_t)WideCfg<true>::SMEM_BYTES,
+        SENTRY_CUDA_TRY(launch_chained(k1, dim3((unsigned)wide_grid_cols(d.k_c), nt), dim3(kWThreads), (size_t)WideCfg<true>::SMEM_BYTES,
                                        st, ah, al, m1, (const __nv_bfloat16*)a.X, hh, hl, nullptr, plan, d.n_lists, t0, (int)nt, d.D,
                                        d.k_c, kc_pad, ctx->sm_count, a.status));
-        SENTRY_CUDA_TRY(launch_chained(k2, dim3((unsigned)(d.D / 64), nt), dim3(kWThreads), (size_t)WideCfg<false>::SMEM_BYTES, st, ah,
+        SENTRY_CUDA_TRY(launch_chained(k2, dim3((unsigned)wide_grid_cols(d.D), nt), dim3(kWThreads), (size_t)WideCfg<false>::SMEM_BYTES, st, ah,
                                        al, m2, nullptr, nullptr, nullptr, (__nv_bfloat16*)a.Y, plan, d.n_lists, t0, (int)nt, d.D,
                                        d.k_c, kc_pad, ctx->sm_count, a.status));
     }
@@ -314,6 +302,10 @@ int ffn_wide_kc_pad(int k_c) { return (k_c + 127) / 128 * 128; }
 // The hidden buffer for a call of at most max_tiles row tiles.
 size_t ffn_wide_hidden_bytes(int kc_pad, long long max_tiles) {
     return (size_t)(max_tiles < kWideTiles ? max_tiles : kWideTiles) * 128 * kc_pad * 2 * 2;
+}
+// CTAs of GEMM 1's first launch
+long long ffn_wide_first_ctas(int k_c, long long max_tiles) {
+    return (max_tiles < kWideTiles ? max_tiles : kWideTiles) * wide_grid_cols(k_c);
 }
 int launch_ffn_wide(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c, int kc_pad, int max_tiles,
                     void* hidden, cudaStream_t st) {

@@ -1,4 +1,5 @@
-// Arithmetic of ffn_wide.cu that needs no GPU, so that a CPU test can compile it too: the GELU of GEMM 1's epilogue.
+// Arithmetic of ffn_wide.cu that needs no GPU, so that a CPU test can compile it too: the GELU of GEMM 1's epilogue, and
+// the tiles' widths.
 #pragma once
 #include <math.h>
 
@@ -33,4 +34,21 @@ SENTRY_HD float gelu_two_part(float z, Rcp rcp, Ex2 ex2) {
     p = fmaf(p, s, 0.398942199f);
     const float near = fmaf(s, p, 0.5f * z), far = fmaf(-a, r * e, fmaxf(z, 0.f));
     return s < 1.f ? near : far;
+}
+
+// Columns of a tile of GEMM 1 (first) and 2: a multiple of 32 from 64 to wide_bn_max; wide_ctas of them run on an SM.
+SENTRY_HD constexpr int wide_bn_max(bool first) { return first ? 160 : 192; }
+SENTRY_HD constexpr int wide_ctas(bool first) { return first ? 2 : 1; }
+// Column tiles that a launch has CTAs for: what the narrowest tiles need, since the width is chosen on the device.
+SENTRY_HD constexpr int wide_grid_cols(int cols) { return (cols + 63) / 64; }
+// The width where R row tiles have `cols` columns: the rounds times what a K block costs in shared-memory traffic, which is that
+// of A and the columns of B (in units of B's).
+SENTRY_HD int wide_bn(bool first, int R, int cols, int sm_count) {
+    const int slots = sm_count * wide_ctas(first);
+    int best = 64, best_cost = 0x7fffffff;
+    for (int bn = 64; bn <= wide_bn_max(first); bn += 32) {
+        const int items = R * ((cols + bn - 1) / bn), cost = (items + slots - 1) / slots * ((first ? 128 : 170) + bn);
+        if (cost < best_cost) { best = bn; best_cost = cost; }
+    }
+    return best;
 }

@@ -1,5 +1,5 @@
 """The arithmetic of the wide FFN that needs no GPU (csrc/ffn_wide_math.cuh), compiled for the host: the error of its GELU
-against float64 and against the erf form of the math library."""
+against float64 and against the erf form of the math library, and the widths of its tiles."""
 import ctypes
 import os
 import subprocess
@@ -21,6 +21,9 @@ extern "C" void gelu(const float* z, float* out, long n, int rcp_ulps, int ex2_u
         out[i] = gelu_two_part(z[i], [=](float x) { return ulps((float)(1.0 / (double)x), rcp_ulps); },
                                [=](float x) { return ulps((float)exp2((double)x), ex2_ulps); });
 }
+extern "C" int bn(int first, int R, int cols, int sm_count) { return wide_bn(first != 0, R, cols, sm_count); }
+extern "C" int bn_max(int first) { return wide_bn_max(first != 0); }
+extern "C" int grid_cols(int cols) { return wide_grid_cols(cols); }
 extern "C" void gelu_erf(const float* z, float* out, long n) {
     for (long i = 0; i < n; ++i) out[i] = 0.5f * z[i] * (1.f + erff(z[i] * 0.70710678f));
 }
@@ -76,3 +79,16 @@ def test_gelu_of_special_values(lib):
     finite = z[:-3].astype(np.float64)
     np.testing.assert_allclose(g[:-3], np.where(np.abs(finite) < 1, finite / 2, np.maximum(finite, 0)), rtol=1e-7, atol=0)
     assert np.isnan(g[-3:]).all()
+
+
+@pytest.mark.parametrize("first", [1, 0])
+def test_every_column_has_a_block(lib, first):
+    """The launch's blocks cover the columns at whichever width the device takes, and every width is taken."""
+    taken = set()
+    for sm_count in (148, 132):
+        for R in list(range(1, 129)):
+            for cols in range(64, 1665, 64) if first else range(64, 1025, 64):
+                bn = lib.bn(first, R, cols, sm_count)
+                assert 64 <= bn <= lib.bn_max(first) and bn % 32 == 0 and -(-cols // bn) <= lib.grid_cols(cols)
+                taken.add(bn)
+    assert taken == set(range(64, lib.bn_max(first) + 1, 32))
