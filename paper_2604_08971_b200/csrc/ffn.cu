@@ -762,10 +762,11 @@ int launch_ffn(sentry_ctx* ctx, const FfnArgs& a, void* ws, size_t ws_bytes, con
         if (zsplit > 32) zsplit = 32;
         const size_t pack_blocks = packed != nullptr ? 0
                                    : (tc ? k_major_blocks(d, kc_pad) : 2 * (size_t)d.n_lists * ((per + 255) / 256));
-        // the next kernel starts early where the CTAs of its launch leave half of the SMs free: one window of 64 tokens 31.7 -> 31.3 us
-        // a step; on 64 windows x 1024 tokens, whose FFN has a CTA for every SM, 116 -> 119.  The wide form (its launch has a CTA for
-        // every 64 channels), a call early / not: 32 CTAs (46 rows of d_model 768, 967 channels) 23.4 / 23.8 us, 40 25.3 / 25.4, 60 22.1 / 22.1,
-        // 84 24.2 / 24.0, 100 26.3 / 26.1, 132 27.9 / 27.4, 180 29.6 / 29.6; at d_model 192 not early is faster on few, too (12 CTAs 14.0 / 13.4)
+        // the next kernel starts early where the CTAs of its launch leave half of the SMs free: one window of 64 tokens 31.7 -> 31.3
+        // us a step; on 64 windows x 1024 tokens, whose FFN has a CTA for every SM, 116 -> 119.  The wide form, whose launch has a
+        // CTA for every 64 channels, a call early / not: 32 CTAs (46 rows of d_model 768, 967 channels) 23.4 / 23.8 us, 40
+        // 25.3 / 25.4, 60 22.1 / 22.1, 84 24.2 / 24.0, 96 21.6 / 21.8, 100 26.3 / 26.1, 132 27.9 / 27.4, 180 29.6 / 29.6; at d_model
+        // 192 not early is faster on few, too (12 CTAs 14.0 / 13.4)
         const long long next = ffn_wide_supported(d) ? ffn_wide_first_ctas(d.k_c, tiles_bound(d)) : tiles_bound(d);
         const int early = next <= ctx->sm_count / 2;
         const bool grouped = d.B >= kGroupPlanB;

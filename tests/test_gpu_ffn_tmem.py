@@ -44,11 +44,12 @@ def test_one_row(D):
         sn.close()
 
 
-@pytest.mark.parametrize("k_c,n_lists", [(65, 7), (200, 3), (384, 1), (130, 64)])
-def test_pairs_equal_single_ctas(k_c, n_lists):
-    """A large call (pairs of CTAs) against the same samples in small calls (single CTAs): equal bits, and equal again."""
+@pytest.mark.parametrize("k_c,n_lists,B", [(65, 7, 1280), (200, 3, 1800), (384, 1, 1280), (130, 64, 1800), (512, 7, 900), (512, 1, 640)])
+def test_pairs_equal_single_ctas(k_c, n_lists, B):
+    """A large call (pairs of CTAs where there is more than one chunk of 128 channels) against the same samples in small calls
+    (single CTAs): equal bits, and equal again."""
     gen = torch.Generator(device="cuda").manual_seed(k_c)
-    B, T, D, F = 1280, 100, 256, 512
+    T, D, F = 100, 256, 512
     X = torch.randn((B, T, D), generator=gen, device="cuda").bfloat16()
     W1 = torch.randn((D, F), generator=gen, device="cuda").mul_(0.05).bfloat16()
     W2 = torch.randn((F, D), generator=gen, device="cuda").mul_(0.05).bfloat16()

@@ -67,6 +67,34 @@ def test_moe_ffn_matches_oracle(case):
         sn.close()
 
 
+@pytest.mark.parametrize("E,k_c,N", [(5, 450, 24000), (16, 512, 24000), (3, 256, 48000)])
+def test_moe_pairs_equal_single_ctas(E, k_c, N):
+    """A call whose row tiles go to pairs of CTAs (d_model 256; results scattered by the plan's destination rows) against the same tokens in
+    small calls (single CTAs): equal bits, tokens without an expert zero."""
+    D, F, top_k, step = 256, 1024, 2, 3000
+    gen = torch.Generator(device="cuda").manual_seed(E)
+    X = torch.randn((N, D), generator=gen, device="cuda").bfloat16()
+    W1 = torch.randn((E, D, F), generator=gen, device="cuda").mul_(0.05).bfloat16()
+    W2 = torch.randn((E, F, D), generator=gen, device="cuda").mul_(0.05).bfloat16()
+    kept = torch.rand((E, F), generator=gen, device="cuda").topk(k_c, dim=1).indices.sort(dim=1).values.int().contiguous()
+    # expert e is as popular as 1 / (e + 1); one token in twenty has no expert
+    pop = torch.log(1.0 / torch.arange(1, E + 1, device="cuda"))
+    u = torch.rand((N, E), generator=gen, device="cuda").clamp_(1e-9, 1 - 1e-7)
+    ids = (pop - torch.log(-torch.log(u))).topk(top_k, dim=1).indices.int()
+    ids[torch.rand((N,), generator=gen, device="cuda") < 0.05] = -1
+    ids = ids.contiguous()
+    wts = torch.rand((N, top_k), generator=gen, device="cuda")
+    sn = sentry.Sentry(0)
+    try:
+        packed = sn.moe_prepack(W1, W2, kept)
+        call = lambda a, b: sn.moe_ffn_fwd(X[a:b].contiguous(), ids[a:b].contiguous(), wts[a:b].contiguous(), packed=packed, F=F, E=E, k_c=k_c)
+        Y = call(0, N)
+        assert torch.equal(Y, torch.cat([call(a, min(a + step, N)) for a in range(0, N, step)]))
+        assert torch.all(Y[ids[:, 0] < 0] == 0) and sn.last_status() == 0
+    finally:
+        sn.close()
+
+
 def test_moe_one_expert_top1_equals_plain_ffn():
     """E = 1, top-1, weight 1: bit for bit the channel-compacted FFN on the same rows."""
     m = synth.generate_moe(640, 256, 512, 1, 1, 256, "bf16", seed=9)
