@@ -45,14 +45,15 @@ namespace {
 // holds 128 elements instead of 64), the accumulators stay fp32, Y is stored as bf16.
 template <int D, bool FP8 = false>
 struct Cfg {
+    static_assert(FP8 || D == 384, "16-bit operands at the other widths: ffn_tmem.cu");
     static constexpr int EPB = FP8 ? 128 : 64;         // elements per 128-byte operand row
     static constexpr int CH = (D == 384) ? 128 : 256;  // kept channels per chunk
     static constexpr int CH16 = FP8 ? CH / 2 : CH;     // a chunk's width in the 16-bit units of the weight maps
     static constexpr int KB1 = D / EPB;                // X blocks per tile = K blocks of GEMM1
     static constexpr int H_COL0 = (D == 384) ? 384 : 256;  // TMEM column of the hidden accumulator
-    static constexpr int NXS = (D == 128 || FP8) ? 4 : KB1;   // X block slots (two tiles' worth where they are few)
+    static constexpr int NXS = FP8 ? 4 : KB1;          // X block slots (two tiles' worth where they are few)
     static constexpr int NHS = CH / EPB;               // hidden blocks per chunk
-    static constexpr int NBATCH = CH / 128;            // 64-column batches per epilogue warp
+    static constexpr int NBATCH = CH / 128;            // 64-column batches per epilogue warp (16-bit: one)
     static constexpr int SPG = (D == 384) ? 3 : KB1;   // weight stages per chunk of GEMM1 (= of GEMM2)
     static constexpr bool COLSPLIT = (D == 384);   // tail tiles shared by three CTAs, a third of Y each
     // FP8 with d_model = 384: one 128-channel hidden block, written by all eight epilogue warps, and two more
@@ -448,11 +449,8 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__
         // lane holds one row; 64 columns at a time go through this warp's 4 KB piece of the
         // hidden-block buffer (free while Y is complete and this warp has not yet written its
         // next hidden block there) so that the global stores cover whole 128-byte row segments.
-        constexpr int kDrainBlk = C::NBATCH - 1;
-        // (FP8: a warp writes one 128-channel hidden block, rows of its own quarter: that piece)
-        const uint32_t stg = C::FP8_384 ? hs + (uint32_t)(1 + half) * kBlockBytes + (uint32_t)quarter * 4096u
-                           : FP8 ? hs + (uint32_t)half * kBlockBytes + (uint32_t)quarter * 4096u
-                                 : hs + (uint32_t)(half * C::NBATCH + kDrainBlk) * kBlockBytes + (uint32_t)quarter * 4096u;
+        // (FP8 at 384: the two blocks that only stage Y)
+        const uint32_t stg = hs + (uint32_t)((C::FP8_384 ? 1 : 0) + half) * kBlockBytes + (uint32_t)quarter * 4096u;
         auto drain_y = [&](uint32_t t_idx, int32_t grow, int third) {
             if (!warp_wait(&misc->y_full, t_idx & 1u, abort_flag)) { ok = false; return; }
             ptx::tc_fence_after_sync();
@@ -524,10 +522,10 @@ ffn_tc_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__
                     // 32 rows x 64 columns of the hidden accumulator -> registers
                     const int blk = half * C::NBATCH + j;        // hidden block = 64 channels (FP8: column batch)
                     // Y of the previous tile is complete about now (its last GEMM2 was queued right
-                    // after this tile's first GEMM1): store it before this warp's last batch of the
-                    // chunk is loaded, while no accumulator values are held in registers
-                    // (FP8: before the first batch -- the staging piece is the block this warp is about to write)
-                    if (j == (FP8 ? 0 : C::NBATCH - 1) && c == 0 && ti > 0) {
+                    // after this tile's first GEMM1): store it before this warp's first batch of the
+                    // chunk is loaded, while no accumulator values are held in registers and the staging
+                    // piece is the block this warp is about to write
+                    if (j == 0 && c == 0 && ti > 0) {
                         drain_y((uint32_t)(ti - 1), prev_row, -1);   // a split tile is the last one: never drained here
                         if (!ok) break;
                     }
@@ -625,14 +623,15 @@ __global__ void __launch_bounds__(128, 1) wait_expiry_selftest_kernel(long long 
     tc_cta_teardown(abort_flag, status, tmem, 32);
 }
 
-template <int D, bool F16>
-int launch_d(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c, int kc_pad,
+template <bool F16>
+int launch_384(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1c, void* w2c, int kc_pad,
              int max_tiles, cudaStream_t st) {
+    constexpr int D = 384;
     const sentry_ffn_desc& d = a.d;
     CUtensorMap m1, m2a, m2b;
     const uint64_t r1 = (uint64_t)d.n_lists * kc_pad, r2 = (uint64_t)d.n_lists * D;
-    if (!make_weight_map(&m1, w1c, r1, D, Cfg<D>::CH == 256 ? 256 : 128)) return SENTRY_ERR_CUDA;
-    if (!make_weight_map(&m2a, w2c, r2, kc_pad, D >= 256 ? 256 : 128)) return SENTRY_ERR_CUDA;
+    if (!make_weight_map(&m1, w1c, r1, D, Cfg<D>::CH)) return SENTRY_ERR_CUDA;
+    if (!make_weight_map(&m2a, w2c, r2, kc_pad, 256)) return SENTRY_ERR_CUDA;
     if (!make_weight_map(&m2b, w2c, r2, kc_pad, 128)) return SENTRY_ERR_CUDA;
     auto kern = ffn_tc_kernel<D, F16>;
     SENTRY_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<D>::SMEM_BYTES));
@@ -706,8 +705,8 @@ int launch_ffn_tc(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* 
     const bool f16 = a.d.dtype == SENTRY_F16;
     if (ffn_tmem_supported(a.d)) rc = launch_ffn_tmem(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
     else if (a.d.D != 384) return SENTRY_ERR_UNSUPPORTED;
-    else rc = f16 ? launch_d<384, true>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
-                  : launch_d<384, false>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
+    else rc = f16 ? launch_384<true>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
+                  : launch_384<false>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
     if (rc != SENTRY_OK) return rc;
     SENTRY_CUDA_TRY(cudaGetLastError());
     return SENTRY_OK;
