@@ -629,7 +629,7 @@ __device__ __forceinline__ void fused_score_pass(const __nv_bfloat16* __restrict
 // are not unrolled: attention of 4096 x 256 tokens took 560 us with bodies of four keys and three for the rest, 456 with two and
 // one, 427 with two alone, 422 with the other loops rolled.  Larger CTAs do not gain by the last steps (256 x 1024: 124 us with
 // bodies of two and one, 128 with TIGHT).  FOUR false: four heads of d = 32 go in two passes, and the other bodies keep more
-// registers: 408 us; a single wave of CTAs, which waits for the slowest, takes the one pass (256 x 192 tokens 31 us, 37 with two).
+// registers: 408 us (launch_d has the line).
 template <int D, bool TIGHT, bool FOUR>
 __global__ void __launch_bounds__(512, 1)
 attend_fused_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16* __restrict__ K,
@@ -1114,6 +1114,12 @@ int launch_d(sentry_ctx* ctx, const AttendArgs& a, cudaStream_t st) {
         // one big CTA, or two per SM; short sequences get small CTAs (more of them per SM: their
         // phases are a few barrier-separated microseconds each, so concurrency is what helps)
         const int threads = fused_bytes > 100 * 1024 ? 512 : (d.T <= kSmallT ? 128 : 256);
+        // groups that keep all four of their heads of d = 32, in two passes from four waves of 128-thread CTAs on.  Change
+        // against the one pass in %, T = 64, 128, 192, 256 (8 heads in 2 groups): 4 kept, samples missing modalities, 4 waves
+        // -2.4 -2.5 -2.2 -1.0, 8 waves -3.0 -3.1 -2.3 -1.9, 24 and 16 waves -3.7 -4.1; 6 kept -3.8 -2.3 -1.3 -0.4, -4.3 -3.9
+        // -2.3 -2.0, -5.9 -4.9; all kept -1.2 +0.6 +1.6 +1.9, +0.2 +0.5 +1.4 +1.9, -0.9 +0.4; every token present within 1 of
+        // these.  Up to three waves either way (1 wave -3.0 to +0.9, 1.5 -3.6 to +4.4, 2 and 3 -2.8 to +2.3).  At d = 16 two
+        // passes are slower at every size (all kept +7 to +22, 4 kept -1 to +18); d = 64 takes two heads a pass anyway
         const long long waves = (long long)d.B * d.Hk / ((long long)ctx->sm_count * (512 / threads));
         auto kern = threads != 128 ? attend_fused_bf16_kernel<D, false, true>
                     : (D == 32 && waves >= 4) ? attend_fused_bf16_kernel<D, true, D != 32>

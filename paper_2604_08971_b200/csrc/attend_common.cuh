@@ -48,9 +48,9 @@ constexpr int kScoreThreads = 256;
 constexpr int kCoreThreads = 256;
 constexpr int kCoreWarps = kCoreThreads / 32;
 constexpr int kKeyTile = 64;
-constexpr int kMaxActive = 48;
+constexpr int kMaxActive = 48; // U <= 45 for T <= 8103 with c = 5 (checked on the host)
 constexpr int kSmallT = 256;   // fused attention: sequences up to this length run in 128-thread CTAs
-constexpr int kOrderMaxBatch = 1024; // batches up to this size are walked heaviest-sample-first     // U <= 45 for T <= 8103 with c = 5 (checked on the host)
+constexpr int kOrderMaxBatch = 1024; // batches up to this size are walked heaviest-sample-first
 
 // Row layout in shared memory: rows of D bf16, 16-byte chunks XOR-swizzled so that both
 // 8-consecutive-row matrix loads and random row gathers spread over the banks.

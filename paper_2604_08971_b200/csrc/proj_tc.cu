@@ -12,12 +12,16 @@
 // Before the stages warp 0 allocates tensor memory, warp 1 sets up barriers and slices and warps 2-7 list the tile's tokens, at
 // once.  Then warp 0 feeds the weights by TMA, warp 1 issues the UMMAs, warps 4-7 gather the rows, and all eight store: 64
 // accumulator columns at a time pass through shared memory so that eight lanes write 128 consecutive bytes.
-// Bound by what a CTA does one after the other (19 K cycles at B = 128, T = 512, D = 384 with 15 slices of 32: 3.4 K to the first
-// copy, 4.5 K until X and weights of the first stage are there, 7.5 K for six stages of 48 KB, two in flight, 3.5 K to store), which
-// two CTAs per SM overlap in part.  One after the other with four storing warps, list and set-up took 2 and 3 K cycles:
-// 128 x 512 tokens, 9 of 12 heads, QKV 63.4 -> 61.5 us, OUT 40.9 -> 37.7; 16 x 4096 at D = 256 46.5 -> 42.4 and 26.4 -> 20.9; 256 x 256 36.6 -> 35.4
-// and 22.9 -> 17.9.  Slower: two row tiles to a CTA that share the weights, one CTA per SM (63 -> 74 and 41 -> 53), three CTAs per SM with
-// 128 columns (65 and 42; 46 -> 65 on 16 x 4096); without effect: box coordinates kept in registers (issue of a stage 1.2 -> 0.7 K cycles).
+// Bound by what a CTA does one after the other (19 K cycles at B = 128, T = 512, D = 384 with 15 slices of 32: 3.4 K to the
+// first copy, 4.5 K until X and weights of the first stage are there, 7.5 K for six stages of 48 KB, two in flight, 3.5 K to
+// store), which two CTAs per SM overlap in part.  One after the other with four storing warps, list and set-up took 2 and 3 K
+// cycles: 128 x 512 tokens, 9 of 12 heads, QKV 63.4 -> 61.5 us, OUT 40.9 -> 37.7; 16 x 4096 at D = 256 46.5 -> 42.4 and 26.4 ->
+// 20.9; 256 x 256 36.6 -> 35.4 and 22.9 -> 17.9.  Slower: two row tiles to a CTA that share the weights, one CTA per SM (63 ->
+// 74 and 41 -> 53), three CTAs per SM with 128 columns (65 and 42; 46 -> 65 on 16 x 4096); without effect: box coordinates kept
+// in registers (issue of a stage 1.2 -> 0.7 K cycles).
+// A tile without a present token (missing modalities at T above 128) sets up and frees before it leaves, at once with its token
+// count.  Calls full of them gained with the rest: 256 x 1024, 12 % present, QKV 29.0 -> 26.7 and OUT 47.4 -> 38.5; 16 x 4096,
+// 3 % 15.0 -> 12.5 and 21.8 -> 14.3; 1024 x 256, 50 % 47.7 -> 48.0 and 54.2 -> 48.5.
 // Measured there, the whole layer 262 -> 206 us: one CTA per SM that loaded X, multiplied slice by slice and then stored
 // took 73 us for QKV and 61 for OUT.
 // Every wait is bounded; on expiry the CTA raises SENTRY_STATUS_BIT_TIMEOUT and unwinds.

@@ -86,8 +86,12 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// Arrival at another CTA's barrier.  What it announces is ordered by the fences of its own proxy (tcgen05.fence, fence.proxy.async
-// before it); a release at cluster scope would wait about 600 ns for every write in flight.
+// Arrival at another CTA's barrier, in the default form; a release at cluster scope would wait about 600 ns for every write in
+// flight. What it announces is ordered by the fence of the proxy that reads it, which every announcing lane executes before the
+// warp's one arrival: accumulator reads and hidden values written to tensor memory by tcgen05.fence::before_thread_sync (behind
+// tcgen05.wait), operand rows in shared memory by fence.proxy.async, which covers the rows that cp.async copied (behind its
+// wait) and the zero rows of plain st.shared alike.  Each CTA's rows are read from its own memory; the weights, which both
+// read from both, are announced by their TMA.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
