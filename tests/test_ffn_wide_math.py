@@ -92,3 +92,13 @@ def test_every_column_has_a_block(lib, first):
                 assert 64 <= bn <= lib.bn_max(first) and bn % 32 == 0 and -(-cols // bn) <= lib.grid_cols(cols)
                 taken.add(bn)
     assert taken == set(range(64, lib.bn_max(first) + 1, 32))
+
+
+def test_gpu_shapes_take_every_width(lib):
+    from tests.test_gpu_ffn_wide import WIDTHS
+    first, second, last = set(), set(), set()
+    for D, k_c, tiles in WIDTHS:
+        cols = (k_c + 63) // 64 * 64
+        a, b = lib.bn(1, tiles, cols, 148), lib.bn(0, tiles, D, 148)
+        first.add(a), second.add(b), last.update((cols % a, D % b))
+    assert first == set(range(64, 161, 32)) and second == set(range(64, 193, 32)) and {32, 64, 128} <= last

@@ -91,6 +91,35 @@ def test_wide_ffn_hidden_value_beyond_the_storage_type(dtype, x, scale):
         sn.close()
 
 
+# (d_model, kept channels, row tiles): with 148 SMs every width of both GEMMs' column tiles, and last tiles of 32 to 128 columns
+# (tests/test_ffn_wide_math.py holds the list to that)
+WIDTHS = [(64, 100, 1), (192, 300, 60), (320, 129, 99), (192, 385, 60), (320, 300, 75), (192, 385, 75), (320, 385, 75),
+          (320, 300, 99), (768, 1229, 33)]
+
+
+@pytest.mark.parametrize("D,k_c,tiles", WIDTHS)
+def test_wide_ffn_tile_widths(D, k_c, tiles):
+    """Against the same sums in float64.  A stored hidden value is off by up to 2^-17 of itself (head and remainder), its GELU and
+    the fp32 sums by less; the sum of a result's absolute terms is about 0.65 sqrt(k_c) times the results' RMS, twice that
+    in the largest rows: 2^-16 sqrt(k_c) RMS, beside the half unit of the stored result."""
+    gen = torch.Generator(device="cuda").manual_seed(D + k_c)
+    rows, F = tiles * 128 - 37, k_c + 50
+    X = torch.randn((1, rows, D), generator=gen, device="cuda").bfloat16()
+    W1 = torch.randn((D, F), generator=gen, device="cuda").mul_(D ** -0.5).bfloat16()
+    W2 = torch.randn((F, D), generator=gen, device="cuda").mul_(k_c ** -0.5).bfloat16()
+    kept = torch.rand((F,), generator=gen, device="cuda").topk(k_c).indices.sort().values
+    sn = sentry.Sentry(0)
+    try:
+        Y = sn.ffn_fwd(X, W1, W2, kept.int().reshape(1, -1).contiguous(), torch.zeros(1, dtype=torch.int32, device="cuda"))
+        want = torch.nn.functional.gelu(X[0].double() @ W1.double()[:, kept]) @ W2.double()[kept]
+        half_ulp = torch.exp2(torch.floor(torch.log2(want.abs().clamp_min(1e-30))) - 8)
+        excess = ((Y[0].double() - want).abs() - half_ulp).clamp_min(0).max()
+        assert float(excess) <= 2.0 ** -16 * k_c ** 0.5 * float(want.square().mean().sqrt())
+        assert sn.last_status() == 0
+    finally:
+        sn.close()
+
+
 def test_wide_moe_matches_oracle():
     m = synth.generate_moe(300, 512, 256, 5, 2, 100, "bf16", seed=3, skew=1.0)
     sn = sentry.Sentry(0)
