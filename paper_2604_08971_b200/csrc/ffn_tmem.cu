@@ -273,12 +273,15 @@ ffn_tmem_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant
         auto wait_all = [&](uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1, uint32_t b2, uint32_t p2) -> bool {
             // (in a pair, the other CTA's copies and threads arrive on them too)
             auto probe = [&](uint32_t b, uint32_t ph_) { return P == 2 ? ptx::mbar_try_wait_cluster(b, ph_) : ptx::mbar_try_wait(b, ph_); };
-            bool p = probe(b0, p0);
-            if (b1 != 0u) p &= probe(b1, p1);
-            if (b2 != 0u) p &= probe(b2, p2);
-            if (!__all_sync(0xffffffffu, p)) {
+            auto probe_all = [&]() {
+                bool p = probe(b0, p0);
+                if (b1 != 0u) p &= probe(b1, p1);
+                if (b2 != 0u) p &= probe(b2, p2);
+                return p;
+            };
+            if (!__all_sync(0xffffffffu, probe_all())) {
                 if (!__all_sync(0xffffffffu, wait_each_slow(b0, p0, b1, p1, b2, p2, 0u, 0u, abort_flag))) return false;
-                if constexpr (P == 2) asm volatile("fence.acq_rel.cluster;" ::: "memory");
+                if constexpr (P == 2) probe_all();   // acquired at cluster scope too: no phase moves on before this warp does
             }
             ptx::tc_fence_after_sync();
             return true;
@@ -356,6 +359,7 @@ ffn_tmem_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant
         auto publish_oldest = [&]() {
             cp_async_wait_pending((int)(gx - published) - 1);
             ptx::fence_proxy_async_smem();
+            if constexpr (P == 2) ptx::fence_release_smem_cluster();
             arrive_issuer(TM_BAR(mb, x_full) + 8u * (published % C::NXS));
             ++published;
         };
