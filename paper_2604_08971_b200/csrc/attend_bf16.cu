@@ -511,7 +511,7 @@ attend_core_bf16_kernel(const __nv_bfloat16* __restrict__ Q, const __nv_bfloat16
 // One CTA per (sample, KV group) does the whole of SentryAttend for the group's kept heads
 // when the group's present K and V rows fit in shared memory (T up to ~1.5 k at d = 32):
 //   stage K, V (gathered present rows, once) -> sparsity scores from shared memory ->
-//   top-U per head (one warp per head, radix selection) -> Eq. 6 on the active rows with the
+//   top-U per head (one warp per head; long lists: the whole block) -> Eq. 6 on the active rows with the
 //   warp-level tensor-core MMA straight from the resident K/V -> context rows and zero rows.
 // Q, K, V are read from HBM once and O is written once: the algorithmic traffic.
 
@@ -622,7 +622,7 @@ __device__ __forceinline__ void fused_score_pass(const __nv_bfloat16* __restrict
     }
 }
 
-// grid B*Hk, 256 or 512 threads.  Dynamic smem: valid[T] u16 | kind[T] u8 | actbits[4][T/32] u32 |
+// grid B*Hk, 128 (TIGHT), 256 or 512 threads.  Dynamic smem: valid[T] u16 | kind[T] u8 | actbits[4][T/32] u32 |
 // keys[4][T] u32 | hist[4][256] | K[Tpad][D] | V[Tpad][D]   (Tpad = T rounded up to 64).
 // TIGHT (128-thread CTAs, four to an SM, T <= kSmallT): CTAs of an SM are in different phases, and the instructions of all phases
 // together are what an SM's instruction cache has to hold.  The score loop is then a body of two keys, and loops that are not hot

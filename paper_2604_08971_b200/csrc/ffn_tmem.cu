@@ -20,7 +20,7 @@
 // both: 2300 cycles a chunk.  Per call with the row plan, hidden tile in shared memory / P = 1 / P = 2: 149 k rows, d_model 256,
 // 512 channels 80 / 79 / 72 us; 599 k rows 303 / 298 / 270; 65 k rows 38.6 / 37.4 / 36.1; 37 k rows 26.2 / 24.4 / 25.5; 2.2 k rows
 // 15.4 / 14.4 / 15.1; 35 k rows of d_model 128, 256 channels 16.7 / 14.1 / 16.0.  So pairs at d_model 256, where the weights are what is
-// moved, from a number of rounds and chunks on (launch_ffn_tmem), and single CTAs otherwise.
+// moved, from a number of rounds and chunks on (ffn_pair_rule.cuh), and single CTAs otherwise.
 //
 // Warp roles (512 threads): warp 0 = weight TMA producer (owns TMEM), warp 1 = UMMA issuer, warps 3-6 = X row gather, warps 7-14 =
 // epilogue (two warps per TMEM lane quarter), warp 15 = zero rows of absent tokens.  Every wait is bounded; on expiry the CTA
@@ -29,6 +29,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "ffn_pair_rule.cuh"
 #include "ffn_plan.cuh"
 #include "ffn_tc_common.cuh"
 #include "tc_common.cuh"
@@ -529,20 +530,7 @@ int launch_ffn_tmem(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void
     const bool f16 = a.d.dtype == SENTRY_F16;
     if (a.d.D == 128) return f16 ? launch_d<128, true, 1>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
                                  : launch_d<128, false, 1>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
-    // Pairs save about a fifth of a chunk's time and cost 1.2 us once, so they pay from a number of rounds of tiles times chunks
-    // on: 9.  Measured with every token present, single CTAs / pairs in us: 2 chunks, 3.0 rounds 25.5 / 25.4, 5.3 rounds 35.6 / 35.0,
-    // 9.5 56.8 / 53.8; 3 chunks, 2.1 rounds 28.7 / 28.8, 3.5 31.4 / 30.4; 4 chunks, 2.1 rounds 33.0 / 32.7, 3.5 37.1 / 35.3; 8 chunks,
-    // 2.1 rounds 60.2 / 55.7.  A single chunk gains nothing at any number (3.0 rounds 18.4 / 19.5, 26 103.3 / 103.3).
-    // With masks max_tiles is what there is when every token is present, and a list with an odd number of tiles leaves half of
-    // a pair idle.  Several lists are the sign of samples that miss modalities: 18, so that half of the tokens still pay.  What
-    // pairs change where 100, 80, 60 and 45 % of the tokens are present, in %:
-    //   7 lists   512 channels  3.5 rounds  -1.3 +0.9 +3.2 +3.8    4.8  -5.2 -2.2 +1.0 +3.4    6.1  -7.9 -8.1 -4.8  0.0
-    //             256           6.1         -1.2  0.0 +1.6 +1.0    9.5  -5.1 -5.7 -0.2  0.0
-    //   1 list    512           3.0         -3.8 -2.3 +2.1 +2.6    3.5  -3.6 -1.7 -0.2 +1.4    4.1  -5.8 -3.4 -0.2 +2.9
-    //             256           4.1         -2.0 -0.3 +3.4 +2.5    6.1  -2.9 -1.5 +0.3 +0.2
-    // so 13 with one list.  Every thread adds up the lists: at most 64.
-    const int chunks = (a.d.k_c + 127) / 128, need = a.ids == nullptr ? 9 : a.d.n_lists == 1 ? 13 : 18;
-    if (chunks > 1 && (long long)max_tiles * chunks >= (long long)need * ctx->sm_count && a.d.n_lists <= 64)
+    if (ffn_takes_pairs(a.ids != nullptr, a.d.n_lists, a.d.k_c, max_tiles, ctx->sm_count))
         return f16 ? launch_d<256, true, 2>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)
                    : launch_d<256, false, 2>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st);
     return f16 ? launch_d<256, true, 1>(ctx, a, plan, w1c, w2c, kc_pad, max_tiles, st)

@@ -44,15 +44,22 @@ def test_one_row(D):
         sn.close()
 
 
-@pytest.mark.parametrize("k_c,n_lists,B", [(65, 7, 1280), (200, 3, 1800), (384, 1, 1280), (130, 64, 1800), (512, 7, 900), (512, 1, 640)])
-def test_pairs_equal_single_ctas(k_c, n_lists, B):
+# kept channels, lists, samples, element type; with 148 SMs all but the first go to pairs (tests/test_ffn_pair_rule.py holds them to that)
+PAIRS = [(65, 7, 1280, "bf16"), (200, 3, 1800, "bf16"), (384, 1, 1280, "bf16"), (130, 64, 1800, "bf16"), (512, 7, 900, "bf16"),
+         (512, 1, 640, "bf16"), (129, 5, 1900, "f16"), (257, 1, 900, "f16"), (512, 7, 900, "f16")]
+PAIR_T, PAIR_STEP = 100, 160
+
+
+@pytest.mark.parametrize("k_c,n_lists,B,dtype", PAIRS)
+def test_pairs_equal_single_ctas(k_c, n_lists, B, dtype):
     """A large call (pairs of CTAs where there is more than one chunk of 128 channels) against the same samples in small calls
     (single CTAs): equal bits, and equal again."""
     gen = torch.Generator(device="cuda").manual_seed(k_c)
-    T, D, F = 100, 256, 512
-    X = torch.randn((B, T, D), generator=gen, device="cuda").bfloat16()
-    W1 = torch.randn((D, F), generator=gen, device="cuda").mul_(0.05).bfloat16()
-    W2 = torch.randn((F, D), generator=gen, device="cuda").mul_(0.05).bfloat16()
+    T, D, F = PAIR_T, 256, 512
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float16
+    X = torch.randn((B, T, D), generator=gen, device="cuda").to(dt)
+    W1 = torch.randn((D, F), generator=gen, device="cuda").mul_(0.05).to(dt)
+    W2 = torch.randn((F, D), generator=gen, device="cuda").mul_(0.05).to(dt)
     u = torch.rand((n_lists, F), generator=gen, device="cuda")
     kept = u.topk(k_c, dim=1).indices.sort(dim=1).values.int().contiguous()
     ids = torch.tensor([0] * 41 + [1] * 33 + [2] * 26, dtype=torch.int32, device="cuda")
@@ -63,7 +70,7 @@ def test_pairs_equal_single_ctas(k_c, n_lists, B):
     try:
         Y = sn.ffn_fwd(X, W1, W2, kept, lists, ids, masks)
         assert torch.equal(Y, sn.ffn_fwd(X, W1, W2, kept, lists, ids, masks))
-        step = 160
+        step = PAIR_STEP
         for b in range(0, B, step):
             part = sn.ffn_fwd(X[b:b + step].contiguous(), W1, W2, kept, lists[b:b + step].contiguous(), ids, masks[b:b + step].contiguous())
             assert torch.equal(Y[b:b + step], part)

@@ -67,11 +67,15 @@ def test_moe_ffn_matches_oracle(case):
         sn.close()
 
 
-@pytest.mark.parametrize("E,k_c,N", [(5, 450, 24000), (16, 512, 24000), (3, 256, 48000)])
+PAIRS = [(5, 450, 24000), (16, 512, 24000), (3, 256, 48000)]   # experts, kept channels, tokens
+PAIR_TOP_K, PAIR_STEP = 2, 3000
+
+
+@pytest.mark.parametrize("E,k_c,N", PAIRS)
 def test_moe_pairs_equal_single_ctas(E, k_c, N):
     """A call whose row tiles go to pairs of CTAs (d_model 256; results scattered by the plan's destination rows) against the same tokens in
     small calls (single CTAs): equal bits, tokens without an expert zero."""
-    D, F, top_k, step = 256, 1024, 2, 3000
+    D, F, top_k, step = 256, 1024, PAIR_TOP_K, PAIR_STEP
     gen = torch.Generator(device="cuda").manual_seed(E)
     X = torch.randn((N, D), generator=gen, device="cuda").bfloat16()
     W1 = torch.randn((E, D, F), generator=gen, device="cuda").mul_(0.05).bfloat16()
