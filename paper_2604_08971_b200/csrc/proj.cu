@@ -11,8 +11,11 @@ namespace {
 constexpr int kProjThreads = 256;
 constexpr int kMaxSlices = 128;  // kept heads (at most 64) + 2 x referenced groups (at most 32)
 
+// Bound by the weight columns' round trips, so by the CTAs that an SM holds: four, at 64 registers.  Left to itself the compiler takes 80
+// and fewer loads on the way: 500 tokens of d_model 768, 7 of 12 heads of 64, 336 us (now 126, and 128 before the slice list was made by a
+// warp), 64 k tokens 25.0 ms (12.8, 13.4); fp32, 1600 tokens of d_model 64, 13.9 us (11.8, 14.7).
 template <typename T>
-__global__ void __launch_bounds__(kProjThreads)
+__global__ void __launch_bounds__(kProjThreads, 4)
 project_qkv_kernel(const T* __restrict__ X, const T* __restrict__ WQ, const T* __restrict__ WK,
                    const T* __restrict__ WV, const int32_t* __restrict__ kept_heads,
                    const int32_t* __restrict__ ids, const uint32_t* __restrict__ masks, int Tlen, int D, int Hq,
