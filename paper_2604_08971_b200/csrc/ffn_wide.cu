@@ -2,7 +2,7 @@
 // and an X tile must fit one SM beside the hidden tile: 128, 256, 384): any other multiple of 64 up to 1024, bf16 or fp16.
 //
 // Two tcgen05 GEMMs over the row plan, a CTA per tile of 128 rows and BN columns:
-//   1  H = gelu(X[rows] . W1c^T)   X rows gathered by 16-byte async copies, W1c by TMA; erf form
+//   1  H = gelu(X[rows] . W1c^T)   X rows gathered by 16-byte async copies, W1c by TMA
 //   2  Y[rows] = H . W2c^T         both operands by TMA
 // The hidden activations pass through a buffer of kWideTiles row tiles that stays in L2 (84 MB at 1280 channels); more
 // rows than that go in turns.  They are stored as a 16-bit head plus a 16-bit remainder (h = hi + lo to 2^-17), and
@@ -11,7 +11,9 @@
 // What bounds them: GEMM 1 its epilogue (two special-function and twenty other instructions per element, ffn_wide_math.cuh, by all
 // eight warps; with the library's erff and four warps 6 us of 13 a tile) and its row gather, GEMM 2 the shared memory that serves the UMMAs'
 // operands and the copies (128 bytes a cycle).  The column tile follows the number of row tiles, which only the device
-// knows: small calls spread over more SMs, large ones read A less often.
+// knows: small calls spread over more SMs, large ones read A less often.  GEMM 2 has one CTA per SM where an SM has a single
+// tile, and two otherwise (wide_second_one has both sides): alone from the second tile on, with its epilogues beside
+// nothing, it was slower than 128 x 128 tiles of two CTAs by up to 25 % (30 k rows of d_model 1024, 512 channels 549 -> 692 us; now 534).
 // Measured, a call with its row plan on materialised weights, before (128 x 128 tiles, erff, four epilogue warps that stored row
 // by row) and now: 3.7 k rows of d_model 768, 1229 channels in seven lists 55.1 -> 47.1 us; 524 rows, 765 channels 29.0 -> 23.8;
 // 46 rows, 967 channels 30.2 -> 24.8; 233 rows of d_model 192, 340 channels 19.0 -> 15.1; 5.6 k rows, 384 channels 21.6 -> 18.4.
@@ -32,12 +34,13 @@ constexpr int kWThreads = 256;
 constexpr int kWBlock = 128 * 128;      // bytes of 128 rows x 64 elements
 constexpr int kWideTiles = 128;         // row tiles the hidden buffer holds
 
-template <bool FIRST>
+template <int FORM>
 struct WideCfg {
+    static constexpr bool FIRST = FORM == kWideFirst;
     static constexpr int A_BLOCKS = FIRST ? 1 : 2;          // A, or A's head and remainder
-    static constexpr int BN_MAX = wide_bn_max(FIRST);
-    static constexpr int CTAS = wide_ctas(FIRST);           // per SM
-    static constexpr int STAGES = FIRST ? 3 : 4;
+    static constexpr int BN_MAX = wide_bn_max(FORM);
+    static constexpr int CTAS = wide_ctas(FORM);            // per SM
+    static constexpr int STAGES = FIRST ? 3 : CTAS == 1 ? 4 : 2;
     static constexpr int STAGE_BYTES = A_BLOCKS * kWBlock + BN_MAX * 128;
     static constexpr int TMEM_COLS = 256;
     static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 /* misc */ + 1024 /* alignment */;
@@ -83,16 +86,18 @@ __device__ __forceinline__ float gelu_wide(float z) {
         });
 }
 
-// grid (column tiles of 64, row tiles of this turn); a CTA beyond the tiles that there are at the width taken has nothing to do.
+// grid: a CTA for every 64 columns of every row tile of this turn.  The tiles that there are at the width taken go to the first ones: with
+// the idle ones among them a call of 59 row tiles, d_model 640, 500 channels took 38.2 us (now 33.1).
 // FIRST: tm_b = W1c [lists * kc_pad, D], out_h / out_l = the hidden buffer's two planes.  Otherwise tm_a_hi / tm_a_lo = those
 // planes, tm_b = W2c [lists * D, kc_pad], Y the result.
-template <bool FIRST, bool F16>
-__global__ void __launch_bounds__(kWThreads, WideCfg<FIRST>::CTAS)
+template <int FORM, bool F16>
+__global__ void __launch_bounds__(kWThreads, WideCfg<FORM>::CTAS)
 ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_constant__ CUtensorMap tm_a_lo,
                 const __grid_constant__ CUtensorMap tm_b, const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ out_h,
                 __nv_bfloat16* __restrict__ out_l, __nv_bfloat16* __restrict__ Y, FfnPlan plan, int n_lists, int tile0, int turn,
                 int D, int k_c, int kc_pad, int sm_count, unsigned int* status) {
-    using C = WideCfg<FIRST>;
+    using C = WideCfg<FORM>;
+    constexpr bool FIRST = C::FIRST;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = ptx::smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;
@@ -100,13 +105,13 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
     volatile int* abort_flag = &misc->abort_flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     grid_dependency_wait();
-    int l, row0, n_rows;
-    if (!ffn_tile_lookup(plan, n_lists, tile0 + (int)blockIdx.y, 128, l, row0, n_rows)) return;
     const int kc = (k_c + 63) / 64 * 64;                   // channels that are computed (padded ones carry zero weights)
     const int cols = FIRST ? kc : D;
-    const int bn = wide_bn(FIRST, min(plan.tile_start[n_lists] - tile0, turn), cols, sm_count);
-    const int n0 = blockIdx.x * bn;                        // first output column
-    if (n0 >= cols) return;
+    const int row_tiles = min(plan.tile_start[n_lists] - tile0, turn);
+    const int bn = wide_bn(FORM, row_tiles, cols, sm_count), across = (cols + bn - 1) / bn;
+    const int tile = (int)blockIdx.x / across, n0 = ((int)blockIdx.x - tile * across) * bn;   // row tile, first output column
+    int l, row0, n_rows;
+    if (tile >= row_tiles || !ffn_tile_lookup(plan, n_lists, tile0 + tile, 128, l, row0, n_rows)) return;
     const int n_cols = min(bn, cols - n0);                 // a multiple of 32
     const int KB = (FIRST ? D : kc) / 64;                  // 64-element K blocks
 
@@ -139,8 +144,8 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
                 const uint32_t bar = ptx::smem_u32(&misc->full[s]), dst = base + s * C::STAGE_BYTES;
                 ptx::mbar_arrive_expect_tx(bar, (FIRST ? 0 : 2 * kWBlock) + n_cols * 128);
                 if constexpr (!FIRST) {
-                    ptx::tma_load_2d(dst, &tm_a_hi, kb * 64, (int)blockIdx.y * 128, bar);
-                    ptx::tma_load_2d(dst + kWBlock, &tm_a_lo, kb * 64, (int)blockIdx.y * 128, bar);
+                    ptx::tma_load_2d(dst, &tm_a_hi, kb * 64, tile * 128, bar);
+                    ptx::tma_load_2d(dst + kWBlock, &tm_a_lo, kb * 64, tile * 128, bar);
                 }
                 for (int c = 0; c < n_cols; c += 32)
                     ptx::tma_load_2d(dst + C::A_BLOCKS * kWBlock + c * 128, &tm_b, kb * 64, l * (FIRST ? kc_pad : D) + n0 + c, bar);
@@ -219,7 +224,7 @@ ffn_wide_kernel(const __grid_constant__ CUtensorMap tm_a_hi, const __grid_consta
         int32_t grs[4];                                    // where the rows go that this lane stores pieces of
         {
             int32_t mine = -1;
-            if (row < n_rows) mine = FIRST ? (int)blockIdx.y * 128 + row : (plan.rowout ? plan.rowout : plan.rowidx)[row0 + row];
+            if (row < n_rows) mine = FIRST ? tile * 128 + row : (plan.rowout ? plan.rowout : plan.rowidx)[row0 + row];
 #pragma unroll
             for (int i = 0; i < 4; ++i) grs[i] = __shfl_sync(0xffffffffu, mine, i * 8 + (lane >> 2));
         }
@@ -275,19 +280,22 @@ int launch_wide(sentry_ctx* ctx, const FfnArgs& a, const FfnPlan& plan, void* w1
         !make_weight_map(&m2, w2c, (uint64_t)d.n_lists * d.D, kc_pad, 32) ||
         !make_weight_map(&ah, hh, (uint64_t)turn * 128, kc_pad, 128) || !make_weight_map(&al, hl, (uint64_t)turn * 128, kc_pad, 128))
         return SENTRY_ERR_CUDA;
-    auto k1 = ffn_wide_kernel<true, F16>;
-    auto k2 = ffn_wide_kernel<false, F16>;
-    SENTRY_CUDA_TRY(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, WideCfg<true>::SMEM_BYTES));
-    SENTRY_CUDA_TRY(cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, WideCfg<false>::SMEM_BYTES));
+    auto k1 = ffn_wide_kernel<kWideFirst, F16>;
+    const bool one = wide_second_one(d.D, d.k_c, (max_tiles - d.n_lists) * 128LL, a.ids != nullptr, d.n_lists, kWideTiles, ctx->sm_count);
+    auto k2 = one ? ffn_wide_kernel<kWideSecondOne, F16> : ffn_wide_kernel<kWideSecondTwo, F16>;
+    constexpr size_t smem1 = WideCfg<kWideFirst>::SMEM_BYTES;
+    const size_t smem2 = one ? WideCfg<kWideSecondOne>::SMEM_BYTES : WideCfg<kWideSecondTwo>::SMEM_BYTES;
+    SENTRY_CUDA_TRY(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
+    SENTRY_CUDA_TRY(cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
     for (int t0 = 0; t0 < max_tiles; t0 += turn) {
         const unsigned nt = (unsigned)(max_tiles - t0 < turn ? max_tiles - t0 : turn);
         LaunchScope ls(ctx, KS_FFN_MAIN, st, 2);
-        SENTRY_CUDA_TRY(launch_chained(k1, dim3((unsigned)wide_grid_cols(d.k_c), nt), dim3(kWThreads), (size_t)WideCfg<true>::SMEM_BYTES,
-                                       st, ah, al, m1, (const __nv_bfloat16*)a.X, hh, hl, nullptr, plan, d.n_lists, t0, (int)nt, d.D,
-                                       d.k_c, kc_pad, ctx->sm_count, a.status));
-        SENTRY_CUDA_TRY(launch_chained(k2, dim3((unsigned)wide_grid_cols(d.D), nt), dim3(kWThreads), (size_t)WideCfg<false>::SMEM_BYTES, st, ah,
-                                       al, m2, nullptr, nullptr, nullptr, (__nv_bfloat16*)a.Y, plan, d.n_lists, t0, (int)nt, d.D,
-                                       d.k_c, kc_pad, ctx->sm_count, a.status));
+        SENTRY_CUDA_TRY(launch_chained(k1, dim3(nt * (unsigned)wide_grid_cols(d.k_c)), dim3(kWThreads), smem1, st, ah, al, m1,
+                                       (const __nv_bfloat16*)a.X, hh, hl, nullptr, plan, d.n_lists, t0, (int)nt, d.D, d.k_c, kc_pad,
+                                       ctx->sm_count, a.status));
+        SENTRY_CUDA_TRY(launch_chained(k2, dim3(nt * (unsigned)wide_grid_cols(d.D)), dim3(kWThreads), smem2, st, ah, al, m2, nullptr,
+                                       nullptr, nullptr, (__nv_bfloat16*)a.Y, plan, d.n_lists, t0, (int)nt, d.D, d.k_c, kc_pad,
+                                       ctx->sm_count, a.status));
     }
     return SENTRY_OK;
 }

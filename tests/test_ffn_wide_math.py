@@ -21,8 +21,11 @@ extern "C" void gelu(const float* z, float* out, long n, int rcp_ulps, int ex2_u
         out[i] = gelu_two_part(z[i], [=](float x) { return ulps((float)(1.0 / (double)x), rcp_ulps); },
                                [=](float x) { return ulps((float)exp2((double)x), ex2_ulps); });
 }
-extern "C" int bn(int first, int R, int cols, int sm_count) { return wide_bn(first != 0, R, cols, sm_count); }
-extern "C" int bn_max(int first) { return wide_bn_max(first != 0); }
+extern "C" int bn(int form, int R, int cols, int sm_count) { return wide_bn(form, R, cols, sm_count); }
+extern "C" int bn_max(int form) { return wide_bn_max(form); }
+extern "C" int second_one(int D, int k_c, long long rows, int token_ids, int n_lists) {
+    return wide_second_one(D, k_c, rows, token_ids != 0, n_lists, 128, 148);
+}
 extern "C" int grid_cols(int cols) { return wide_grid_cols(cols); }
 extern "C" void gelu_erf(const float* z, float* out, long n) {
     for (long i = 0; i < n; ++i) out[i] = 0.5f * z[i] * (1.f + erff(z[i] * 0.70710678f));
@@ -81,24 +84,39 @@ def test_gelu_of_special_values(lib):
     assert np.isnan(g[-3:]).all()
 
 
-@pytest.mark.parametrize("first", [1, 0])
-def test_every_column_has_a_block(lib, first):
+FIRST, ONE, TWO = 0, 1, 2     # forms: GEMM 1, GEMM 2 with one and with two CTAs per SM
+WIDEST = {FIRST: 160, ONE: 192, TWO: 128}
+
+
+@pytest.mark.parametrize("form", [FIRST, ONE, TWO])
+def test_every_column_has_a_block(lib, form):
     """The launch's blocks cover the columns at whichever width the device takes, and every width is taken."""
     taken = set()
+    assert lib.bn_max(form) == WIDEST[form]
     for sm_count in (148, 132):
         for R in list(range(1, 129)):
-            for cols in range(64, 1665, 64) if first else range(64, 1025, 64):
-                bn = lib.bn(first, R, cols, sm_count)
-                assert 64 <= bn <= lib.bn_max(first) and bn % 32 == 0 and -(-cols // bn) <= lib.grid_cols(cols)
+            for cols in range(64, 1665, 64) if form == FIRST else range(64, 1025, 64):
+                bn = lib.bn(form, R, cols, sm_count)
+                assert 64 <= bn <= WIDEST[form] and bn % 32 == 0 and -(-cols // bn) <= lib.grid_cols(cols)
                 taken.add(bn)
-    assert taken == set(range(64, lib.bn_max(first) + 1, 32))
+    assert taken == set(range(64, WIDEST[form] + 1, 32))
+
+
+def test_second_form(lib):
+    one = lambda D, k_c, rows, ids=0, lists=1: bool(lib.second_one(D, k_c, ctypes.c_longlong(rows), ids, lists))
+    assert one(768, 1229, 37 * 128) and not one(768, 1229, 37 * 128 + 1)      # 148 tiles of 192 columns
+    assert not one(768, 199, 128) and one(192, 200, 10 ** 9)                  # few K blocks; one column tile a row tile
+    # several lists: two thirds of the rows of a call with masks, all of a call without
+    assert one(768, 1229, 51 * 128, 1, 7) and not one(768, 1229, 53 * 128, 1, 7)
+    assert one(768, 1229, 33 * 128, 0, 8) and not one(768, 1229, 34 * 128, 0, 8)
 
 
 def test_gpu_shapes_take_every_width(lib):
     from tests.test_gpu_ffn_wide import WIDTHS
-    first, second, last = set(), set(), set()
+    taken, last = {FIRST: set(), ONE: set(), TWO: set()}, set()
     for D, k_c, tiles in WIDTHS:
         cols = (k_c + 63) // 64 * 64
-        a, b = lib.bn(1, tiles, cols, 148), lib.bn(0, tiles, D, 148)
-        first.add(a), second.add(b), last.update((cols % a, D % b))
-    assert first == set(range(64, 161, 32)) and second == set(range(64, 193, 32)) and {32, 64, 128} <= last
+        form = ONE if lib.second_one(D, k_c, ctypes.c_longlong(tiles * 128 - 37), 0, 1) else TWO
+        a, b = lib.bn(FIRST, tiles, cols, 148), lib.bn(form, tiles, D, 148)
+        taken[FIRST].add(a), taken[form].add(b), last.update((cols % a, D % b))
+    assert taken == {form: set(range(64, WIDEST[form] + 1, 32)) for form in taken} and {32, 64, 128} <= last

@@ -91,10 +91,10 @@ def test_wide_ffn_hidden_value_beyond_the_storage_type(dtype, x, scale):
         sn.close()
 
 
-# (d_model, kept channels, row tiles): with 148 SMs every width of both GEMMs' column tiles, and last tiles of 32 to 128 columns
-# (tests/test_ffn_wide_math.py holds the list to that)
-WIDTHS = [(64, 100, 1), (192, 300, 60), (320, 129, 99), (192, 385, 60), (320, 300, 75), (192, 385, 75), (320, 385, 75),
-          (320, 300, 99), (768, 1229, 33)]
+# (d_model, kept channels, row tiles): with 148 SMs every width of the column tiles of GEMM 1 and of both forms of GEMM 2, and last
+# tiles of 32 to 128 columns (tests/test_ffn_wide_math.py holds the list to that)
+WIDTHS = [(64, 100, 1), (64, 300, 33), (192, 100, 99), (192, 300, 60), (320, 100, 40), (320, 129, 99), (320, 300, 40), (192, 300, 75),
+          (320, 300, 60), (512, 300, 45), (192, 385, 60), (320, 385, 75), (768, 1229, 33), (640, 500, 59)]
 
 
 @pytest.mark.parametrize("D,k_c,tiles", WIDTHS)
