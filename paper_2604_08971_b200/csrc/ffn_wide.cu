@@ -15,10 +15,11 @@
 // tile, and two otherwise (wide_second_one has both sides): alone from the second tile on, with its epilogues beside
 // nothing, it was slower than 128 x 128 tiles of two CTAs by up to 25 % (30 k rows of d_model 1024, 512 channels 549 -> 692 us; now 534).
 // Measured, a call with its row plan on materialised weights, before (128 x 128 tiles, erff, four epilogue warps that stored row
-// by row) and now: 3.7 k rows of d_model 768, 1229 channels in seven lists 55.1 -> 47.1 us; 524 rows, 765 channels 29.0 -> 23.8;
-// 46 rows, 967 channels 30.2 -> 24.8; 233 rows of d_model 192, 340 channels 19.0 -> 15.1; 5.6 k rows, 384 channels 21.6 -> 18.4.
-// The GELU alone, as the erff form / the tail form without the polynomial / both parts: 3.7 k rows 47.9 / 46.3 / 47.1; 30.7 k rows of
-// d_model 512, 1024 channels 191.4 / 182.7 / 187.5; 46 rows 24.9 / 24.6 / 24.8.
+// by row) and now: 3.7 k rows of d_model 768, 1229 channels in seven lists 56.7 -> 41.9 us; 524 rows, 765 channels 28.8 -> 22.8;
+// 46 rows, 967 channels 27.1 -> 23.1; 233 rows of d_model 192, 340 channels 19.5 -> 15.3; 5.6 k rows, 384 channels 21.8 -> 18.4;
+// 30.7 k rows of d_model 512, 1024 channels 185.0 -> 163.9.
+// The GELU alone, as the erff form / the tail form without the polynomial / both parts (GEMM 2 with one CTA per SM throughout): 3.7 k
+// rows 47.9 / 46.3 / 47.1; 30.7 k rows 191.4 / 182.7 / 187.5; 46 rows 24.9 / 24.6 / 24.8.
 #include <cuda.h>
 #include <math.h>
 
